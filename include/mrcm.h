@@ -379,20 +379,19 @@ int mrcm_set_root_form(mrcm_ctx* ctx, int form);
 /*
  * mrcm_autotune -- picks the launch shapes of every blocked merge level by
  * timing them on this device: CTAs per SM of the cooperative Gauss-Jordan
- * sweep (1 to 4), rows of X per CTA (32 or 64), side of an R tile (16 or
- * 32); each candidate is run `reps` times (1..100) on the context's stream
- * and the fastest kept per launch and tree height.  Every shape computes the
+ * sweep (1 to 4); each candidate is run `reps` times (1..100) on the
+ * context's stream and the fastest kept per tree height.  Every shape computes the
  * same numbers, so the basis stays valid; later builds use the choices (the
  * captured build graph is dropped).  The paper has no counterpart.  Needs a
  * built basis (MRCM_ERR_NOT_BUILT otherwise).  Errors: MRCM_ERR_INVALID_ARG,
  * MRCM_ERR_NOT_BUILT, MRCM_ERR_TIMEOUT, MRCM_ERR_CUDA.
  *
  * mrcm_tune_info -- the choices for tree height `height` (1 = the leaves'
- * parents): out[0] CTAs per SM of the sweep, out[1] X rows, out[2] R tile;
- * 0 where the built-in heuristic applies (before mrcm_autotune, and on
- * heights merged by the small-system kernel); out[0] is also 0 on heights
- * inverted one system per CTA (2g <= 128 with at least one node per two
- * SMs: a fixed rule, no launch shape to choose).
+ * parents): out[0] CTAs per SM of the sweep; 0 where the built-in heuristic
+ * applies (before mrcm_autotune, and on heights merged by the small-system
+ * kernel) and on heights inverted one system per CTA (2g <= 128 with at
+ * least one node per two SMs: a fixed rule, no launch shape to choose).
+ * out[1] and out[2] (the products X and R) are 0: they have one shape.
  */
 int mrcm_autotune(mrcm_ctx* ctx, int reps);
 int mrcm_tune_info(const mrcm_ctx* ctx, int height, int out[3]);

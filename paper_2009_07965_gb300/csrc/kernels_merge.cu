@@ -59,7 +59,7 @@
 // (merge_small_kernel).  Larger systems: the form T is written into W, then a
 // blocked Gauss-Jordan sweep (block kGJ) across many CTAs, the back
 // transform, and X and R by output tiles.
-#include "mrcm_internal.h"
+#include "merge_common.cuh"
 
 #include <algorithm>
 
@@ -70,68 +70,8 @@ constexpr int kGJ = kMergeBlock; // block size of the blocked Gauss-Jordan sweep
 constexpr int kGJTile = 32;       // output tile of the blocked update (kGJTile^2 per CTA)
 constexpr int kSmallMax = 32;     // largest 2g merged by the per-node register kernel
 constexpr int kNodeMax = 128;     // largest 2g inverted by the per-node kernel of the blocked path
-constexpr int kRTile = 32;       // R update tile
-constexpr double kTinyPivot = 1e-14;   // pivots of the scaled form are O(1)
 constexpr double kRsqrt2 = 0.70710678118654752440;   // 1 / sqrt(2), the sum / difference transform
 
-struct NodeRefs {
-    int g, g2, m, o1, m1, m2;
-    const int *gpos1, *gpos2, *opos1, *opos2;
-    const double *R1, *R2;
-};
-
-__device__ __forceinline__ NodeRefs node_refs(const DevView& v, const MergeDesc& D) {
-    NodeRefs r;
-    r.g = D.g; r.g2 = 2 * D.g; r.m = D.m; r.o1 = D.o1; r.m1 = D.m1; r.m2 = D.m2;
-    r.gpos1 = v.node_map + D.map_off;
-    r.gpos2 = r.gpos1 + D.g;
-    r.opos1 = r.gpos2 + D.g;
-    r.opos2 = r.opos1 + D.o1;
-    r.R1 = v.R + D.R1_off;
-    r.R2 = v.R + D.R2_off;
-    return r;
-}
-
-__device__ __forceinline__ double gamma_D(const DevView& v, const MergeDesc& D, int i) {
-    return v.seg_D[v.gamma_segs[D.gamma_off + i]];
-}
-
-// Entry of T at (row r, column c), r, c in [0, 2g): d block first.  sd* =
-// D^-1/2 and sq* = D^1/2 of the two gamma segments, inv_sum = 1 / sum D for
-// the regularised all-Neumann root (0 otherwise).
-__device__ __forceinline__ double t_entry(const NodeRefs& N, int r, int c, double sdi, double sdj, double sqi,
-                                          double sqj, double inv_sum) {
-    const int g = N.g;
-    const bool dr = r < g, dc = c < g;
-    const int i = dr ? r : r - g, j = dc ? c : c - g;
-    // R is stored symmetric: read it along the column of j, so that
-    // consecutive r (consecutive i) read consecutive entries
-    const double ra = N.R1[N.gpos1[j] * N.m1 + N.gpos1[i]] * sdi * sdj;
-    const double rb = N.R2[N.gpos2[j] * N.m2 + N.gpos2[i]] * sdi * sdj;
-    if (dr && dc) return 0.5 * (ra + rb) + (i == j ? 2.0 : 0.0);
-    if (!dr && !dc) return 0.5 * (ra + rb) - sqi * sqj * inv_sum;
-    return 0.5 * (rb - ra);
-}
-
-// Expected pivot sign of step k: positive on the d block, negative on s.
-__device__ __forceinline__ bool pivot_ok(double p, bool d_row) {
-    return d_row ? (p > kTinyPivot) : (p < -kTinyPivot);
-}
-// The same test on the bit pattern (integer instructions only; an FP64
-// compare takes a full FP64 instruction): sign as expected, magnitude above
-// kTinyPivot and finite.
-__device__ __forceinline__ bool pivot_ok_bits(double p, bool d_row) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(p);
-    const unsigned long long mag = b & 0x7fffffffffffffffull;
-    const unsigned long long tiny = (unsigned long long)__double_as_longlong(kTinyPivot);
-    return ((b >> 63) == (d_row ? 0ull : 1ull)) && mag > tiny && mag < 0x7ff0000000000000ull;
-}
-__device__ __forceinline__ bool pivot_ok_bits(float p, bool d_row) {
-    const unsigned int b = __float_as_uint(p);
-    const unsigned int mag = b & 0x7fffffffu;
-    const unsigned int tiny = __float_as_uint((float)kTinyPivot);
-    return ((b >> 31) == (d_row ? 0u : 1u)) && mag > tiny && mag < 0x7f800000u;
-}
 // The interface matrix being inverted in place: the W storage itself in
 // FP64, or the FP32 work array of the mixed form (same offsets).
 template <class T> __device__ __forceinline__ T* gj_work(const DevView& v);
@@ -1020,14 +960,6 @@ __global__ void __launch_bounds__(256, 4) gj_sweep_kernel(DevView v, int first, 
     __syncthreads();
     if (tid == 0 && s_bad) atomicOr(v.status, kStatusSingular);
 }
-// (row, column) of entry r of a row-packed lower triangle
-__device__ __forceinline__ void tri_rc(int r, int& a, int& b) {
-    a = (int)((sqrtf(8.0f * r + 1.0f) - 1.0f) * 0.5f);
-    while ((a + 1) * (a + 2) / 2 <= r) ++a;
-    while (a * (a + 1) / 2 > r) --a;
-    b = r - a * (a + 1) / 2;
-}
-
 // ---------------------------------------------------------------------------
 // Per-node inversion for levels of many mid-sized systems (32 < 2g <= 128,
 // at least half as many nodes as SMs): one CTA per node holds the lower triangle
@@ -1446,146 +1378,6 @@ __global__ void __launch_bounds__(256, 4) ldl_sweep_kernel(DevView v, int first,
     if (tid == 0 && s_bad) atomicOr(v.status, kStatusSingular);
 }
 
-
-// X = -W C with C = blockdiag(R^a_go, R^b_go): column j < o1 uses the first
-// g columns of W, the others the last g.  A CTA computes 64 rows x 16
-// columns; the gathered entries of C are staged in shared memory in chunks.
-constexpr int kXColsOut = 16, kXChunk = 64;
-// XROWS rows x kXColsOut columns of X per CTA: 32 unless the level has
-// CTAs in great excess (then 64, fewer staged loads per product); with few
-// long rows per node the smaller CTAs keep more SMs busy.
-// F: the arithmetic (double; float for the FP32 levels of the mixed form,
-// which read W and the children's maps in double and write X in double).
-template <int XROWS, class F>
-__global__ void __launch_bounds__(256) merge_x_kernel(DevView v, int first) {
-    constexpr int kXRows = XROWS, kQ = kXRows * kXColsOut / 256;   // outputs per thread
-    __shared__ F Cs[kXChunk][kXColsOut];
-    const MergeDesc D = v.merges[first + blockIdx.x];
-    const NodeRefs N = node_refs(v, D);
-    const int g = N.g, g2 = N.g2, m = N.m;
-    const int rt = (g2 + kXRows - 1) / kXRows;
-    const int r0 = (blockIdx.y % rt) * kXRows, j0 = (blockIdx.y / rt) * kXColsOut;
-    if (j0 >= m) return;                              // uniform per CTA
-    const double* W = v.W + D.W_off;
-    double* X = v.X + D.X_off;
-    const int tid = threadIdx.x, rl = tid % kXRows, cg = tid / kXRows;   // column groups of kQ
-    const int r = r0 + rl;
-    F acc[kQ];
-#pragma unroll
-    for (int q = 0; q < kQ; ++q) acc[q] = 0;
-    // columns of this CTA may straddle o1: treat the two halves separately
-    for (int half = 0; half < 2; ++half) {
-        const int jlo = half == 0 ? 0 : N.o1, jhi = half == 0 ? N.o1 : m;
-        if (j0 + kXColsOut <= jlo || j0 >= jhi) continue;  // uniform
-        for (int k0 = 0; k0 < g; k0 += kXChunk) {
-            const int kn = min(kXChunk, g - k0);
-            __syncthreads();
-            for (int idx = tid; idx < kXChunk * kXColsOut; idx += 256) {
-                const int kk = idx / kXColsOut, jj = idx % kXColsOut, j = j0 + jj;
-                double c = 0.0;
-                if (kk < kn && j >= jlo && j < jhi) {
-                    c = half == 0 ? N.R1[N.gpos1[k0 + kk] * N.m1 + N.opos1[j]]
-                                  : N.R2[N.gpos2[k0 + kk] * N.m2 + N.opos2[j - N.o1]];
-                }
-                Cs[kk][jj] = (F)c;
-            }
-            __syncthreads();
-            if (r < g2) {
-                const double* wcol = W + (long long)(half * g + k0) * g2 + r;
-                for (int kk = 0; kk < kn; ++kk) {
-                    const F wv = (F)wcol[(long long)kk * g2];
-#pragma unroll
-                    for (int q = 0; q < kQ; ++q) acc[q] += wv * Cs[kk][cg * kQ + q];
-                }
-            }
-        }
-    }
-    if (r < g2) {
-#pragma unroll
-        for (int q = 0; q < kQ; ++q) {
-            const int j = j0 + cg * kQ + q;
-            if (j < m) X[(long long)j * g2 + r] = (double)(-acc[q]);
-        }
-    }
-}
-
-// R = blockdiag(R_oo) + blockdiag(R_og) X on (16 TS)^2 output tiles (the
-// lower triangle, mirrored: R is symmetric): row i
-// of the tile uses the gathered row of R^a (i < o1) or R^b and the matching
-// half of X; both are staged in shared memory in chunks of kRTile.
-// staged in shared memory in chunks of kRTile.  TS = 1 (16 x 16 tiles, one
-// entry per thread) unless the level has tiles in great excess (then TS = 2,
-// 32 x 32 tiles, 2 x 2 per thread): with few nodes per height the small
-// tiles keep more SMs busy behind the long k loops.
-template <int TS, class F>
-__global__ void __launch_bounds__(256) merge_rupdate_kernel(DevView v, int first) {
-    constexpr int kTile = 16 * TS;
-    __shared__ F Cs[kTile][kRTile + 1];         // Cs[row][k]
-    __shared__ F Xs[2][kRTile][kTile + 1];      // Xs[half][k][col]
-    const MergeDesc D = v.merges[first + blockIdx.x];
-    const NodeRefs N = node_refs(v, D);
-    const int m = N.m, g = N.g, g2 = N.g2, o1 = N.o1;
-    const int tiles = (m + kTile - 1) / kTile;
-    if ((int)blockIdx.y >= tiles * (tiles + 1) / 2) return;
-    // R is symmetric: lower-triangle tiles (ti >= tj) only, mirrored on write
-    int ti = (int)((sqrtf(8.0f * blockIdx.y + 1.0f) - 1.0f) * 0.5f);
-    while ((ti + 1) * (ti + 2) / 2 <= (int)blockIdx.y) ++ti;
-    while (ti * (ti + 1) / 2 > (int)blockIdx.y) --ti;
-    const int tj = blockIdx.y - ti * (ti + 1) / 2;
-    const int i0 = ti * kTile, jt = tj * kTile;
-    const double* X = v.X + D.X_off;
-    double* Rp = v.R + D.R_off;
-    const int tid = threadIdx.x;
-    const int tr = (tid % 16) * TS, tc = (tid / 16) * TS;
-    F acc[TS][TS];
-#pragma unroll
-    for (int a = 0; a < TS; ++a)
-#pragma unroll
-        for (int b = 0; b < TS; ++b) acc[a][b] = 0;
-    for (int k0 = 0; k0 < g; k0 += kRTile) {
-        const int kn = min(kRTile, g - k0);
-        __syncthreads();
-        for (int idx = tid; idx < kTile * kRTile; idx += 256) {
-            const int rr = idx / kRTile, kk = idx % kRTile, i = i0 + rr;
-            double c = 0.0;
-            if (kk < kn && i < m)
-                c = i < o1 ? N.R1[N.opos1[i] * N.m1 + N.gpos1[k0 + kk]]
-                           : N.R2[N.opos2[i - o1] * N.m2 + N.gpos2[k0 + kk]];
-            Cs[rr][kk] = (F)c;
-        }
-        for (int idx = tid; idx < 2 * kRTile * kTile; idx += 256) {
-            const int half = idx / (kRTile * kTile), rem = idx % (kRTile * kTile);
-            const int kk = rem % kRTile, jj = rem / kRTile, j = jt + jj;
-            Xs[half][kk][jj] = (kk < kn && j < m) ? (F)X[(long long)j * g2 + half * g + k0 + kk] : (F)0;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int a = 0; a < TS; ++a) {
-            const int half = (i0 + tr + a) < o1 ? 0 : 1;
-            for (int kk = 0; kk < kRTile; ++kk) {
-                const F cv = Cs[tr + a][kk];
-#pragma unroll
-                for (int b = 0; b < TS; ++b) acc[a][b] += cv * Xs[half][kk][tc + b];
-            }
-        }
-    }
-#pragma unroll
-    for (int a = 0; a < TS; ++a) {
-        const int i = i0 + tr + a;
-        if (i >= m) continue;
-        const double* row = i < o1 ? N.R1 + N.opos1[i] * N.m1 : N.R2 + N.opos2[i - o1] * N.m2;
-#pragma unroll
-        for (int b = 0; b < TS; ++b) {
-            const int j = jt + tc + b;
-            if (j >= m || j > i) continue;
-            double val = (double)acc[a][b];
-            if (i < o1 && j < o1) val += row[N.opos1[j]];
-            if (i >= o1 && j >= o1) val += row[N.opos2[j - o1]];
-            Rp[(long long)i * m + j] = val;
-            Rp[(long long)j * m + i] = val;
-        }
-    }
-}
 
 // ---------------------------------------------------------------------------
 // Block triangular sweeps with the factor Lt of a root level, in blocks of
@@ -2077,10 +1869,10 @@ static cudaError_t launch_small(const DevView& v, int first, int count, int max_
     return go(merge_small_kernel<F, kSmallThreads>, kSmallThreads);
 }
 
-// The three launches of a blocked level, each with its tuning choice (0:
-// the heuristic below).  Every choice computes the same numbers: a tile,
-// an X block or an R tile is formed by the same thread arithmetic whichever
-// CTA shape runs it, so the tuner may pick any of them.
+// The sweep of a blocked level with its tuning choice (0: the heuristic
+// below).  Every choice computes the same numbers: a tile is formed by the
+// same thread arithmetic whichever CTA shape runs it, so the tuner may pick
+// any of them.
 template <class F>
 static cudaError_t sweep_launch(const DevView& v, int first, int count, int max_g2, double* scratch, void* barrier,
                                 int sms, int per_sm, bool factor, cudaStream_t s) {
@@ -2140,33 +1932,6 @@ static cudaError_t node_launch(const DevView& v, int first, int count, int max_g
     }
     return cudaGetLastError();
 }
-template <class F>
-static cudaError_t x_launch(const DevView& v, int first, int count, int max_g2, int max_m, int sms, int rows,
-                            cudaStream_t s) {
-    const int ct = (max_m + kXColsOut - 1) / kXColsOut;
-    const int rt64 = (max_g2 + 63) / 64;
-    if (rows == 0) rows = (long long)count * rt64 * ct >= 64LL * sms ? 64 : 32;
-    if (rows == 64) {
-        merge_x_kernel<64, F><<<dim3(count, rt64 * ct), 256, 0, s>>>(v, first);
-    } else {
-        const int rt32 = (max_g2 + 31) / 32;
-        merge_x_kernel<32, F><<<dim3(count, rt32 * ct), 256, 0, s>>>(v, first);
-    }
-    return cudaGetLastError();
-}
-template <class F>
-static cudaError_t r_launch(const DevView& v, int first, int count, int max_m, int sms, int tile, cudaStream_t s) {
-    const int rt32 = (max_m + 31) / 32;
-    if (tile == 0) tile = (long long)count * rt32 * (rt32 + 1) / 2 >= 64LL * sms ? 32 : 16;
-    if (tile == 32) {
-        merge_rupdate_kernel<2, F><<<dim3(count, rt32 * (rt32 + 1) / 2), 256, 0, s>>>(v, first);
-    } else {
-        const int rt16 = (max_m + 15) / 16;
-        merge_rupdate_kernel<1, F><<<dim3(count, rt16 * (rt16 + 1) / 2), 256, 0, s>>>(v, first);
-    }
-    return cudaGetLastError();
-}
-
 static cudaError_t device_sms(int* sms) {
     int dev = 0;
     cudaError_t e;
@@ -2213,12 +1978,12 @@ static cudaError_t launch_merge_build_t(const DevView& v, int first, int count, 
     if (max_m > 0) {
         {
             HookScope hs(hook, kPhMergeX);
-            e = x_launch<F>(v, first, count, max_g2, max_m, sms, tune.x_rows, s);
+            e = launch_merge_x(v, first, count, max_g2, max_m, sizeof(F) == sizeof(float), s);
             ++*launches;
             if (e != cudaSuccess) return e;
         }
         HookScope hs(hook, kPhMergeR);
-        e = r_launch<F>(v, first, count, max_m, sms, tune.r_tile, s);
+        e = launch_merge_r(v, first, count, max_m, sizeof(F) == sizeof(float), s);
         ++*launches;
         if (e != cudaSuccess) return e;
     }
@@ -2278,25 +2043,6 @@ static cudaError_t tune_level_t(const DevView& v, int first, int count, int max_
         }, &t);
         if (e != cudaSuccess) break;
         if (t < best) { best = t; out->sweep_per_sm = per_sm; }
-    }
-    if (e == cudaSuccess && max_m > 0) {
-        best = 1e30f;
-        for (int rows : {32, 64}) {
-            float t = 0.f;
-            e = best_time(s, reps, e0, e1, [&] { return x_launch<F>(v, first, count, max_g2, max_m, sms, rows, s); },
-                          &t);
-            if (e != cudaSuccess) break;
-            if (t < best) { best = t; out->x_rows = rows; }
-        }
-    }
-    if (e == cudaSuccess && max_m > 0) {
-        best = 1e30f;
-        for (int tile : {16, 32}) {
-            float t = 0.f;
-            e = best_time(s, reps, e0, e1, [&] { return r_launch<F>(v, first, count, max_m, sms, tile, s); }, &t);
-            if (e != cudaSuccess) break;
-            if (t < best) { best = t; out->r_tile = tile; }
-        }
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);

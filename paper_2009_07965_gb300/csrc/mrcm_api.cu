@@ -1504,8 +1504,7 @@ int mrcm_tune_info(const mrcm_ctx* c, int height, int out[3]) {
     if (!c || !out || height < 1 || height > c->P.height) return MRCM_ERR_INVALID_ARG;
     const MergeTune t = c->tune.empty() ? MergeTune{} : c->tune[height - 1];
     out[0] = t.sweep_per_sm;
-    out[1] = t.x_rows;
-    out[2] = t.r_tile;
+    out[1] = out[2] = 0;           // the products have one launch shape
     return MRCM_OK;
 }
 

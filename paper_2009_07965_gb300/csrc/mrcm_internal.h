@@ -378,12 +378,15 @@ struct PhaseHook {
 // one tree height of merges; scratch: merge_scratch_doubles(count, max_g2,
 // max_m) values; barrier: kMergeBarrierBytes of device memory (reset by the
 // call); *launches is increased by the number of kernels launched
-// Launch shapes of one blocked merge level (0 everywhere: the built-in
-// heuristic).  sweep_per_sm: CTAs per SM of the cooperative sweep (1-4);
-// x_rows: rows of X per CTA (32, 64); r_tile: side of an R tile (16, 32).
+// Launch shape of one blocked merge level (0: the built-in
+// heuristic).  sweep_per_sm: CTAs per SM of the cooperative sweep (1-4).
 struct MergeTune {
-    int sweep_per_sm = 0, x_rows = 0, r_tile = 0;
+    int sweep_per_sm = 0;
 };
+// X = -W C and the merged R of one height of blocked merges
+// (kernels_merge_mma.cu).  fp32: the mixed form's precision.
+cudaError_t launch_merge_x(const DevView& v, int first, int count, int max_g2, int max_m, bool fp32, cudaStream_t s);
+cudaError_t launch_merge_r(const DevView& v, int first, int count, int max_m, bool fp32, cudaStream_t s);
 // fp32: the mixed form's FP32 arithmetic for this level (T of the blocked
 // sweep in v.W32; W, X and R stored in double either way).  factor: a
 // blocked level without outer segments (a root level) keeps the block

@@ -1,0 +1,74 @@
+"""The merged maps of blocked merges (2g > 32), whose products X = -W C and
+R = R_oo + C^T X run as split products on the tensor cores, against the same
+merge formed on the host from the children's maps.
+
+The sizes put 2g, m and the two children's shares of m on and off the edges
+of the 64 x 32 product tiles and of the 64-entry chunks of k, odd ones among
+them.  FP64: the host's own partial-pivot LU and products are good to about
+2g u times the condition of the interface matrix (below 1e3 for these
+fields), so 2g u 1e3 < 256 * 1.1e-16 * 1e3 = 3e-11 bounds both sides'
+errors; the maps of the mixed form carry FP32 merges, 2g 2^-24 1e3 / 10 per
+merge with the same reasoning, below 1.5e-3 at 2g = 256 (the FP32 LU-free
+elimination of the quasi-definite form stays far inside it).
+"""
+import numpy as np
+import pytest
+
+import inputs
+from conftest import rel
+
+pytestmark = pytest.mark.gpu
+
+# nx, ny, seg, alpha
+GRIDS = [(96, 512, 1, 1.0),        # 2g up to 192, chunks of 64 and 32
+         (80, 330, 1, 0.5),        # truncated leaves: odd g and m
+         (333, 70, 2, 2.0),
+         (272, 272, 4, 1.0)]       # 2g = 68 and 72: one entry row past a tile
+
+
+def _merge_on_host(mr, ctx, prob, node):
+    info = mr.mrcm_node_info(ctx, node)
+    s1, s2 = (mr.mrcm_node_segments(ctx, info[c]) for c in ("c1", "c2"))
+    R1, R2 = (mr.mrcm_node_operator(ctx, info[c]) for c in ("c1", "c2"))
+    pos2 = {t: k for k, t in enumerate(s2)}
+    gam = [t for t in s1 if t in pos2]
+    g1, g2 = [k for k, t in enumerate(s1) if t in pos2], [pos2[t] for t in gam]
+    gs = set(gam)
+    o1, o2 = ([k for k, t in enumerate(s) if t not in gs] for s in (s1, s2))
+    D = []
+    for t in gam:
+        si = mr.mrcm_segment_info(ctx, t)
+        e = np.arange(si["lo"], si["lo"] + si["len"])
+        ka, kb = ((prob.K[e, si["line"] - 1], prob.K[e, si["line"]]) if si["axis"] == 0 else
+                  (prob.K[si["line"] - 1, e], prob.K[si["line"], e]))
+        D.append(np.mean(2 * ka * kb / (ka + kb)) / (2 * prob.alpha))
+    g = len(gam)
+    M = np.block([[R1[np.ix_(g1, g1)] + np.diag(D), -np.diag(D)], [-np.diag(D), R2[np.ix_(g2, g2)] + np.diag(D)]])
+    C = np.zeros((2 * g, len(o1) + len(o2)))
+    C[:g, :len(o1)] = R1[np.ix_(g1, o1)]
+    C[g:, len(o1):] = R2[np.ix_(g2, o2)]
+    R = -C.T @ np.linalg.solve(M, C)
+    R[:len(o1), :len(o1)] += R1[np.ix_(o1, o1)]
+    R[len(o1):, len(o1):] += R2[np.ix_(o2, o2)]
+    return R
+
+
+@pytest.mark.parametrize("precision,tol", [("fp64", 3e-11), ("mixed", 1.5e-3)])
+@pytest.mark.parametrize("nx,ny,seg,alpha", GRIDS)
+def test_blocked_merges_match_the_host(mrcm_lib, nx, ny, seg, alpha, precision, tol):
+    import torch
+    import paper_2009_07965_gb300 as mr
+    prob = inputs.darcy_problem(nx, ny, sigma2=2.0, corr=0.1, seed=nx, bc="left_right", seg=(seg, seg), alpha=alpha)
+    s = mr.Solver(torch.from_numpy(prob.K).cuda(), prob.Lx, prob.Ly, prob.sub, prob.seg, prob.alpha, prob.bc_type,
+                  precision=mr.binding.MRCM_FP64 if precision == "fp64" else mr.binding.MRCM_MIXED)
+    s.build_basis()
+    seen = {}
+    for v in range(mr.mrcm_query(s.ctx, "LEAVES"), mr.mrcm_query(s.ctx, "NODES")):
+        i = mr.mrcm_node_info(s.ctx, v)
+        if i["g"] > 16 and i["m"] > 0:
+            seen.setdefault((i["g"], i["m"]), v)      # one node of every shape
+    assert len(seen) >= 3
+    for shape, v in seen.items():
+        e = rel(mr.mrcm_node_operator(s.ctx, v), _merge_on_host(mr, s.ctx, prob, v))
+        assert e <= tol, (shape, e)
+    s.close()
