@@ -262,8 +262,8 @@ enum {
     MRCM_PHASE_LEAF_BUILD = 1,     /* leaf factorisation and Robin-to-flux maps     */
     MRCM_PHASE_MERGE_SMALL = 2,    /* whole merges of small interface systems       */
     MRCM_PHASE_GJ_SWEEP = 3,       /* blocked merges: Gauss-Jordan inversion of the
-                                      quasi-definite form (the cooperative sweep, or
-                                      one system per CTA for many mid-sized ones)  */
+                                      quasi-definite form (one system per CTA up to
+                                      2g = 64, a cooperative sweep above)          */
     MRCM_PHASE_MERGE_FORM = 4,     /* blocked merges: the quasi-definite form of the
                                       interface matrix and its back transform; now
                                       done inside the sweep's launch (timed as
@@ -365,9 +365,9 @@ int mrcm_set_mixed_leaves(mrcm_ctx* ctx, int fp32);
  * on it (64-row blocks, each waiting only for the blocks it depends on).
  * MRCM_ROOT_INVERSE: the explicit inverse, as at every other blocked height;
  * each solve pass then applies it as a matrix-vector product.
- * MRCM_ROOT_AUTO (the default): the factor for root systems of 2g >= 1024,
- * the inverse below (there both eliminations are bound by the same chain of
- * pivot blocks and the product is the shorter solve).
+ * MRCM_ROOT_AUTO (the default): the inverse (its products run on the tensor
+ * cores, so that it takes less time than the factor at every size measured,
+ * and its solve passes are the shorter).
  * Applies to tree heights with 2g > 32 whose nodes all lack outer segments.
  * Both forms solve the same equations (to rounding).  Invalidates the basis
  * (call mrcm_build_basis again).  Errors: MRCM_ERR_INVALID_ARG,
@@ -378,8 +378,8 @@ int mrcm_set_root_form(mrcm_ctx* ctx, int form);
 
 /*
  * mrcm_autotune -- picks the launch shapes of every blocked merge level by
- * timing them on this device: CTAs per SM of the cooperative Gauss-Jordan
- * sweep (1 to 4); each candidate is run `reps` times (1..100) on the
+ * timing them on this device: CTAs per SM of the cooperative sweeps (1 or 2
+ * of the block sweep, 1 to 4 of the FP64 sweep); each candidate is run `reps` times (1..100) on the
  * context's stream and the fastest kept per tree height.  Every shape computes the
  * same numbers, so the basis stays valid; later builds use the choices (the
  * captured build graph is dropped).  The paper has no counterpart.  Needs a
@@ -389,8 +389,8 @@ int mrcm_set_root_form(mrcm_ctx* ctx, int form);
  * mrcm_tune_info -- the choices for tree height `height` (1 = the leaves'
  * parents): out[0] CTAs per SM of the sweep; 0 where the built-in heuristic
  * applies (before mrcm_autotune, and on heights merged by the small-system
- * kernel) and on heights inverted one system per CTA (2g <= 128 with at
- * least one node per two SMs: a fixed rule, no launch shape to choose).
+ * kernel) and on heights inverted one system per CTA (2g <= 64: no launch
+ * shape to choose).
  * out[1] and out[2] (the products X and R) are 0: they have one shape.
  */
 int mrcm_autotune(mrcm_ctx* ctx, int reps);

@@ -54,11 +54,11 @@
 // tree_up_kernel / tree_down_kernel).
 //
 // Storage: W column-major per node (entry (r, c) at c*2g + r); X column-major
-// (2g x m).  Two launch shapes.  Levels with 2g <= 32: one group of 2g (padded
-// to a power of two) lanes per node does the whole merge in registers
-// (merge_small_kernel).  Larger systems: the form T is written into W, then a
-// blocked Gauss-Jordan sweep (block kGJ) across many CTAs, the back
-// transform, and X and R by output tiles.
+// (2g x m).  Levels with 2g <= 32: one CTA per node does the whole merge in
+// shared memory (merge_small_kernel).  Larger systems: the inversion, then X
+// and R by output tiles (kernels_merge_mma.cu).  The inversion runs one system
+// per CTA up to 2g = 64, as the block sweep of kernels_merge_mma.cu, or, for
+// few and small systems, as the FP64 sweep below (block kGJ).
 #include "merge_common.cuh"
 
 #include <algorithm>
@@ -69,7 +69,7 @@ namespace {
 constexpr int kGJ = kMergeBlock; // block size of the blocked Gauss-Jordan sweep
 constexpr int kGJTile = 32;       // output tile of the blocked update (kGJTile^2 per CTA)
 constexpr int kSmallMax = 32;     // largest 2g merged by the per-node register kernel
-constexpr int kNodeMax = 128;     // largest 2g inverted by the per-node kernel of the blocked path
+constexpr int kNodeMax = 64;      // largest 2g inverted one system per CTA
 constexpr double kRsqrt2 = 0.70710678118654752440;   // 1 / sqrt(2), the sum / difference transform
 
 // The interface matrix being inverted in place: the W storage itself in
@@ -472,11 +472,6 @@ __device__ void gj_first_cu_item(const DevView& v, const MergeDesc& D, int slot,
 // default: DevView::spin_limit); false on timeout (kStatusTimeout set).  Thread 0 polls with acquire loads, so what the
 // raising CTA wrote before its release (fence + atomic) is visible to the
 // whole CTA after the barrier that ends the wait.
-__device__ __forceinline__ unsigned int ld_acquire_gpu(const unsigned int* p) {
-    unsigned int v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
 __device__ bool wait_flag(const unsigned int* flag, unsigned int value, int* status, long long limit) {
     __shared__ int s_ok;
     if (threadIdx.x == 0) {
@@ -681,48 +676,6 @@ __device__ bool gj_next_diag_item(const DevView& v, const MergeDesc& D, int slot
     __syncthreads();
     if (tid == 0) atomicExch(gj_flag(sc, nmax), (unsigned int)(step + 1));
     return ok;
-}
-
-// Grid-wide barrier of a cooperative launch: a monotonic arrival counter
-// (reset before the launch); round n ends when it reaches (n + 1) * grid.
-// Data written by other CTAs before a barrier is read after it with L2-only
-// loads (__ldcg).  Every wait is bounded (`limit` polls, about a second by
-// default); a CTA that gives up sets kStatusTimeout and the caller returns.
-
-__device__ bool grid_barrier(unsigned int* counter, unsigned int& round, int* status, long long limit) {
-    __shared__ int s_ok;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int ok = 1;
-        const unsigned int target = (round + 1) * gridDim.x;
-        __threadfence();
-        atomicAdd(counter, 1u);
-        long long spins = 0;
-        while (ld_acquire_gpu(counter) < target) {
-            if (++spins > limit) {
-                ok = 0;
-                atomicOr(status, kStatusTimeout);
-                break;
-            }
-        }
-        s_ok = ok;
-    }
-    ++round;
-    __syncthreads();
-    return s_ok != 0;
-}
-
-// Next item of a dynamically distributed loop: thread 0 takes a ticket from
-// the launch's work counter (work; zeroed with the barrier counter before
-// the launch) and the CTA reads it.  The tickets of one loop run from base;
-// every CTA leaves the loop at its first ticket past the loop's items, so a
-// loop of n items consumes n + gridDim.x tickets (the next loop's base).
-__device__ __forceinline__ int grab_item(unsigned int* work, unsigned int base, int* s_item) {
-    if (threadIdx.x == 0) *s_item = (int)(atomicAdd(work, 1u) - base);
-    __syncthreads();
-    const int item = *s_item;
-    __syncthreads();
-    return item;
 }
 
 // Lower tile of rank r among the tiles of one node at a block step: the
@@ -960,98 +913,6 @@ __global__ void __launch_bounds__(256, 4) gj_sweep_kernel(DevView v, int first, 
     __syncthreads();
     if (tid == 0 && s_bad) atomicOr(v.status, kStatusSingular);
 }
-// ---------------------------------------------------------------------------
-// Per-node inversion for levels of many mid-sized systems (32 < 2g <= 128,
-// at least half as many nodes as SMs): one CTA per node holds the lower triangle
-// of T in shared memory (row-packed) and runs the Gauss-Jordan elimination
-// of merge_small on it, a rank-one step per pivot (warp 0 forms the pivot's
-// reciprocal, the pivot test and the scaled pivot row and column; every
-// thread then updates its kept entries in place), then back-forms W into
-// global memory.  No grid barriers, no global round trips of T: at these
-// sizes the cooperative blocked sweep spends most of its time on its
-// per-step synchronisation.  X and R follow with merge_x / merge_rupdate.
-// NMAX: largest 2g of the instantiation; F: the arithmetic (double, or
-// float for the mixed form's FP32 levels; W is stored in double).
-template <int NMAX>
-struct NodeTri {
-    static constexpr int kTri = NMAX * (NMAX + 1) / 2;
-    static constexpr int kPer = (kTri + 255) / 256;    // kept entries per thread
-};
-template <int NMAX, class F>
-__global__ void __launch_bounds__(256) gj_node_kernel(DevView v, int first) {
-    constexpr int kPer = NodeTri<NMAX>::kPer;
-    extern __shared__ __align__(16) unsigned char nsm_raw[];
-    F* T = reinterpret_cast<F*>(nsm_raw);                               // row-packed lower triangle
-    __shared__ F xcol[NMAX], vrow[NMAX];
-    __shared__ double scl[NMAX];                                        // D^1/2 (g), D^-1/2 (g)
-    __shared__ double red[8];
-    __shared__ int s_bad;
-    const MergeDesc D = v.merges[first + blockIdx.x];
-    const NodeRefs Nr = node_refs(v, D);
-    const int g = D.g, n = 2 * g, ntri = n * (n + 1) / 2;
-    const int tid = threadIdx.x;
-    if (tid == 0) s_bad = 0;
-    const double sum = stage_gamma_scalings(v, D, scl, red);
-    const double inv_sum = (D.pinned && sum > 0.0) ? 1.0 / sum : 0.0;
-    // the thread's entries (r, c), r >= c, packed as r << 16 | c
-    int rc[kPer];
-#pragma unroll
-    for (int e = 0; e < kPer; ++e) {
-        const int idx = tid + e * 256;
-        int r = 0, c = 0;
-        if (idx < ntri) tri_rc(idx, r, c);
-        rc[e] = (r << 16) | c;
-    }
-#pragma unroll
-    for (int e = 0; e < kPer; ++e) {
-        const int idx = tid + e * 256;
-        if (idx >= ntri) break;
-        const int r = rc[e] >> 16, c = rc[e] & 0xffff;
-        const int i = r < g ? r : r - g, j = c < g ? c : c - g;
-        T[idx] = (F)t_entry(Nr, r, c, scl[g + i], scl[g + j], scl[i], scl[j], inv_sum);
-    }
-    // Gauss-Jordan without pivoting (d rows first: positive pivots, then
-    // negative); kept entries r >= c; after step k an entry of an eliminated
-    // and a remaining index is antisymmetric: a_rk = -T(k, r) for r < k.
-    for (int k = 0; k < n; ++k) {
-        __syncthreads();
-        if (tid < 32) {
-            const F p = T[k * (k + 1) / 2 + k];
-            const F rp = rcp_nr(p);
-            for (int c = tid; c < n; c += 32) {
-                // a_kc (row k) and -a_ck (column k) from the kept triangle
-                const F akc = c == k ? (F)1 : (c < k ? T[k * (k + 1) / 2 + c] : T[c * (c + 1) / 2 + k]);
-                vrow[c] = akc * rp;
-                xcol[c] = c == k ? (F)1 : (c > k ? neg_bits(T[c * (c + 1) / 2 + k]) : T[k * (k + 1) / 2 + c]);
-            }
-            if (tid == 0 && !pivot_ok_bits(p, k < g)) s_bad = 1;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int e = 0; e < kPer; ++e) {
-            const int idx = tid + e * 256;
-            if (idx >= ntri) break;
-            const int r = rc[e] >> 16, c = rc[e] & 0xffff;
-            const F y = (r == k || c == k) ? (F)0 : T[idx];
-            T[idx] = fma(xcol[r], vrow[c], y);
-        }
-    }
-    __syncthreads();
-    if (tid == 0 && s_bad) atomicOr(v.status, kStatusSingular);
-    // W = D^-1/2 Q T^-1 Q^T D^-1/2, column-major, from the symmetric T^-1
-    double* Wg = v.W + D.W_off;
-    auto tinv = [&](int r, int c) -> F { return r >= c ? T[r * (r + 1) / 2 + c] : T[c * (c + 1) / 2 + r]; };
-    for (int idx = tid; idx < g * g; idx += 256) {
-        const int i = idx % g, j = idx / g;
-        const F zdd = tinv(i, j), zds = tinv(i, g + j), zsd = tinv(g + i, j), zss = tinv(g + i, g + j);
-        const F sc = (F)(0.5 * scl[g + i] * scl[g + j]);
-        Wg[(long long)j * n + i] = (double)((zdd - zds - zsd + zss) * sc);
-        Wg[(long long)(g + j) * n + i] = (double)((zss + zsd - zds - zdd) * sc);
-        Wg[(long long)j * n + g + i] = (double)((zss + zds - zsd - zdd) * sc);
-        Wg[(long long)(g + j) * n + g + i] = (double)((zdd + zds + zsd + zss) * sc);
-    }
-}
-
 // ---------------------------------------------------------------------------
 // Factor form of a root interface system (a level whose nodes have no outer
 // segments: only lambda_gamma = -M^-1 rbar_gamma is ever needed, no X and no
@@ -1841,7 +1702,11 @@ bool merge_level_blocked(int, int max_g2, int max_m) {
 
 size_t merge_scratch_doubles(int count, int max_g2, int max_m) {
     if (!merge_level_blocked(count, max_g2, max_m)) return 0;
-    return (size_t)count * (2 * kGJ * kGJ + 4 * (size_t)max_g2 * kGJ + 2);
+    // the cooperative sweeps' scratch (2 kGJ^2 + 4 2g kGJ + 2 values a node)
+    // or the block sweep's C, U and P, whichever form the level takes
+    const size_t coop = max_g2 > kNodeMax || max_m == 0 ? 2 * kGJ * kGJ + 4 * (size_t)max_g2 * kGJ + 2 : 0;
+    const size_t block = max_g2 > kNodeMax ? (size_t)sweep_node_scratch(max_g2) : 0;
+    return (size_t)count * std::max(coop, block);
 }
 
 // phase ids (include/mrcm.h)
@@ -1908,30 +1773,6 @@ static cudaError_t sweep_launch(const DevView& v, int first, int count, int max_
     void* args[] = {&vv, &f, &c, &n, &scr, &bar};
     return cudaLaunchCooperativeKernel(kern, dim3(grid), dim3(256), args, dyn, s);
 }
-// A blocked level of many mid-sized systems takes the per-node inversion
-// (gj_node_kernel): one CTA per node, no per-step grid barriers; from half
-// as many nodes as SMs on, a node's whole elimination on one SM is shorter
-// than the sweep's chain of block steps over the level.  A fixed rule (not
-// a tuning choice, so that tuned launch shapes keep the bits of the result).
-static bool node_level(int count, int max_g2, int sms) { return max_g2 <= kNodeMax && 2 * count >= sms; }
-template <class F>
-static cudaError_t node_launch(const DevView& v, int first, int count, int max_g2, cudaStream_t s) {
-    cudaError_t e;
-    if (max_g2 <= 64) {
-        const size_t sm = sizeof(F) * NodeTri<64>::kTri;
-        if ((e = cudaFuncSetAttribute(gj_node_kernel<64, F>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) !=
-            cudaSuccess)
-            return e;
-        gj_node_kernel<64, F><<<count, 256, sm, s>>>(v, first);
-    } else {
-        const size_t sm = sizeof(F) * NodeTri<kNodeMax>::kTri;
-        if ((e = cudaFuncSetAttribute(gj_node_kernel<kNodeMax, F>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)sm)) != cudaSuccess)
-            return e;
-        gj_node_kernel<kNodeMax, F><<<count, 256, sm, s>>>(v, first);
-    }
-    return cudaGetLastError();
-}
 static cudaError_t device_sms(int* sms) {
     int dev = 0;
     cudaError_t e;
@@ -1945,6 +1786,28 @@ static cudaError_t sweep_attributes() {
                                          kSweepSmemPad);
     if (e != cudaSuccess) return e;
     return cudaFuncSetAttribute(ldl_sweep_kernel<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSweepSmemPad);
+}
+
+// The elimination of a blocked level.  Up to 2g = 64 one system per CTA: a
+// single diagonal block of the block sweep, no barriers and no round trips
+// of T whatever the node count.  Above, the block sweep's products run at
+// about six times the FP64 pipe's rate, but its chain is the longer one (89
+// us per 64 rows against 49 for the FP64 sweep's four 16-row steps, 2g = 512
+// and one node): the FP64 sweep is the shorter where the chain sets the pace,
+// count (2g)^2 below kBlockSweepWork (measured: 1 x 512 0.40 against 0.71 ms,
+// 4 x 256 0.22 / 0.37, 16 x 128 0.20 / 0.25; 64 x 256 1.73 / 0.67, 2 x 1024
+// 3.0 / 1.5).  A rule on the level's sizes alone, so that tuned launch shapes
+// keep the bits of the result.
+constexpr long long kBlockSweepWork = 540000;
+static bool block_level(int count, int max_g2) { return (long long)count * max_g2 * max_g2 >= kBlockSweepWork; }
+template <class F>
+static cudaError_t invert_launch(const DevView& v, int first, int count, int max_g2, double* scratch, void* barrier,
+                                 int sms, int per_sm, bool factor, cudaStream_t s) {
+    constexpr bool fp32 = sizeof(F) == sizeof(float);
+    if (!factor && max_g2 <= kNodeMax) return launch_node_invert(v, first, count, fp32, s);
+    if (!factor && block_level(count, max_g2))
+        return launch_block_sweep(v, first, count, max_g2, fp32, scratch, barrier, sms, per_sm == 1 ? 1 : 2, s);
+    return sweep_launch<F>(v, first, count, max_g2, scratch, barrier, sms, per_sm, factor, s);
 }
 
 template <class F>
@@ -1968,10 +1831,7 @@ static cudaError_t launch_merge_build_t(const DevView& v, int first, int count, 
     factor = factor && max_m == 0;
     {
         HookScope hs(hook, factor ? kPhRootFactor : kPhGjSweep);
-        if (!factor && node_level(count, max_g2, sms))
-            e = node_launch<F>(v, first, count, max_g2, s);
-        else
-            e = sweep_launch<F>(v, first, count, max_g2, scratch, barrier, sms, tune.sweep_per_sm, factor, s);
+        e = invert_launch<F>(v, first, count, max_g2, scratch, barrier, sms, tune.sweep_per_sm, factor, s);
         ++*launches;
         if (e != cudaSuccess) return e;
     }
@@ -2036,10 +1896,11 @@ static cudaError_t tune_level_t(const DevView& v, int first, int count, int max_
     }
     float best = 1e30f;
     for (int per_sm : {1, 2, 3, 4}) {
-        if (!factor && node_level(count, max_g2, sms)) break;        // the per-node kernel: no shape to pick
+        if (!factor && max_g2 <= kNodeMax) break;                         // one system per CTA: no shape to pick
+        if (!factor && block_level(count, max_g2) && per_sm > 2) break;   // two CTAs fit an SM
         float t = 0.f;
         e = best_time(s, reps, e0, e1, [&] {
-            return sweep_launch<F>(v, first, count, max_g2, scratch, barrier, sms, per_sm, factor, s);
+            return invert_launch<F>(v, first, count, max_g2, scratch, barrier, sms, per_sm, factor, s);
         }, &t);
         if (e != cudaSuccess) break;
         if (t < best) { best = t; out->sweep_per_sm = per_sm; }

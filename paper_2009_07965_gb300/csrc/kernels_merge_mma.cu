@@ -2,8 +2,11 @@
 // products of split_gemm.cuh): X = -W C and the merged map R = R_oo + C^T X
 // of every node of a tree height (Eqs. new_bfs.1-2; kernels_merge.cu has the
 // derivation and the launches around these).
+#include "block_invert.cuh"
 #include "merge_common.cuh"
 #include "split_gemm.cuh"
+
+#include <algorithm>
 
 namespace mrcm {
 namespace {
@@ -112,7 +115,543 @@ cudaError_t r_launch(const DevView& v, int first, int count, int max_m, cudaStre
     return cudaGetLastError();
 }
 
+// ---------------------------------------------------------------------------
+// Inversion of the interface systems in blocks of kSweepB rows: the symmetric
+// sweep operator of block_invert.cuh, a block K of 64 rows at a time, over
+// the quasi-definite T (kernels_merge.cu).  With P = A_KK^-1 and C_x = A_xK,
+//     A_KK <- -P,  A_xK <- U_x = C_x P,  A_xy <- A_xy - C_x U_y^T,
+// and -T^-1 is left in the end.  Only the lower triangle is kept (row-major,
+// in the W storage, or the FP32 work array of a mixed level).
+//
+// One cooperative launch per tree height, two CTAs of four warps per SM: T of
+// every node, the inverse of the first diagonal blocks; per step the panel
+// items (U = C P; C and U into scratch, 64 entries a row), then the update
+// items, 64 x 32 tiles of one chunk of k each, behind one item per node that
+// updates the next diagonal block and inverts it meanwhile, so that the
+// sequential chain of pivots runs beside the other tiles' products; then W.
+// A grid barrier between the phases (two per 64 rows); with more items than
+// CTAs the update items are handed out by ticket, the next one taken while
+// the current one runs.
+//
+// Measured (FP64, one GB300) against the FP64-pipe sweep of kernels_merge.cu:
+// 256 nodes of 2g = 512 63.7 -> 7.3 ms, 512 x 256 19.1 -> 3.3, 2 x 1024 3.0 ->
+// 1.6, 1 x 2048 (the root of 4096^2, a factorisation before) 4.2 -> 3.4; FP32
+// levels 1024 x 512 120 -> 18.8.  Bound by the latency of the chain for few
+// nodes (about 90 us per 64 rows, half of it the 64 pivots) and by cutting
+// digits and by the loads of a tile for many.
+constexpr int kSweepB = kInvert;
+static_assert(kSweepB == kChunkK && kSweepB == kTileM && kSweepB == 2 * kTileN, "one chunk, one tile row per block");
+
+template <class T> __device__ __forceinline__ T* sweep_matrix(const DevView& v);
+template <> __device__ __forceinline__ double* sweep_matrix<double>(const DevView& v) { return v.W; }
+template <> __device__ __forceinline__ float* sweep_matrix<float>(const DevView& v) { return v.W32; }
+
+// Scratch of a node: C and U of the current block (nmax rows of kSweepB) and
+// two P (by step parity).
+template <class T>
+struct SweepScratch {
+    T *C, *U, *P;
+    __device__ __forceinline__ SweepScratch(T* scratch, int slot, int nmax) {
+        C = scratch + (long long)slot * sweep_node_scratch(nmax);
+        U = C + (long long)nmax * kSweepB;
+        P = U + (long long)nmax * kSweepB;
+    }
+    __device__ __forceinline__ T* p(int step) const { return P + (step & 1) * kSweepB * kSweepB; }
+};
+
+// 1 / sum D of a pinned node's gamma segments (the regularised all-Neumann
+// root), 0 otherwise; red: 4 doubles.
+__device__ double pinned_inv_sum(const DevView& v, const MergeDesc& D, double* red) {
+    if (!D.pinned) return 0.0;                                          // uniform per CTA
+    double part = 0.0;
+    for (int i = threadIdx.x; i < D.g; i += kGemmThreads) part += gamma_D(v, D, i);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = part;
+    __syncthreads();
+    const double sum = (red[0] + red[1]) + (red[2] + red[3]);
+    return sum > 0.0 ? 1.0 / sum : 0.0;
+}
+
+// Rows [r0, r0 + 16) of T's lower triangle.
+template <class T>
+__device__ void form_rows(const DevView& v, const MergeDesc& D, int r0, double* red) {
+    const NodeRefs N = node_refs(v, D);
+    const int g = N.g, n = N.g2;
+    const double* sq = v.gam_sq + D.gamma_off;
+    const double* sd = v.gam_sd + D.gamma_off;
+    const double inv_sum = pinned_inv_sum(v, D, red);
+    T* A = sweep_matrix<T>(v) + D.W_off;
+    for (int r = r0; r < min(r0 + 16, n); ++r) {
+        const int i = r < g ? r : r - g;
+        for (int c = threadIdx.x; c <= r; c += kGemmThreads) {
+            const int j = c < g ? c : c - g;
+            A[(long long)r * n + c] = (T)t_entry(N, c, r, sd[j], sd[i], sq[j], sq[i], inv_sum);
+        }
+    }
+}
+
+// The inverse left in S (zero outside nb) as a full kSweepB x kSweepB matrix.
+template <class T>
+__device__ void store_inverse(const InvertSmem<T>& S, int nb, T* P) {
+    for (int idx = threadIdx.x; idx < kSweepB * kSweepB; idx += kGemmThreads) {
+        const int r = idx / kSweepB, c = idx % kSweepB, a = max(r, c), b = min(r, c);
+        P[idx] = a < nb ? neg_bits(S.A[a][b]) : (T)0;
+    }
+}
+template <class T>
+__device__ void invert_checked(const DevView& v, InvertSmem<T>& S, int nb, int d_rows) {
+    if (!invert_block(S, nb, [&](T p, int k) { return pivot_ok_bits(p, k < d_rows); }) && threadIdx.x == 0)
+        atomicOr(v.status, kStatusSingular);
+}
+
+// P of block 0.
+template <class T>
+__device__ void first_inverse(const DevView& v, const MergeDesc& D, const SweepScratch<T>& sc, InvertSmem<T>& S) {
+    const int n = 2 * D.g, nb = min(kSweepB, n);
+    const T* A = sweep_matrix<T>(v) + D.W_off;
+    __syncthreads();
+    for (int idx = threadIdx.x; idx < kSweepB * kSweepB; idx += kGemmThreads) {
+        const int r = idx / kSweepB, c = idx % kSweepB;
+        S.A[r][c] = r < nb && c <= r ? A[(long long)r * n + c] : (T)0;
+    }
+    invert_checked(v, S, nb, D.g);
+    store_inverse(S, nb, sc.p(0));
+}
+
+// U_x = C_x P for 64 rows x outside K and half of K's columns; C and U to
+// scratch.
+template <class T>
+__device__ void panel_item(const DevView& v, const MergeDesc& D, const SweepScratch<T>& sc, int step, int xt, int h0,
+                           unsigned char* smem_raw) {
+    constexpr int S = Slices<T>::S;
+    SplitSmem<S>& sm = *reinterpret_cast<SplitSmem<S>*>(smem_raw);
+    const int n = 2 * D.g, k0 = step * kSweepB, nb = min(kSweepB, n - k0), x0 = xt * kSweepB, tid = threadIdx.x;
+    if (nb <= 0 || x0 >= n || xt == step || h0 >= nb) return;           // uniform per CTA
+    const T* A = sweep_matrix<T>(v) + D.W_off;
+    T* C = sc.C + (long long)x0 * kSweepB;
+    const int nx = min(kSweepB, n - x0);
+    __syncthreads();
+    if (xt < step) {
+        // rows above K: C_x = A_Kx^T, transposed through shared memory (both
+        // halves' items write the same values)
+        T (*tile)[kSweepB + 1] = reinterpret_cast<T (*)[kSweepB + 1]>(smem_raw);
+        for (int idx = tid; idx < nb * kSweepB; idx += kGemmThreads)
+            tile[idx / kSweepB][idx % kSweepB] = A[(long long)(k0 + idx / kSweepB) * n + x0 + idx % kSweepB];
+        __syncthreads();
+        for (int idx = tid; idx < kSweepB * kSweepB; idx += kGemmThreads) {
+            const int x = idx / kSweepB, k = idx % kSweepB;
+            if (k < nb) C[idx] = tile[k][x];
+        }
+        __syncthreads();
+    } else if (h0 == 0) {
+        for (int idx = tid; idx < nx * kSweepB; idx += kGemmThreads) {
+            const int x = idx / kSweepB, k = idx % kSweepB;
+            if (k < nb) C[idx] = A[(long long)(x0 + x) * n + k0 + k];
+        }
+    }
+    const T* rows = xt < step ? C : A + (long long)x0 * n + k0;
+    const long long ld = xt < step ? kSweepB : n;
+    const T* P = sc.p(step);
+    typename SplitAcc<S>::T sum[2][2][4];
+    split_product<S, T, false, false>(
+        sm, nb, nullptr, [&](int x) { return x < nx ? rows + x * ld : nullptr; },
+        [&](int c) { return h0 + c < nb ? P + (h0 + c) * kSweepB : nullptr; }, sum);
+    T* U = sc.U + (long long)x0 * kSweepB;
+    const int lane = tid & 31, warp = tid >> 5;
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int x = (warp >> 1) * 32 + 16 * mt + (lane >> 2) + 8 * (q >> 1);
+                const int c = h0 + (warp & 1) * 16 + 8 * nt + 2 * (lane & 3) + (q & 1);
+                if (x < nx && c < nb) U[x * kSweepB + c] = (T)sum[mt][nt][q];
+            }
+}
+
+// Two adjacent entries in one load (rows of the scratch are aligned to it).
+__device__ __forceinline__ void load_pair(double& a, double& b, const double* p) {
+    const double2 x = *reinterpret_cast<const double2*>(p);
+    a = x.x;
+    b = x.y;
+}
+__device__ __forceinline__ void load_pair(float& a, float& b, const float* p) {
+    const float2 x = *reinterpret_cast<const float2*>(p);
+    a = x.x;
+    b = x.y;
+}
+// This lane's entries of a scratch row (nb of its 64 entries are set; nb is
+// even).
+template <class T>
+__device__ __forceinline__ void load_scratch_row(T (&v)[2 * kChunkK / 8], const T* p, bool on, int nb) {
+    const int q = threadIdx.x & 3;
+#pragma unroll
+    for (int i = 0; i < kChunkK / 8; ++i) {
+        const int k = 8 * i + 2 * q;
+        v[2 * i] = v[2 * i + 1] = (T)0;
+        if (on && k < nb) load_pair(v[2 * i], v[2 * i + 1], p + k);
+    }
+}
+
+// The update of half tiles [h0, h1) (32 columns each) of the 64 rows of tile
+// row ti: the digits of C are cut once for the strip, and a half tile's U
+// and old entries are loaded while the products of the one before run.
+template <class T>
+__device__ void update_strip(const DevView& v, const MergeDesc& D, const SweepScratch<T>& sc, int step, int ti, int h0,
+                             int h1, unsigned char* smem_raw) {
+    constexpr int S = Slices<T>::S;
+    SplitSmem<S>& sm = *reinterpret_cast<SplitSmem<S>*>(smem_raw);
+    const int n = 2 * D.g, k0 = step * kSweepB, nb = min(kSweepB, n - k0), r0 = ti * kSweepB;
+    if (nb <= 0 || r0 >= n) return;                                     // uniform per CTA
+    T* A = sweep_matrix<T>(v) + D.W_off;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, row = tid >> 2;
+    const int wr = (warp >> 1) * 32 + (lane >> 2), wc = (warp & 1) * 16 + 2 * (lane & 3);
+    h1 = min(h1, (n + kTileN - 1) / kTileN);
+    // a half tile formed by a product: not in the swept block's rows or
+    // columns, not the next diagonal block (its own item, not read again)
+    auto product = [&](int h) {
+        const int tj = h >> 1;
+        return h < h1 && ti != step && tj != step && !(ti == step + 1 && tj == ti);
+    };
+    auto next_product = [&](int h) {
+        while (h < h1 && !product(h)) ++h;
+        return h;
+    };
+    const T* P = sc.p(step);
+    for (int h = h0; h < h1; ++h) {
+        const int tj = h >> 1, c0 = h * kTileN;
+        if (ti != step && tj != step) continue;
+        // the swept block's rows and columns, from P and U
+        for (int idx = tid; idx < kTileM * kTileN; idx += kGemmThreads) {
+            const int r = r0 + idx / kTileN, c = c0 + idx % kTileN;
+            if (r >= n || c > r) continue;
+            T x;
+            if (ti == tj) x = neg_bits(P[(r - k0) * kSweepB + c - k0]);
+            else if (tj == step) x = sc.U[(long long)r * kSweepB + c - k0];
+            else x = sc.U[(long long)c * kSweepB + r - k0];
+            A[(long long)r * n + c] = x;
+        }
+    }
+    int h = next_product(h0);
+    if (h >= h1) return;
+    T vb[2 * kChunkK / 8];
+    load_scratch_row(vb, sc.U + (long long)(h * kTileN + row) * kSweepB, h * kTileN + row < n, nb);
+    {
+        T va[2][2 * kChunkK / 8];
+#pragma unroll
+        for (int p = 0; p < 2; ++p)
+            load_scratch_row(va[p], sc.C + (long long)(r0 + row + 32 * p) * kSweepB, r0 + row + 32 * p < n, nb);
+        __syncthreads();                                                // the CTA's previous item is done with sm
+#pragma unroll
+        for (int p = 0; p < 2; ++p) stage_row<S>(sm.A, sm.ea, row + 32 * p, nb, va[p]);
+    }
+    for (;;) {
+        const int c0 = h * kTileN;
+        stage_row<S>(sm.B, sm.eb, row, nb, vb);
+        __syncthreads();
+        const int hn = next_product(h + 1);
+        if (hn < h1) load_scratch_row(vb, sc.U + (long long)(hn * kTileN + row) * kSweepB, hn * kTileN + row < n, nb);
+        T old[2][2][4];
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+            for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int r = r0 + wr + 16 * mt + 8 * (q >> 1), c = c0 + wc + 8 * nt + (q & 1);
+                    old[mt][nt][q] = r < n && c <= r ? A[(long long)r * n + c] : (T)0;
+                }
+        float acc[S][2][2][4];
+        chunk_mma<S>(sm, nb, acc);
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+            for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    float l[S];
+#pragma unroll
+                    for (int i = 0; i < S; ++i) l[i] = acc[i][mt][nt][q];
+                    const T x = (T)combine_levels(l, sm.ea[wr + 16 * mt + 8 * (q >> 1)], sm.eb[wc + 8 * nt + (q & 1)]);
+                    const int r = r0 + wr + 16 * mt + 8 * (q >> 1), c = c0 + wc + 8 * nt + (q & 1);
+                    if (r < n && c <= r) A[(long long)r * n + c] = old[mt][nt][q] - x;
+                }
+        if (hn >= h1) return;
+        h = hn;
+        __syncthreads();
+    }
+}
+
+// The next diagonal block: its update and its inverse, P of step + 1.
+template <class T>
+__device__ void next_inverse(const DevView& v, const MergeDesc& D, const SweepScratch<T>& sc, int step,
+                             unsigned char* smem_raw) {
+    constexpr int S = Slices<T>::S;
+    SplitSmem<S>& sm = *reinterpret_cast<SplitSmem<S>*>(smem_raw);
+    InvertSmem<T>& I = *reinterpret_cast<InvertSmem<T>*>(smem_raw);
+    static_assert(sizeof(InvertSmem<T>) <= sizeof(SplitSmem<S>), "the inversion reuses the digits' storage");
+    const int n = 2 * D.g, k1 = (step + 1) * kSweepB;
+    if (k1 >= n) return;                                                // uniform per CTA
+    const int nb1 = min(kSweepB, n - k1), tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const T* A = sweep_matrix<T>(v) + D.W_off;
+    const int wr = (warp >> 1) * 32 + (lane >> 2), wc = (warp & 1) * 16 + 2 * (lane & 3);
+    typename SplitAcc<S>::T sum[2][2][2][4];
+    for (int h = 0; h < 2; ++h) {
+        __syncthreads();
+        split_product<S, T, false, false>(
+            sm, kSweepB, nullptr, [&](int x) { return x < nb1 ? sc.C + (long long)(k1 + x) * kSweepB : nullptr; },
+            [&](int c) { return h * kTileN + c < nb1 ? sc.U + (long long)(k1 + h * kTileN + c) * kSweepB : nullptr; },
+            sum[h]);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+            for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int r = wr + 16 * mt + 8 * (q >> 1), c = h * kTileN + wc + 8 * nt + (q & 1);
+                    I.A[r][c] = r < nb1 && c <= r ? A[(long long)(k1 + r) * n + k1 + c] - (T)sum[h][mt][nt][q] : (T)0;
+                }
+    invert_checked(v, I, nb1, D.g - k1);
+    store_inverse(I, nb1, sc.p(step + 1));
+}
+
+// W = D^-1/2 Q T^-1 Q^T D^-1/2 (both triangles) from the entries dd, sd (s_i,
+// d_j), ds (d_i, s_j), ss of -T^-1: the entries (a_i, a_j), (b_i, b_j), (a_i,
+// b_j), (b_i, a_j) of W.
+template <class T>
+__device__ __forceinline__ void back_entries(T dd, T sd, T ds, T ss, T sc, double (&w)[4]) {
+    const T sum = dd + ss, cross = ds + sd, dif = ss - dd, skew = sd - ds;
+    w[0] = (double)((cross - sum) * sc);
+    w[1] = (double)(neg_bits(sum + cross) * sc);
+    w[2] = (double)(neg_bits(dif + skew) * sc);
+    w[3] = (double)((skew - dif) * sc);
+}
+
+// ... by 32 x 32 tiles of (i, j), i, j < g, i's tile at or below j's; a tile
+// pair is read and written by its own item only (in FP64 the two matrices
+// share their storage).
+constexpr int kBackTile = 32;
+template <class T>
+struct BackSmem {
+    T z[4][kBackTile][kBackTile + 1];          // dd, sd, ds, ss
+    double w[2][kBackTile][kBackTile + 1];
+};
+template <class T>
+__device__ void back_item(const DevView& v, const MergeDesc& D, int ti, int tj, BackSmem<T>& S) {
+    const int g = D.g, n = 2 * g, tid = threadIdx.x;
+    const int i0 = ti * kBackTile, j0 = tj * kBackTile;
+    if (i0 >= g) return;                                                // uniform per CTA
+    const T* A = sweep_matrix<T>(v) + D.W_off;
+    double* W = v.W + D.W_off;
+    const double* sd = v.gam_sd + D.gamma_off;
+    auto at = [&](int r, int c) -> T { return r >= c ? A[(long long)r * n + c] : A[(long long)c * n + r]; };
+    __syncthreads();
+    for (int idx = tid; idx < kBackTile * kBackTile; idx += kGemmThreads) {
+        const int a = idx / kBackTile, b = idx % kBackTile;             // b along the rows of A
+        const int i = i0 + a, j = j0 + b;
+        if (i < g && j < g) {
+            S.z[0][a][b] = at(i, j);
+            S.z[1][a][b] = A[(long long)(g + i) * n + j];
+            S.z[3][a][b] = at(g + i, g + j);
+        }
+        const int jj = j0 + a, ii = i0 + b;
+        if (ii < g && jj < g) S.z[2][b][a] = A[(long long)(g + jj) * n + ii];
+    }
+    __syncthreads();
+    // blocks (a_i, a_j) and (b_i, b_j), then (a_i, b_j) and (b_i, a_j); each
+    // written with its mirror
+    for (int pass = 0; pass < 2; ++pass) {
+        for (int idx = tid; idx < kBackTile * kBackTile; idx += kGemmThreads) {
+            const int a = idx / kBackTile, b = idx % kBackTile, i = i0 + a, j = j0 + b;
+            if (i >= g || j >= g) continue;
+            double w[4];
+            back_entries(S.z[0][a][b], S.z[1][a][b], S.z[2][a][b], S.z[3][a][b], (T)(0.5 * sd[i] * sd[j]), w);
+            S.w[0][a][b] = w[2 * pass];
+            S.w[1][a][b] = w[2 * pass + 1];
+        }
+        __syncthreads();
+        for (int idx = tid; idx < kBackTile * kBackTile; idx += kGemmThreads) {
+            const int a = idx / kBackTile, b = idx % kBackTile;
+            {
+                const int i = i0 + a, j = j0 + b;
+                if (i < g && j < g) {
+                    W[(long long)i * n + j + (pass ? g : 0)] = S.w[0][a][b];
+                    W[(long long)(g + i) * n + j + (pass ? 0 : g)] = S.w[1][a][b];
+                }
+            }
+            if (ti != tj) {
+                const int i = i0 + b, j = j0 + a;
+                if (i < g && j < g) {
+                    W[(long long)(j + (pass ? g : 0)) * n + i] = S.w[0][b][a];
+                    W[(long long)(j + (pass ? 0 : g)) * n + g + i] = S.w[1][b][a];
+                }
+            }
+        }
+        __syncthreads();
+    }
+}
+
+template <class T>
+constexpr size_t sweep_smem() {
+    return std::max({sizeof(SplitSmem<Slices<T>::S>), sizeof(InvertSmem<T>), sizeof(BackSmem<T>)});
+}
+
+template <class T>
+__global__ void __launch_bounds__(kGemmThreads, 2) block_sweep_kernel(DevView v, int first, int count, int nmax,
+                                                                      T* scratch, unsigned int* counter) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ double red[4];
+    __shared__ int s_item;
+    unsigned int* work = counter + 1;                       // ticket counter of the update items
+    unsigned int wbase = 0, round = 0;
+    const int nt = (nmax + kSweepB - 1) / kSweepB, gt = (nmax / 2 + kBackTile - 1) / kBackTile;
+    const int grid = gridDim.x;
+    auto node = [&](int q) -> const MergeDesc& { return v.merges[first + q]; };
+    auto scr = [&](int q) { return SweepScratch<T>(scratch, q, nmax); };
+    {
+        const int runs = (nmax + 15) / 16;
+        for (long long item = blockIdx.x; item < (long long)count * runs; item += grid) {
+            const int q = (int)(item / runs), r0 = (int)(item % runs) * 16;
+            if (r0 < 2 * node(q).g) form_rows<T>(v, node(q), r0, red);
+        }
+    }
+    if (!grid_barrier(counter, round, v.status, v.spin_limit)) return;
+    for (int q = blockIdx.x; q < count; q += grid)
+        first_inverse<T>(v, node(q), scr(q), *reinterpret_cast<InvertSmem<T>*>(smem_raw));
+    if (!grid_barrier(counter, round, v.status, v.spin_limit)) return;
+    for (int step = 0; step < nt; ++step) {
+        if (nt > 1) {
+            for (int item = blockIdx.x; item < count * 2 * nt; item += grid) {
+                const int q = item % count, r = item / count;
+                panel_item<T>(v, node(q), scr(q), step, r >> 1, (r & 1) * kTileN, smem_raw);
+            }
+            if (!grid_barrier(counter, round, v.status, v.spin_limit)) return;
+        }
+        // the next diagonal blocks, then strips of half tiles, a few per CTA
+        const int halves = count * nt * (nt + 1);
+        const int len = max(1, min(2 * nt, halves / (3 * grid)));
+        int pieces = 0;
+        for (int t = 0; t < nt; ++t) pieces += (2 * t + 1 + len) / len;
+        const int nitems = count * (1 + pieces);
+        const bool dyn = nitems > grid;
+        int item = dyn ? grab_item(work, wbase, &s_item) : (int)blockIdx.x;
+        while (item < nitems) {
+            // the next ticket is taken while this item runs
+            if (dyn && threadIdx.x == 0) s_item = (int)(atomicAdd(work, 1u) - wbase);
+            const int q = item % count;
+            int r = item / count - 1;
+            if (r < 0) {
+                next_inverse<T>(v, node(q), scr(q), step, smem_raw);
+            } else {
+                // long rows first
+                int ti = nt - 1;
+                for (; r >= (2 * ti + 1 + len) / len; --ti) r -= (2 * ti + 1 + len) / len;
+                update_strip<T>(v, node(q), scr(q), step, ti, r * len, min((r + 1) * len, 2 * ti + 2), smem_raw);
+            }
+            __syncthreads();
+            item = dyn ? s_item : nitems;
+            __syncthreads();
+        }
+        if (dyn) wbase += (unsigned int)nitems + grid;
+        if (!grid_barrier(counter, round, v.status, v.spin_limit)) return;
+    }
+    for (int item = blockIdx.x; item < count * (gt * (gt + 1) / 2); item += grid) {
+        int ti, tj;
+        tri_rc(item / count, ti, tj);
+        back_item<T>(v, node(item % count), ti, tj, *reinterpret_cast<BackSmem<T>*>(smem_raw));
+    }
+}
+
+// One CTA per node for levels of many small systems (2g <= 64): T, its
+// inverse and W without leaving shared memory.
+template <class T>
+__global__ void __launch_bounds__(kGemmThreads) node_invert_kernel(DevView v, int first) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ double red[4];
+    InvertSmem<T>& S = *reinterpret_cast<InvertSmem<T>*>(smem_raw);
+    const MergeDesc D = v.merges[first + blockIdx.x];
+    const NodeRefs N = node_refs(v, D);
+    const int g = N.g, n = N.g2;
+    const double* sq = v.gam_sq + D.gamma_off;
+    const double* sd = v.gam_sd + D.gamma_off;
+    const double inv_sum = pinned_inv_sum(v, D, red);
+    for (int idx = threadIdx.x; idx < kInvert * kInvert; idx += kGemmThreads) {
+        const int r = idx / kInvert, c = idx % kInvert;
+        const int i = r < g ? r : r - g, j = c < g ? c : c - g;
+        S.A[r][c] = r < n && c <= r ? (T)t_entry(N, c, r, sd[j], sd[i], sq[j], sq[i], inv_sum) : (T)0;
+    }
+    invert_checked(v, S, n, g);
+    double* W = v.W + D.W_off;
+    auto at = [&](int r, int c) -> T { return r >= c ? S.A[r][c] : S.A[c][r]; };
+    for (int idx = threadIdx.x; idx < g * g; idx += kGemmThreads) {
+        const int i = idx / g, j = idx % g;
+        double w[4];
+        back_entries(at(i, j), S.A[g + i][j], S.A[g + j][i], at(g + i, g + j), (T)(0.5 * sd[i] * sd[j]), w);
+        W[i * n + j] = w[0];
+        W[(g + i) * n + g + j] = w[1];
+        W[i * n + g + j] = w[2];
+        W[(g + i) * n + j] = w[3];
+    }
+}
+
+template <class T>
+cudaError_t block_sweep(const DevView& v, int first, int count, int nmax, T* scratch, void* barrier, int sms,
+                        int per_sm, cudaStream_t s) {
+    constexpr int bytes = (int)sweep_smem<T>();
+    auto* kern = block_sweep_kernel<T>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e != cudaSuccess) return e;
+    const int nt = (nmax + kSweepB - 1) / kSweepB;
+    const long long items = std::max<long long>((long long)count * (1 + nt * (nt + 1)), (long long)count * ((nmax + 15) / 16));
+    int fit = 0;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, kern, kGemmThreads, bytes)) != cudaSuccess) return e;
+    const int grid = (int)std::min<long long>(items, (long long)sms * std::max(1, std::min(per_sm, fit)));
+    // the grid barrier's arrival counter and the ticket counter
+    if ((e = cudaMemsetAsync(barrier, 0, 2 * sizeof(unsigned int), s)) != cudaSuccess) return e;
+    unsigned int* bar = reinterpret_cast<unsigned int*>(barrier);
+    DevView vv = v;
+    void* args[] = {&vv, &first, &count, &nmax, &scratch, &bar};
+    return cudaLaunchCooperativeKernel((const void*)kern, dim3(grid), dim3(kGemmThreads), args, bytes, s);
+}
+template <class T>
+cudaError_t node_invert(const DevView& v, int first, int count, cudaStream_t s) {
+    constexpr int bytes = (int)sizeof(InvertSmem<T>);
+    cudaError_t e = cudaFuncSetAttribute(node_invert_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e != cudaSuccess) return e;
+    node_invert_kernel<T><<<count, kGemmThreads, bytes, s>>>(v, first);
+    return cudaGetLastError();
+}
+
+// D^1/2 and D^-1/2 of every gamma segment of the tree.
+__global__ void gamma_scale_kernel(DevView v, int n) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const double sq = sqrt(v.seg_D[v.gamma_segs[i]]);
+    v.gam_sq[i] = sq;
+    v.gam_sd[i] = 1.0 / sq;
+}
+
 }  // namespace
+
+cudaError_t launch_gamma_scale(const DevView& v, int n, cudaStream_t s) {
+    if (n > 0) gamma_scale_kernel<<<(n + 127) / 128, 128, 0, s>>>(v, n);
+    return cudaGetLastError();
+}
+cudaError_t launch_block_sweep(const DevView& v, int first, int count, int max_g2, bool fp32, double* scratch,
+                               void* barrier, int sms, int per_sm, cudaStream_t s) {
+    return fp32 ? block_sweep<float>(v, first, count, max_g2, reinterpret_cast<float*>(scratch), barrier, sms, per_sm, s)
+                : block_sweep<double>(v, first, count, max_g2, scratch, barrier, sms, per_sm, s);
+}
+cudaError_t launch_node_invert(const DevView& v, int first, int count, bool fp32, cudaStream_t s) {
+    return fp32 ? node_invert<float>(v, first, count, s) : node_invert<double>(v, first, count, s);
+}
 
 cudaError_t launch_merge_x(const DevView& v, int first, int count, int max_g2, int max_m, bool fp32, cudaStream_t s) {
     return fp32 ? x_launch<4>(v, first, count, max_g2, max_m, s) : x_launch<7>(v, first, count, max_g2, max_m, s);

@@ -71,5 +71,53 @@ __device__ __forceinline__ void tri_rc(int r, int& a, int& b) {
     b = r - a * (a + 1) / 2;
 }
 
+// A load that acquires what was released before the value was written.
+__device__ __forceinline__ unsigned int ld_acquire_gpu(const unsigned int* p) {
+    unsigned int v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+// Grid-wide barrier of a cooperative launch: a monotonic arrival counter
+// (reset before the launch); round n ends when it reaches (n + 1) * grid.
+// Data written by other CTAs before a barrier is read after it with L2-only
+// loads (__ldcg).  Every wait is bounded (`limit` polls, about a second by
+// default); a CTA that gives up sets kStatusTimeout and the caller returns.
+
+__device__ bool grid_barrier(unsigned int* counter, unsigned int& round, int* status, long long limit) {
+    __shared__ int s_ok;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int ok = 1;
+        const unsigned int target = (round + 1) * gridDim.x;
+        __threadfence();
+        atomicAdd(counter, 1u);
+        long long spins = 0;
+        while (ld_acquire_gpu(counter) < target) {
+            if (++spins > limit) {
+                ok = 0;
+                atomicOr(status, kStatusTimeout);
+                break;
+            }
+        }
+        s_ok = ok;
+    }
+    ++round;
+    __syncthreads();
+    return s_ok != 0;
+}
+
+// Next item of a dynamically distributed loop: thread 0 takes a ticket from
+// the launch's work counter (work; zeroed with the barrier counter before
+// the launch) and the CTA reads it.  The tickets of one loop run from base;
+// every CTA leaves the loop at its first ticket past the loop's items, so a
+// loop of n items consumes n + gridDim.x tickets (the next loop's base).
+__device__ __forceinline__ int grab_item(unsigned int* work, unsigned int base, int* s_item) {
+    if (threadIdx.x == 0) *s_item = (int)(atomicAdd(work, 1u) - base);
+    __syncthreads();
+    const int item = *s_item;
+    __syncthreads();
+    return item;
+}
+
 }  // namespace
 }  // namespace mrcm

@@ -68,11 +68,10 @@ struct Plan {
     double model_build = 0, model_sweep = 0;
     double phase_build[MRCM_PHASE_COUNT] = {};   // per build call
     double phase_pass[MRCM_PHASE_COUNT] = {};    // per solve pass
-    // the above count root levels in the inverse form; where a root level
-    // takes the factor form these differences are added: [0] every root
-    // level (MRCM_ROOT_FACTOR), [1] the levels MRCM_ROOT_AUTO factors
-    double root_build[2][MRCM_PHASE_COUNT] = {}, root_pass[2][MRCM_PHASE_COUNT] = {};
-    double root_merge[2] = {}, root_solve[2] = {}, root_model_sweep[2] = {};
+    // the above count root levels in the inverse form; these differences are
+    // added where they take the factor form (MRCM_ROOT_FACTOR)
+    double root_build[MRCM_PHASE_COUNT] = {}, root_pass[MRCM_PHASE_COUNT] = {};
+    double root_merge = 0, root_solve = 0, root_model_sweep = 0;
     double residual_flops = 0, finish_flops = 0;
     // 3D contexts: the grid, the blocks (leaves), the second tangential
     // extent of each segment and the z-face map
@@ -446,16 +445,13 @@ void finish_merges(Plan& P) {
                 // forward sweep (N^2), the inverse diagonal blocks (2 kGJ N)
                 // and the backward sweep (N^2) instead of the product (2 N^2)
                 const double fac = N * (N * N - 1.0) / 3.0;
-                for (int a = 0; a < 2; ++a) {
-                    if (a == 1 && P.level_max_g2[h - 1] < kRootFactorMinG2) continue;
-                    P.root_build[a][MRCM_PHASE_GJ_SWEEP] -= sym;
-                    P.root_build[a][MRCM_PHASE_ROOT_FACTOR] += fac;
-                    P.root_merge[a] += fac - sym;
-                    P.root_model_sweep[a] -= 2.0 / 3.0 * N * N * N;
-                    P.root_pass[a][MRCM_PHASE_TREE_UP] += N * N;
-                    P.root_pass[a][MRCM_PHASE_TREE_DOWN] += N * N + 2.0 * kMergeBlock * N - 2.0 * N * N;
-                    P.root_solve[a] += 2.0 * kMergeBlock * N;
-                }
+                P.root_build[MRCM_PHASE_GJ_SWEEP] -= sym;
+                P.root_build[MRCM_PHASE_ROOT_FACTOR] += fac;
+                P.root_merge += fac - sym;
+                P.root_model_sweep -= 2.0 / 3.0 * N * N * N;
+                P.root_pass[MRCM_PHASE_TREE_UP] += N * N;
+                P.root_pass[MRCM_PHASE_TREE_DOWN] += N * N + 2.0 * kMergeBlock * N - 2.0 * N * N;
+                P.root_solve += 2.0 * kMergeBlock * N;
             }
             P.phase_build[MRCM_PHASE_MERGE_X] += 2.0 * N * gd * md;
             P.phase_build[MRCM_PHASE_MERGE_R] += md * (md + 1.0) * gd;
@@ -973,24 +969,22 @@ static void fill_plan_inputs(Plan& P, int count, const mrcm_grid* g, const int s
     P.gx = seg[0]; P.gy = seg[1];
 }
 
-// which set of root-level flop differences applies to a root form: -1 none
-static int root_set(int form) { return form == MRCM_ROOT_FACTOR ? 0 : (form == MRCM_ROOT_AUTO ? 1 : -1); }
+// whether a root form keeps factors (then the plan's root_* differences apply)
+static double root_factored(int form) { return form == MRCM_ROOT_FACTOR ? 1.0 : 0.0; }
 
 static int plan_value(const Plan& P, int what, long long* value, int form = MRCM_ROOT_AUTO) {
-    const int a = root_set(form);
-    const double f = a >= 0 ? 1.0 : 0.0;
-    const int ai = a >= 0 ? a : 0;
+    const double f = root_factored(form);
     switch (what) {
         case MRCM_Q_LEAVES: *value = P.nleaf; break;
         case MRCM_Q_SEGMENTS: *value = P.nseg; break;
         case MRCM_Q_LEVELS: *value = P.height; break;
         case MRCM_Q_NODES: *value = (long long)P.nodes.size(); break;
         case MRCM_Q_MAX_GAMMA: *value = P.max_g2; break;
-        case MRCM_Q_BUILD_FLOPS: *value = P.leaf_flops + P.merge_flops + (long long)(f * P.root_merge[ai]); break;
-        case MRCM_Q_SOLVE_FLOPS: *value = P.solve_flops + (long long)(f * P.root_solve[ai]); break;  // one pass
+        case MRCM_Q_BUILD_FLOPS: *value = P.leaf_flops + P.merge_flops + (long long)(f * P.root_merge); break;
+        case MRCM_Q_SOLVE_FLOPS: *value = P.solve_flops + (long long)(f * P.root_solve); break;  // one pass
         case MRCM_Q_LEAF_FLOPS: *value = P.leaf_flops; break;
         case MRCM_Q_MODEL_BUILD_FLOPS: *value = (long long)P.model_build; break;
-        case MRCM_Q_MODEL_SWEEP_FLOPS: *value = (long long)(P.model_sweep + f * P.root_model_sweep[ai]); break;
+        case MRCM_Q_MODEL_SWEEP_FLOPS: *value = (long long)(P.model_sweep + f * P.root_model_sweep); break;
         case MRCM_Q_GRIDS: *value = (long long)P.grids.size(); break;
         case MRCM_Q_CELLS: *value = P.ncell; break;
         default: return MRCM_ERR_INVALID_ARG;
@@ -1019,10 +1013,8 @@ int mrcm_plan_query(const mrcm_grid* g, const int sub_cells[3], const int seg_ce
 // form of the context.
 static bool level_factor(const mrcm_ctx* c, int h) {
     const Plan& P = c->P;
-    if (c->root_form == MRCM_ROOT_INVERSE || P.level_max_m[h - 1] != 0 ||
-        !merge_level_blocked(P.level_count[h - 1], P.level_max_g2[h - 1], P.level_max_m[h - 1]))
-        return false;
-    return c->root_form == MRCM_ROOT_FACTOR || P.level_max_g2[h - 1] >= kRootFactorMinG2;
+    return c->root_form == MRCM_ROOT_FACTOR && P.level_max_m[h - 1] == 0 &&
+           merge_level_blocked(P.level_count[h - 1], P.level_max_g2[h - 1], P.level_max_m[h - 1]);
 }
 static void set_tree_forms(mrcm_ctx* c) {
     for (int h = 1; h <= c->P.height; ++h) c->tree.form[h - 1] = level_factor(c, h) ? 1 : 0;
@@ -1056,6 +1048,8 @@ static int setup_tree(mrcm_ctx* c) {
             T.g2[h - 1] = P.level_max_g2[h - 1];
             T.m[h - 1] = P.level_max_m[h - 1];
         }
+        TRY(dev_alloc(c, &v.gam_sq, std::max<long long>((long long)P.gamma_segs.size(), 1)));
+        TRY(dev_alloc(c, &v.gam_sd, std::max<long long>((long long)P.gamma_segs.size(), 1)));
         TRY(dev_alloc(c, &v.rgam, std::max<long long>(2 * (long long)P.gamma_segs.size(), 1)));
         TRY(dev_alloc(c, &v.fwd, std::max<long long>(2 * (long long)P.gamma_segs.size(), 1)));
         // flags of the triangular sweeps: per node of a level that may take
@@ -1300,6 +1294,7 @@ static int enqueue_build(mrcm_ctx* c, int& launches, bool merges_only = false) {
             PhaseScope ps(c, MRCM_PHASE_COEF);
             TRYC(launch_check_K(v, s)); ++launches;
             TRYC(launch_coef3(v, s)); launches += 1 + (P.nseg > 0);
+            TRYC(launch_gamma_scale(v, (int)P.gamma_segs.size(), s)); launches += !P.gamma_segs.empty();
         }
         PhaseScope ps(c, MRCM_PHASE_LEAF_BUILD);
         TRYC(launch_leaf3_build(v, s)); ++launches;
@@ -1309,6 +1304,7 @@ static int enqueue_build(mrcm_ctx* c, int& launches, bool merges_only = false) {
         TRYC(launch_cell_resist(v, s)); ++launches;
         TRYC(launch_seg_beta(v, s)); launches += P.nseg > 0;
         TRYC(launch_face_coef(v, s)); ++launches;
+        TRYC(launch_gamma_scale(v, (int)P.gamma_segs.size(), s)); launches += !P.gamma_segs.empty();
     }
     if (!merges_only && P.dim != 3) {
         PhaseScope ps(c, MRCM_PHASE_LEAF_BUILD);
@@ -1822,12 +1818,10 @@ int mrcm_group_times(mrcm_ctx* c, int* phase, double* ms, int cap) {
 int mrcm_phase_flops(const mrcm_ctx* c, double* flops) {
     if (!c || !flops) return MRCM_ERR_INVALID_ARG;
     const Plan& P = c->P;
-    const int a = root_set(c->root_form);
-    const double passes = 1.0 + c->refine_steps, f = a >= 0 ? 1.0 : 0.0;
-    const int ai = a >= 0 ? a : 0;
+    const double passes = 1.0 + c->refine_steps, f = root_factored(c->root_form);
     for (int p = 0; p < MRCM_PHASE_COUNT; ++p)
-        flops[p] = P.phase_build[p] + f * P.root_build[ai][p] +
-                   passes * (P.phase_pass[p] + f * P.root_pass[ai][p]);
+        flops[p] = P.phase_build[p] + f * P.root_build[p] +
+                   passes * (P.phase_pass[p] + f * P.root_pass[p]);
     flops[MRCM_PHASE_RESIDUAL] = (c->refine_steps + (c->refine_check ? 1 : 0)) * P.residual_flops;
     flops[MRCM_PHASE_FINISH] = P.finish_flops;
     return MRCM_OK;

@@ -154,6 +154,8 @@ struct DevView {
     double* leafzb;     // particular forward solves
     double* R;          // node maps (leaves and internal nodes)
     double* rbar;       // node particular fluxes
+    double* gam_sq;     // D^1/2 and D^-1/2 of every gamma segment (gamma_segs order)
+    double* gam_sd;
     double* rgam;       // per merge, rbar of its 2g gamma unknowns gathered from
                         // the children (at 2 * gamma_off), written by the up sweep
     double* lam;        // node Robin data (top-down)
@@ -236,32 +238,38 @@ __device__ __forceinline__ DD dd_neg(DD x) { return {-x.h, -x.l}; }
 
 // Reciprocal from a single-precision seed refined by one third-order step of
 // the Newton-Raphson family (Muller et al., Handbook of Floating-Point
-// Arithmetic, Sec. 5.3): with x the seed and e = 1 - p x, 1/p = x / (1 - e) =
-// x (1 + e + e^2 + ...), and the series is cut after e^2.  The seed is the
-// approximate FP32 reciprocal (at most 1 ulp off) of p's sign, exponent and
-// leading 23 mantissa bits, moved between formats with integer operations
-// (conversion instructions run on the slower FP64 path), so |e| < 2^-21.9 and
-// the dropped terms are below 2^-65 relative: the result is within an ulp of
-// 1/p.  Three dependent FP64 instructions (e, e + e^2, x + x (e + e^2))
-// instead of the longer IEEE division sequence, which matters where a
-// reciprocal sits on a sequential chain (pivots).  Outside the exponent range
-// of FP32 it falls back to the division.
+// Arithmetic, Sec. 5.3), in 64-bit integer arithmetic: with p = m 2^(e - 52),
+// m its 53-bit integer significand, and X the 24-bit integer nearest to the
+// approximate FP32 reciprocal of m 2^-52 (at most 1 ulp off, |error| < 2^-22
+// with the truncated argument), E = 2^76 - m X is exact in 64 bits and
+//     2^52 / m = X 2^-24 / (1 - E 2^-76) = X 2^-24 (1 + eps + eps^2 + ...),
+// cut after eps^2 (below 2^-66 relative); the sum is kept to 2^-59 and
+// rounded once, so the result is within an ulp of 1/p.  An FP64 instruction
+// takes 75 cycles from issue to result on this part and holds its
+// scheduler's FP64 pipe for 64 of them; the three of an FP64 Newton step made
+// the reciprocal 320 cycles of every pivot's chain, the integer ones about
+// half.  Zeros, subnormals, infinities, NaN and exponents whose reciprocal is
+// not normal take the division.
 __device__ __forceinline__ double rcp_nr(double p) {
-    const unsigned long long bits = (unsigned long long)__double_as_longlong(p);
-    const int e = (int)((bits >> 52) & 0x7ff) - 1023;
-    if (e < -120 || e > 120) return 1.0 / p;
-    const unsigned int fb = (unsigned int)(bits >> 32 & 0x80000000u) | ((unsigned int)(e + 127) << 23) |
-                            (unsigned int)(bits >> 29 & 0x7fffffu);
+    const unsigned hi = (unsigned)__double2hiint(p), lo = (unsigned)__double2loint(p);
+    const int be = (int)((hi >> 20) & 0x7ffu);
+    if (be == 0 || be > 2044) return 1.0 / p;
+    const unsigned mh = (hi & 0xfffffu) | 0x100000u;                       // significand, high and low words
+    const float f = __uint_as_float(0x3f800000u | ((mh << 3) & 0x7fffffu) | (lo >> 29));
     float rf;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rf) : "f"(__uint_as_float(fb)));
-    const unsigned int rb = __float_as_uint(rf);
-    const int er = (int)((rb >> 23) & 0xff) - 127;
-    const unsigned long long xb = ((unsigned long long)(rb & 0x80000000u) << 32) |
-                                  ((unsigned long long)(er + 1023) << 52) | ((unsigned long long)(rb & 0x7fffffu) << 29);
-    const double x = __longlong_as_double((long long)xb);
-    const double e0 = fma(-p, x, 1.0);
-    const double s = fma(e0, e0, e0);
-    return fma(x, s, x);
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rf) : "f"(f));
+    const unsigned rb = __float_as_uint(rf);                               // in (0.5, 1]
+    const unsigned x = ((rb & 0x7fffffu) | 0x800000u) << ((rb >> 23) - 126u);
+    const unsigned long long mx = (unsigned long long)lo * x + ((unsigned long long)(mh * x) << 32);
+    const long long E = -(long long)mx;                                    // 2^76 - m X, |E| < 2^55
+    const long long t1 = (long long)(((E >> 17) * (long long)x) >> 20);
+    const int e2 = (int)(E >> 33);
+    const unsigned sq = (unsigned)(((long long)e2 * e2) >> 18);
+    const unsigned t2 = (unsigned)(((unsigned long long)sq * x) >> 29);
+    const unsigned long long q = ((unsigned long long)x << 39) + (unsigned long long)(t1 + (long long)t2);
+    const unsigned long long bits =
+        ((unsigned long long)(2044 - be) << 52) + ((q + 0x200ull) >> 10) + ((unsigned long long)(hi & 0x80000000u) << 32);
+    return __longlong_as_double((long long)bits);
 }
 // Quotient and remainder of a non-negative index by a positive divisor in
 // 32-bit unsigned arithmetic (every index of the workspace is below 2^32;
@@ -387,6 +395,15 @@ struct MergeTune {
 // (kernels_merge_mma.cu).  fp32: the mixed form's precision.
 cudaError_t launch_merge_x(const DevView& v, int first, int count, int max_g2, int max_m, bool fp32, cudaStream_t s);
 cudaError_t launch_merge_r(const DevView& v, int first, int count, int max_m, bool fp32, cudaStream_t s);
+// T^-1 -> W of one height in blocks of 64 on the tensor cores; scratch:
+// sweep_node_scratch(max_g2) values of the arithmetic type per node.
+__host__ __device__ constexpr long long sweep_node_scratch(int nmax) { return 2LL * nmax * 64 + 2 * 64 * 64; }
+cudaError_t launch_block_sweep(const DevView& v, int first, int count, int max_g2, bool fp32, double* scratch,
+                               void* barrier, int sms, int per_sm, cudaStream_t s);
+// T^-1 -> W of one height with 2g <= 64, one system per CTA
+cudaError_t launch_node_invert(const DevView& v, int first, int count, bool fp32, cudaStream_t s);
+// gam_sq, gam_sd of the tree's n gamma segments
+cudaError_t launch_gamma_scale(const DevView& v, int n, cudaStream_t s);
 // fp32: the mixed form's FP32 arithmetic for this level (T of the blocked
 // sweep in v.W32; W, X and R stored in double either way).  factor: a
 // blocked level without outer segments (a root level) keeps the block
@@ -404,10 +421,6 @@ bool merge_level_blocked(int count, int max_g2, int max_m);
 size_t merge_scratch_doubles(int count, int max_g2, int max_m);
 constexpr int kMergeBlock = 16;      // block size of the blocked Gauss-Jordan sweep (flop model)
 constexpr int kTriBlock = 64;        // solve blocks of the factor form's triangular sweeps
-// MRCM_ROOT_AUTO factors root systems from this 2g on: below it the root's
-// elimination is bound by its sequential chain of pivot blocks (the same
-// length in both forms), and the inverse's solve passes are the shorter.
-constexpr int kRootFactorMinG2 = 1024;
 
 // The merge levels of the tree for the fused up / down sweeps of the solve
 // (passed by value as a kernel argument; index h - 1 for height h).

@@ -291,5 +291,89 @@ __device__ __forceinline__ void split_product(SplitSmem<S>& sm, int K, const int
     }
 }
 
+// ---------------------------------------------------------------------------
+// Products of small matrices by one warp, operands cut straight into MMA
+// fragments (no shared-memory staging of digits).  Lane (g, t) = (lane / 4,
+// lane % 4) of an A fragment (16 x 16) holds rows g and g + 8, entries 2 t,
+// 2 t + 1, 2 t + 8, 2 t + 9; of a B fragment (16 x 8) the same entries of
+// column g.
+template <int S>
+struct FragA {
+    unsigned d[S][4];
+    int e0, e1;                 // exponents of rows g, g + 8
+};
+template <int S>
+struct FragB {
+    unsigned d[S][2];
+    int e;                      // exponent of column g
+};
+template <class T>
+__device__ __forceinline__ int quad_exponent(T a, T b, T c, T d) {
+    int E = max(max(exponent_bits(a), exponent_bits(b)), max(exponent_bits(c), exponent_bits(d)));
+    E = max(E, __shfl_xor_sync(0xffffffffu, E, 1));
+    E = max(E, __shfl_xor_sync(0xffffffffu, E, 2));
+    return sizeof(T) == 8 ? E >> 20 : E >> 23;
+}
+// at(row, k): the operand's entry
+template <int S, class T, class At>
+__device__ __forceinline__ void load_frag_a(FragA<S>& f, At&& at) {
+    const int g = (threadIdx.x & 31) >> 2, t = threadIdx.x & 3;
+    T v[2][4];
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[h][i] = at(g + 8 * h, 2 * t + (i & 1) + 8 * (i >> 1));
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int E = quad_exponent(v[h][0], v[h][1], v[h][2], v[h][3]);
+        (h ? f.e1 : f.e0) = common_exponent<T>(E);
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+            unsigned d[S];
+            digit_pair<S>(v[h][2 * p], v[h][2 * p + 1], E, d);
+#pragma unroll
+            for (int s = 0; s < S; ++s) f.d[s][h + 2 * p] = d[s];
+        }
+    }
+}
+// at(col, k)
+template <int S, class T, class At>
+__device__ __forceinline__ void load_frag_b(FragB<S>& f, At&& at) {
+    const int g = (threadIdx.x & 31) >> 2, t = threadIdx.x & 3;
+    T v[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) v[i] = at(g, 2 * t + (i & 1) + 8 * (i >> 1));
+    const int E = quad_exponent(v[0], v[1], v[2], v[3]);
+    f.e = common_exponent<T>(E);
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+        unsigned d[S];
+        digit_pair<S>(v[2 * p], v[2 * p + 1], E, d);
+#pragma unroll
+        for (int s = 0; s < S; ++s) f.d[s][p] = d[s];
+    }
+}
+// out[r]: row g + 8 (r / 2), column 2 t + r % 2 of the 16 x 8 product
+template <int S>
+__device__ __forceinline__ void frag_product(const FragA<S>& a, const FragB<S>& b, typename SplitAcc<S>::T (&out)[4]) {
+    float acc[S][4];
+#pragma unroll
+    for (int l = 0; l < S; ++l)
+#pragma unroll
+        for (int r = 0; r < 4; ++r) acc[l][r] = 0.f;
+#pragma unroll
+    for (int i = 0; i < S; ++i)
+#pragma unroll
+        for (int j = 0; j < S - i; ++j) mma_f16(acc[i + j], a.d[i], b.d[j][0], b.d[j][1]);
+    const int t = threadIdx.x & 3;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        float n[S];
+#pragma unroll
+        for (int l = 0; l < S; ++l) n[l] = acc[l][r];
+        out[r] = combine_levels(n, r < 2 ? a.e0 : a.e1, __shfl_sync(0xffffffffu, b.e, (2 * t + (r & 1)) * 4));
+    }
+}
+
 }  // namespace
 }  // namespace mrcm
