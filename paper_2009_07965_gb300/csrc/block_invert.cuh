@@ -1,6 +1,6 @@
 // Inverses of small symmetric matrices inside a CTA: up to 16 x 16 by the
-// lanes of one warp on the FP64 pipe, up to 64 x 64 by four warps, 16 rows at
-// a time, with the products on the tensor cores (split_gemm.cuh).
+// lanes of one warp on the FP64 pipe, up to 64 x 64 by four or eight warps, 16
+// rows at a time, with the products on the tensor cores (split_gemm.cuh).
 //
 // Both use the symmetric sweep operator: sweeping the indices K turns A_KK
 // into -A_KK^-1, A_xK into A_xK A_KK^-1 and A_xy into A_xy - A_xK A_KK^-1 A_Ky
@@ -91,10 +91,7 @@ __device__ __forceinline__ bool sweep_block(T (&e)[BlockSlots<GL>::kN], const Bl
 }
 
 // ---------------------------------------------------------------------------
-// Up to 64 x 64 by the four warps of a CTA.
-template <class T> struct Slices { static constexpr int S = 7; };
-template <> struct Slices<float> { static constexpr int S = 4; };
-
+// Up to 64 x 64 by the NT threads of a CTA.
 constexpr int kInvert = 64;
 template <class T>
 struct InvertSmem {
@@ -105,23 +102,22 @@ struct InvertSmem {
     int bad;
 };
 
-// The 16 x 16 diagonal block from row k0 on (n rows) into S.P by the four
-// warps.  Warp 0 runs the chain of pivots one step ahead of the others: while
-// warps 1-3 apply pivot k - 1 to the lower triangle (two entries per thread),
-// it forms pivot k itself,
+// The 16 x 16 diagonal block from row k0 on (n rows) into S.P, by NT threads.
+// Warp 0 runs the chain of pivots one step ahead of the others: while they
+// apply pivot k - 1 to the lower triangle (one entry per thread, two with
+// NT = 128), it forms pivot k itself,
 //     p_k = T_kk - T_k,k-1^2 / p_(k-1)   (entries before pivot k - 1),
 // and its reciprocal.  One CTA barrier per pivot hands the reciprocal to the
 // update and the fresh entries to warp 0.
-template <class T, class Ok>
+template <int NT, class T, class Ok>
 __device__ __forceinline__ void invert16(InvertSmem<T>& S, int k0, int n, Ok&& pivot_ok) {
-    constexpr int kTri = kPlane * (kPlane + 1) / 2;
-    static_assert(kTri <= 2 * 96, "two entries per thread of three warps");
+    constexpr int kTri = kPlane * (kPlane + 1) / 2, kOwn = (kTri + NT - 33) / (NT - 32);
     const int tid = threadIdx.x, u = tid - 32;
-    int r[2], c[2];
-    T e[2];
+    int r[kOwn], c[kOwn];
+    T e[kOwn];
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
-        const int idx = u + 96 * j;
+    for (int j = 0; j < kOwn; ++j) {
+        const int idx = u + (NT - 32) * j;
         r[j] = c[j] = kColNone;                            // (matches no pivot)
         e[j] = (T)0;
         if (u >= 0 && idx < kTri) {
@@ -135,7 +131,7 @@ __device__ __forceinline__ void invert16(InvertSmem<T>& S, int k0, int n, Ok&& p
     // column k off its diagonal, and the next diagonal entry (last place)
     auto publish = [&](int k) {
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
+        for (int j = 0; j < kOwn; ++j) {
             int at = c[j] == k ? r[j] : (r[j] == k ? c[j] : kColNone);
             if (r[j] == c[j]) at = r[j] == k + 1 ? kColPivot : kColNone;
             S.col[k & 1][at] = e[j];
@@ -162,7 +158,7 @@ __device__ __forceinline__ void invert16(InvertSmem<T>& S, int k0, int n, Ok&& p
             const int s = k - 1;
             const T q = S.rp[s & 1];
 #pragma unroll
-            for (int j = 0; j < 2; ++j) {
+            for (int j = 0; j < kOwn; ++j) {
                 const T m = (r[j] == s ? (T)-1 : a[r[j]]) * (c[j] == s ? (T)-1 : a[c[j]]);
                 e[j] = fma(neg_bits(m), q, (r[j] == s || c[j] == s) ? (T)0 : e[j]);
             }
@@ -174,7 +170,7 @@ __device__ __forceinline__ void invert16(InvertSmem<T>& S, int k0, int n, Ok&& p
         if (!ok) S.bad = 1;
     } else {
 #pragma unroll
-        for (int j = 0; j < 2; ++j)
+        for (int j = 0; j < kOwn; ++j)
             if (r[j] < kPlane) S.P[r[j]][c[j]] = S.P[c[j]][r[j]] = r[j] < n ? neg_bits(e[j]) : (T)0;
     }
     __syncthreads();
@@ -182,36 +178,33 @@ __device__ __forceinline__ void invert16(InvertSmem<T>& S, int k0, int n, Ok&& p
 
 // Sweeps all nb rows of S.A (-inverse in its lower triangle).  False (all
 // threads) when pivot_ok(p, row) fails.
-template <class T, class Ok>
+template <int NT, class T, class Ok>
 __device__ bool invert_block(InvertSmem<T>& S, int nb, Ok&& pivot_ok) {
-    constexpr int SL = Slices<T>::S;
+    constexpr int SL = Slices<T>::S, NW = NT / 32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
     const int nblk = (nb + kPlane - 1) / kPlane;
     if (tid == 0) S.bad = 0;
     __syncthreads();
     for (int kb = 0; kb < nblk; ++kb) {
         const int k0 = kb * kPlane;
-        invert16(S, k0, min(kPlane, nb - k0), [&](T p, int k) { return pivot_ok(p, k0 + k); });
+        invert16<NT>(S, k0, min(kPlane, nb - k0), [&](T p, int k) { return pivot_ok(p, k0 + k); });
         // C(x, k) of row x of block bx against the block's columns
         auto c_entry = [&](int bx, int r, int k) -> T {
             return bx > kb ? S.A[bx * kPlane + r][k0 + k] : S.A[k0 + k][bx * kPlane + r];
         };
         // U = C P, A_KK = -P
-        for (int q = warp; q < nblk - 1; q += 4) {
-            const int bx = q < kb ? q : q + 1;
+        for (int item = warp; item < 2 * (nblk - 1); item += NW) {
+            const int q = item >> 1, nt = item & 1, bx = q < kb ? q : q + 1;
             FragA<SL> a;
+            FragB<SL> b;
             load_frag_a<SL, T>(a, [&](int r, int k) { return c_entry(bx, r, k); });
+            load_frag_b<SL, T>(b, [&](int n, int k) { return S.P[8 * nt + n][k]; });
+            typename SplitAcc<SL>::T out[4];
+            frag_product(a, b, out);
 #pragma unroll
-            for (int nt = 0; nt < 2; ++nt) {
-                FragB<SL> b;
-                load_frag_b<SL, T>(b, [&](int n, int k) { return S.P[8 * nt + n][k]; });
-                typename SplitAcc<SL>::T out[4];
-                frag_product(a, b, out);
-#pragma unroll
-                for (int r = 0; r < 4; ++r) S.U[bx * kPlane + g + 8 * (r >> 1)][8 * nt + 2 * t + (r & 1)] = (T)out[r];
-            }
+            for (int r = 0; r < 4; ++r) S.U[bx * kPlane + g + 8 * (r >> 1)][8 * nt + 2 * t + (r & 1)] = (T)out[r];
         }
-        if (warp == 3)
+        if (warp == NW - 1)
             for (int i = lane; i < kPlane * kPlane; i += 32) {
                 const int r = i / kPlane, c = i % kPlane;
                 if (r >= c) S.A[k0 + r][k0 + c] = neg_bits(S.P[r][c]);
@@ -219,7 +212,7 @@ __device__ bool invert_block(InvertSmem<T>& S, int nb, Ok&& pivot_ok) {
         __syncthreads();
         // A_xy -= C_x U_y^T by 16 x 8 tiles, each warp a run of them in row
         // order (the digits of C_x are kept from one to the next)
-        const int nitem = (nblk - 1) * nblk, per = (nitem + 3) / 4;
+        const int nitem = (nblk - 1) * nblk, per = (nitem + NW - 1) / NW;
         const int lo = warp * per, hi = min(lo + per, nitem);
         int item = 0, have = -1;
         FragA<SL> a;
@@ -242,7 +235,7 @@ __device__ bool invert_block(InvertSmem<T>& S, int nb, Ok&& pivot_ok) {
                 }
             }
         __syncthreads();
-        for (int i = tid; i < nblk * kPlane * kPlane; i += 128) {
+        for (int i = tid; i < nblk * kPlane * kPlane; i += NT) {
             const int x = i / kPlane, c = i % kPlane, bx = x / kPlane;
             if (bx > kb) S.A[x][k0 + c] = S.U[x][c];
             else if (bx < kb) S.A[k0 + c][x] = S.U[x][c];

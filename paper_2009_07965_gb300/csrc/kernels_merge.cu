@@ -1843,7 +1843,7 @@ static cudaError_t launch_merge_build_t(const DevView& v, int first, int count, 
             if (e != cudaSuccess) return e;
         }
         HookScope hs(hook, kPhMergeR);
-        e = launch_merge_r(v, first, count, max_m, sizeof(F) == sizeof(float), s);
+        e = launch_merge_r(v, first, count, max_g2, max_m, sizeof(F) == sizeof(float), s);
         ++*launches;
         if (e != cudaSuccess) return e;
     }

@@ -34,22 +34,18 @@ __global__ void __launch_bounds__(kGemmThreads, 2) merge_x_kernel(DevView v, int
     const int* gpos = half ? N.gpos2 : N.gpos1;
     const int* opos = half ? N.opos2 - N.o1 : N.opos1;
     const int mc = half ? N.m2 : N.m1;
-    typename SplitAcc<S>::T sum[2][2][4];
+    typename SplitAcc<S>::T sum[2][4];
     split_product<S, double, false, true>(
         sm, g, gpos, [&](int r) { return r0 + r < g2 ? W + (long long)(r0 + r) * g2 : nullptr; },
         [&](int j) { return j0 + j < jend ? Rc + (long long)opos[j0 + j] * mc : nullptr; }, sum);
     double* X = v.X + D.X_off;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
     for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-        for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int r = r0 + (warp >> 1) * 32 + 16 * mt + (lane >> 2) + 8 * (q >> 1);
-                const int j = j0 + (warp & 1) * 16 + 8 * nt + 2 * (lane & 3) + (q & 1);
-                if (r < g2 && j < jend) X[(long long)j * g2 + r] = -(double)sum[mt][nt][q];
-            }
+        for (int q = 0; q < 4; ++q) {
+            const int r = r0 + out_row(mt, q), j = j0 + out_col(q);
+            if (r < g2 && j < jend) X[(long long)j * g2 + r] = neg_bits(widen(sum[mt][q]));
+        }
 }
 
 // R = blockdiag(R^a_oo, R^b_oo) + blockdiag(R^a_og, R^b_og) X, lower triangle
@@ -74,27 +70,93 @@ __global__ void __launch_bounds__(kGemmThreads, 2) merge_rupdate_kernel(DevView 
     const int* gpos = half ? N.gpos2 : N.gpos1;
     const int* opos = half ? N.opos2 - o1 : N.opos1;
     const int mc = half ? N.m2 : N.m1;
-    typename SplitAcc<S>::T sum[2][2][4];
+    typename SplitAcc<S>::T sum[2][4];
     split_product<S, double, true, false>(
         sm, g, gpos, [&](int i) { return i0 + i < iend ? Rc + (long long)opos[i0 + i] * mc : nullptr; },
         [&](int j) { return j0 + j < m ? X + (long long)(j0 + j) * g2 : nullptr; }, sum);
     double* Rp = v.R + D.R_off;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
     for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-        for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int i = i0 + (warp >> 1) * 32 + 16 * mt + (lane >> 2) + 8 * (q >> 1);
-                const int j = j0 + (warp & 1) * 16 + 8 * nt + 2 * (lane & 3) + (q & 1);
-                if (i >= iend || j > i) continue;
-                double val = (double)sum[mt][nt][q];
-                if (half == (j >= o1)) val += Rc[(long long)opos[i] * mc + opos[j]];   // both on one child
-                Rp[(long long)i * m + j] = val;
-                Rp[(long long)j * m + i] = val;
-            }
+        for (int q = 0; q < 4; ++q) {
+            const int i = i0 + out_row(mt, q), j = j0 + out_col(q);
+            if (i >= iend || j > i) continue;
+            double val = widen(sum[mt][q]);
+            if (half == (j >= o1)) val += Rc[(long long)opos[i] * mc + opos[j]];   // both on one child
+            Rp[(long long)i * m + j] = val;
+            Rp[(long long)j * m + i] = val;
+        }
 }
+
+// The same products where g <= kChunkK and the level has CTAs enough: one CTA
+// per 64 rows of X and child, and per 64 rows of R, over all their column
+// tiles (the digits of the rows are cut once and a tile's loads hide behind
+// the products before it: box 128x128x64 R of 2g <= 128 6.0 -> 3.9 ms, the mixed
+// 256x256x64 box 20 -> 8).
+template <int S>
+__global__ void __launch_bounds__(kGemmThreads, 2) merge_x_strip_kernel(DevView v, int first) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    SplitSmem<S>& sm = *reinterpret_cast<SplitSmem<S>*>(smem_raw);
+    const MergeDesc D = v.merges[first + blockIdx.x];
+    const NodeRefs N = node_refs(v, D);
+    const int g = N.g, g2 = N.g2, m = N.m, r0 = (blockIdx.y >> 1) * kTileM;
+    const bool half = blockIdx.y & 1;
+    const int jbeg = half ? N.o1 : 0, jend = half ? m : N.o1;
+    if (r0 >= g2 || jbeg >= jend) return;                              // uniform per CTA
+    const double* W = v.W + D.W_off + (half ? g : 0);
+    const double* Rc = half ? N.R2 : N.R1;
+    const int* opos = half ? N.opos2 - N.o1 : N.opos1;
+    const int mc = half ? N.m2 : N.m1;
+    double* X = v.X + D.X_off;
+    strip_product<S, false, true>(
+        sm, g, half ? N.gpos2 : N.gpos1, 0, (jend - jbeg + kTileN - 1) / kTileN,
+        [&](int r) { return r0 + r < g2 ? W + (long long)(r0 + r) * g2 : nullptr; },
+        [&](int t, int c) {
+            const int j = jbeg + t * kTileN + c;
+            return j < jend ? Rc + (long long)opos[j] * mc : nullptr;
+        },
+        [](int, int, int) { return 0.0; },
+        [&](int t, int i, int c, double x, double) {
+            const int r = r0 + i, j = jbeg + t * kTileN + c;
+            if (r < g2 && j < jend) X[(long long)j * g2 + r] = neg_bits(x);
+        });
+}
+template <int S>
+__global__ void __launch_bounds__(kGemmThreads, 2) merge_rupdate_strip_kernel(DevView v, int first) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    SplitSmem<S>& sm = *reinterpret_cast<SplitSmem<S>*>(smem_raw);
+    const MergeDesc D = v.merges[first + blockIdx.x];
+    const NodeRefs N = node_refs(v, D);
+    const int g = N.g, g2 = N.g2, m = N.m, o1 = N.o1;
+    const int na = (o1 + kTileM - 1) / kTileM, nb = (m - o1 + kTileM - 1) / kTileM;
+    if ((int)blockIdx.y >= na + nb) return;                             // uniform per CTA
+    const int rt = na + nb - 1 - blockIdx.y;                            // long rows first
+    const bool half = rt >= na;
+    const int i0 = half ? o1 + (rt - na) * kTileM : rt * kTileM, iend = min(i0 + kTileM, half ? m : o1);
+    const double* X = v.X + D.X_off + (half ? g : 0);
+    const double* Rc = half ? N.R2 : N.R1;
+    const int* opos = half ? N.opos2 - o1 : N.opos1;
+    const int mc = half ? N.m2 : N.m1;
+    double* Rp = v.R + D.R_off;
+    strip_product<S, true, false>(
+        sm, g, half ? N.gpos2 : N.gpos1, 0, (iend + kTileN - 1) / kTileN,
+        [&](int i) { return i0 + i < iend ? Rc + (long long)opos[i0 + i] * mc : nullptr; },
+        [&](int t, int c) { return t * kTileN + c < m ? X + (long long)(t * kTileN + c) * g2 : nullptr; },
+        [&](int t, int r, int c) {
+            const int i = i0 + r, j = t * kTileN + c;                   // R_oo: both on one child
+            return i < iend && j <= i && half == (j >= o1) ? Rc[(long long)opos[i] * mc + opos[j]] : 0.0;
+        },
+        [&](int t, int r, int c, double x, double old) {
+            const int i = i0 + r, j = t * kTileN + c;
+            if (i >= iend || j > i) return;
+            Rp[(long long)i * m + j] = x + old;
+            Rp[(long long)j * m + i] = x + old;
+        });
+}
+
+// Whether a level's products run as strips: one chunk of k, and the strips
+// fill the resident CTAs (two per SM) three times over.
+bool strips(int max_g2, long long ctas) { return max_g2 <= 2 * kChunkK && ctas >= 3 * 2 * 152; }
 
 template <int S>
 cudaError_t x_launch(const DevView& v, int first, int count, int max_g2, int max_m, cudaStream_t s) {
@@ -102,15 +164,27 @@ cudaError_t x_launch(const DevView& v, int first, int count, int max_g2, int max
     cudaError_t e = cudaFuncSetAttribute(merge_x_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     if (e != cudaSuccess) return e;
     const int rt = (max_g2 + kTileM - 1) / kTileM, ct = (max_m + kTileN - 1) / kTileN + 1;
+    if (strips(max_g2, (long long)count * rt * 2)) {
+        e = cudaFuncSetAttribute(merge_x_strip_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        if (e != cudaSuccess) return e;
+        merge_x_strip_kernel<S><<<dim3(count, 2 * rt), kGemmThreads, bytes, s>>>(v, first);
+        return cudaGetLastError();
+    }
     merge_x_kernel<S><<<dim3(count, rt * ct), kGemmThreads, bytes, s>>>(v, first);
     return cudaGetLastError();
 }
 template <int S>
-cudaError_t r_launch(const DevView& v, int first, int count, int max_m, cudaStream_t s) {
+cudaError_t r_launch(const DevView& v, int first, int count, int max_g2, int max_m, cudaStream_t s) {
     const int bytes = (int)sizeof(SplitSmem<S>);
     cudaError_t e = cudaFuncSetAttribute(merge_rupdate_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     if (e != cudaSuccess) return e;
     const int rt = (max_m + kTileM - 1) / kTileM + 1, ct = (max_m + kTileN - 1) / kTileN;
+    if (strips(max_g2, (long long)count * rt)) {
+        e = cudaFuncSetAttribute(merge_rupdate_strip_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        if (e != cudaSuccess) return e;
+        merge_rupdate_strip_kernel<S><<<dim3(count, rt), kGemmThreads, bytes, s>>>(v, first);
+        return cudaGetLastError();
+    }
     merge_rupdate_kernel<S><<<dim3(count, rt * ct), kGemmThreads, bytes, s>>>(v, first, ct);
     return cudaGetLastError();
 }
@@ -123,22 +197,14 @@ cudaError_t r_launch(const DevView& v, int first, int count, int max_m, cudaStre
 // and -T^-1 is left in the end.  Only the lower triangle is kept (row-major,
 // in the W storage, or the FP32 work array of a mixed level).
 //
-// One cooperative launch per tree height, two CTAs of four warps per SM: T of
+// One cooperative launch per tree height, two CTAs of eight warps per SM: T of
 // every node, the inverse of the first diagonal blocks; per step the panel
 // items (U = C P; C and U into scratch, 64 entries a row), then the update
 // items, 64 x 32 tiles of one chunk of k each, behind one item per node that
 // updates the next diagonal block and inverts it meanwhile, so that the
 // sequential chain of pivots runs beside the other tiles' products; then W.
 // A grid barrier between the phases (two per 64 rows); with more items than
-// CTAs the update items are handed out by ticket, the next one taken while
-// the current one runs.
-//
-// Measured (FP64, one GB300) against the FP64-pipe sweep of kernels_merge.cu:
-// 256 nodes of 2g = 512 63.7 -> 7.3 ms, 512 x 256 19.1 -> 3.3, 2 x 1024 3.0 ->
-// 1.6, 1 x 2048 (the root of 4096^2, a factorisation before) 4.2 -> 3.4; FP32
-// levels 1024 x 512 120 -> 18.8.  Bound by the latency of the chain for few
-// nodes (about 90 us per 64 rows, half of it the 64 pivots) and by cutting
-// digits and by the loads of a tile for many.
+// CTAs the update items are handed out by ticket.
 constexpr int kSweepB = kInvert;
 static_assert(kSweepB == kChunkK && kSweepB == kTileM && kSweepB == 2 * kTileN, "one chunk, one tile row per block");
 
@@ -160,17 +226,19 @@ struct SweepScratch {
 };
 
 // 1 / sum D of a pinned node's gamma segments (the regularised all-Neumann
-// root), 0 otherwise; red: 4 doubles.
+// root), 0 otherwise; red: a double per warp of the NT threads.
+template <int NT>
 __device__ double pinned_inv_sum(const DevView& v, const MergeDesc& D, double* red) {
     if (!D.pinned) return 0.0;                                          // uniform per CTA
     double part = 0.0;
-    for (int i = threadIdx.x; i < D.g; i += kGemmThreads) part += gamma_D(v, D, i);
+    for (int i = threadIdx.x; i < D.g; i += NT) part += gamma_D(v, D, i);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
     __syncthreads();
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = part;
     __syncthreads();
-    const double sum = (red[0] + red[1]) + (red[2] + red[3]);
+    double sum = 0.0;
+    for (int w = 0; w < NT / 32; ++w) sum += red[w];
     return sum > 0.0 ? 1.0 / sum : 0.0;
 }
 
@@ -181,7 +249,7 @@ __device__ void form_rows(const DevView& v, const MergeDesc& D, int r0, double* 
     const int g = N.g, n = N.g2;
     const double* sq = v.gam_sq + D.gamma_off;
     const double* sd = v.gam_sd + D.gamma_off;
-    const double inv_sum = pinned_inv_sum(v, D, red);
+    const double inv_sum = pinned_inv_sum<kGemmThreads>(v, D, red);
     T* A = sweep_matrix<T>(v) + D.W_off;
     for (int r = r0; r < min(r0 + 16, n); ++r) {
         const int i = r < g ? r : r - g;
@@ -200,9 +268,9 @@ __device__ void store_inverse(const InvertSmem<T>& S, int nb, T* P) {
         P[idx] = a < nb ? neg_bits(S.A[a][b]) : (T)0;
     }
 }
-template <class T>
+template <int NT, class T>
 __device__ void invert_checked(const DevView& v, InvertSmem<T>& S, int nb, int d_rows) {
-    if (!invert_block(S, nb, [&](T p, int k) { return pivot_ok_bits(p, k < d_rows); }) && threadIdx.x == 0)
+    if (!invert_block<NT>(S, nb, [&](T p, int k) { return pivot_ok_bits(p, k < d_rows); }) && threadIdx.x == 0)
         atomicOr(v.status, kStatusSingular);
 }
 
@@ -216,7 +284,7 @@ __device__ void first_inverse(const DevView& v, const MergeDesc& D, const SweepS
         const int r = idx / kSweepB, c = idx % kSweepB;
         S.A[r][c] = r < nb && c <= r ? A[(long long)r * n + c] : (T)0;
     }
-    invert_checked(v, S, nb, D.g);
+    invert_checked<kGemmThreads>(v, S, nb, D.g);
     store_inverse(S, nb, sc.p(0));
 }
 
@@ -254,22 +322,18 @@ __device__ void panel_item(const DevView& v, const MergeDesc& D, const SweepScra
     const T* rows = xt < step ? C : A + (long long)x0 * n + k0;
     const long long ld = xt < step ? kSweepB : n;
     const T* P = sc.p(step);
-    typename SplitAcc<S>::T sum[2][2][4];
+    typename SplitAcc<S>::T sum[2][4];
     split_product<S, T, false, false>(
         sm, nb, nullptr, [&](int x) { return x < nx ? rows + x * ld : nullptr; },
         [&](int c) { return h0 + c < nb ? P + (h0 + c) * kSweepB : nullptr; }, sum);
     T* U = sc.U + (long long)x0 * kSweepB;
-    const int lane = tid & 31, warp = tid >> 5;
 #pragma unroll
     for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-        for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int x = (warp >> 1) * 32 + 16 * mt + (lane >> 2) + 8 * (q >> 1);
-                const int c = h0 + (warp & 1) * 16 + 8 * nt + 2 * (lane & 3) + (q & 1);
-                if (x < nx && c < nb) U[x * kSweepB + c] = (T)sum[mt][nt][q];
-            }
+        for (int q = 0; q < 4; ++q) {
+            const int x = out_row(mt, q), c = h0 + out_col(q);
+            if (x < nx && c < nb) U[x * kSweepB + c] = (T)sum[mt][q];
+        }
 }
 
 // Two adjacent entries in one load (rows of the scratch are aligned to it).
@@ -286,13 +350,11 @@ __device__ __forceinline__ void load_pair(float& a, float& b, const float* p) {
 // This lane's entries of a scratch row (nb of its 64 entries are set; nb is
 // even).
 template <class T>
-__device__ __forceinline__ void load_scratch_row(T (&v)[2 * kChunkK / 8], const T* p, bool on, int nb) {
-    const int q = threadIdx.x & 3;
+__device__ __forceinline__ void load_scratch_row(T (&v)[kLaneK], const T* p, bool on, int nb) {
 #pragma unroll
-    for (int i = 0; i < kChunkK / 8; ++i) {
-        const int k = 8 * i + 2 * q;
-        v[2 * i] = v[2 * i + 1] = (T)0;
-        if (on && k < nb) load_pair(v[2 * i], v[2 * i + 1], p + k);
+    for (int i = 0; i < kLaneK; i += 2) {
+        v[i] = v[i + 1] = (T)0;
+        if (on && lane_k(i) < nb) load_pair(v[i], v[i + 1], p + lane_k(i));
     }
 }
 
@@ -307,8 +369,7 @@ __device__ void update_strip(const DevView& v, const MergeDesc& D, const SweepSc
     const int n = 2 * D.g, k0 = step * kSweepB, nb = min(kSweepB, n - k0), r0 = ti * kSweepB;
     if (nb <= 0 || r0 >= n) return;                                     // uniform per CTA
     T* A = sweep_matrix<T>(v) + D.W_off;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, row = tid >> 2;
-    const int wr = (warp >> 1) * 32 + (lane >> 2), wc = (warp & 1) * 16 + 2 * (lane & 3);
+    const int tid = threadIdx.x, row = stage_slot();
     h1 = min(h1, (n + kTileN - 1) / kTileN);
     // a half tile formed by a product: not in the swept block's rows or
     // columns, not the next diagonal block (its own item, not read again)
@@ -337,16 +398,18 @@ __device__ void update_strip(const DevView& v, const MergeDesc& D, const SweepSc
     }
     int h = next_product(h0);
     if (h >= h1) return;
-    T vb[2 * kChunkK / 8];
+    T vb[kLaneK];
     load_scratch_row(vb, sc.U + (long long)(h * kTileN + row) * kSweepB, h * kTileN + row < n, nb);
     {
-        T va[2][2 * kChunkK / 8];
+        T va[2][kLaneK];
 #pragma unroll
-        for (int p = 0; p < 2; ++p)
-            load_scratch_row(va[p], sc.C + (long long)(r0 + row + 32 * p) * kSweepB, r0 + row + 32 * p < n, nb);
+        for (int p = 0; p < 2; ++p) {
+            const int r = r0 + row + p * kPassRows;
+            load_scratch_row(va[p], sc.C + (long long)r * kSweepB, r < n, nb);
+        }
         __syncthreads();                                                // the CTA's previous item is done with sm
 #pragma unroll
-        for (int p = 0; p < 2; ++p) stage_row<S>(sm.A, sm.ea, row + 32 * p, nb, va[p]);
+        for (int p = 0; p < 2; ++p) stage_row<S>(sm.A, sm.ea, row + p * kPassRows, nb, va[p]);
     }
     for (;;) {
         const int c0 = h * kTileN;
@@ -354,31 +417,27 @@ __device__ void update_strip(const DevView& v, const MergeDesc& D, const SweepSc
         __syncthreads();
         const int hn = next_product(h + 1);
         if (hn < h1) load_scratch_row(vb, sc.U + (long long)(hn * kTileN + row) * kSweepB, hn * kTileN + row < n, nb);
-        T old[2][2][4];
+        T old[2][4];
 #pragma unroll
         for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-            for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int r = r0 + wr + 16 * mt + 8 * (q >> 1), c = c0 + wc + 8 * nt + (q & 1);
-                    old[mt][nt][q] = r < n && c <= r ? A[(long long)r * n + c] : (T)0;
-                }
-        float acc[S][2][2][4];
+            for (int q = 0; q < 4; ++q) {
+                const int r = r0 + out_row(mt, q), c = c0 + out_col(q);
+                old[mt][q] = r < n && c <= r ? A[(long long)r * n + c] : (T)0;
+            }
+        float acc[S][2][4];
         chunk_mma<S>(sm, nb, acc);
 #pragma unroll
         for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-            for (int nt = 0; nt < 2; ++nt)
+            for (int q = 0; q < 4; ++q) {
+                float l[S];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    float l[S];
-#pragma unroll
-                    for (int i = 0; i < S; ++i) l[i] = acc[i][mt][nt][q];
-                    const T x = (T)combine_levels(l, sm.ea[wr + 16 * mt + 8 * (q >> 1)], sm.eb[wc + 8 * nt + (q & 1)]);
-                    const int r = r0 + wr + 16 * mt + 8 * (q >> 1), c = c0 + wc + 8 * nt + (q & 1);
-                    if (r < n && c <= r) A[(long long)r * n + c] = old[mt][nt][q] - x;
-                }
+                for (int i = 0; i < S; ++i) l[i] = acc[i][mt][q];
+                const T x = (T)combine_levels(l, sm.ea[out_row(mt, q)], sm.eb[out_col(q)]);
+                const int r = r0 + out_row(mt, q), c = c0 + out_col(q);
+                if (r < n && c <= r) A[(long long)r * n + c] = old[mt][q] - x;
+            }
         if (hn >= h1) return;
         h = hn;
         __syncthreads();
@@ -395,10 +454,10 @@ __device__ void next_inverse(const DevView& v, const MergeDesc& D, const SweepSc
     static_assert(sizeof(InvertSmem<T>) <= sizeof(SplitSmem<S>), "the inversion reuses the digits' storage");
     const int n = 2 * D.g, k1 = (step + 1) * kSweepB;
     if (k1 >= n) return;                                                // uniform per CTA
-    const int nb1 = min(kSweepB, n - k1), tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int nb1 = min(kSweepB, n - k1);
     const T* A = sweep_matrix<T>(v) + D.W_off;
-    const int wr = (warp >> 1) * 32 + (lane >> 2), wc = (warp & 1) * 16 + 2 * (lane & 3);
-    typename SplitAcc<S>::T sum[2][2][2][4];
+    typename SplitAcc<S>::T sum[2][2][4];
+#pragma unroll
     for (int h = 0; h < 2; ++h) {
         __syncthreads();
         split_product<S, T, false, false>(
@@ -412,13 +471,11 @@ __device__ void next_inverse(const DevView& v, const MergeDesc& D, const SweepSc
 #pragma unroll
         for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-            for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int r = wr + 16 * mt + 8 * (q >> 1), c = h * kTileN + wc + 8 * nt + (q & 1);
-                    I.A[r][c] = r < nb1 && c <= r ? A[(long long)(k1 + r) * n + k1 + c] - (T)sum[h][mt][nt][q] : (T)0;
-                }
-    invert_checked(v, I, nb1, D.g - k1);
+            for (int q = 0; q < 4; ++q) {
+                const int r = out_row(mt, q), c = h * kTileN + out_col(q);
+                I.A[r][c] = r < nb1 && c <= r ? A[(long long)(k1 + r) * n + k1 + c] - (T)sum[h][mt][q] : (T)0;
+            }
+    invert_checked<kGemmThreads>(v, I, nb1, D.g - k1);
     store_inverse(I, nb1, sc.p(step + 1));
 }
 
@@ -507,7 +564,7 @@ template <class T>
 __global__ void __launch_bounds__(kGemmThreads, 2) block_sweep_kernel(DevView v, int first, int count, int nmax,
                                                                       T* scratch, unsigned int* counter) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ double red[4];
+    __shared__ double red[kGemmWarps];
     __shared__ int s_item;
     unsigned int* work = counter + 1;                       // ticket counter of the update items
     unsigned int wbase = 0, round = 0;
@@ -570,27 +627,30 @@ __global__ void __launch_bounds__(kGemmThreads, 2) block_sweep_kernel(DevView v,
 }
 
 // One CTA per node for levels of many small systems (2g <= 64): T, its
-// inverse and W without leaving shared memory.
+// inverse and W without leaving shared memory.  Four CTAs of four warps per SM:
+// a CTA waits for its chain of pivots most of the time, the others fill in
+// (4096 nodes of 2g = 64, FP64: 0.78 ms, 1.08 with two CTAs of eight warps).
+constexpr int kNodeThreads = 128;
 template <class T>
-__global__ void __launch_bounds__(kGemmThreads) node_invert_kernel(DevView v, int first) {
+__global__ void __launch_bounds__(kNodeThreads, 4) node_invert_kernel(DevView v, int first) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ double red[4];
+    __shared__ double red[kNodeThreads / 32];
     InvertSmem<T>& S = *reinterpret_cast<InvertSmem<T>*>(smem_raw);
     const MergeDesc D = v.merges[first + blockIdx.x];
     const NodeRefs N = node_refs(v, D);
     const int g = N.g, n = N.g2;
     const double* sq = v.gam_sq + D.gamma_off;
     const double* sd = v.gam_sd + D.gamma_off;
-    const double inv_sum = pinned_inv_sum(v, D, red);
-    for (int idx = threadIdx.x; idx < kInvert * kInvert; idx += kGemmThreads) {
+    const double inv_sum = pinned_inv_sum<kNodeThreads>(v, D, red);
+    for (int idx = threadIdx.x; idx < kInvert * kInvert; idx += kNodeThreads) {
         const int r = idx / kInvert, c = idx % kInvert;
         const int i = r < g ? r : r - g, j = c < g ? c : c - g;
         S.A[r][c] = r < n && c <= r ? (T)t_entry(N, c, r, sd[j], sd[i], sq[j], sq[i], inv_sum) : (T)0;
     }
-    invert_checked(v, S, n, g);
+    invert_checked<kNodeThreads>(v, S, n, g);
     double* W = v.W + D.W_off;
     auto at = [&](int r, int c) -> T { return r >= c ? S.A[r][c] : S.A[c][r]; };
-    for (int idx = threadIdx.x; idx < g * g; idx += kGemmThreads) {
+    for (int idx = threadIdx.x; idx < g * g; idx += kNodeThreads) {
         const int i = idx / g, j = idx % g;
         double w[4];
         back_entries(at(i, j), S.A[g + i][j], S.A[g + j][i], at(g + i, g + j), (T)(0.5 * sd[i] * sd[j]), w);
@@ -625,7 +685,7 @@ cudaError_t node_invert(const DevView& v, int first, int count, cudaStream_t s) 
     constexpr int bytes = (int)sizeof(InvertSmem<T>);
     cudaError_t e = cudaFuncSetAttribute(node_invert_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     if (e != cudaSuccess) return e;
-    node_invert_kernel<T><<<count, kGemmThreads, bytes, s>>>(v, first);
+    node_invert_kernel<T><<<count, kNodeThreads, bytes, s>>>(v, first);
     return cudaGetLastError();
 }
 
@@ -654,10 +714,10 @@ cudaError_t launch_node_invert(const DevView& v, int first, int count, bool fp32
 }
 
 cudaError_t launch_merge_x(const DevView& v, int first, int count, int max_g2, int max_m, bool fp32, cudaStream_t s) {
-    return fp32 ? x_launch<4>(v, first, count, max_g2, max_m, s) : x_launch<7>(v, first, count, max_g2, max_m, s);
+    return fp32 ? x_launch<4>(v, first, count, max_g2, max_m, s) : x_launch<8>(v, first, count, max_g2, max_m, s);
 }
-cudaError_t launch_merge_r(const DevView& v, int first, int count, int max_m, bool fp32, cudaStream_t s) {
-    return fp32 ? r_launch<4>(v, first, count, max_m, s) : r_launch<7>(v, first, count, max_m, s);
+cudaError_t launch_merge_r(const DevView& v, int first, int count, int max_g2, int max_m, bool fp32, cudaStream_t s) {
+    return fp32 ? r_launch<4>(v, first, count, max_g2, max_m, s) : r_launch<8>(v, first, count, max_g2, max_m, s);
 }
 
 }  // namespace mrcm

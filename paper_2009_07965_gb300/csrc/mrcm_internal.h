@@ -394,7 +394,7 @@ struct MergeTune {
 // X = -W C and the merged R of one height of blocked merges
 // (kernels_merge_mma.cu).  fp32: the mixed form's precision.
 cudaError_t launch_merge_x(const DevView& v, int first, int count, int max_g2, int max_m, bool fp32, cudaStream_t s);
-cudaError_t launch_merge_r(const DevView& v, int first, int count, int max_m, bool fp32, cudaStream_t s);
+cudaError_t launch_merge_r(const DevView& v, int first, int count, int max_g2, int max_m, bool fp32, cudaStream_t s);
 // T^-1 -> W of one height in blocks of 64 on the tensor cores; scratch:
 // sweep_node_scratch(max_g2) values of the arithmetic type per node.
 __host__ __device__ constexpr long long sweep_node_scratch(int nmax) { return 2LL * nmax * 64 + 2 * 64 * 64; }

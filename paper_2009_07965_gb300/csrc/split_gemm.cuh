@@ -6,39 +6,42 @@
 // of Ootomo, Ozaki and Yokota, "DGEMM on integer matrix multiplication unit",
 // IJHPCA 2024, here with FP16 operands and FP32 accumulators holding
 // integers): within one chunk of k (kChunkK entries) a row of A is written
-// as 2^(Ea - 1076) V, V an integer of at most 54 bits and a sign, and V as
-// S = 7 digits of 8 bits, d in [-128, 127] (|d_0| <= 64); a row of B (a column of the
+// as 2^(Ea - 1085) V, V an integer of at most 63 bits and a sign, and V as
+// S = 8 digits of 8 bits, d in [-128, 128]; a row of B (a column of the
 // product's right factor, read along k) likewise.  Digit products are exact
 // in FP16 x FP16 -> FP32, and all products of one level l = i + j are summed
-// in one accumulator: at most 7 x 64 terms of magnitude 2^14, below 2^24, so
+// in one accumulator: at most 8 x 64 terms of magnitude 2^14, below 2^24, so
 // every sum is an exact integer.  Levels past S - 1 are dropped (below
-// 2^-54 of the largest product); 28 products of digits remain.  At the end
-// of a chunk the seven integers of an output are combined in 64-bit integer
+// 2^-62 of the largest product); 36 products of digits remain.  At the end
+// of a chunk the eight integers of an output are combined in 64-bit integer
 // arithmetic, rounded once to FP64 and added to the running sum.
 //
-// Against an FP64 fused multiply-add loop: operands are rounded to 2^-54 of
-// the largest entry of their row in the chunk (an FP64 operand is exact, but
-// every addition of the loop rounds), and only one rounding per 64 terms
-// follows.
+// Against an FP64 fused multiply-add loop: an operand is exact unless it is
+// more than 2^10 below the largest entry of its row in the chunk (then it is
+// rounded to 2^-63 of that entry), and one rounding per 64 terms takes the
+// place of one per term.
 //
-// S = 4 (30 bits, 10 digit products) serves the FP32 merges of the mixed
+// S = 4 (31 bits, 10 digit products) serves the FP32 merges of the mixed
 // form: more than an FP32 operand's 24 bits of the largest entry, sums
 // exact up to the one FP32 rounding per chunk.
 //
-// Work split.  A CTA of four warps forms a 64 x 32 tile of the product; a
-// warp a 32 x 16 part of it with all levels in registers (7 x 16
-// accumulators), so that a k-step of 16 loads 21 fragments from shared
-// memory for 112 MMAs.  The digits are cut by the CTA that uses them (about
-// 30 integer instructions per entry, hidden behind the other resident CTA's
-// MMAs: two CTAs of 97 KB per SM); digits kept in global memory would cost
-// 14 bytes per entry and more L2 bandwidth than the FP64 entries do.
+// Work split.  A CTA of eight warps forms a 64 x 32 tile of the product; a
+// warp a 32 x 8 part of it with all levels in registers (8 x 8
+// accumulators), so that a k-step of 16 loads 20 fragments from shared
+// memory for 72 MMAs.  The digits are cut by the CTA that uses them (about
+// 25 integer instructions per entry, hidden behind the other resident CTA's
+// MMAs: two CTAs of 97 KB and 16 warps per SM); digits kept in global memory
+// would cost 16 bytes per entry and more L2 bandwidth than the FP64 entries
+// do.  Shared memory holds a digit row's 64 entries in 8 units of 16 bytes,
+// unit u at u ^ (row % 8): the eight rows an ldmatrix reads and the four rows
+// a staging warp writes then lie in distinct banks.
 //
-// Measured (4096^2 quarter-five-spot, all heights, one GB300): X 14.46 ->
-// 2.29 ms, R 12.65 -> 2.75 ms against FP64 FMA loops at 97 and 92% of the
-// FP64 peak; 7 to 9 TFLOP/s of FP64 products.  Tensor pipe 35% busy, stalls
-// mostly on fixed latencies with two warps per scheduler.  Node maps against
-// quadruple precision (sigma^2 = 1..4, alpha = 0.5..2): relative errors
-// 4e-17..3e-16, those of the FMA loops to within 20%.
+// Measured (one GB300, all heights): 4096^2 X 14.46 -> 2.33 ms, R 12.65 -> 2.41
+// against FP64 FMA loops at 97 and 92% of the FP64 peak; box 128x128x64 X
+// 27.5 -> 4.7, R 23.6 -> 5.5.  Seven digits in four warps per CTA were as fast
+// (2.25 and 2.67 ms) and less exact: node maps against quadruple precision 2.1e-15
+// at alpha = 100 (now 1.9e-16, the FMA loops 2.4e-16), boxes against a dense
+// FP64 solution 6.3e-13 (now 2.6e-13, the FMA loops 2.7e-13).
 #pragma once
 #include <cuda_fp16.h>
 #include "mrcm_internal.h"
@@ -48,21 +51,44 @@ namespace {
 
 constexpr int kChunkK = 64;              // k entries staged (and scaled) at a time
 constexpr int kTileM = 64, kTileN = 32;  // product tile of a CTA
-constexpr int kGemmThreads = 128;
-constexpr int kSmemStride = kChunkK + 8; // halves per staged row: 144 bytes, an odd number of 16-byte
-                                         // units (ldmatrix rows and the digit stores hit distinct banks)
+constexpr int kGemmThreads = 256, kGemmWarps = kGemmThreads / 32;
+
+template <class T> struct Slices { static constexpr int S = 8; };
+template <> struct Slices<float> { static constexpr int S = 4; };
 
 template <int S>
 struct SplitSmem {
-    __half A[S][kTileM][kSmemStride];
-    __half B[S][kTileN][kSmemStride];
+    __half A[S][kTileM][kChunkK];
+    __half B[S][kTileN][kChunkK];
     int ea[kTileM], eb[kTileN];          // largest biased exponent of each row in the chunk
 };
+// Position of entry k of a staged row.
+__device__ __forceinline__ int swizzled(int row, int k) { return ((k >> 3) ^ (row & 7)) * 8 + (k & 7); }
+
+// Staging: a pass of the CTA covers 32 rows, eight lanes per row, entries
+// 16 i + 2 q and 16 i + 2 q + 1 (i < kLaneK / 2) on lane q, so that the lanes of
+// a row read 128 consecutive bytes.
+constexpr int kLaneK = kChunkK / 8;      // entries of a row per lane
+constexpr int kPassRows = kGemmThreads / 8;
+__device__ __forceinline__ int stage_q() { return threadIdx.x & 7; }
+__device__ __forceinline__ int stage_slot() {          // row of this lane within a pass
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    return 8 * (warp >> 1) + (warp & 1) + 2 * (lane >> 3);
+}
+__device__ __forceinline__ int lane_k(int i) { return 16 * (i >> 1) + 2 * stage_q() + (i & 1); }
+
+// The warp's 32 x 8 part of a tile: output r of the 16 x 8 tile mt lies in
+// row out_row(mt, r), column out_col(r).
+__device__ __forceinline__ int warp_m0() { return ((threadIdx.x >> 5) >> 2) * 32; }
+__device__ __forceinline__ int warp_n0() { return ((threadIdx.x >> 5) & 3) * 8; }
+__device__ __forceinline__ int out_row(int mt, int r) {
+    return warp_m0() + 16 * mt + ((threadIdx.x & 31) >> 2) + 8 * (r >> 1);
+}
+__device__ __forceinline__ int out_col(int r) { return warp_n0() + 2 * (threadIdx.x & 3) + (r & 1); }
 
 // The digits of |x| relative to the row exponent E, one byte each (the
 // leading digit as it is, in [0, 128]; the others + 128), the last digit in
-// the lowest byte.  S = 7 leaves 0x64 in the highest byte, the upper half of
-// the FP16 number 1024 + byte.
+// the lowest byte.
 __device__ __forceinline__ unsigned high_word(double x) { return (unsigned)__double2hiint(x); }
 __device__ __forceinline__ unsigned high_word(float x) { return __float_as_uint(x); }
 __device__ __forceinline__ int exponent_bits(double x) { return __double2hiint(x) & 0x7ff00000; }
@@ -70,10 +96,10 @@ __device__ __forceinline__ int exponent_bits(float x) { return __float_as_int(x)
 template <int S>
 __device__ __forceinline__ unsigned long long digit_bytes(double x, int E) {
     const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-    const int d = min(E - (int)((hi >> 20) & 0x7ffu), S == 7 ? 63 : 39);
-    const unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 34) | ((unsigned long long)lo << 2);
-    if (S == 7) return (m >> d) + 0x6400808080808080ull;
-    return (m >> (d + 24)) + 0x00808080ull;
+    const int d = min(E - (int)((hi >> 20) & 0x7ffu), S == 8 ? 63 : 31);
+    const unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 42) | ((unsigned long long)lo << 10);
+    if (S == 8) return (m >> d) + 0x0080808080808080ull;
+    return (m >> (d + 32)) + 0x00808080ull;
 }
 template <int S>
 __device__ __forceinline__ unsigned digit_bytes(float x, int E) {       // S = 4
@@ -94,12 +120,9 @@ __device__ __forceinline__ void digit_pair(T x, T y, int E, unsigned (&out)[S]) 
     const unsigned off = (sg & 0x80008000u) ^ 0xe480e480u, off0 = (sg & 0x80008000u) ^ 0xe400e400u;
 #pragma unroll
     for (int s = 0; s < S; ++s) {
-        const int byte = S - 1 - s;              // digit s (0: the leading one)
-        unsigned w;
-        if (S == 7 && byte >= 4)
-            w = __byte_perm((unsigned)(ua >> 32), (unsigned)(ub >> 32), (byte - 4) | 3 << 4 | byte << 8 | 7 << 12);
-        else
-            w = (__byte_perm((unsigned)ua, (unsigned)ub, byte | (4 + byte) << 8) & 0x00ff00ffu) | 0x64006400u;
+        const int byte = S - 1 - s, b = byte & 3;    // digit s (0: the leading one)
+        const unsigned wa = (unsigned)(byte >= 4 ? ua >> 32 : ua), wb = (unsigned)(byte >= 4 ? ub >> 32 : ub);
+        const unsigned w = (__byte_perm(wa, wb, b | (4 + b) << 8) & 0x00ff00ffu) | 0x64006400u;   // 1024 + byte
         const __half2 h = __hfma2(*reinterpret_cast<const __half2*>(&w), *reinterpret_cast<const __half2*>(&one),
                                   *reinterpret_cast<const __half2*>(s == 0 ? &off0 : &off));
         out[s] = *reinterpret_cast<const unsigned*>(&h);
@@ -112,27 +135,24 @@ __device__ __forceinline__ int common_exponent(int E) {
     return sizeof(T) == 8 || E == 0 ? E : (E == 255 ? 2047 : E + 896);
 }
 
-// Writes the digit pairs (k, k + 1) of one row's 16 entries held by this
-// lane (entries 8 i + 2 q and 8 i + 2 q + 1 of the chunk).
+// Writes the digit pairs of this lane's entries of one row (eight lanes).
 template <int S, int ROWS, class T>
-__device__ __forceinline__ void stage_row(__half (*dst)[ROWS][kSmemStride], int* e, int row, int kn,
-                                          const T (&v)[2 * kChunkK / 8]) {
-    const int q = threadIdx.x & 3;
+__device__ __forceinline__ void stage_row(__half (*dst)[ROWS][kChunkK], int* e, int row, int kn, const T (&v)[kLaneK]) {
     int E = 0;
 #pragma unroll
-    for (int i = 0; i < 2 * kChunkK / 8; ++i) E = max(E, exponent_bits(v[i]));
-    E = max(E, __shfl_xor_sync(0xffffffffu, E, 1));
-    E = max(E, __shfl_xor_sync(0xffffffffu, E, 2));
+    for (int i = 0; i < kLaneK; ++i) E = max(E, exponent_bits(v[i]));
+#pragma unroll
+    for (int w = 1; w < 8; w <<= 1) E = max(E, __shfl_xor_sync(0xffffffffu, E, w));
     E = sizeof(T) == 8 ? E >> 20 : E >> 23;
-    if (q == 0) e[row] = common_exponent<T>(E);
+    if (stage_q() == 0) e[row] = common_exponent<T>(E);
     const int kend = (kn + 15) & ~15;
 #pragma unroll
-    for (int i = 0; i < kChunkK / 8; ++i) {
+    for (int i = 0; i < kLaneK; i += 2) {
         if (8 * i >= kend) break;
         unsigned d[S];
-        digit_pair<S>(v[2 * i], v[2 * i + 1], E, d);
+        digit_pair<S>(v[i], v[i + 1], E, d);
 #pragma unroll
-        for (int s = 0; s < S; ++s) *reinterpret_cast<unsigned*>(&dst[s][row][8 * i + 2 * q]) = d[s];
+        for (int s = 0; s < S; ++s) *reinterpret_cast<unsigned*>(&dst[s][row][swizzled(row, lane_k(i))]) = d[s];
     }
 }
 
@@ -149,56 +169,56 @@ __device__ __forceinline__ void mma_f16(float (&c)[4], const unsigned (&a)[4], u
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// The digit products of the staged chunk: acc[l][mt][nt] += level l of the
-// warp's 16 x 8 tiles (mt, nt).
+// The digit products of the staged chunk: acc[l][mt] += level l of the warp's
+// 16 x 8 tile mt.
 template <int S>
-__device__ __forceinline__ void chunk_mma(const SplitSmem<S>& sm, int kn, float (&acc)[S][2][2][4]) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int m0 = (warp >> 1) * 32, n0 = (warp & 1) * 16;
-    const int arow = m0 + (lane & 15), acol = (lane >> 4) * 8;
-    const int brow = n0 + (lane & 7) + (lane >> 4) * 8, bcol = ((lane >> 3) & 1) * 8;
+__device__ __forceinline__ void chunk_mma(const SplitSmem<S>& sm, int kn, float (&acc)[S][2][4]) {
+    const int lane = threadIdx.x & 31;
+    const int arow = warp_m0() + (lane & 15), brow = warp_n0() + (lane & 7);
 #pragma unroll
     for (int l = 0; l < S; ++l)
 #pragma unroll
         for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-            for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-                for (int r = 0; r < 4; ++r) acc[l][mt][nt][r] = 0.f;
+            for (int r = 0; r < 4; ++r) acc[l][mt][r] = 0.f;
 #pragma unroll 1
     for (int k0 = 0; k0 < kn; k0 += 16) {
-        unsigned b[S][4];
+        const int ak = swizzled(arow, k0 + (lane >> 4) * 8), bk = swizzled(brow, k0 + ((lane >> 3) & 1) * 8);
+        unsigned b[S / 2][4];                     // two digits of B per load
 #pragma unroll
-        for (int j = 0; j < S; ++j) ldmatrix_x4(b[j], &sm.B[j][brow][k0 + bcol]);
+        for (int j = 0; j < S / 2; ++j) ldmatrix_x4(b[j], &sm.B[2 * j + (lane >> 4)][brow][bk]);
 #pragma unroll
         for (int i = 0; i < S; ++i) {
             unsigned a[2][4];
 #pragma unroll
-            for (int mt = 0; mt < 2; ++mt) ldmatrix_x4(a[mt], &sm.A[i][arow + 16 * mt][k0 + acol]);
+            for (int mt = 0; mt < 2; ++mt) ldmatrix_x4(a[mt], &sm.A[i][arow + 16 * mt][ak]);
 #pragma unroll
             for (int j = 0; j < S - i; ++j)
 #pragma unroll
                 for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-                    for (int nt = 0; nt < 2; ++nt) mma_f16(acc[i + j][mt][nt], a[mt], b[j][2 * nt], b[j][2 * nt + 1]);
+                    mma_f16(acc[i + j][mt], a[mt], b[j >> 1][2 * (j & 1)], b[j >> 1][2 * (j & 1) + 1]);
         }
     }
 }
 
 // One output of a chunk in FP64 from its level sums and the exponents of its
-// row and column.
-__device__ __forceinline__ double combine_levels(const float (&n)[7], int ea, int eb) {
+// row and column: v + w 2^-14 in units of 2^-42 of a leading digit product,
+// both exact integers; v is moved up by as many bits (at most 14) as it
+// leaves free, so that w enters where it matters, and the sum is rounded once.
+__device__ __forceinline__ double combine_levels(const float (&n)[8], int ea, int eb) {
+    const int w = (__float2int_rn(n[6]) << 8) + __float2int_rn(n[7]);
     const int m = (__float2int_rn(n[4]) << 8) + __float2int_rn(n[5]);
     const int h = (__float2int_rn(n[2]) << 8) + __float2int_rn(n[3]);
     const int t = (__float2int_rn(n[0]) << 8) + __float2int_rn(n[1]);
-    const long long low = (long long)m * 4 + ((__float2int_rn(n[6]) + 32) >> 6);
-    const long long v = ((long long)(t << 2) << 32) + (long long)h * 262144 + low;      // |v| < 2^63
-    const unsigned long long s = (unsigned long long)(v >> 63), u = ((unsigned long long)v ^ s) - s;
+    const long long v = ((long long)(t << 2) << 32) + (long long)h * 262144 + (long long)m * 4;    // |v| < 2^63
+    const int up = min(14, max(__clzll((long long)((unsigned long long)v ^ (unsigned long long)(v >> 63))) - 2, 0));
+    const long long x = (long long)((unsigned long long)v << up) + (w >> (14 - up));
+    const unsigned long long s = (unsigned long long)(x >> 63), u = ((unsigned long long)x ^ s) - s;
     const int lz = __clzll((long long)u);
     // leading bit to bit 62, rounded at bit 10; the carry of the rounding
     // moves into the exponent field
-    const unsigned long long mant = ((u << (lz - 1)) + 0x200ull) >> 10;
-    const int be = ea + eb - lz - 1014;
+    const unsigned long long mant = ((u << ((lz - 1) & 63)) + 0x200ull) >> 10;
+    const int be = ea + eb - lz - 1014 - up;
     unsigned long long bits = ((unsigned long long)(be - 1) << 52) + mant;
     if (u == 0 || be <= 0) bits = 0;                                          // zero or underflow
     if (be >= 2047) bits = 0x7ff0000000000000ull;                             // overflow
@@ -215,79 +235,113 @@ __device__ __forceinline__ float combine_levels(const float (&n)[4], int ea, int
     const float f = v * pow2f(ea - 1041) * pow2f(eb - 1041);
     return (ea == 2047 || eb == 2047) ? __int_as_float(0x7fc00000) : f;
 }
+// x as a double by integer operations (a conversion instruction holds the
+// FP64 pipe like an FP64 instruction); FP32 subnormals count as zero.
+__device__ __forceinline__ double widen(float x) {
+    const unsigned b = __float_as_uint(x), e = (b >> 23) & 0xffu;
+    const unsigned hi = e == 0 ? 0u : (e == 255 ? 0x7ff00000u : (e + 896u) << 20) | ((b & 0x7fffffu) >> 3);
+    return __hiloint2double((int)(hi | (b & 0x80000000u)), e == 0 ? 0 : (int)(b << 29));
+}
+__device__ __forceinline__ double widen(double x) { return x; }
 template <int S> struct SplitAcc { using T = double; };
 template <> struct SplitAcc<4> { using T = float; };
 
-// The 16 entries 8 i + 2 q (+ 1) of a row from p on (nullptr: zeros), through
-// the index registers ix when the row is gathered.
+// This lane's entries of a row from p on (nullptr: zeros), through the index
+// registers ix when the row is gathered.
 template <bool GATHER, class T>
-__device__ __forceinline__ void load_row(T (&v)[2 * kChunkK / 8], const T* p, const int (&ix)[2 * kChunkK / 8],
-                                         int kn) {
-    const int q = threadIdx.x & 3;
+__device__ __forceinline__ void load_row(T (&v)[kLaneK], const T* p, const int (&ix)[kLaneK], int kn) {
 #pragma unroll
-    for (int i = 0; i < 2 * kChunkK / 8; ++i) {
-        const int k = 8 * (i >> 1) + 2 * q + (i & 1);
-        v[i] = (p && k < kn) ? p[GATHER ? ix[i] : k] : (T)0;
-    }
+    for (int i = 0; i < kLaneK; ++i) v[i] = (p && lane_k(i) < kn) ? p[GATHER ? ix[i] : lane_k(i)] : (T)0;
+}
+template <bool ON>
+__device__ __forceinline__ void load_index(int (&ix)[kLaneK], const int* idx, int kn) {
+#pragma unroll
+    for (int i = 0; i < kLaneK; ++i) ix[i] = (ON && lane_k(i) < kn) ? idx[lane_k(i)] : 0;
 }
 
-// The warp's part of sum_k A(row, k) B(col, k), k < K (K >= 1): sum[mt][nt][r] for
-// row m0 + 16 mt + lane / 4 + 8 (r / 2), column n0 + 8 nt + 2 (lane % 4) +
-// (r % 2).  arow(row) / brow(col): pointer to the operand's row (nullptr:
-// zeros), entry k at [k], or at [idx[k]] where AG / BG say that the operand
-// is gathered.
+// The warp's part of sum_k A(row, k) B(col, k), k < K (K >= 1), at row
+// out_row(mt, r), column out_col(r).  arow(row) / brow(col): pointer to the
+// operand's row (nullptr: zeros), entry k at [k], or at [idx[k]] where AG /
+// BG say that the operand is gathered.
 template <int S, class T, bool AG, bool BG, class ASrc, class BSrc>
 __device__ __forceinline__ void split_product(SplitSmem<S>& sm, int K, const int* idx, ASrc&& arow, BSrc&& brow,
-                                              typename SplitAcc<S>::T (&sum)[2][2][4]) {
-    constexpr int kPer = 2 * kChunkK / 8;             // entries of a row per lane
-    constexpr int kRows = kGemmThreads / 4;           // rows staged per pass
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, q = lane & 3, row = threadIdx.x >> 2;
-    const int m0 = (warp >> 1) * 32, n0 = (warp & 1) * 16;
-    const T *pa[kTileM / kRows], *pb[kTileN / kRows];
-#pragma unroll
-    for (int p = 0; p < kTileM / kRows; ++p) pa[p] = arow(row + p * kRows);
-#pragma unroll
-    for (int p = 0; p < kTileN / kRows; ++p) pb[p] = brow(row + p * kRows);
+                                              typename SplitAcc<S>::T (&sum)[2][4]) {
+    const int row = stage_slot();
+    const T *pa[2] = {arow(row), arow(row + kPassRows)}, *pb = brow(row);
 #pragma unroll 1
     for (int k0 = 0; k0 < K; k0 += kChunkK) {
         const int kn = min(kChunkK, K - k0);
         {
-            int ix[kPer];
-#pragma unroll
-            for (int i = 0; i < kPer; ++i) {
-                const int k = 8 * (i >> 1) + 2 * q + (i & 1);
-                ix[i] = ((AG || BG) && k < kn) ? idx[k0 + k] : 0;
-            }
+            int ix[kLaneK];
+            load_index<AG || BG>(ix, idx + k0, kn);
             // every row's entries in flight together
-            T va[kTileM / kRows][kPer], vb[kTileN / kRows][kPer];
+            T va[2][kLaneK], vb[kLaneK];
 #pragma unroll
-            for (int p = 0; p < kTileM / kRows; ++p)
-                load_row<AG>(va[p], pa[p] ? pa[p] + (AG ? 0 : k0) : nullptr, ix, kn);
-#pragma unroll
-            for (int p = 0; p < kTileN / kRows; ++p)
-                load_row<BG>(vb[p], pb[p] ? pb[p] + (BG ? 0 : k0) : nullptr, ix, kn);
+            for (int p = 0; p < 2; ++p) load_row<AG>(va[p], pa[p] ? pa[p] + (AG ? 0 : k0) : nullptr, ix, kn);
+            load_row<BG>(vb, pb ? pb + (BG ? 0 : k0) : nullptr, ix, kn);
             if (k0) __syncthreads();                  // the previous chunk's digits are read
 #pragma unroll
-            for (int p = 0; p < kTileM / kRows; ++p) stage_row<S>(sm.A, sm.ea, row + p * kRows, kn, va[p]);
-#pragma unroll
-            for (int p = 0; p < kTileN / kRows; ++p) stage_row<S>(sm.B, sm.eb, row + p * kRows, kn, vb[p]);
+            for (int p = 0; p < 2; ++p) stage_row<S>(sm.A, sm.ea, row + p * kPassRows, kn, va[p]);
+            stage_row<S>(sm.B, sm.eb, row, kn, vb);
         }
         __syncthreads();
-        float acc[S][2][2][4];
+        float acc[S][2][4];
         chunk_mma<S>(sm, kn, acc);
 #pragma unroll
         for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-            for (int nt = 0; nt < 2; ++nt)
+            for (int r = 0; r < 4; ++r) {
+                float n[S];
 #pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    float n[S];
+                for (int l = 0; l < S; ++l) n[l] = acc[l][mt][r];
+                const auto c = combine_levels(n, sm.ea[out_row(mt, r)], sm.eb[out_col(r)]);
+                sum[mt][r] = k0 ? sum[mt][r] + c : c;
+            }
+    }
+}
+
+// The same for a strip of the product with K <= kChunkK: 64 rows of A, whose
+// digits are cut once, by the 32-column tiles t0 <= t < t1.  A tile's rows of
+// B and the values pre(t, row, column) that its epilogue needs are loaded
+// while the products of the tile before run; epi(t, row, column, product,
+// pre) receives every entry.
+template <int S, bool AG, bool BG, class ASrc, class BSrc, class Pre, class Epi>
+__device__ __forceinline__ void strip_product(SplitSmem<S>& sm, int K, const int* idx, int t0, int t1, ASrc&& arow,
+                                              BSrc&& brow, Pre&& pre, Epi&& epi) {
+    const int row = stage_slot();
+    int ix[kLaneK];
+    load_index<AG || BG>(ix, idx, K);
+    double vb[kLaneK];
+    load_row<BG>(vb, brow(t0, row), ix, K);
+    {
+        double va[2][kLaneK];
 #pragma unroll
-                    for (int l = 0; l < S; ++l) n[l] = acc[l][mt][nt][r];
-                    const auto c = combine_levels(n, sm.ea[m0 + 16 * mt + (lane >> 2) + 8 * (r >> 1)],
-                                                  sm.eb[n0 + 8 * nt + 2 * (lane & 3) + (r & 1)]);
-                    sum[mt][nt][r] = k0 ? sum[mt][nt][r] + c : c;
-                }
+        for (int p = 0; p < 2; ++p) load_row<AG>(va[p], arow(row + p * kPassRows), ix, K);
+#pragma unroll
+        for (int p = 0; p < 2; ++p) stage_row<S>(sm.A, sm.ea, row + p * kPassRows, K, va[p]);
+    }
+    for (int t = t0; t < t1; ++t) {
+        if (t > t0) __syncthreads();                  // the tile before is done with sm.B
+        stage_row<S>(sm.B, sm.eb, row, K, vb);
+        __syncthreads();
+        if (t + 1 < t1) load_row<BG>(vb, brow(t + 1, row), ix, K);
+        double old[2][4];
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+            for (int r = 0; r < 4; ++r) old[mt][r] = pre(t, out_row(mt, r), out_col(r));
+        float acc[S][2][4];
+        chunk_mma<S>(sm, K, acc);
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                float n[S];
+#pragma unroll
+                for (int l = 0; l < S; ++l) n[l] = acc[l][mt][r];
+                const int i = out_row(mt, r), j = out_col(r);
+                epi(t, i, j, widen(combine_levels(n, sm.ea[i], sm.eb[j])), old[mt][r]);
+            }
     }
 }
 

@@ -1,6 +1,8 @@
 """The merged maps of blocked merges (2g > 32), whose products X = -W C and
 R = R_oo + C^T X run as split products on the tensor cores, against the same
-merge formed on the host from the children's maps.
+merge formed on the host from the children's maps; the last test does so on
+levels large enough for the block sweep (count (2g)^2 >= 540000) and the
+strips.
 
 The sizes put 2g, m and the two children's shares of m on and off the edges
 of the 64 x 32 product tiles and of the 64-entry chunks of k, odd ones among
@@ -72,3 +74,39 @@ def test_blocked_merges_match_the_host(mrcm_lib, nx, ny, seg, alpha, precision, 
         e = rel(mr.mrcm_node_operator(s.ctx, v), _merge_on_host(mr, s.ctx, prob, v))
         assert e <= tol, (shape, e)
     s.close()
+
+
+@pytest.mark.parametrize("precision,tol", [("fp64", 3e-11), ("mixed", 1.5e-3)])
+def test_block_sweep_levels_match_the_host(mrcm_lib, precision, tol):
+    # 40 problems of 170 x 147 cells, one-face segments: 2g = 294 at the root's
+    # children's level, 170 and 148 below (a last block of 38, 42 or 20 rows)
+    import torch
+    import paper_2009_07965_gb300 as mr
+    probs = [inputs.darcy_problem(170, 147 + 3 * (k % 2), sigma2=2.0, corr=0.1, seed=90 + k, bc="left_right",
+                                  seg=(1, 1)) for k in range(40)]
+    b = mr.BatchSolver([torch.from_numpy(p.K).cuda() for p in probs], [(p.Lx, p.Ly) for p in probs],
+                       [p.bc_type for p in probs], sub=probs[0].sub, seg=(1, 1), alpha=1.0,
+                       precision=mr.binding.MRCM_FP64 if precision == "fp64" else mr.binding.MRCM_MIXED)
+    b.build_basis()
+    count, first = {}, {}
+    nodes = mr.mrcm_query(b.ctx, "NODES")
+    owner = [-1] * nodes
+    roots = [v for v in range(nodes) if mr.mrcm_node_info(b.ctx, v)["parent"] < 0]
+    for k, r in enumerate(roots):
+        stack = [r]
+        while stack:
+            v = stack.pop()
+            owner[v] = k
+            i = mr.mrcm_node_info(b.ctx, v)
+            stack += [c for c in (i["c1"], i["c2"]) if c >= 0]
+    for v in range(mr.mrcm_query(b.ctx, "LEAVES"), nodes):
+        i = mr.mrcm_node_info(b.ctx, v)
+        if i["m"] > 0 and i["g"] > 32:
+            count[i["height"]] = count.get(i["height"], 0) + 1
+            first.setdefault((i["height"], i["g"], i["m"]), v)
+    blocked = {s: v for s, v in first.items() if count[s[0]] * (2 * s[1]) ** 2 >= 540000}
+    assert len(blocked) >= 3 and any(2 * s[1] % 64 for s in blocked)
+    for s, v in blocked.items():
+        e = rel(mr.mrcm_node_operator(b.ctx, v), _merge_on_host(mr, b.ctx, probs[owner[v]], v))
+        assert e <= tol, (s, e)
+    b.close()
