@@ -1,4 +1,5 @@
-// Leaf kernels: the local Robin problems of every finest-level subdomain.
+// Leaf kernels: the local Robin problems of every finest-level block, 2D
+// leaves and 3D patch-shaped blocks alike.
 //
 // arXiv 2009.07965, Eqs. (11.2)-(12.2) on one leaf with lumped RT0 (two-point
 // fluxes).  On a skeleton face e of segment t the Robin term gives the
@@ -13,540 +14,674 @@
 // the traces of all MMBFs of the leaf (coefficient-tracking remark, Section
 // 3.2); bbar carries the source and external boundary data (Eqs. addu, addp).
 //
-// Layout and mapping.  16 threads own one leaf (two leaves per warp, four
-// per CTA so that a 64 x 64-leaf grid fits in one wave); cells are ordered x
-// fastest, so A is banded with half-bandwidth w (leaf width).  A = L D L^T
-// is factored right-looking over a circular window of w+2 band rows in
-// shared memory; each step also advances the multi-right-hand-side forward
-// solve Z = L^-1 B and accumulates R += z_k z_k^T / d_k, so no column of L is
-// read twice.  The columns of B are taken in the order of their first
-// nonzero row, so the structurally zero upper part of Z is skipped and the
-// remaining work is spread evenly over the 16 lanes (a masked FP64 lane
-// costs as much as a busy one).  The multipliers L, 1/d and Z are written to
-// global memory for the solve phase.
+// Elimination.  A leaf is a stack of H planes of nb <= 16 cells (2D: the grid
+// rows of the leaf; 3D: its x-y planes), and the two-point coupling between
+// neighbouring planes is diagonal: A is block tridiagonal with diagonal
+// off-diagonal blocks -T_k.  It is eliminated plane by plane from both ends
+// towards a middle plane M = H / 2 (half the sequential chain of an
+// elimination from one end, and fewer columns of B meet each plane):
+//     S_k = A_k - T P T (P of the plane eliminated before),   P_k = S_k^-1,
+//     Z_k = B_k + T P Z,   y_k = b_k + T P y                   (likewise),
+// with both neighbours' contributions at M.  Then
+//     R = sum_k Z_k^T P_k Z_k - W,   rbar = sum_k Z_k^T P_k y_k,
+//     x_M = P_M y_M,   x_k = P_k (y_k + T x of the plane next to it towards M).
+// The explicit P_k make every pass of the solve phase a chain of H / 2 + 1
+// small matrix-vector products.
+//
+// Arithmetic.  An FP64 instruction holds its scheduler's FP64 pipe for 64
+// cycles, so the FP64 instructions of a warp set the pace: only the
+// inversions of S_k (Gauss-Jordan on the lower triangle, no pivot search: S_k
+// is SPD) and the diagonal scalings run there; the products V = P Z and
+// Z^T V go to the tensor cores as split products (split_gemm.cuh) on
+// fragments cut from shared memory.
+//
+// Measured against the elimination cell by cell (banded LDL^T, FP64 FMA loops)
+// of before: build 4096^2 13.4 -> 9.4 ms, 333x517 with two-face segments 2.86 ->
+// 0.47, box 256x256x64 34.9 -> 16.8; particular problems and pressures of
+// 1500x700 per pass 0.20 and 0.22 -> 0.11 and 0.12, of 256x256x64 3.3 and 3.0 ->
+// 2.1 and 1.1 (4096^2 1.21 and 1.08 -> 1.22 and 1.11: FP64 pipe either way).
+// Of the build's 9.4 ms, 6.0 are FP64 instructions (1690 per leaf, 64 cycles
+// each).
+//
+// Stored for the solve phase: P_k (nb x nb per plane, planes in order) and Z_k
+// (nb x c_k, column-major, only the c_k columns that have met the plane): the
+// planes below M, then M, then the planes from H - 1 down to M + 1.
+#include "block_invert.cuh"
+#include "leaf_geometry.cuh"
 #include "mrcm_internal.h"
+#include "split_gemm.cuh"
+
+#include <algorithm>
 
 namespace mrcm {
 namespace {
 
-constexpr int kWin = kMaxLeafSide + 2;   // circular window rows
+constexpr int kTeams = 4;         // independent warps of a build CTA (leaf_build_kernel)
 
-// T: the arithmetic of the factorisation (double; float in the mixed form).
-template <int MMAX, class T>
+// Shared memory of one leaf of a build CTA; mp, cz: the launch's largest
+// segment count and the largest column count off the middle plane.
+constexpr int kTriP = kPlane * (kPlane + 1) / 2;
+__host__ __device__ __forceinline__ int tri_at(int r, int c) {
+    const int hi = r > c ? r : c, lo = r > c ? c : r;
+    return hi * (hi + 1) / 2 + lo;
+}
+template <int DIM, class T>
 struct LeafBuildSmem {
-    T win[kWin][kMaxLeafSide + 1];       // win[row % (w+2)][o] = A[row][row - o]
-    T zw[kWin][MMAX + 1];                // rows of Z being updated (ordered columns)
-    T R[MMAX][MMAX + 1];                 // lower triangle of B^T A^-1 B (ordered)
-    double W[MMAX];                      // sum of rho per segment (ordered)
-    T lcol[kMaxLeafSide];                // column k of L below the diagonal
-    T zk[MMAX];                          // row k of Z (ordered)
-    T uk[MMAX];                          // row k of Z / d_k (ordered)
-    int order[MMAX];                     // ordered column q -> local segment
-    int pos[MMAX];                       // local segment -> ordered column
-    int start[MMAX];                     // first row with a nonzero, per ordered column
-    double dg[kLeafThreads];             // diagonal entries of the next rows to enter (row % 16)
+    T (*P)[kTriP];                  // [2]: the halves' current P (lower triangle, zero outside nb)
+    T (*Z)[kPlane + 1];             // [2 cz]: the halves' current Z, by column; V of the middle plane
+    T (*V)[kPlane + 1];             // [mp]: P Z; Z of the middle plane
+    double* R;                      // packed lower triangle (local segments)
+    T (*col)[2][kColSize];          // [2]: pivot columns of each half (sweep_block)
+    double (*dg)[kPlane];           // [2]: diagonal of the plane, couplings to cell i - 1 and
+    double (*cx)[kPlane];           // i - w0, to the plane before and to the one after
+    double (*cy)[kPlane];           // (3D)
+    double (*tp)[kPlane];
+    double (*tn)[kPlane];
+    short *ord, *pos;               // [2 mp]: column -> segment and back, per half
+    __host__ __device__ static int zrows(int mp, int cz) { return 2 * cz > mp ? 2 * cz : mp; }
+    __host__ __device__ static size_t bytes(int mp, int cz) {
+        size_t t = sizeof(T) * (2 * kTriP + (zrows(mp, cz) + mp) * (kPlane + 1) + 4 * kColSize);
+        t = (t + 7) / 8 * 8 + sizeof(double) * ((size_t)mp * (mp + 1) / 2 + (DIM == 3 ? 10 : 8) * kPlane) + sizeof(short) * 4 * mp;
+        return (t + 15) / 16 * 16;
+    }
+    __device__ LeafBuildSmem(unsigned char* p, int mp, int cz) {
+        T* t = reinterpret_cast<T*>(p);
+        P = reinterpret_cast<T (*)[kTriP]>(t); t += 2 * kTriP;
+        Z = reinterpret_cast<T (*)[kPlane + 1]>(t); t += zrows(mp, cz) * (kPlane + 1);
+        V = reinterpret_cast<T (*)[kPlane + 1]>(t); t += mp * (kPlane + 1);
+        col = reinterpret_cast<T (*)[2][kColSize]>(t); t += 4 * kColSize;
+        size_t o = (size_t)(reinterpret_cast<unsigned char*>(t) - p);
+        double* d = reinterpret_cast<double*>(p + (o + 7) / 8 * 8);
+        R = d; d += (size_t)mp * (mp + 1) / 2;
+        dg = reinterpret_cast<double (*)[kPlane]>(d); d += 2 * kPlane;
+        cx = reinterpret_cast<double (*)[kPlane]>(d); d += 2 * kPlane;
+        cy = reinterpret_cast<double (*)[kPlane]>(d); d += DIM == 3 ? 2 * kPlane : 0;
+        tp = reinterpret_cast<double (*)[kPlane]>(d); d += 2 * kPlane;
+        tn = reinterpret_cast<double (*)[kPlane]>(d); d += 2 * kPlane;
+        ord = reinterpret_cast<short*>(d);
+        pos = ord + 2 * mp;
+    }
 };
 
-// (row, col) of entry idx of a lower triangle stored row by row.
-__device__ __forceinline__ void tri_index(int idx, int& r, int& c) {
-    r = (int)((sqrtf(8.0f * idx + 1.0f) - 1.0f) * 0.5f);
-    while ((r + 1) * (r + 2) / 2 <= idx) ++r;
-    while (r * (r + 1) / 2 > idx) --r;
-    c = idx - r * (r + 1) / 2;
+template <int NW>
+__device__ __forceinline__ void leaf_sync() {
+    if (NW == 1) __syncwarp();
+    else __syncthreads();
 }
 
-// Face coefficients around local cell (i, j) of leaf L.
-struct CellFaces {
-    double w_, e_, s_, n_;   // coefficient seen from the cell: west, east, south, north
-    double tx, ty;           // couplings to the west / south neighbour inside the leaf
-};
+// A team of NW warps builds LPC leaves (LPC = 2: two leaves in one warp, four
+// blocks inverted at a time; LPC = 1: one leaf, two blocks at a time, the
+// tensor-core products spread over the warps); a CTA holds TM teams.  The
+// teams are independent, but start each inversion and each round of products
+// together: the code of a plane is larger than the instruction caches next to
+// the schedulers, and warps at different places of it waited for instructions
+// a third of their time (4096^2: one warp per CTA 13.0 ms; two 9.7, four 9.4,
+// six 9.8, twelve 10.5).
+template <int DIM, class T, int NW, int LPC, int TM>
+__global__ void __launch_bounds__(32 * NW * TM, NW == 1 ? 12 / TM : (DIM == 3 ? 3 : 4))
+leaf_build_kernel(DevView v, int mp, int cz, int bytes) {
+    constexpr int GL = 16 / LPC, S = Slices<T>::S, NT = 32 * NW;
+    static_assert(LPC == 1 || NW == 1, "two leaves per team only in one warp");
+    static_assert(TM == 1 || NW == 1, "several teams only of one warp each");
+    extern __shared__ __align__(16) unsigned char smem_all[];
+    __shared__ LeafGeo geo_all[LPC * TM];
+    const int team = NW == 1 ? threadIdx.x >> 5 : 0;
+    unsigned char* smem_raw = smem_all + (size_t)team * LPC * bytes;
+    LeafGeo* geos = geo_all + team * LPC;
+    const int tid = threadIdx.x - 32 * team, lane = tid & 31, warp = tid >> 5;
+    const int leaf0 = (blockIdx.x * TM + team) * LPC;
+    // the warp that inverts: warps of one index share a scheduler, so CTAs
+    // take turns (152 of them are dealt to the SMs at a time)
+    const int wsweep = NW == 1 ? 0 : (blockIdx.x / 152) % NW;
+    // this lane's block in the inversions: half hf of leaf lf
+    const int q = lane / GL, lf = q >> 1, hf = q & 1, gl = lane & (GL - 1);
+    const bool present = leaf0 + lf < v.nleaf;
+    if (tid < LPC) geos[tid] = leaf_geo<DIM>(v, min(leaf0 + tid, v.nleaf - 1));
+    if (TM > 1) __syncthreads();
+    leaf_sync<NW>();
+    const LeafGeo& G = geos[lf];
+    const LeafBuildSmem<DIM, T> Sm(smem_raw + (size_t)lf * bytes, mp, cz);
+    bool bad = false;
 
-__device__ __forceinline__ CellFaces cell_faces(const DevView& v, const LeafDesc& L, int i, int j) {
-    const GridDesc& G = v.grids[L.grid];
-    const int gi = L.i0 + i, gj = L.j0 + j;
-    const long long fx = G.fx0 + gi + (long long)(G.nx + 1) * gj;
-    const long long fy = G.fy0 + gi + (long long)G.nx * gj;
-    CellFaces c;
-    c.w_ = v.cxU[fx];
-    c.e_ = v.cxL[fx + 1];
-    c.s_ = v.cyU[fy];
-    c.n_ = v.cyL[fy + G.nx];
-    c.tx = (i > 0) ? v.cxL[fx] : 0.0;
-    c.ty = (j > 0) ? v.cyL[fy] : 0.0;
-    return c;
-}
-
-// Local segments of the Robin faces of cell (i, j), -1 where the face is not
-// on the skeleton.
-__device__ __forceinline__ void cell_robin_segments(const DevView& v, const LeafDesc& L, int i, int j,
-                                                    int& sw, int& se, int& ss, int& sn) {
-    sw = (i == 0 && L.side_off[0] >= 0) ? L.side_off[0] + j / v.gy : -1;
-    se = (i == L.w - 1 && L.side_off[1] >= 0) ? L.side_off[1] + j / v.gy : -1;
-    ss = (j == 0 && L.side_off[2] >= 0) ? L.side_off[2] + i / v.gx : -1;
-    sn = (j == L.h - 1 && L.side_off[3] >= 0) ? L.side_off[3] + i / v.gx : -1;
-}
-
-// Diagonal entry of row `row` of the leaf matrix: the sum of the cell's face
-// coefficients.
-__device__ __forceinline__ double row_diag(const DevView& v, const LeafDesc& L, int row) {
-    const CellFaces f = cell_faces(v, L, row % L.w, row / L.w);
-    return (f.w_ + f.e_) + (f.s_ + f.n_);
-}
-
-// Row `row` of the band into the window and its Robin columns into zw.  The
-// diagonal entry comes from S.dg (formed 16 rows at a time, one row per
-// lane: an FP64 instruction costs a whole warp's issue however few lanes it
-// uses), or is formed here when `fresh` (the rows before the elimination).
-template <int MMAX, class T>
-__device__ __forceinline__ void init_row(const DevView& v, const LeafDesc& L, LeafBuildSmem<MMAX, T>& S,
-                                         int row, int t, bool fresh) {
-    const int w = L.w, m = L.m;
-    const int i = row % w, j = row / w;
-    const int slot = row % (w + 2);
-    const CellFaces f = cell_faces(v, L, i, j);
-    for (int o = t; o <= w; o += kLeafThreads) {
-        double a = 0.0;
-        if (o == 0) a = fresh ? (f.w_ + f.e_) + (f.s_ + f.n_) : S.dg[row % kLeafThreads];
-        if (o == 1 && i > 0) a = neg_bits(f.tx);
-        if (o == w && j > 0) a = neg_bits(f.ty);   // w == 1: the y neighbour sits at offset 1
-        S.win[slot][o] = (T)a;
-    }
-    int sw, se, ss, sn;
-    cell_robin_segments(v, L, i, j, sw, se, ss, sn);
-    for (int q = t; q < m; q += kLeafThreads) {
-        const int s = S.order[q];
-        double b = 0.0;
-        if (s == sw) b = f.w_;
-        if (s == se) b = f.e_;
-        if (s == ss) b = f.s_;
-        if (s == sn) b = f.n_;
-        S.zw[slot][q] = (T)b;
-    }
-}
-
-// Sum of the Robin coefficients rho_e over the faces of local segment s,
-// seen from the leaf's own cells (the diagonal W_s of B^T A^-1 B - W).
-__device__ __forceinline__ double segment_rho_sum(const DevView& v, const LeafDesc& L, int s) {
-    int side = 0;
-    for (int d = 1; d < 4; ++d)
-        if (L.side_off[d] >= 0 && s >= L.side_off[d]) side = d;
-    const int p = s - L.side_off[side];
-    const int len = side < 2 ? L.h : L.w, g = side < 2 ? v.gy : v.gx;
-    const GridDesc& G = v.grids[L.grid];
-    const double* cxL = v.cxL + G.fx0;
-    const double* cxU = v.cxU + G.fx0;
-    const double* cyL = v.cyL + G.fy0;
-    const double* cyU = v.cyU + G.fy0;
-    double sum = 0.0;
-    for (int e = p * g; e < min((p + 1) * g, len); ++e) {
-        if (side == 0) sum += cxU[(long long)L.i0 + (long long)(G.nx + 1) * (L.j0 + e)];
-        else if (side == 1) sum += cxL[(long long)(L.i0 + L.w) + (long long)(G.nx + 1) * (L.j0 + e)];
-        else if (side == 2) sum += cyU[(long long)(L.i0 + e) + (long long)G.nx * L.j0];
-        else sum += cyL[(long long)(L.i0 + e) + (long long)G.nx * (L.j0 + L.h)];
-    }
-    return sum;
-}
-
-// First row of the leaf whose cell touches local segment s (the first
-// nonzero of column s of B).
-__device__ __forceinline__ int segment_start_row(const DevView& v, const LeafDesc& L, int s) {
-    const int w = L.w, h = L.h;
-    if (L.side_off[3] >= 0 && s >= L.side_off[3]) return (h - 1) * w + (s - L.side_off[3]) * v.gx;
-    if (L.side_off[2] >= 0 && s >= L.side_off[2]) return (s - L.side_off[2]) * v.gx;
-    if (L.side_off[1] >= 0 && s >= L.side_off[1]) return (s - L.side_off[1]) * v.gy * w + w - 1;
-    return (s - L.side_off[0]) * v.gy * w;
-}
-
-// Body of the leaf build for one leaf; WF > 0 fixes the leaf to WF x WF
-// cells at compile time (the full leaf), 0 reads the size from the
-// descriptor (truncated leaves).  T: arithmetic and storage of the factors
-// (double, or float in the mixed form; the map R is stored in double).
-template <int MMAX, int WF, class T>
-__device__ __forceinline__ void leaf_build_body(const DevView& v, LeafBuildSmem<MMAX, T>& S, const LeafDesc& L,
-                                                int t, unsigned mask) {
-    const int w = WF ? WF : L.w, n = WF ? WF * WF : L.w * L.h, m = L.m, W2 = w + 2;
-    T* Lg = leaf_L<T>(v) + L.L_off;          // n x 16 multipliers
-    T* Dg = Lg + (long long)n * kLeafThreads;   // n reciprocal pivots
-    T* Zg = leaf_Z<T>(v) + L.Z_off;          // n x m, column-major (local segment order)
-
-    // Columns of B ordered by their first nonzero row: column q of Z stays
-    // zero above start[q], so only the first c_k ordered columns take part
-    // in step k of the forward solve and of the R accumulation.
-    if (t == 0) {
-        for (int s = 0; s < m; ++s) {
-            const int st = segment_start_row(v, L, s);
-            int q = s;
-            while (q > 0 && S.start[q - 1] > st) {
-                S.start[q] = S.start[q - 1];
-                S.order[q] = S.order[q - 1];
-                --q;
+    // column orders, zeroed R
+#pragma unroll 1
+    for (int f = 0; f < LPC; ++f) {
+        const LeafGeo& g = geos[f];
+        const LeafBuildSmem<DIM, T> s(smem_raw + (size_t)f * bytes, mp, cz);
+        for (int i = tid; i < 2 * g.m; i += NT) s.pos[(i / g.m) * mp + i % g.m] = (short)-1;
+        leaf_sync<NW>();
+        for (int h = 0; h < 2; ++h)
+            for (int p = tid; p < g.ncols(h); p += NT) {
+                const int t = g.segment(h, p);
+                s.ord[h * mp + p] = (short)t;
+                s.pos[h * mp + t] = (short)p;
             }
-            S.start[q] = st;
-            S.order[q] = s;
-        }
-        for (int q = 0; q < m; ++q) S.pos[S.order[q]] = q;
+        for (int i = tid; i < g.m * (g.m + 1) / 2; i += NT) s.R[i] = 0.0;
+        for (int i = tid; i < 2 * cz * (kPlane + 1); i += NT) (&s.Z[0][0])[i] = (T)0;
+        for (int i = tid; i < 2 * kTriP; i += NT) s.P[0][i] = (T)0;
     }
-    __syncwarp(mask);
+    leaf_sync<NW>();
 
-    for (int idx = t; idx < m * (MMAX + 1); idx += kLeafThreads) S.R[idx / (MMAX + 1)][idx % (MMAX + 1)] = (T)0;
-    const int first = min(w, n - 1);
-    for (int r = 0; r <= first; ++r) init_row(v, L, S, r, t, true);
-    __syncwarp(mask);
+    const BlockSlots<GL> B;
+    int steps = 0;                                             // uniform over the CTA
+#pragma unroll 1
+    for (int f = 0; f < LPC * TM; ++f) steps = max(steps, max(geo_all[f].M, geo_all[f].H - 1 - geo_all[f].M));
+    // entry (r, c), r >= c, of the plane's matrix block
+    auto plane_entry = [&](const LeafGeo& g, const LeafBuildSmem<DIM, T>& s, int h, int r, int c) -> double {
+        if (r == c) return s.dg[h][r];
+        double a = 0.0;
+        if (r - c == 1 && (DIM == 2 || r % g.w0 != 0)) a = neg_bits(s.cx[h][r]);
+        if (DIM == 3 && r - c == g.w0) a = neg_bits(s.cy[h][r]);
+        return a;
+    };
+    const int r16 = tid >> 4, c16 = tid & 15;                  // a half warp per row of 16
 
-    // per-thread index patterns of the two triangles (band update: rows a >=
-    // b of the w x w trailing block; R update: r >= c of the active columns),
-    // fixed for the whole elimination: entry idx = t + 16 e
-    constexpr int kBandEnt = (kMaxLeafSide * (kMaxLeafSide + 1) / 2 + kLeafThreads - 1) / kLeafThreads;
-    constexpr int kREnt = (MMAX * (MMAX + 1) / 2 + kLeafThreads - 1) / kLeafThreads;
-    constexpr bool kRPre = kREnt <= 12;       // keep the R pattern in registers when it is small
-    constexpr int kRReg = kRPre ? kREnt : 1;
-    int band_a[kBandEnt], band_b[kBandEnt], tri_r[kRReg], tri_c[kRReg];
-#pragma unroll
-    for (int e = 0; e < kBandEnt; ++e) tri_index(t + e * kLeafThreads, band_a[e], band_b[e]);
-    if constexpr (kRPre) {
-#pragma unroll
-        for (int e = 0; e < kREnt; ++e) tri_index(t + e * kLeafThreads, tri_r[e], tri_c[e]);
-    }
-
-    bool bad_pivot = false;
-    int ck = 0;                      // active ordered columns
-    int sk = 0;                      // window slot of row k (k mod W2)
-    for (int k = 0; k < n; ++k) {
-        // diagonals of the rows entering the window in steps k .. k + 15 (read
-        // after the warp barrier of phase A)
-        if ((k & (kLeafThreads - 1)) == 0) {
-            const int r = k + w + 1 + t;
-            if (r < n) S.dg[r % kLeafThreads] = row_diag(v, L, r);
-        }
-        while (ck < m && S.start[ck] <= k) ++ck;
-        const int s1 = sk + 1 == W2 ? 0 : sk + 1;        // slot of row k + 1
-        // ---- phase A: pivot, multipliers, row k of Z -------------------------
-        const T dk = S.win[sk][0];
-        // dk > 0 and finite, tested on the bit pattern (no FP64 compare)
-        bad_pivot |= !positive_finite_bits(dk);
-        const T rcp = rcp_nr(dk);
-        const int wk = min(w, n - 1 - k);
-        if (t < wk) {
-            int sl = s1 + t;
-            sl -= sl >= W2 ? W2 : 0;
-            const T l = S.win[sl][1 + t] * rcp;
-            S.lcol[t] = l;
-            Lg[(long long)k * kLeafThreads + t] = l;
-        }
-        if (t == 0) Dg[k] = rcp;
-        for (int q = t; q < ck; q += kLeafThreads) {
-            const T z = S.zw[sk][q];
-            S.zk[q] = z;
-            S.uk[q] = z * rcp;
-        }
-        __syncwarp(mask);
-        for (int s = t; s < m; s += kLeafThreads) {
-            const int q = S.pos[s];
-            Zg[(long long)s * n + k] = q < ck ? S.zk[q] : (T)0;
-        }
-        // ---- phase B: trailing band update, Z update, R update, new row -----
-        const int ntri_w = wk * (wk + 1) / 2;
-#pragma unroll
-        for (int e = 0; e < kBandEnt; ++e) {
-            if (t + e * kLeafThreads >= ntri_w) break;
-            const int a = band_a[e], b = band_b[e];
-            int ra = s1 + a, rb = s1 + b;
-            ra -= ra >= W2 ? W2 : 0;
-            rb -= rb >= W2 ? W2 : 0;
-            T& x = S.win[ra][a - b];
-            x = fma(-S.lcol[a], S.win[rb][1 + b], x);
-        }
-        if (ck > 0) {
-            // (row a, column q) of entry idx = a ck + q, stepped by 16 entries
-            const int nz = wk * ck, da = kLeafThreads / ck, dq = kLeafThreads - da * ck;
-            int a = t / ck, q = t - a * ck;
-            for (int idx = t; idx < nz; idx += kLeafThreads) {
-                int ra = s1 + a;
-                ra -= ra >= W2 ? W2 : 0;
-                T& x = S.zw[ra][q];
-                x = fma(-S.lcol[a], S.zk[q], x);
-                a += da;
-                q += dq;
-                if (q >= ck) {
-                    q -= ck;
-                    ++a;
+    for (int j = 0; j <= steps; ++j) {
+        const bool mid = j == steps;
+        if (TM > 1) __syncthreads();
+        // ---- the planes' coefficients and blocks; inversion (one warp) ------
+        if (NW == 1 || warp == wsweep) {
+            const int k = mid ? G.M : (hf ? G.H - 1 - j : j);
+            const bool act = present && (mid ? hf == 0 : j < G.halfplanes(hf));
+            if (act) {
+                for (int i = gl; i < G.nb; i += GL) {
+                    const CellFaces<DIM> c = cell_faces<DIM>(v, leaf0 + lf, G, k, i);
+                    Sm.dg[hf][i] = c.diag();
+                    Sm.cx[hf][i] = c.c[0];
+                    if (DIM == 3) Sm.cy[hf][i] = c.c[2];
+                    Sm.tp[hf][i] = mid || !hf ? c.down() : c.up();  // coupling to the plane before (mid: below)
+                    Sm.tn[hf][i] = mid || !hf ? c.up() : c.down();  // after (mid: above)
+                    if (!mid)                                       // B's entries of the plane
+                        plane_faces<DIM>(v, G, c, k, i,
+                                         [&](int t, double rho) { Sm.Z[hf * cz + Sm.pos[hf * mp + t]][i] += (T)rho; });
                 }
             }
-        }
-        const int ntri_m = ck * (ck + 1) / 2;
-        if constexpr (kRPre) {
+            __syncwarp();
+            T e[BlockSlots<GL>::kN];
 #pragma unroll
-            for (int e = 0; e < kREnt; ++e) {
-                if (t + e * kLeafThreads >= ntri_m) break;
-                const int r = tri_r[e], c = tri_c[e];
-                S.R[r][c] = fma(S.zk[r], S.uk[c], S.R[r][c]);
+            for (int s = 0; s < BlockSlots<GL>::kN; ++s) {
+                e[s] = (T)0;
+                if (!B.valid(s)) continue;
+                const int r = B.row(s), c = B.colm(s);
+                if (!act || r >= G.nb) continue;
+                double x = plane_entry(G, Sm, hf, r, c);
+                if (!mid) {
+                    if (j > 0) x -= (double)Sm.P[hf][tri_at(r, c)] * (Sm.tp[hf][r] * Sm.tp[hf][c]);
+                } else {
+                    if (G.halfplanes(0) > 0) x -= (double)Sm.P[0][tri_at(r, c)] * (Sm.tp[0][r] * Sm.tp[0][c]);
+                    if (G.halfplanes(1) > 0) x -= (double)Sm.P[1][tri_at(r, c)] * (Sm.tn[0][r] * Sm.tn[0][c]);
+                }
+                e[s] = (T)x;
             }
-        } else {
-            for (int idx = t; idx < ntri_m; idx += kLeafThreads) {
-                int r, c;
-                tri_index(idx, r, c);
-                S.R[r][c] = fma(S.zk[r], S.uk[c], S.R[r][c]);
-            }
+            __syncwarp();
+            // lanes of absent or smaller blocks follow the longest one
+            const int nb = act ? G.nb : 0;
+            const int nbmax = __reduce_max_sync(0xffffffffu, nb);
+            bad |= !sweep_block<GL, T>(e, B, Sm.col[hf], nb, nbmax, [](T p, int) { return positive_finite_bits(p); });
+            if (act)
+#pragma unroll
+                for (int s = 0; s < BlockSlots<GL>::kN; ++s) {
+                    if (!B.valid(s)) continue;
+                    const int r = B.row(s), c = B.colm(s);
+                    if (r < G.nb) Sm.P[hf][tri_at(r, c)] = neg_bits(e[s]);
+                }
         }
-        if (k + w + 1 < n) init_row(v, L, S, k + w + 1, t, false);
-        __syncwarp(mask);
-        sk = s1;
+        if (TM > 1) __syncthreads();
+        leaf_sync<NW>();
+        // ---- products, per leaf and half (loops kept rolled: one copy of the
+        // code of a product, or the instruction fetch sets the pace)
+#pragma unroll 1
+        for (int fh = 0; fh < 2 * LPC; ++fh) {
+            const int f = fh >> 1, h = fh & 1;
+            const LeafGeo& g = geos[f];
+            if (leaf0 + f >= v.nleaf || (mid ? h : j >= g.halfplanes(h))) continue;
+            const LeafBuildSmem<DIM, T> s(smem_raw + (size_t)f * bytes, mp, cz);
+            const int k = mid ? g.M : (h ? g.H - 1 - j : j), cc = mid ? g.m : g.cols(h, k);
+            // Z of the plane by column, V = P Z, column -> segment
+            T (*zs)[kPlane + 1] = mid ? s.V : s.Z + h * cz;
+            T (*vs)[kPlane + 1] = mid ? s.Z : s.V;
+            const short* ord = s.ord + h * mp;
+            if (mid) {
+                // Z of the middle plane: both halves' contributions and B
+                for (int t = r16; t < g.m; t += NT / 16) {
+                    const int pt = s.pos[t], pb = s.pos[mp + t];
+                    T z = (T)0;
+                    if (g.M > 0 && pt >= 0 && pt < g.cols(0, g.M - 1)) z += s.Z[pt][c16];
+                    if (g.H - 1 - g.M > 0 && pb >= 0 && pb < g.cols(1, g.M + 1)) z += s.Z[cz + pb][c16];
+                    s.V[t][c16] = z;
+                }
+                leaf_sync<NW>();
+                for (int i = tid; i < g.nb; i += NT)
+                    plane_faces<DIM>(v, g, cell_faces<DIM>(v, leaf0 + f, g, g.M, i), g.M, i,
+                                     [&](int t, double rho) { s.V[t][i] += (T)rho; });
+                leaf_sync<NW>();
+            }
+            {
+                T* Lk = leaf_L<T>(v) + g.L_off + (long long)k * g.nb * g.nb;
+                T* Zk = leaf_Z<T>(v) + g.Z_off + g.zoff(mid ? 0 : h, k);
+                if (c16 < g.nb) {
+                    for (int r = r16; r < g.nb; r += NT / 16) Lk[r * g.nb + c16] = s.P[h][tri_at(r, c16)];
+                    for (int n = r16; n < cc; n += NT / 16) Zk[n * g.nb + c16] = zs[n][c16];
+                }
+            }
+            // stage 0: V = P Z; stage 1: R += Z^T V, entries (row, n), row >= n, of
+            // the column order; 16 x 8 tiles dealt to the warps
+            int item = 0;
+#pragma unroll 1
+            for (int stage = 0; stage < 2; ++stage) {
+                const int mt = stage ? (cc + 15) / 16 : 1;
+#pragma unroll 1
+                for (int ri = 0; ri < mt; ++ri) {
+                    const int nt = stage ? min((cc + 7) / 8, 2 * ri + 2) : (cc + 7) / 8;
+                    const int rows = stage ? min(cc - 16 * ri, 16) : g.nb;
+                    FragA<S> a;
+                    bool loaded = false;
+#pragma unroll 1
+                    for (int ni = 0; ni < nt; ++ni) {
+                        if (NW > 1 && (item + ni) % NW != warp) continue;
+                        if (!loaded) {
+                            const T *zp = &zs[16 * ri][0], *pp = s.P[h];
+                            load_frag_a<S, T>(a, [&](int r, int k) {
+                                return r < rows ? (stage ? zp[r * (kPlane + 1) + k] : pp[tri_at(r, k)]) : (T)0;
+                            });
+                            loaded = true;
+                        }
+                        const T* bp = &(stage ? vs : zs)[8 * ni][0];
+                        FragB<S> b;
+                        load_frag_b<S, T>(
+                            b, [&](int n, int k) { return 8 * ni + n < cc ? bp[n * (kPlane + 1) + k] : (T)0; });
+                        typename SplitAcc<S>::T out[4];
+                        frag_product(a, b, out, rows);
+#pragma unroll
+                        for (int r = 0; r < 4; ++r) {
+                            const int i = (lane >> 2) + 8 * (r >> 1), row = 16 * ri + i;
+                            const int n = 8 * ni + 2 * (lane & 3) + (r & 1);
+                            if (!stage) {
+                                if (n < cc) vs[n][i] = (T)out[r];
+                            } else if (row < cc && n <= row)
+                                s.R[mid ? tri_at(row, n) : tri_at(ord[row], ord[n])] += (double)out[r];
+                        }
+                    }
+                    item += nt;
+                }
+                leaf_sync<NW>();
+            }
+            if (mid) continue;
+            // what the next plane receives: T V
+            for (int p = r16; p < cc; p += NT / 16)
+                zs[p][c16] = c16 < g.nb ? (T)(s.tn[h][c16] * (double)s.V[p][c16]) : (T)0;
+            leaf_sync<NW>();
+        }
     }
-    if (bad_pivot) atomicOr(v.status, kStatusSingular);
-    // W_s = sum of rho over the faces of segment s (seen from this leaf)
-    for (int q = t; q < m; q += kLeafThreads) S.W[q] = segment_rho_sum(v, L, S.order[q]);
-    __syncwarp(mask);
-    double* Rg = v.R + L.R_off;
-    for (int idx = t; idx < m * m; idx += kLeafThreads) {
-        const int r = S.pos[idx / m], c = S.pos[idx % m];
-        double val = (r >= c) ? (double)S.R[r][c] : (double)S.R[c][r];
-        if (r == c) val -= S.W[r];
-        Rg[idx] = val;
-    }}
-
-// Residency: the FP64 full-leaf variant holds 31 KB of shared memory per
-// CTA, so 7 CTAs fit an SM; the register cap keeps all 7 resident (one wave
-// of 1064 CTAs covers the 4096 leaves of a 1024^2 grid).
-template <int MMAX, int LPB, class T>
-__global__ void __launch_bounds__(kLeafThreads * LPB, MMAX == 16 ? (sizeof(T) == 8 ? 7 : 8) : 1)
-leaf_build_kernel(DevView v) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int t = threadIdx.x & (kLeafThreads - 1);
-    const int slot_leaf = threadIdx.x / kLeafThreads;
-    const int leaf = blockIdx.x * LPB + slot_leaf;
-    if (leaf >= v.nleaf) return;     // uniform over the 16 threads of the leaf
-    const unsigned mask = 0xFFFFu << (threadIdx.x & 16);
-    LeafBuildSmem<MMAX, T>& S = reinterpret_cast<LeafBuildSmem<MMAX, T>*>(smem_raw)[slot_leaf];
-    const LeafDesc L = v.leaves[leaf];
-    if (L.w == kMaxLeafSide && L.h == kMaxLeafSide)
-        leaf_build_body<MMAX, kMaxLeafSide, T>(v, S, L, t, mask);
-    else
-        leaf_build_body<MMAX, 0, T>(v, S, L, t, mask);
+    if (bad) atomicOr(v.status, kStatusSingular);
+    // R = Z^T P Z - W
+#pragma unroll 1
+    for (int f = 0; f < LPC; ++f) {
+        if (leaf0 + f >= v.nleaf) break;
+        const LeafGeo& g = geos[f];
+        const LeafBuildSmem<DIM, T> s(smem_raw + (size_t)f * bytes, mp, cz);
+        for (int t = tid; t < g.m; t += NT) s.R[t * (t + 1) / 2 + t] -= segment_rho_sum<DIM>(v, leaf0 + f, g, t);
+        leaf_sync<NW>();
+        double* Rg = v.R + g.R_off;
+        for (int r = r16; r < g.m; r += NT / 16)
+            for (int c = c16; c < g.m; c += 16) Rg[r * g.m + c] = s.R[tri_at(r, c)];
+    }
 }
 
 // ---------------------------------------------------------------------------
-// Solve phase.  Right-hand side of the particular problem (Eqs. addu/addp):
-// source plus Dirichlet and Neumann data of the leaf's domain-boundary faces.
-__device__ __forceinline__ double particular_rhs(const DevView& v, const LeafDesc& L, const double* q,
-                                                 const double* bc_val, int row) {
-    const GridDesc& G = v.grids[L.grid];
-    const int i = row % L.w, j = row / L.w;
-    const int gi = L.i0 + i, gj = L.j0 + j;
-    double b = q[G.c0 + (long long)gj * G.nx + gi];
+// Solve phase, one warp per leaf: lanes 0-15 the planes below the middle one
+// (lane = cell), lanes 16-31 those above, in step; the middle plane by both
+// (each half of the warp takes half of the products).
+constexpr int kSolveWarps = 4;
+
+// Right-hand side of the particular problem at one cell (Eqs. addu/addp):
+// the source plus Dirichlet and Neumann data of its domain-boundary faces.
+template <int DIM>
+__device__ __forceinline__ double particular_rhs(const DevView& v, int leaf, const CellFaces<DIM>& f,
+                                                 const double* q, const double* bc_val) {
+    double b = q[f.cell];
     if (!bc_val) return b;
-    const double* bv = bc_val + G.b0;
-    if (gi == 0) {
-        const double g = bv[gj];
-        b += G.bc[0] ? v.cxU[G.fx0 + (long long)(G.nx + 1) * gj] * g : -G.hy * g;
-    }
-    if (gi == G.nx - 1) {
-        const double g = bv[G.ny + gj];
-        b += G.bc[1] ? v.cxL[G.fx0 + G.nx + (long long)(G.nx + 1) * gj] * g : -G.hy * g;
-    }
-    if (gj == 0) {
-        const double g = bv[2 * G.ny + gi];
-        b += G.bc[2] ? v.cyU[G.fy0 + gi] * g : -G.hx * g;
-    }
-    if (gj == G.ny - 1) {
-        const double g = bv[2 * G.ny + G.nx + gi];
-        b += G.bc[3] ? v.cyL[G.fy0 + gi + (long long)G.nx * G.ny] * g : -G.hx * g;
+    if constexpr (DIM == 2) {
+        const GridDesc& G = v.grids[v.leaves[leaf].grid];
+        const double* bv = bc_val + G.b0;
+        if (f.x == 0) b += G.bc[0] ? f.c[0] * bv[f.y] : -G.hy * bv[f.y];
+        if (f.x == G.nx - 1) b += G.bc[1] ? f.c[1] * bv[G.ny + f.y] : -G.hy * bv[G.ny + f.y];
+        if (f.y == 0) b += G.bc[2] ? f.c[2] * bv[2 * G.ny + f.x] : -G.hx * bv[2 * G.ny + f.x];
+        if (f.y == G.ny - 1) {
+            const double g = bv[2 * G.ny + G.nx + f.x];
+            b += G.bc[3] ? f.c[3] * g : -G.hx * g;
+        }
+    } else {
+        const Grid3& G = v.g3;
+#pragma unroll
+        for (int s = 0; s < 6; ++s) {
+            const int pos = s < 2 ? f.x : (s < 4 ? f.y : f.z), n = s < 2 ? G.nx : (s < 4 ? G.ny : G.nz);
+            if (s & 1 ? pos != n - 1 : pos != 0) continue;
+            const double g = bc_value3(G, bc_val, s, f.x, f.y, f.z);
+            b += G.bc[s] ? f.c[s] * g : -(area3(G, s >> 1) * g);
+        }
     }
     return b;
 }
 
-struct LeafSolveSmem {
-    double y[kMaxLeafSide * kMaxLeafSide];             // right-hand side, swept in place
-};
-
-// Depth of the register ring that prefetches the band multipliers of the
-// sweeps (rows streamed from HBM ahead of the sequential elimination chain).
-constexpr int kSweepAhead = 16;
-
-// Body of the particular solve for one leaf; NF, WF > 0 fix the row count
-// and the band width at compile time (the full kMaxLeafSide^2 leaf: the
-// sweep's bounds and end tests then fold away, which makes it ~3x faster),
-// 0 reads them from the descriptor (truncated leaves).  TS: storage type of
-// the factors (float in the mixed form); the sweep itself runs in FP64.
-template <int NF, int WF, class TS>
-__device__ __forceinline__ void leaf_particular_body(const DevView& v, const double* __restrict__ q,
-                                                     const double* __restrict__ bc_val, bool with_sadj,
-                                                     LeafSolveSmem& S, const LeafDesc& L, int t, unsigned mask) {
-    const int w = WF ? WF : L.w, n = NF ? NF : L.w * L.h, m = L.m;
-    const TS* Lg = leaf_L<TS>(v) + L.L_off;
-    const TS* Dg = Lg + (long long)n * kLeafThreads;
-    const TS* Zg = leaf_Z<TS>(v) + L.Z_off;
-    double* zb = v.leafzb + L.zb_off;
-
-    // forward sweep zbar = L^-1 bbar (unit lower band); the right-hand side
-    // is formed for all rows first, the multipliers stream through a
-    // register ring kSweepAhead steps ahead of their use
-    for (int r = t; r < n; r += kLeafThreads) S.y[r] = particular_rhs(v, L, q, bc_val, r);
-    __syncwarp(mask);
-    double ring[kSweepAhead];
+// Column l of the stored P of plane k (P is symmetric: entry j is P(l, j)).
+template <class TS>
+__device__ __forceinline__ void load_p(TS (&p)[kPlane], const TS* Lg, int nb, int k, int l, bool on) {
+    const TS* c = Lg + (long long)k * nb * nb + l;
 #pragma unroll
-    for (int d = 0; d < kSweepAhead; ++d) ring[d] = (d < n && t < min(w, n - 1 - d)) ? Lg[(long long)d * kLeafThreads + t] : 0.0;
-    for (int k0 = 0; k0 < n; k0 += kSweepAhead) {
+    for (int j = 0; j < kPlane; ++j) p[j] = (on && l < nb && j < nb) ? c[j * nb] : (TS)0;
+}
+// sum_j p[j] y[j], and column l of plane k in p's place: each entry is loaded
+// as soon as the one before it is used, a plane ahead of its own use.  One
+// chain: its latency (75 cycles) is little above what an FP64 instruction
+// holds the pipe for, and partial sums would only add to it.
+template <class TS>
+__device__ __forceinline__ double row_product_next(TS (&p)[kPlane], const double* y, const TS* Lg, int nb, int k, int l,
+                                                   bool on) {
+    const TS* c = Lg + (long long)k * nb * nb + l;
+    const int n = on && l < nb ? nb : 0;
+    double a = 0.0;
 #pragma unroll
-        for (int d = 0; d < kSweepAhead; ++d) {
-            const int k = k0 + d;
-            if (k >= n) break;
-            const double lk = ring[d];
-            const int kn = k + kSweepAhead;
-            ring[d] = (kn < n && t < min(w, n - 1 - kn)) ? Lg[(long long)kn * kLeafThreads + t] : 0.0;
-            const double zk = S.y[k];
-            if (t < min(w, n - 1 - k)) S.y[k + 1 + t] = fma(-lk, zk, S.y[k + 1 + t]);
-            __syncwarp(mask);
-        }
+    for (int j = 0; j < kPlane; ++j) {
+        a = fma((double)p[j], y[j], a);
+        p[j] = j < n ? c[j * nb] : (TS)0;
     }
-    for (int k = t; k < n; k += kLeafThreads) zb[k] = S.y[k];
-    // y = D^-1 zbar ; rbar = Z^T y  (= B^T A^-1 bbar): the 16 lanes share
-    // every column of Z (consecutive rows, coalesced) and reduce by shuffles;
-    // the lane's y stay in registers and all of its kRows loads of a column
-    // are in flight together
-    constexpr int kRows = kMaxLeafSide * kMaxLeafSide / kLeafThreads;
-    double yv[kRows];
+    return a;
+}
+// the half of the product over j in [8 part, 8 part + 8)
+template <class TS>
+__device__ __forceinline__ double half_product(const TS (&p)[kPlane], const double* y, int part) {
+    double a = 0.0;
 #pragma unroll
-    for (int r = 0; r < kRows; ++r) {
-        const int k = t + r * kLeafThreads;
-        yv[r] = k < n ? S.y[k] * (double)Dg[k] : 0.0;
-    }
-    double* rb = v.rbar + L.r_off;
-    for (int s = 0; s < m; ++s) {
-        const TS* zc = Zg + (long long)s * n;
-        double zv[kRows];
-#pragma unroll
-        for (int r = 0; r < kRows; ++r) {
-            const int k = t + r * kLeafThreads;
-            zv[r] = k < n ? (double)zc[k] : 0.0;
-        }
-        double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-#pragma unroll
-        for (int r = 0; r < kRows; r += 4) {
-            a0 = fma(zv[r], yv[r], a0);
-            a1 = fma(zv[r + 1], yv[r + 1], a1);
-            a2 = fma(zv[r + 2], yv[r + 2], a2);
-            a3 = fma(zv[r + 3], yv[r + 3], a3);
-        }
-        double acc = (a0 + a1) + (a2 + a3);
-#pragma unroll
-        for (int o = kLeafThreads / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(mask, acc, o);
-        // a right-hand side sigma on this segment's interface row,
-        // F - D (lambda_other - lambda_own) = sigma, acts as rbar - sigma
-        if (t == 0) rb[s] = with_sadj ? acc - v.sadj[L.r_off + s] : acc;
-    }}
-
-template <int LPB, class TS>
-__global__ void __launch_bounds__(kLeafThreads * LPB)
-leaf_particular_kernel(DevView v, const double* __restrict__ q, const double* __restrict__ bc_val,
-                       bool with_sadj) {
-    __shared__ LeafSolveSmem smem[LPB];
-    const int t = threadIdx.x & (kLeafThreads - 1);
-    const int slot_leaf = threadIdx.x / kLeafThreads;
-    const int leaf = blockIdx.x * LPB + slot_leaf;
-    if (leaf >= v.nleaf) return;
-    const unsigned mask = 0xFFFFu << (threadIdx.x & 16);
-    LeafSolveSmem& S = smem[slot_leaf];
-    const LeafDesc L = v.leaves[leaf];
-    if (L.w == kMaxLeafSide && L.h == kMaxLeafSide)
-        leaf_particular_body<kMaxLeafSide * kMaxLeafSide, kMaxLeafSide, TS>(v, q, bc_val, with_sadj, S, L, t,
-                                                                            mask);
-    else
-        leaf_particular_body<0, 0, TS>(v, q, bc_val, with_sadj, S, L, t, mask);
+    for (int j = 0; j < kPlane / 2; ++j)
+        a = fma((double)(part ? p[j + kPlane / 2] : p[j]), y[j + part * (kPlane / 2)], a);
+    return a;
 }
 
-// p = A^-1 (bbar + B lambda) = L^-T D^-1 (zbar + Z lambda), written into the
-// state (p_hi, p_lo) or added to it in double-double (refinement corrections).
-// Body of the final solve for one leaf; NF, WF as for the particular solve.
-template <int NF, int WF, class TS>
-__device__ __forceinline__ void leaf_pressure_body(const DevView& v, bool accumulate, LeafSolveSmem& S,
-                                                   double* lam, const LeafDesc& L, int t, unsigned mask) {
-    const int w = WF ? WF : L.w, n = NF ? NF : L.w * L.h, m = L.m;
-    const TS* Lg = leaf_L<TS>(v) + L.L_off;
-    const TS* Dg = Lg + (long long)n * kLeafThreads;
-    const TS* Zg = leaf_Z<TS>(v) + L.Z_off;
-    const double* zb = v.leafzb + L.zb_off;
-    for (int s = t; s < m; s += kLeafThreads) lam[s] = v.lam[L.r_off + s];
-    __syncwarp(mask);
-    // y = D^-1 (zbar + Z lambda), Z column-major: the lane's rows
-    // k = t + 16 r accumulate together, one column at a time, so that
-    // kRows independent loads are in flight per lane
-    constexpr int kRows = kMaxLeafSide * kMaxLeafSide / kLeafThreads;
-    double acc[kRows];
+// Sums x[c], c < 8, over the 16 lanes of each half warp; lane l returns
+// column l / 2 (both lanes of a pair the same).
+__device__ __forceinline__ double reduce_columns8(double (&x)[8], int l) {
 #pragma unroll
-    for (int r = 0; r < kRows; ++r) {
-        const int k = t + r * kLeafThreads;
-        acc[r] = k < n ? zb[k] : 0.0;
-    }
-    for (int s = 0; s < m; ++s) {
-        const double ls = lam[s];
-        const TS* zc = Zg + (long long)s * n;
+    for (int w = 8, n = 4; w >= 2; w >>= 1, n >>= 1) {
+        const bool up = l & w;
 #pragma unroll
-        for (int r = 0; r < kRows; ++r) {
-            const int k = t + r * kLeafThreads;
-            if (k < n) acc[r] = fma((double)zc[k], ls, acc[r]);
+        for (int c = 0; c < n; ++c) {
+            const double mine = up ? x[c + n] : x[c], theirs = up ? x[c] : x[c + n];
+            x[c] = mine + __shfl_xor_sync(0xffffffffu, theirs, w);
         }
     }
+    return x[0] + __shfl_xor_sync(0xffffffffu, x[0], 1);
+}
+
+// y_k (into leafzb), w_k = P_k y_k and rbar = sum_k Z_k^T w_k.  SMALL: at most
+// 8 columns meet a plane off the middle one and m <= 16 (partial sums in
+// registers); otherwise they go through shared memory (acc: (2 cz + mp) rows
+// of 17 doubles per warp).  TS: storage type of the factors (float in the
+// mixed form's FP32 leaves); the arithmetic is FP64.
+template <int DIM, class TS, bool SMALL>
+__global__ void __launch_bounds__(32 * kSolveWarps)
+leaf_particular_kernel(DevView v, const double* __restrict__ q, const double* __restrict__ bc_val, bool with_sadj,
+                       int mp, int cz) {
+    __shared__ double ysh[kSolveWarps][2][kPlane];
+    extern __shared__ __align__(16) double acc_raw[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, h = lane >> 4, l = lane & 15;
+    const int leaf = blockIdx.x * kSolveWarps + warp;
+    if (leaf >= v.nleaf) return;                      // uniform over the warp
+    const LeafGeo g = leaf_geo<DIM>(v, leaf);
+    const int nb = g.nb, hp = g.halfplanes(h), steps = max(g.halfplanes(0), g.halfplanes(1));
+    const TS* Lg = leaf_L<TS>(v) + g.L_off;
+    const TS* Zg = leaf_Z<TS>(v) + g.Z_off;
+    double* zb = v.leafzb + g.zb_off;
+    double (*acc)[kPlane + 1] = reinterpret_cast<double (*)[kPlane + 1]>(acc_raw) + (size_t)warp * (2 * cz + mp);
+    double part[8];
 #pragma unroll
-    for (int r = 0; r < kRows; ++r) {
-        const int k = t + r * kLeafThreads;
-        if (k < n) S.y[k] = acc[r] * (double)Dg[k];
-    }
-    __syncwarp(mask);
-    // backward sweep L^T p = y in place, right-looking from the last row,
-    // reading row k of L from the column layout (L[k][k-1-t] is multiplier t
-    // of column k-1-t, at Lg[16 (k-1-t) + t]: a diagonal of the layout, whose
-    // lines the next steps read again from L1); the multipliers stream
-    // through a register ring kSweepAhead steps ahead
-    double ring[kSweepAhead];
+    for (int p = 0; p < 8; ++p) part[p] = 0.0;
+    if constexpr (!SMALL)
+        for (int p = 0; p < cz; ++p) acc[h * cz + p][l] = 0.0;
+    TS p[kPlane];
+    double w = 0.0, yn = 0.0, tn = 0.0;
+    // right-hand side and coupling to the plane before, a plane ahead
+    auto ahead = [&](int j) {
+        if (j >= hp || l >= nb) return;
+        const CellFaces<DIM> f = cell_faces<DIM>(v, leaf, g, h ? g.H - 1 - j : j, l);
+        yn = particular_rhs<DIM>(v, leaf, f, q, bc_val);
+        tn = h ? f.up() : f.down();
+    };
+    ahead(0);
+    load_p(p, Lg, nb, h ? g.H - 1 : 0, l, hp > 0);
+    const int ccw = __reduce_max_sync(0xffffffffu, g.ncols(h));    // columns of the warp's widest plane
+    for (int j = 0; j < steps; ++j) {
+        const bool act = j < hp && l < nb;
+        const int k = h ? g.H - 1 - j : j;
+        const double y = act ? (j > 0 ? fma(tn, w, yn) : yn) : 0.0;
+        if (act) zb[k * nb + l] = y;
+        const int cc = j < hp ? g.cols(h, k) : 0;
+        const TS* Zk = Zg + g.zoff(h, k);
+        TS z[8];
+        if (SMALL)
 #pragma unroll
-    for (int d = 0; d < kSweepAhead; ++d) {
-        const int k = n - 1 - d;
-        ring[d] = (k >= 1 && t < min(w, k)) ? Lg[(long long)(k - 1 - t) * kLeafThreads + t] : 0.0;
-    }
-    for (int k0 = n - 1; k0 >= 0; k0 -= kSweepAhead) {
+            for (int c = 0; c < 8; ++c) z[c] = act && c < cc ? Zk[c * nb + l] : (TS)0;
+        ysh[warp][h][l] = y;
+        __syncwarp();
+        ahead(j + 1);
+        const double wn = row_product_next(p, ysh[warp][h], Lg, nb, h ? k - 1 : k + 1, l, j + 1 < hp);
+        if (act) w = wn;
+        if (SMALL) {
 #pragma unroll
-        for (int d = 0; d < kSweepAhead; ++d) {
-            const int k = k0 - d;
-            if (k < 0) break;
-            const double lk = ring[d];
-            const int kn = k - kSweepAhead;
-            ring[d] = (kn >= 1 && t < min(w, kn)) ? Lg[(long long)(kn - 1 - t) * kLeafThreads + t] : 0.0;
-            const double pk = S.y[k];
-            if (t < min(w, k)) S.y[k - 1 - t] = fma(-lk, pk, S.y[k - 1 - t]);   // entry L[k][k-1-t]
-            __syncwarp(mask);
-        }
-    }
-    const GridDesc& G = v.grids[L.grid];
-    for (int k = t; k < n; k += kLeafThreads) {
-        const int i = k % w, j = k / w;
-        const long long c = G.c0 + (long long)(L.j0 + j) * G.nx + L.i0 + i;
-        if (accumulate) {
-            const DD x = dd_add(DD{v.p_hi[c], v.p_lo[c]}, DD{S.y[k], 0.0});
-            v.p_hi[c] = x.h;
-            v.p_lo[c] = x.l;
+            for (int c = 0; c < 8; ++c)
+                if (c < ccw) part[c] = fma((double)z[c], wn, part[c]);
         } else {
-            v.p_hi[c] = S.y[k];
+            for (int c = 0; c < cc; ++c)
+                acc[h * cz + c][l] = fma(act ? (double)Zk[c * nb + l] : 0.0, wn, acc[h * cz + c][l]);
+        }
+        __syncwarp();
+    }
+    // the middle plane
+    {
+        load_p(p, Lg, nb, g.M, l, true);
+        const double other = __shfl_xor_sync(0xffffffffu, w, 16);
+        const double wt = h ? other : w, wb = h ? w : other;       // (0 for a half without planes)
+        double y = 0.0;
+        if (l < nb) {
+            const CellFaces<DIM> f = cell_faces<DIM>(v, leaf, g, g.M, l);
+            y = particular_rhs<DIM>(v, leaf, f, q, bc_val);
+            if (g.halfplanes(0) > 0) y = fma(f.down(), wt, y);
+            if (g.halfplanes(1) > 0) y = fma(f.up(), wb, y);
+            if (h == 0) zb[g.M * nb + l] = y;
+        }
+        ysh[warp][h][l] = y;
+        __syncwarp();
+        w = half_product(p, ysh[warp][h], h);
+        w += __shfl_xor_sync(0xffffffffu, w, 16);
+    }
+    const TS* Zm = Zg + g.zoff(0, g.M);
+    double* rb = v.rbar + g.r_off;
+    auto store = [&](int t, double x) {
+        // a right-hand side sigma on this segment's interface row,
+        // F - D (lambda_other - lambda_own) = sigma, acts as rbar - sigma
+        rb[t] = with_sadj ? x - v.sadj[g.r_off + t] : x;
+    };
+    if (SMALL) {
+        // columns 8 h + c of the middle plane
+        double zm[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+            const int t = 8 * h + c;
+            zm[c] = l < nb && t < g.m ? (double)Zm[t * nb + l] * w : 0.0;
+        }
+        double* rs = &ysh[warp][0][0];                             // rbar by segment (m <= 16)
+        const double r = reduce_columns8(zm, l);
+        __syncwarp();
+        if (!(l & 1) && 8 * h + (l >> 1) < g.m) rs[8 * h + (l >> 1)] = r;
+        __syncwarp();
+        const double o = reduce_columns8(part, l);
+        for (int s = 0; s < 2; ++s) {
+            if (h == s && !(l & 1) && (l >> 1) < g.ncols(s)) rs[g.segment(s, l >> 1)] += o;
+            __syncwarp();
+        }
+        if (lane < g.m) store(lane, rs[lane]);
+        return;
+    }
+    for (int t = h; t < g.m; t += 2) acc[2 * cz + t][l] = l < nb ? (double)Zm[t * nb + l] * w : 0.0;
+    __syncwarp();
+    // each row summed by one lane (over the 16 cells), then the halves' rows
+    // added to their segments
+    for (int p = lane; p < 2 * cz + g.m; p += 32) {
+        double s0 = 0.0, s1 = 0.0;
+#pragma unroll
+        for (int c = 0; c < kPlane; c += 2) {
+            s0 += acc[p][c];
+            s1 += acc[p][c + 1];
+        }
+        acc[p][0] = s0 + s1;
+    }
+    __syncwarp();
+    for (int s = 0; s < 2; ++s) {
+        for (int p = lane; p < g.ncols(s); p += 32) acc[2 * cz + g.segment(s, p)][0] += acc[s * cz + p][0];
+        __syncwarp();
+    }
+    for (int t = lane; t < g.m; t += 32) store(t, acc[2 * cz + t][0]);
+}
+
+// x = A^-1 (A-elimination's right-hand sides), from the middle plane outwards;
+// rhs(h, k, l, Zk, cc): y_k + Z_k lambda at cell l (h < 0: the middle plane,
+// where each half warp returns its share), out(k, l, x).
+template <int DIM, class TS, class Rhs, class Out>
+__device__ __forceinline__ void solve_outward(const DevView& v, int leaf, const LeafGeo& g, const TS* Lg,
+                                              double (*ysh)[kPlane], int lane, Rhs&& rhs, Out&& out) {
+    const int h = lane >> 4, l = lane & 15, nb = g.nb, hp = g.halfplanes(h);
+    const int steps = max(g.halfplanes(0), g.halfplanes(1));
+    TS p[kPlane];
+    double x, tn = 0.0;
+    auto ahead = [&](int d) {                                      // coupling to the plane before, a plane ahead
+        if (d > hp || l >= nb) return;
+        const CellFaces<DIM> f = cell_faces<DIM>(v, leaf, g, h ? g.M + d : g.M - d, l);
+        tn = h ? f.down() : f.up();
+    };
+    ahead(1);
+    {
+        TS pm[kPlane];
+        load_p(pm, Lg, nb, g.M, l, true);
+        load_p(p, Lg, nb, h ? g.M + 1 : g.M - 1, l, hp > 0);
+        double y = rhs(-1, g.M, l);
+        y += __shfl_xor_sync(0xffffffffu, y, 16);
+        ysh[h][l] = y;
+        __syncwarp();
+        x = half_product(pm, ysh[h], h);
+        x += __shfl_xor_sync(0xffffffffu, x, 16);
+        __syncwarp();
+        if (h == 0 && l < nb) out(g.M, l, x);
+    }
+    double r = steps > 0 && hp > 0 ? rhs(h, h ? g.M + 1 : g.M - 1, l) : 0.0;
+    for (int d = 1; d <= steps; ++d) {
+        const bool act = d <= hp;
+        const int k = h ? g.M + d : g.M - d;
+        ysh[h][l] = act && l < nb ? fma(tn, x, r) : 0.0;
+        __syncwarp();
+        ahead(d + 1);
+        const double xn = row_product_next(p, ysh[h], Lg, nb, h ? k + 1 : k - 1, l, d + 1 <= hp);
+        if (d + 1 <= hp) r = rhs(h, h ? k + 1 : k - 1, l);         // the next plane's
+        if (act) x = xn;
+        if (act && l < nb) out(k, l, x);
+        __syncwarp();
+    }
+}
+
+// Final pressures p = A^-1 (bbar + B lambda), written into the state (p_hi,
+// p_lo) or added to it in double-double (refinement corrections).
+template <int DIM, class TS>
+__global__ void __launch_bounds__(32 * kSolveWarps) leaf_pressure_kernel(DevView v, bool accumulate, int mp, int cz) {
+    __shared__ double ysh[kSolveWarps][2][kPlane];
+    extern __shared__ __align__(16) double lam_raw[];              // per warp: lambda in the halves' orders
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int leaf = blockIdx.x * kSolveWarps + warp;
+    if (leaf >= v.nleaf) return;                                   // uniform over the warp
+    const LeafGeo g = leaf_geo<DIM>(v, leaf);
+    double* lam = lam_raw + (size_t)warp * (2 * cz + mp);
+    for (int t = lane; t < g.m; t += 32) lam[2 * cz + t] = v.lam[g.r_off + t];
+    __syncwarp();
+    for (int s = 0; s < 2; ++s)
+        for (int p = lane; p < g.ncols(s); p += 32) lam[s * cz + p] = lam[2 * cz + g.segment(s, p)];
+    __syncwarp();
+    const TS* Zg = leaf_Z<TS>(v) + g.Z_off;
+    const double* zb = v.leafzb + g.zb_off;
+    const int nb = g.nb;
+    auto rhs = [&](int h, int k, int l) -> double {
+        const bool mid = h < 0;
+        const int half = lane >> 4, cc = mid ? g.m : g.cols(h, k), step = mid ? 2 : 1;
+        const TS* Zk = Zg + g.zoff(mid ? 0 : h, k) + l;
+        const double* lm = lam + (mid ? 2 * cz : h * cz);
+        if (l >= nb) return 0.0;
+        double a = mid && half ? 0.0 : zb[k * nb + l];
+        int c = mid ? half : 0;
+        for (; c + 7 * step < cc; c += 8 * step) {                 // eight loads in flight
+            TS z[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) z[u] = Zk[(c + u * step) * nb];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) a = fma((double)z[u], lm[c + u * step], a);
+        }
+        TS z[8];
+#pragma unroll
+        for (int u = 0; u < 7; ++u) z[u] = c + u * step < cc ? Zk[(c + u * step) * nb] : (TS)0;
+#pragma unroll
+        for (int u = 0; u < 7; ++u)
+            if (c + u * step < cc) a = fma((double)z[u], lm[c + u * step], a);
+        return a;
+    };
+    solve_outward<DIM, TS>(v, leaf, g, leaf_L<TS>(v) + g.L_off, ysh[warp], lane, rhs, [&](int k, int l, double x) {
+        long long c;
+        if constexpr (DIM == 2) {
+            const LeafDesc& L = v.leaves[leaf];
+            const GridDesc& G = v.grids[L.grid];
+            c = G.c0 + (long long)(L.j0 + k) * G.nx + L.i0 + l;
+        } else {
+            const LeafDesc3& L = v.leaves3[leaf];
+            c = cell3(v.g3, L.i0 + l % g.w0, L.j0 + l / g.w0, L.k0 + k);
+        }
+        if (accumulate) {
+            const DD s = dd_add_d(DD{v.p_hi[c], v.p_lo[c]}, x);
+            v.p_hi[c] = s.h;
+            v.p_lo[c] = s.l;
+        } else {
+            v.p_hi[c] = x;
             v.p_lo[c] = 0.0;
         }
-    }}
+    });
+}
 
-template <int LPB, class TS>
-__global__ void __launch_bounds__(kLeafThreads * LPB)
-leaf_pressure_kernel(DevView v, bool accumulate) {
-    __shared__ LeafSolveSmem smem[LPB];
-    __shared__ double lam_s[LPB][64];
-    const int t = threadIdx.x & (kLeafThreads - 1);
-    const int slot_leaf = threadIdx.x / kLeafThreads;
-    const int leaf = blockIdx.x * LPB + slot_leaf;
-    if (leaf >= v.nleaf) return;
-    const unsigned mask = 0xFFFFu << (threadIdx.x & 16);
-    LeafSolveSmem& S = smem[slot_leaf];
-    double* lam = lam_s[slot_leaf];
-    const LeafDesc L = v.leaves[leaf];
-    if (L.w == kMaxLeafSide && L.h == kMaxLeafSide)
-        leaf_pressure_body<kMaxLeafSide * kMaxLeafSide, kMaxLeafSide, TS>(v, accumulate, S, lam, L, t, mask);
-    else
-        leaf_pressure_body<0, 0, TS>(v, accumulate, S, lam, L, t, mask);
+// Training targets of the learned surrogate: psi[item][k][s] (float; cell
+// k = i + 16 j, segment s fastest) = A^-1 B e_s of the leaves ids[item], from
+// the stored factors.
+template <class TS>
+__global__ void __launch_bounds__(32 * kSolveWarps) leaf_fields_kernel(DevView v, const int* __restrict__ ids,
+                                                                      int count, float* __restrict__ psi) {
+    __shared__ double ysh[kSolveWarps][2][kPlane];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int item = blockIdx.x * kSolveWarps + warp;
+    if (item >= count) return;                                     // uniform over the warp
+    const int id = ids[item];
+    if ((unsigned)id >= (unsigned)v.nleaf || v.leaves[id].m > 16) {
+        if (lane == 0) atomicOr(v.status, kStatusBadIndex);
+        return;
+    }
+    const LeafGeo g = leaf_geo<2>(v, id);
+    const TS* Zg = leaf_Z<TS>(v) + g.Z_off;
+    const int nb = g.nb;
+    for (int s = 0; s < g.m; ++s) {
+        int pos[2] = {-1, -1};
+        for (int h = 0; h < 2; ++h)
+            for (int p = 0; p < g.ncols(h); ++p)
+                if (g.segment(h, p) == s) pos[h] = p;
+        auto rhs = [&](int h, int k, int l) -> double {
+            if (l >= nb) return 0.0;
+            if (h < 0) return lane < 16 ? (double)Zg[g.zoff(0, k) + s * nb + l] : 0.0;
+            return pos[h] >= 0 && pos[h] < g.cols(h, k) ? (double)Zg[g.zoff(h, k) + pos[h] * nb + l] : 0.0;
+        };
+        solve_outward<2, TS>(v, id, g, leaf_L<TS>(v) + g.L_off, ysh[warp], lane, rhs, [&](int k, int l, double x) {
+            psi[((long long)item * 256 + k * nb + l) * 16 + s] = (float)x;
+        });
+    }
 }
 
 constexpr int kRedBlocks = 256;
@@ -611,46 +746,84 @@ __global__ void mean_subtract_kernel(DevView v, long long n) {
     }
 }
 
+template <int DIM, class T, int NW, int LPC, int TM = 1>
+cudaError_t build_launch(const DevView& v, int mp, int cz, cudaStream_t s) {
+    const int bytes = (int)LeafBuildSmem<DIM, T>::bytes(mp, cz), per = LPC * TM;
+    auto* kern = leaf_build_kernel<DIM, T, NW, LPC, TM>;
+    // set on every launch (a host call; the attribute belongs to the current device)
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes * per);
+    if (e != cudaSuccess) return e;
+    kern<<<(v.nleaf + per - 1) / per, 32 * NW * TM, bytes * per, s>>>(v, mp, cz, bytes);
+    return cudaGetLastError();
+}
+template <int DIM, class T>
+cudaError_t build_dispatch(const DevView& v, int mp, int cz, cudaStream_t s) {
+    // 2D leaves of up to 16 segments: one warp per two leaves (the FP64
+    // instructions of the inversions serve four blocks: a quarter fewer per
+    // leaf).  One leaf per warp while two would leave a last wave nearly empty
+    // (a wave of the former is 3648 leaves; 4096 leaves: 0.76 ms, two per warp
+    // 0.85; 24576: two per warp 5.2), and four warps to a leaf where not even
+    // that fills the schedulers (16 leaves: 0.20 ms; one warp per leaf in the
+    // elimination by cells before 0.62).  More segments: four warps per leaf
+    // share the products.
+    if (DIM == 2 && mp <= 16) {
+        if (v.nleaf <= 152 * 2) return build_launch<2, T, 4, 1>(v, mp, cz, s);
+        if (v.nleaf <= 152 * 32) return build_launch<2, T, 1, 1, kTeams>(v, mp, cz, s);
+        return build_launch<2, T, 1, 2, kTeams>(v, mp, cz, s);
+    }
+    return build_launch<DIM, T, 4, 1>(v, mp, cz, s);
+}
+template <int DIM, class TS>
+cudaError_t particular_launch(const DevView& v, const double* q, const double* bc_val, bool with_sadj, int mp, int cz,
+                              cudaStream_t s) {
+    const int grid = (v.nleaf + kSolveWarps - 1) / kSolveWarps;
+    if (cz <= 8 && mp <= 16) {
+        leaf_particular_kernel<DIM, TS, true><<<grid, 32 * kSolveWarps, 0, s>>>(v, q, bc_val, with_sadj, mp, cz);
+        return cudaGetLastError();
+    }
+    const int bytes = (int)sizeof(double) * kSolveWarps * (2 * cz + mp) * (kPlane + 1);
+    auto* kern = leaf_particular_kernel<DIM, TS, false>;
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e != cudaSuccess) return e;
+    kern<<<grid, 32 * kSolveWarps, bytes, s>>>(v, q, bc_val, with_sadj, mp, cz);
+    return cudaGetLastError();
+}
+template <int DIM, class TS>
+cudaError_t pressure_launch(const DevView& v, bool accumulate, int mp, int cz, cudaStream_t s) {
+    const int grid = (v.nleaf + kSolveWarps - 1) / kSolveWarps;
+    const int bytes = (int)sizeof(double) * kSolveWarps * (2 * cz + mp);
+    leaf_pressure_kernel<DIM, TS><<<grid, 32 * kSolveWarps, bytes, s>>>(v, accumulate, mp, cz);
+    return cudaGetLastError();
+}
+
 }  // namespace
 
-template <class T>
-static cudaError_t launch_leaf_build_t(const DevView& v, int max_m, cudaStream_t s) {
-    if (max_m <= 16) {
-        constexpr int LPB = 4;
-        const size_t sm = sizeof(LeafBuildSmem<16, T>) * LPB;
-        cudaFuncSetAttribute(leaf_build_kernel<16, LPB, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        leaf_build_kernel<16, LPB, T><<<(v.nleaf + LPB - 1) / LPB, kLeafThreads * LPB, sm, s>>>(v);
-    } else {
-        constexpr int LPB = 2;
-        const size_t sm = sizeof(LeafBuildSmem<64, T>) * LPB;
-        cudaFuncSetAttribute(leaf_build_kernel<64, LPB, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        leaf_build_kernel<64, LPB, T><<<(v.nleaf + LPB - 1) / LPB, kLeafThreads * LPB, sm, s>>>(v);
-    }
-    return cudaGetLastError();
+cudaError_t launch_leaf_build(const DevView& v, int max_m, int max_c, cudaStream_t s) {
+    const int mp = std::max(max_m, 1), cz = std::max(max_c, 1);
+    if (v.dim == 3) return build_dispatch<3, double>(v, mp, cz, s);
+    return v.leaf32 ? build_dispatch<2, float>(v, mp, cz, s) : build_dispatch<2, double>(v, mp, cz, s);
 }
 
-cudaError_t launch_leaf_build(const DevView& v, int max_m, cudaStream_t s) {
-    return v.leaf32 ? launch_leaf_build_t<float>(v, max_m, s) : launch_leaf_build_t<double>(v, max_m, s);
+cudaError_t launch_leaf_particular(const DevView& v, const double* q, const double* bc_val, bool with_sadj, int max_m,
+                                   int max_c, cudaStream_t s) {
+    const int mp = std::max(max_m, 1), cz = std::max(max_c, 1);
+    if (v.dim == 3) return particular_launch<3, double>(v, q, bc_val, with_sadj, mp, cz, s);
+    return v.leaf32 ? particular_launch<2, float>(v, q, bc_val, with_sadj, mp, cz, s)
+                    : particular_launch<2, double>(v, q, bc_val, with_sadj, mp, cz, s);
 }
 
-cudaError_t launch_leaf_particular(const DevView& v, const double* q, const double* bc_val,
-                                   bool with_sadj, cudaStream_t s) {
-    constexpr int LPB = 8;
-    const int grid = (v.nleaf + LPB - 1) / LPB;
-    if (v.leaf32)
-        leaf_particular_kernel<LPB, float><<<grid, kLeafThreads * LPB, 0, s>>>(v, q, bc_val, with_sadj);
-    else
-        leaf_particular_kernel<LPB, double><<<grid, kLeafThreads * LPB, 0, s>>>(v, q, bc_val, with_sadj);
-    return cudaGetLastError();
+cudaError_t launch_leaf_pressure(const DevView& v, bool accumulate, int max_m, int max_c, cudaStream_t s) {
+    const int mp = std::max(max_m, 1), cz = std::max(max_c, 1);
+    if (v.dim == 3) return pressure_launch<3, double>(v, accumulate, mp, cz, s);
+    return v.leaf32 ? pressure_launch<2, float>(v, accumulate, mp, cz, s)
+                    : pressure_launch<2, double>(v, accumulate, mp, cz, s);
 }
 
-cudaError_t launch_leaf_pressure(const DevView& v, bool accumulate, cudaStream_t s) {
-    constexpr int LPB = 8;
-    const int grid = (v.nleaf + LPB - 1) / LPB;
-    if (v.leaf32)
-        leaf_pressure_kernel<LPB, float><<<grid, kLeafThreads * LPB, 0, s>>>(v, accumulate);
-    else
-        leaf_pressure_kernel<LPB, double><<<grid, kLeafThreads * LPB, 0, s>>>(v, accumulate);
+cudaError_t launch_leaf_fields(const DevView& v, const int* ids, int count, float* psi, cudaStream_t s) {
+    if (count == 0) return cudaSuccess;
+    const int grid = (count + kSolveWarps - 1) / kSolveWarps;
+    if (v.leaf32) leaf_fields_kernel<float><<<grid, 32 * kSolveWarps, 0, s>>>(v, ids, count, psi);
+    else leaf_fields_kernel<double><<<grid, 32 * kSolveWarps, 0, s>>>(v, ids, count, psi);
     return cudaGetLastError();
 }
 

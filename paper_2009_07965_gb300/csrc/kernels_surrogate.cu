@@ -31,43 +31,9 @@ constexpr int kS = 16;          // output side (a full leaf)
 constexpr int kIn = kS + 2;     // input side with the halo
 
 // ---------------------------------------------------------------------------
-// Training targets and inputs from the plain method.
+// Network inputs from the plain method (the training targets: leaf_fields_kernel
+// in kernels_leaf.cu).
 //
-// psi[item][k][s] (float; cell k = i + 16 j, segment s fastest: the
-// network's NHWC output layout) for the leaves ids[item]: column s of
-// Z = L^-1 B scaled by D^-1, then the backward sweep L^T psi = y.
-template <class TS>
-__global__ void __launch_bounds__(128) leaf_fields_kernel(DevView v, const int* __restrict__ ids, int count,
-                                                          float* __restrict__ psi) {
-    __shared__ double ys[8][kS * kS];
-    const int t = threadIdx.x & 15, slot = threadIdx.x >> 4;
-    const int item = blockIdx.x * 8 + slot;
-    if (item >= count) return;                        // uniform over the leaf's 16 lanes
-    const unsigned mask = 0xFFFFu << (threadIdx.x & 16);
-    const int id = ids[item];
-    if ((unsigned)id >= (unsigned)v.nleaf || v.leaves[id].m > 16) {
-        if (t == 0) atomicOr(v.status, kStatusBadIndex);
-        return;
-    }
-    const LeafDesc L = v.leaves[id];
-    const int w = L.w, n = L.w * L.h, m = L.m;
-    const TS* Lg = leaf_L<TS>(v) + L.L_off;
-    const TS* Dg = Lg + (long long)n * kLeafThreads;
-    const TS* Zg = leaf_Z<TS>(v) + L.Z_off;
-    double* y = ys[slot];
-    for (int s = 0; s < m; ++s) {
-        for (int k = t; k < n; k += kLeafThreads) y[k] = (double)Zg[(long long)s * n + k] * (double)Dg[k];
-        __syncwarp(mask);
-        for (int k = n - 1; k >= 1; --k) {
-            const double pk = y[k];
-            if (t < min(w, k)) y[k - 1 - t] = fma(-(double)Lg[(long long)(k - 1 - t) * kLeafThreads + t], pk, y[k - 1 - t]);
-            __syncwarp(mask);
-        }
-        for (int k = t; k < n; k += kLeafThreads) psi[((long long)item * (kS * kS) + k) * 16 + s] = (float)y[k];
-        __syncwarp(mask);
-    }
-}
-
 // x[item][18][18][16] (bf16): channel 0 = (log K - its mean over the leaf)
 // / 2 on the leaf and its one-cell halo (0 outside the domain), channel 1 =
 // log10(alpha) / 3, the others 0.  The basis fields do not change when K is
@@ -439,14 +405,6 @@ __global__ void __launch_bounds__(kS * kS) leaf_apply_kernel(DevView v, const in
 
 }  // namespace
 
-cudaError_t launch_leaf_fields(const DevView& v, const int* ids, int count, float* psi, cudaStream_t s) {
-    if (count <= 0) return cudaSuccess;
-    if (v.leaf32)
-        leaf_fields_kernel<float><<<(count + 7) / 8, 128, 0, s>>>(v, ids, count, psi);
-    else
-        leaf_fields_kernel<double><<<(count + 7) / 8, 128, 0, s>>>(v, ids, count, psi);
-    return cudaGetLastError();
-}
 cudaError_t launch_leaf_patches(const DevView& v, const int* ids, int count, void* x, cudaStream_t s) {
     if (count <= 0) return cudaSuccess;
     leaf_patches_kernel<<<count, kIn * kIn, 0, s>>>(v, ids, static_cast<bf16*>(x));

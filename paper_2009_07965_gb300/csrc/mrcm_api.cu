@@ -14,6 +14,7 @@
 #include <unordered_map>
 #include <vector>
 
+#include "leaf_geometry.cuh"
 #include "mrcm_internal.h"
 #include "../../include/mrcm.h"
 
@@ -55,7 +56,7 @@ struct Plan {
     std::vector<MergeDesc> merges;       // grouped by height (ascending)
     std::vector<int> level_first, level_count, level_max_g2, level_max_m;  // index by height-1
     std::vector<int> node_map, gamma_segs;
-    int max_m_leaf = 0, max_g2 = 0;
+    int max_m_leaf = 0, max_c_leaf = 0, max_g2 = 0;
     // storage sizes (doubles / ints)
     long long nR = 0, nr = 0, nW = 0, nX = 0, nL = 0, nZ = 0, nzb = 0;
     std::vector<long long> node_R_off, node_r_off;
@@ -300,13 +301,15 @@ int make_plan(Plan& P) {
         LeafDesc& L = P.leaves[id];
         const long long n = (long long)L.w * L.h;
         L.L_off = P.nL;
-        P.nL += n * (kLeafThreads + 1);
         L.Z_off = P.nZ;
-        P.nZ += n * L.m;
         L.zb_off = P.nzb;
-        P.nzb += n;
         L.R_off = P.node_R_off[id];
         L.r_off = P.node_r_off[id];
+        const LeafGeo geo = leaf_geo2(L, P.gx, P.gy);
+        P.nL += n * L.w;
+        P.nZ += geo.zsize();
+        P.nzb += n;
+        P.max_c_leaf = std::max(P.max_c_leaf, std::max(geo.ncols(0), geo.ncols(1)));
         // flop model of the leaf kernel: LDL^T band steps, forward solve of
         // the Robin columns from their first nonzero row on, SYRK of the
         // lower triangle of the active columns (FMA = 2 flops)
@@ -623,9 +626,11 @@ int make_plan3d(Plan& P) {
     for (int id = 0; id < P.nleaf; ++id) {
         LeafDesc3& B = P.leaves3[id];
         const long long nn = (long long)B.w[0] * B.w[1] * B.w[2], m = B.m;
-        B.L_off = P.nL; P.nL += nn * nn;
-        B.Z_off = P.nZ; P.nZ += nn * m;
+        const LeafGeo geo = leaf_geo3(B);
+        B.L_off = P.nL; P.nL += nn * geo.nb;
+        B.Z_off = P.nZ; P.nZ += geo.zsize();
         B.zb_off = P.nzb; P.nzb += nn;
+        P.max_c_leaf = std::max(P.max_c_leaf, std::max(geo.ncols(0), geo.ncols(1)));
         B.R_off = P.node_R_off[id];
         B.r_off = P.node_r_off[id];
         std::vector<int> key(B.side_off, B.side_off + 6);
@@ -1296,8 +1301,6 @@ static int enqueue_build(mrcm_ctx* c, int& launches, bool merges_only = false) {
             TRYC(launch_coef3(v, s)); launches += 1 + (P.nseg > 0);
             TRYC(launch_gamma_scale(v, (int)P.gamma_segs.size(), s)); launches += !P.gamma_segs.empty();
         }
-        PhaseScope ps(c, MRCM_PHASE_LEAF_BUILD);
-        TRYC(launch_leaf3_build(v, s)); ++launches;
     } else if (!merges_only) {
         PhaseScope ps(c, MRCM_PHASE_COEF);
         TRYC(launch_check_K(v, s)); ++launches;
@@ -1306,9 +1309,9 @@ static int enqueue_build(mrcm_ctx* c, int& launches, bool merges_only = false) {
         TRYC(launch_face_coef(v, s)); ++launches;
         TRYC(launch_gamma_scale(v, (int)P.gamma_segs.size(), s)); launches += !P.gamma_segs.empty();
     }
-    if (!merges_only && P.dim != 3) {
+    if (!merges_only) {
         PhaseScope ps(c, MRCM_PHASE_LEAF_BUILD);
-        TRYC(launch_leaf_build(v, P.max_m_leaf, s)); ++launches;
+        TRYC(launch_leaf_build(v, P.max_m_leaf, P.max_c_leaf, s)); ++launches;
     }
     {
         const PhaseHook hook{c, phase_begin, phase_end};
@@ -1361,8 +1364,7 @@ static int solve_pass(mrcm_ctx* c, const double* q, const double* bc, bool with_
     cudaStream_t s = c->stream;
     {
         PhaseScope ps(c, MRCM_PHASE_LEAF_PART);
-        if (P.dim == 3) TRYC(launch_leaf3_particular(v, q, bc, with_sadj, s));
-        else TRYC(launch_leaf_particular(v, q, bc, with_sadj, s));
+        TRYC(launch_leaf_particular(v, q, bc, with_sadj, P.max_m_leaf, P.max_c_leaf, s));
         ++launches;
     }
     if (P.height > 0) {
@@ -1377,13 +1379,8 @@ static int solve_pass(mrcm_ctx* c, const double* q, const double* bc, bool with_
     }
     {
         PhaseScope ps(c, MRCM_PHASE_LEAF_PRESSURE);
-        if (P.dim == 3) {
-            TRYC(launch_leaf3_pressure(v, accumulate, s)); ++launches;
-            TRYC(launch_lam_to_PU(v, accumulate, s)); launches += P.nseg > 0;
-        } else {
-            TRYC(launch_leaf_pressure(v, accumulate, s)); ++launches;
-            TRYC(launch_lam_to_PU(v, accumulate, s)); launches += P.nseg > 0;
-        }
+        TRYC(launch_leaf_pressure(v, accumulate, P.max_m_leaf, P.max_c_leaf, s)); ++launches;
+        TRYC(launch_lam_to_PU(v, accumulate, s)); launches += P.nseg > 0;
     }
     return MRCM_OK;
 }

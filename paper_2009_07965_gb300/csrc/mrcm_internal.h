@@ -9,8 +9,6 @@ namespace mrcm {
 
 // Largest leaf side handled by the leaf kernels (cells).
 constexpr int kMaxLeafSide = 16;
-// Threads cooperating on one leaf.
-constexpr int kLeafThreads = 16;
 // Device status word bits (host maps them to MRCM_ERR_* codes).
 enum : int {
     kStatusBadK = 1,
@@ -49,10 +47,9 @@ struct LeafDesc {
     int side_off[4];   // local index of the first segment of side x-, x+, y-,
                        // y+ (-1 when the side lies on the domain boundary)
     int seg_off;       // offset of the leaf's segment ids in leaf_segs
-    long long L_off;   // band factor: n x 16 multipliers by column (step k: rows
-                       // k+1..k+16), then n reciprocal pivots
-    long long Z_off;   // Z = L^-1 B: n rows x m
-    long long zb_off;  // particular forward solve: n values
+    long long L_off;   // P_k of every plane (h of w x w)
+    long long Z_off;   // Z_k of every plane (leaf_geometry.cuh)
+    long long zb_off;  // particular right-hand sides y_k: n values
     long long R_off;   // node R (m x m) of the leaf
     long long r_off;   // node rbar / lambda (m values each, separate arrays)
 };
@@ -85,9 +82,9 @@ struct LeafDesc3 {
     int side_off[6];            // local index of the first segment of side x-, x+,
                                 // y-, y+, z-, z+ (-1: the side is on the domain boundary)
     int side_fine[6];           // 1: one segment per face; 0: one patch for the side
-    long long L_off;            // n x n: L below the diagonal (row-major), 1/d on it
-    long long Z_off;            // Z = L^-1 B: m columns of n
-    long long zb_off;           // particular forward solve: n values
+    long long L_off;            // P_k of every x-y plane
+    long long Z_off;            // Z_k of every plane (leaf_geometry.cuh)
+    long long zb_off;           // particular right-hand sides y_k: n values
     long long R_off, r_off;     // node R (m x m) and rbar / lambda (m)
 };
 
@@ -144,14 +141,14 @@ struct DevView {
     const int* node_map;
     const int* gamma_segs;
     // workspace
-    double* leafL;      // band factors
-    double* leafZ;      // Z per leaf
+    double* leafL;      // P_k of every leaf's planes
+    double* leafZ;      // Z_k of every leaf's planes
     float* leafL32;     // the same in FP32 (mixed precision: leaf work in FP32)
     float* leafZ32;
     int mixed;          // 1: the mixed form (the merges of FP32 levels in FP32)
     int leaf32;         // 1: leaf factors in FP32 (mixed form, mrcm_set_mixed_leaves)
     int res_dd;         // 1: refinement residuals in double-double, 0: in FP64 (mrcm_set_residual)
-    double* leafzb;     // particular forward solves
+    double* leafzb;     // particular right-hand sides y_k
     double* R;          // node maps (leaves and internal nodes)
     double* rbar;       // node particular fluxes
     double* gam_sq;     // D^1/2 and D^-1/2 of every gamma segment (gamma_segs order)
@@ -229,6 +226,13 @@ __device__ __forceinline__ DD dd_two_prod(double a, double b) {
 __device__ __forceinline__ DD dd_add(DD x, DD y) {
     const DD s = dd_two_sum(x.h, y.h);
     return dd_two_sum(s.h, __dadd_rn(s.l, __dadd_rn(x.l, y.l)));
+}
+// x + y for a normalised x: dd_add(x, {y, 0}) in 10 instructions instead of
+// 14 (x.h + y is 0 or no smaller than what is left over: a two-sum in order)
+__device__ __forceinline__ DD dd_add_d(DD x, double y) {
+    const DD s = dd_two_sum(x.h, y);
+    const double l = __dadd_rn(s.l, x.l), h = __dadd_rn(s.h, l);
+    return {h, __dsub_rn(l, __dsub_rn(h, s.h))};
 }
 __device__ __forceinline__ DD dd_mul_d(DD x, double b) {
     const DD p = dd_two_prod(x.h, b);
@@ -324,14 +328,16 @@ cudaError_t launch_reciprocal(const double* x, double* r, long long n, cudaStrea
 cudaError_t launch_cell_resist(const DevView& v, cudaStream_t s);
 cudaError_t launch_seg_beta(const DevView& v, cudaStream_t s);
 cudaError_t launch_face_coef(const DevView& v, cudaStream_t s);
-cudaError_t launch_leaf_build(const DevView& v, int max_m, cudaStream_t s);
+// Leaf kernels (2D leaves and 3D blocks); max_m: the most segments of a leaf,
+// max_c: the most columns that meet a plane other than a leaf's middle one.
+cudaError_t launch_leaf_build(const DevView& v, int max_m, int max_c, cudaStream_t s);
 // particular solve: q and bc_val are the data; bc_val == nullptr means zero
 // external data; with_sadj subtracts the interface right-hand sides.
 cudaError_t launch_leaf_particular(const DevView& v, const double* q, const double* bc_val,
-                                   bool with_sadj, cudaStream_t s);
+                                   bool with_sadj, int max_m, int max_c, cudaStream_t s);
 // p = A^-1 (bbar + B lambda) per leaf into the double-double state
 // (p_hi, p_lo): set, or accumulate (double-double add of the correction).
-cudaError_t launch_leaf_pressure(const DevView& v, bool accumulate, cudaStream_t s);
+cudaError_t launch_leaf_pressure(const DevView& v, bool accumulate, int max_m, int max_c, cudaStream_t s);
 // interface unknowns from the two Robin data of each segment (set or add)
 cudaError_t launch_lam_to_PU(const DevView& v, bool accumulate, cudaStream_t s);
 // residual of the discrete equations in double-double; fills rcell, sadj
@@ -345,13 +351,8 @@ cudaError_t launch_face_fluxes(const DevView& v, const double* bc_val, double* p
 // Learned basis surrogate (kernels_surrogate.cu): leaf lists are device
 // arrays of leaf ids (each checked; leaves with more than 16 segments are
 // refused); fields are float [item][16][256], patches bf16 [item][18][18][16].
-// The 3D path (kernels_3d.cu): coefficients, the leaf blocks' local Robin
-// problems, their solve-phase passes and the face fluxes.
+// The 3D path (kernels_3d.cu): coefficients, residuals and the face fluxes.
 cudaError_t launch_coef3(const DevView& v, cudaStream_t s);
-cudaError_t launch_leaf3_build(const DevView& v, cudaStream_t s);
-cudaError_t launch_leaf3_particular(const DevView& v, const double* q, const double* bc_val, bool with_sadj,
-                                    cudaStream_t s);
-cudaError_t launch_leaf3_pressure(const DevView& v, bool accumulate, cudaStream_t s);
 cudaError_t launch_residual3(const DevView& v, const double* q, const double* bc_val, int step, cudaStream_t s);
 cudaError_t launch_face_fluxes3(const DevView& v, const double* bc_val, double* p, double* Fx, double* Fy,
                                 double* Fz, double* iface, cudaStream_t s);

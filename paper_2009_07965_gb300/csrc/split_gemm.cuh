@@ -407,9 +407,11 @@ __device__ __forceinline__ void load_frag_b(FragB<S>& f, At&& at) {
         for (int s = 0; s < S; ++s) f.d[s][p] = d[s];
     }
 }
-// out[r]: row g + 8 (r / 2), column 2 t + r % 2 of the 16 x 8 product
+// out[r]: row g + 8 (r / 2), column 2 t + r % 2 of the 16 x 8 product, of whose
+// rows the first `rows` are wanted (0 past the eighth where there are no more)
 template <int S>
-__device__ __forceinline__ void frag_product(const FragA<S>& a, const FragB<S>& b, typename SplitAcc<S>::T (&out)[4]) {
+__device__ __forceinline__ void frag_product(const FragA<S>& a, const FragB<S>& b, typename SplitAcc<S>::T (&out)[4],
+                                             int rows = 16) {
     float acc[S][4];
 #pragma unroll
     for (int l = 0; l < S; ++l)
@@ -420,12 +422,15 @@ __device__ __forceinline__ void frag_product(const FragA<S>& a, const FragB<S>& 
 #pragma unroll
         for (int j = 0; j < S - i; ++j) mma_f16(acc[i + j], a.d[i], b.d[j][0], b.d[j][1]);
     const int t = threadIdx.x & 3;
+    const int eb[2] = {__shfl_sync(0xffffffffu, b.e, 8 * t), __shfl_sync(0xffffffffu, b.e, 8 * t + 4)};
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
+        out[r] = 0;
+        if (r >= 2 && rows <= 8) continue;
         float n[S];
 #pragma unroll
         for (int l = 0; l < S; ++l) n[l] = acc[l][r];
-        out[r] = combine_levels(n, r < 2 ? a.e0 : a.e1, __shfl_sync(0xffffffffu, b.e, (2 * t + (r & 1)) * 4));
+        out[r] = combine_levels(n, r < 2 ? a.e0 : a.e1, eb[r & 1]);
     }
 }
 
