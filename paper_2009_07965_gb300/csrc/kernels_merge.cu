@@ -1734,6 +1734,12 @@ static cudaError_t launch_small(const DevView& v, int first, int count, int max_
     return go(merge_small_kernel<F, kSmallThreads>, kSmallThreads);
 }
 
+// Items of one step of a sweep: the most CTAs it has work for.
+static long long sweep_items(int count, int max_g2) {
+    const int tiles = (max_g2 + kGJTile - 1) / kGJTile;
+    return (long long)count * (1 + tiles * (tiles + 1) / 2);
+}
+
 // The sweep of a blocked level with its tuning choice (0: the heuristic
 // below).  Every choice computes the same numbers: a tile is formed by the
 // same thread arithmetic whichever CTA shape runs it, so the tuner may pick
@@ -1760,9 +1766,7 @@ static cudaError_t sweep_launch(const DevView& v, int first, int count, int max_
             if (per_sm == 1) dyn = kSweepSmemPad;
         }
     }
-    const int tiles = (max_g2 + kGJTile - 1) / kGJTile;
-    const long long items = (long long)count * (1 + tiles * (tiles + 1) / 2);
-    int grid = (int)std::min<long long>(items, (long long)sms * per_sm);
+    int grid = (int)std::min<long long>(sweep_items(count, max_g2), (long long)sms * per_sm);
     grid = grid < 1 ? 1 : grid;
     // the grid barrier's arrival counter and the tile loops' ticket counter
     if ((e = cudaMemsetAsync(barrier, 0, 2 * sizeof(unsigned int), s)) != cudaSuccess) return e;
@@ -1898,6 +1902,8 @@ static cudaError_t tune_level_t(const DevView& v, int first, int count, int max_
     for (int per_sm : {1, 2, 3, 4}) {
         if (!factor && max_g2 <= kNodeMax) break;                         // one system per CTA: no shape to pick
         if (!factor && block_level(count, max_g2) && per_sm > 2) break;   // two CTAs fit an SM
+        // (past one padded CTA per SM) no more CTAs than at the shape before
+        if (per_sm > 2 && sweep_items(count, max_g2) <= (long long)sms * (per_sm - 1)) break;
         float t = 0.f;
         e = best_time(s, reps, e0, e1, [&] {
             return invert_launch<F>(v, first, count, max_g2, scratch, barrier, sms, per_sm, factor, s);
