@@ -1504,6 +1504,64 @@ __global__ void __launch_bounds__(256) tree_up_kernel(DevView v, TreeLevels L, u
         }
         if (!grid_barrier(counter, round, v.status, v.spin_limit)) return;
         if (mmax == 0) continue;                            // (the root) uniform
+        if (g2max >= 16 && (long long)count * mmax >= 2 * stride) {
+            // enough outputs to give eight of them to eight lanes: X is read
+            // in 64-byte pieces, 16 loads in flight per lane, each term of
+            // rgam serves eight products, and seven additions (not eight
+            // times three) sum the lanes: lane s ends with output s.  Bound by
+            // the FP64 pipe: box 256x256x64 6.2 -> 3.1 ms a pass (its 0.94 G
+            // products hold the pipe 1.6 ms, X takes 1.1 ms to read),
+            // 4096^2 0.67 -> 0.57, 24 ensembles 0.53 -> 0.44.  Heights with
+            // fewer outputs than two per thread need the lanes for
+            // parallelism: 64 merges of 2g = 32 would leave all but 750 of
+            // 77824 threads without work.
+            const int ngrp = (mmax + 7) / 8, sub = lane & 7;
+            const unsigned int m8 = 0xffu << (lane & 24);
+            for (long long t = t0 >> 3; t < (long long)count * ngrp; t += stride >> 3) {
+                int q, ig;
+                udivmod(t, ngrp, q, ig);
+                const MergeDesc& D = v.merges[first + q];
+                const int g2 = 2 * D.g, i0 = 8 * ig, nc = D.m - i0;
+                if (nc <= 0) continue;                      // uniform over the eight lanes
+                const double* rg = v.rgam + 2LL * D.gamma_off;
+                const double* xc = v.X + D.X_off + (long long)i0 * g2;
+                double acc[8];
+#pragma unroll
+                for (int c = 0; c < 8; ++c) acc[c] = 0.0;
+                for (int k = sub; k < g2; k += 16) {
+                    double x0[8], x1[8];
+                    const bool two = k + 8 < g2;
+                    const double r0 = __ldcg(rg + k), r1 = two ? __ldcg(rg + k + 8) : 0.0;
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) {
+                        x0[c] = c < nc ? xc[c * g2 + k] : 0.0;
+                        x1[c] = c < nc && two ? xc[c * g2 + k + 8] : 0.0;
+                    }
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) acc[c] = fma(x0[c], r0, acc[c]);
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) acc[c] = fma(x1[c], r1, acc[c]);
+                }
+#pragma unroll
+                for (int w = 4; w > 0; w >>= 1) {
+                    const bool up = sub & w;
+#pragma unroll
+                    for (int c = 0; c < w; ++c) {
+                        const double mine = up ? acc[c + w] : acc[c], theirs = up ? acc[c] : acc[c + w];
+                        acc[c] = mine + __shfl_xor_sync(m8, theirs, w);
+                    }
+                }
+                if (sub < nc) {
+                    const NodeRefs N = node_refs(v, D);
+                    const int i = i0 + sub;
+                    const double ro = i < N.o1 ? __ldcg(v.rbar + D.r1_off + N.opos1[i])
+                                               : __ldcg(v.rbar + D.r2_off + N.opos2[i - N.o1]);
+                    v.rbar[D.r_off + i] = acc[0] + ro;
+                }
+            }
+            if (h + 1 < L.height && !grid_barrier(counter, round, v.status, v.spin_limit)) return;
+            continue;
+        }
         const int lanes = tree_up_lanes(g2max);
         const unsigned int gmask = (lanes == 32 ? 0xffffffffu : ((1u << lanes) - 1u) << (lane & ~(lanes - 1)));
         const long long total = (long long)count * mmax * lanes;
