@@ -1862,11 +1862,24 @@ static cudaError_t sweep_attributes() {
 // keep the bits of the result.
 constexpr long long kBlockSweepWork = 540000;
 static bool block_level(int count, int max_g2) { return (long long)count * max_g2 * max_g2 >= kBlockSweepWork; }
+// Enough systems to fill the GPU at every phase of every step: one launch per
+// phase, the update on tcgen05 (both sweeps give the same bits; measured
+// against the cooperative one: 64 x 256 0.67 -> 0.57 ms, 128 x 128 0.34 -> 0.24,
+// 256 x 512 8.1 -> 5.8, FP32 8192 x 128 8.2 -> 5.2; with fewer systems the
+// inverse of the next block, which the cooperative sweep hides behind the
+// update, sets the pace: 32 x 256 FP32 0.29 -> 0.33, 16 x 512 0.96 -> 1.02, 8 x
+// 512 FP32 0.46 -> 0.62).
+constexpr int kPhaseSweepNodes = 64;
+constexpr long long kPhaseSweepWork = 1 << 20;
+static bool phase_level(int count, int max_g2) {
+    return count >= kPhaseSweepNodes && (long long)count * max_g2 * max_g2 >= kPhaseSweepWork;
+}
 template <class F>
 static cudaError_t invert_launch(const DevView& v, int first, int count, int max_g2, double* scratch, void* barrier,
                                  int sms, int per_sm, bool factor, cudaStream_t s) {
     constexpr bool fp32 = sizeof(F) == sizeof(float);
     if (!factor && max_g2 <= kNodeMax) return launch_node_invert(v, first, count, fp32, s);
+    if (!factor && phase_level(count, max_g2)) return launch_phase_sweep(v, first, count, max_g2, fp32, scratch, s);
     if (!factor && block_level(count, max_g2))
         return launch_block_sweep(v, first, count, max_g2, fp32, scratch, barrier, sms, per_sm == 1 ? 1 : 2, s);
     return sweep_launch<F>(v, first, count, max_g2, scratch, barrier, sms, per_sm, factor, s);
@@ -1959,6 +1972,7 @@ static cudaError_t tune_level_t(const DevView& v, int first, int count, int max_
     float best = 1e30f;
     for (int per_sm : {1, 2, 3, 4}) {
         if (!factor && max_g2 <= kNodeMax) break;                         // one system per CTA: no shape to pick
+        if (!factor && phase_level(count, max_g2)) break;                 // (plain launches)
         if (!factor && block_level(count, max_g2) && per_sm > 2) break;   // two CTAs fit an SM
         // (past one padded CTA per SM) no more CTAs than at the shape before
         if (per_sm > 2 && sweep_items(count, max_g2) <= (long long)sms * (per_sm - 1)) break;

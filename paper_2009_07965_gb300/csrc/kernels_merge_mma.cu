@@ -5,6 +5,7 @@
 #include "block_invert.cuh"
 #include "merge_common.cuh"
 #include "split_gemm.cuh"
+#include "tc_split.cuh"
 
 #include <algorithm>
 
@@ -555,6 +556,218 @@ __device__ void back_item(const DevView& v, const MergeDesc& D, int ti, int tj, 
     }
 }
 
+// ---------------------------------------------------------------------------
+// The same sweep for levels with work enough to fill the GPU at every step:
+// one launch per phase and step instead of one cooperative launch, each with
+// the CTA shape that suits it, and the update on the fifth-generation tensor
+// cores (tc_split.cuh).
+template <class T>
+__global__ void __launch_bounds__(kGemmThreads) sweep_form_kernel(DevView v, int first, int runs) {
+    __shared__ double red[kGemmWarps];
+    const MergeDesc& D = v.merges[first + blockIdx.x / runs];
+    const int r0 = (int)(blockIdx.x % runs) * 16;
+    if (r0 < 2 * D.g) form_rows<T>(v, D, r0, red);
+}
+// P of block `step`.
+constexpr int kNodeThreads = 128;
+template <class T>
+__global__ void __launch_bounds__(kNodeThreads, 4) sweep_inverse_kernel(DevView v, int first, int nmax, T* scratch,
+                                                                        int step) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    InvertSmem<T>& I = *reinterpret_cast<InvertSmem<T>*>(smem_raw);
+    const MergeDesc& D = v.merges[first + blockIdx.x];
+    const int n = 2 * D.g, k0 = step * kSweepB, nb = min(kSweepB, n - k0);
+    if (nb <= 0) return;
+    const T* A = sweep_matrix<T>(v) + D.W_off + (long long)k0 * n + k0;
+    for (int idx = threadIdx.x; idx < kInvert * kInvert; idx += kNodeThreads) {
+        const int r = idx / kInvert, c = idx % kInvert;
+        I.A[r][c] = r < nb && c <= r ? A[(long long)r * n + c] : (T)0;
+    }
+    invert_checked<kNodeThreads>(v, I, nb, D.g - k0);
+    T* P = SweepScratch<T>(scratch, blockIdx.x, nmax).p(step);
+    for (int idx = threadIdx.x; idx < kSweepB * kSweepB; idx += kNodeThreads) {
+        const int r = idx / kSweepB, c = idx % kSweepB, a = max(r, c), b = min(r, c);
+        P[idx] = a < nb ? neg_bits(I.A[a][b]) : (T)0;
+    }
+}
+template <class T>
+__global__ void __launch_bounds__(kGemmThreads, 2) sweep_panel_kernel(DevView v, int first, int count, int nmax,
+                                                                      T* scratch, int step) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int q = blockIdx.x % count, r = blockIdx.x / count;
+    panel_item<T>(v, v.merges[first + q], SweepScratch<T>(scratch, q, nmax), step, r >> 1, (r & 1) * kTileN, smem_raw);
+}
+// Eight entries of a scratch row (zeros where !on and past the nb set ones).
+template <class T>
+__device__ __forceinline__ void load_eight(T (&x)[8], const T* p, bool on, int nb) {
+    const int j = (threadIdx.x & 7) * 8;
+#pragma unroll
+    for (int i = 0; i < 8; i += 2) {
+        x[i] = x[i + 1] = (T)0;
+        if (on && j + i < nb) load_pair(x[i], x[i + 1], p + j + i);
+    }
+}
+__device__ __forceinline__ void store_pair(double* p, double a, double b) {
+    *reinterpret_cast<double2*>(p) = make_double2(a, b);
+}
+__device__ __forceinline__ void store_pair(float* p, float a, float b) {
+    *reinterpret_cast<float2*>(p) = make_float2(a, b);
+}
+// Half tiles (32 columns) per update item, and the items of a row pair's
+// (128 rows, pair p) half tiles up to the diagonal.
+constexpr int kTcStrip = 8;
+__host__ __device__ __forceinline__ int tc_pieces(int p, int nmax) {
+    const int halves = min(4 * p + 4, (nmax + kTcN - 1) / kTcN);
+    return (halves + kTcStrip - 1) / kTcStrip;
+}
+// The update of a strip of one row pair: the digits of C cut once, U's a half
+// tile ahead of the tensor cores, the results combined a half tile behind
+// them; then the swept block's rows and columns, from P and U.  FP64: one CTA
+// per SM (203 KB of digits, all of tensor memory), 16 warps, because the cutting
+// and combining (about 75 integer instructions an output), not the MMAs, set
+// the pace: a 128 x 32 half tile takes 2.3k cycles of tensor pipe; with eight
+// warps 15.5k cycles in all (256 x 512: 6.3 ms), with sixteen 5.8 ms, as 64 x 32
+// tiles of mma.sync at two CTAs per SM 8.1 ms.
+template <class T>
+__global__ void __launch_bounds__(kTcThreads, sizeof(T) == 8 ? 1 : 2)
+sweep_update_kernel(DevView v, int first, int count, int nmax, T* scratch, int step) {
+    constexpr int S = Slices<T>::S;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    TcSmem<S>& sm = *reinterpret_cast<TcSmem<S>*>(smem_raw);
+    const int q = blockIdx.x % count, tid = threadIdx.x;
+    int piece = blockIdx.x / count, p = (nmax + kTcM - 1) / kTcM - 1;
+    for (; piece >= tc_pieces(p, nmax); --p) piece -= tc_pieces(p, nmax);       // long rows first
+    const MergeDesc& D = v.merges[first + q];
+    const int n = 2 * D.g, k0 = step * kSweepB, nb = min(kSweepB, n - k0), r0 = p * kTcM;
+    if (nb <= 0 || r0 >= n) return;                                     // uniform per CTA
+    const int h0 = piece * kTcStrip, h1 = min(h0 + kTcStrip, min(4 * p + 4, (n + kTcN - 1) / kTcN));
+    const SweepScratch<T> sc(scratch, q, nmax);
+    T* A = sweep_matrix<T>(v) + D.W_off;
+    const bool lo = 2 * p != step, hi = 2 * p + 1 != step && r0 + kSweepB < n;  // the row blocks with products
+    auto next_product = [&](int h) {
+        for (; h < h1; ++h) {
+            const int tj = h >> 1;
+            if (tj != step && ((lo && tj <= 2 * p) || (hi && tj <= 2 * p + 1))) break;
+        }
+        return h;
+    };
+    const T* P = sc.p(step);
+    for (int h = h0; h < h1; ++h) {
+        const int tj = h >> 1, c0 = h * kTcN;
+        for (int ti = 2 * p; ti < 2 * p + 2; ++ti) {
+            if (ti != step && tj != step) continue;
+            // rows of the swept block are columns of U: a warp takes 8 rows x 4
+            // columns, whole sectors on both sides
+            const bool flip = ti == step && tj != step;
+            for (int idx = tid; idx < kSweepB * kTcN; idx += kTcThreads) {
+                const int b = idx >> 5, l = idx & 31;
+                const int r = ti * kSweepB + (flip ? 8 * (b >> 3) + (l >> 2) : b);
+                const int c = c0 + (flip ? 4 * (b & 7) + (l & 3) : l);
+                if (r >= n || c > r) continue;
+                T x;
+                if (ti == tj) x = neg_bits(P[(r - k0) * kSweepB + c - k0]);
+                else if (tj == step) x = sc.U[(long long)r * kSweepB + c - k0];
+                else x = sc.U[(long long)c * kSweepB + r - k0];
+                A[(long long)r * n + c] = x;
+            }
+        }
+    }
+    int h = next_product(h0);
+    if (h >= h1) return;
+    tc_begin(sm);
+    const int row = tid >> 3;                                           // (B: the first 32 of the CTA's 64 rows)
+    const bool stages_b = row < kTcN;                                   // uniform per warp
+    T vb[8];
+    auto load_b = [&](int hh) {
+        const int r = hh * kTcN + row;
+        load_eight(vb, sc.U + (long long)r * kSweepB, stages_b && hh < h1 && r < n, nb);
+    };
+    load_b(h);
+#pragma unroll
+    for (int i = 0; i < kTcM; i += kTcThreads / 8) {
+        const int r = r0 + i + row;
+        T va[8];
+        load_eight(va, sc.C + (long long)r * kSweepB, r < n && r / kSweepB != step, nb);
+        tc_stage_a<S>(sm, i + row, va);
+    }
+    if (stages_b) tc_stage_b<S>(sm, 0, row, vb);
+    tc_staged();
+    if (tid == 0) tc_issue(sm, 0, nb);
+    int hn = next_product(h + 1);
+    load_b(hn);
+    const int r = r0 + tc_row();
+    const bool mine = r < n && r / kSweepB != step;
+    bool ok = true;
+    for (int tile = 0;; ++tile) {
+        const int c0 = h * kTcN + tc_col();
+        T* Ar = A + (long long)r * n + c0;
+        T old[kTcOut];
+#pragma unroll
+        for (int c = 0; c < kTcOut; c += 2) {
+            old[c] = old[c + 1] = (T)0;
+            if (mine && c0 + c <= r) load_pair(old[c], old[c + 1], Ar + c);
+        }
+        if (hn < h1) {
+            if (stages_b) tc_stage_b<S>(sm, tile + 1, row, vb);
+            tc_staged();
+            if (tid == 0) tc_issue(sm, tile + 1, nb);
+        }
+        const int h2 = next_product(hn + 1);
+        load_b(h2);
+        if (ok) ok = tc_wait(sm, tile, v.status);
+#pragma unroll
+        for (int u = 0; u < kTcOut / 4; ++u) {
+            typename SplitAcc<S>::T x[4];
+            tc_outputs(sm, tile, u, x);
+#pragma unroll
+            for (int c = 0; c < 4; c += 2) {
+                const int cc = 4 * u + c;
+                const T y0 = old[cc] - (T)x[c], y1 = old[cc + 1] - (T)x[c + 1];
+                if (mine && c0 + cc + 1 <= r) store_pair(Ar + cc, y0, y1);
+                else if (mine && c0 + cc == r) Ar[cc] = y0;
+            }
+        }
+        if (hn >= h1) break;
+        h = hn;
+        hn = h2;
+    }
+    tc_end(sm);
+}
+template <class T>
+__global__ void __launch_bounds__(kGemmThreads) sweep_back_kernel(DevView v, int first, int tiles) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    int ti, tj;
+    tri_rc((int)(blockIdx.x % tiles), ti, tj);
+    back_item<T>(v, v.merges[first + blockIdx.x / tiles], ti, tj, *reinterpret_cast<BackSmem<T>*>(smem_raw));
+}
+
+template <class T>
+cudaError_t phase_sweep(const DevView& v, int first, int count, int nmax, T* scratch, cudaStream_t s) {
+    constexpr int S = Slices<T>::S;
+    constexpr int panel_bytes = (int)sizeof(SplitSmem<S>), inv_bytes = (int)sizeof(InvertSmem<T>);
+    constexpr int up_bytes = (int)sizeof(TcSmem<S>), back_bytes = (int)sizeof(BackSmem<T>);
+    cudaError_t e;
+    auto allow = [&](auto* kern, int bytes) {
+        return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    };
+    if ((e = allow(sweep_inverse_kernel<T>, inv_bytes)) != cudaSuccess) return e;
+    if ((e = allow(sweep_panel_kernel<T>, panel_bytes)) != cudaSuccess) return e;
+    if ((e = allow(sweep_update_kernel<T>, up_bytes)) != cudaSuccess) return e;
+    if ((e = allow(sweep_back_kernel<T>, back_bytes)) != cudaSuccess) return e;
+    const int nt = (nmax + kSweepB - 1) / kSweepB, runs = (nmax + 15) / 16;
+    const int gt = (nmax / 2 + kBackTile - 1) / kBackTile, tiles = gt * (gt + 1) / 2;
+    int pieces = 0;
+    for (int p = 0; p < (nmax + kTcM - 1) / kTcM; ++p) pieces += tc_pieces(p, nmax);
+    sweep_form_kernel<T><<<count * runs, kGemmThreads, 0, s>>>(v, first, runs);
+    for (int step = 0; step < nt; ++step) {
+        sweep_inverse_kernel<T><<<count, kNodeThreads, inv_bytes, s>>>(v, first, nmax, scratch, step);
+        sweep_panel_kernel<T><<<count * 2 * nt, kGemmThreads, panel_bytes, s>>>(v, first, count, nmax, scratch, step);
+        sweep_update_kernel<T><<<count * pieces, kTcThreads, up_bytes, s>>>(v, first, count, nmax, scratch, step);
+    }
+    sweep_back_kernel<T><<<count * tiles, kGemmThreads, back_bytes, s>>>(v, first, tiles);
+    return cudaGetLastError();
+}
+
 template <class T>
 constexpr size_t sweep_smem() {
     return std::max({sizeof(SplitSmem<Slices<T>::S>), sizeof(InvertSmem<T>), sizeof(BackSmem<T>)});
@@ -630,7 +843,6 @@ __global__ void __launch_bounds__(kGemmThreads, 2) block_sweep_kernel(DevView v,
 // inverse and W without leaving shared memory.  Four CTAs of four warps per SM:
 // a CTA waits for its chain of pivots most of the time, the others fill in
 // (4096 nodes of 2g = 64, FP64: 0.78 ms, 1.08 with two CTAs of eight warps).
-constexpr int kNodeThreads = 128;
 template <class T>
 __global__ void __launch_bounds__(kNodeThreads, 4) node_invert_kernel(DevView v, int first) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -708,6 +920,11 @@ cudaError_t launch_block_sweep(const DevView& v, int first, int count, int max_g
                                void* barrier, int sms, int per_sm, cudaStream_t s) {
     return fp32 ? block_sweep<float>(v, first, count, max_g2, reinterpret_cast<float*>(scratch), barrier, sms, per_sm, s)
                 : block_sweep<double>(v, first, count, max_g2, scratch, barrier, sms, per_sm, s);
+}
+cudaError_t launch_phase_sweep(const DevView& v, int first, int count, int max_g2, bool fp32, double* scratch,
+                               cudaStream_t s) {
+    return fp32 ? phase_sweep<float>(v, first, count, max_g2, reinterpret_cast<float*>(scratch), s)
+                : phase_sweep<double>(v, first, count, max_g2, scratch, s);
 }
 cudaError_t launch_node_invert(const DevView& v, int first, int count, bool fp32, cudaStream_t s) {
     return fp32 ? node_invert<float>(v, first, count, s) : node_invert<double>(v, first, count, s);

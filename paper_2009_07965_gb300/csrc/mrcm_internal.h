@@ -399,6 +399,8 @@ cudaError_t launch_merge_r(const DevView& v, int first, int count, int max_g2, i
 // T^-1 -> W of one height in blocks of 64 on the tensor cores; scratch:
 // sweep_node_scratch(max_g2) values of the arithmetic type per node.
 __host__ __device__ constexpr long long sweep_node_scratch(int nmax) { return 2LL * nmax * 64 + 2 * 64 * 64; }
+cudaError_t launch_phase_sweep(const DevView& v, int first, int count, int max_g2, bool fp32, double* scratch,
+                               cudaStream_t s);
 cudaError_t launch_block_sweep(const DevView& v, int first, int count, int max_g2, bool fp32, double* scratch,
                                void* barrier, int sms, int per_sm, cudaStream_t s);
 // T^-1 -> W of one height with 2g <= 64, one system per CTA

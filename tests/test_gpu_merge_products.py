@@ -110,3 +110,31 @@ def test_block_sweep_levels_match_the_host(mrcm_lib, precision, tol):
         e = rel(mr.mrcm_node_operator(b.ctx, v), _merge_on_host(mr, b.ctx, probs[owner[v]], v))
         assert e <= tol, (s, e)
     b.close()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("nx,ny,seg", [(170, 147, 1), (145, 150, 1), (276, 140, 2)])
+def test_phase_sweep_gives_the_bits_of_the_cooperative_one(mrcm_lib, nx, ny, seg, precision):
+    # 33 problems have 66 systems at the height of two merges per problem (one
+    # launch per phase, tcgen05), 30 have 60 (cooperative, mma.sync); the digit
+    # products are exact in both, so every map agrees bit for bit.  2g = 148 to
+    # 170, 130 and 136: last blocks of 2, 8, 20 and 42 rows, one and two row pairs
+    import torch
+    import paper_2009_07965_gb300 as mr
+    probs = [inputs.darcy_problem(nx, ny, sigma2=2.0, corr=0.1, seed=k % 5, bc="left_right", seg=(seg, seg))
+             for k in range(33)]
+    maps = []
+    for n in (33, 30):
+        b = mr.BatchSolver([torch.from_numpy(p.K).cuda() for p in probs[:n]], [(p.Lx, p.Ly) for p in probs[:n]],
+                           [p.bc_type for p in probs[:n]], sub=probs[0].sub, seg=(seg, seg), alpha=1.0,
+                           precision=mr.binding.MRCM_FP64 if precision == "fp64" else mr.binding.MRCM_MIXED)
+        b.build_basis()
+        nodes = mr.mrcm_query(b.ctx, "NODES")
+        info = [mr.mrcm_node_info(b.ctx, v) for v in range(nodes)]
+        top = max(i["height"] for i in info)
+        maps.append([mr.mrcm_node_operator(b.ctx, v) for h in range(top, 0, -1)
+                     for v in [u for u in range(nodes) if info[u]["height"] == h][:2] if info[v]["m"] > 0])
+        b.close()
+    assert len(maps[0]) == len(maps[1]) > 4
+    for x, y in zip(*maps):
+        assert np.array_equal(x, y)
