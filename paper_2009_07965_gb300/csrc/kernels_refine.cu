@@ -47,20 +47,24 @@ __device__ __forceinline__ DD seg_lam(const DevView& v, int t, int side_b) {
     return {x.x, x.y};
 }
 
-// Largest |x| over the CTA, one atomic per CTA (|x| >= 0: the IEEE bit
-// pattern orders like the value).
+// Largest |x| over the CTA (NaN ignored), one atomic per CTA.  |x| >= 0: the
+// IEEE bit pattern orders like the value, so the integer units find it (five
+// FP64 maxima a warp would be a quarter of what the FP64 residual costs).
+__device__ __forceinline__ unsigned long long warp_max_bits(unsigned long long b) {
+    const unsigned int hi = __reduce_max_sync(0xffffffffu, (unsigned int)(b >> 32));
+    const unsigned int lo = __reduce_max_sync(0xffffffffu, (unsigned int)(b >> 32) == hi ? (unsigned int)b : 0u);
+    return (unsigned long long)hi << 32 | lo;
+}
 __device__ __forceinline__ void block_record_max(unsigned long long* slot, double x) {
-    __shared__ double wmax[32];
-    double a = fabs(x);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) a = fmax(a, __shfl_xor_sync(0xffffffffu, a, o));
-    if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = a;
+    __shared__ unsigned long long wmax[32];
+    unsigned long long b = (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;
+    if (b > 0x7ff0000000000000ull) b = 0;
+    b = warp_max_bits(b);
+    if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = b;
     __syncthreads();
     if (threadIdx.x < 32) {
-        double b = threadIdx.x < (blockDim.x >> 5) ? wmax[threadIdx.x] : 0.0;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) b = fmax(b, __shfl_xor_sync(0xffffffffu, b, o));
-        if (threadIdx.x == 0 && b > 0.0) atomicMax(slot, (unsigned long long)__double_as_longlong(b));
+        b = warp_max_bits(threadIdx.x < (blockDim.x >> 5) ? wmax[threadIdx.x] : 0);
+        if (threadIdx.x == 0 && b > 0) atomicMax(slot, b);
     }
 }
 
@@ -69,18 +73,29 @@ __device__ __forceinline__ void block_record_max(unsigned long long* slot, doubl
 // the Robin datum of the cell's side), coef (pc - g) for a Dirichlet face.
 __device__ __forceinline__ DD face_out_u(DD pc, DD pn, double coef) { return dd_scale_u(dd_sub_u(pc, pn), coef); }
 
-// One face of cell c: its outward flux in the residual sum.  lower: the cell
-// lies below / left of the face (side a of a skeleton segment).
+// What a cell's pressure is compared with across one face: boundary value,
+// Robin datum of the cell's side (lower: the cell lies below / left of the
+// face, side a of a segment) or the neighbour's pressure.  Fetched before any
+// arithmetic: lanes whose faces are of different kinds (every warp of a row
+// crosses a segment) then share one pass of the FP64 pipe, which bounds these
+// kernels (with the integer maximum, FP64 residual of 4096^2 1.27 -> 0.57 ms,
+// double-double of 1024^2 0.25 -> 0.20, fluxes of 1024^2 0.21 -> 0.19).
+__device__ __forceinline__ DD across(const DevView& v, const double* bc_val, bool boundary, int seg, bool lower,
+                                     long long nb, long long bc_index) {
+    DD y = {0.0, 0.0};
+    if (boundary) y.h = bc_val[bc_index];
+    else if (seg >= 0) y = seg_lam(v, seg, lower ? 0 : 1);
+    else y = state_p(v, nb);
+    return y;
+}
+// One face of a cell: its outward flux in the residual sum.
 __device__ __forceinline__ DD cell_face(const DevView& v, const double* bc_val, int dirichlet, bool boundary,
                                         int seg, bool lower, double coef, double area, DD pc, long long nb,
                                         long long bc_index) {
-    if (boundary) {
-        const double g = bc_val[bc_index];
-        if (dirichlet) return face_out_u(pc, DD{g, 0.0}, coef);
-        return dd_two_prod(area, g);                 // Neumann: |e| g_N outward
-    }
-    if (seg >= 0) return face_out_u(pc, seg_lam(v, seg, lower ? 0 : 1), coef);
-    return face_out_u(pc, state_p(v, nb), coef);
+    const DD y = across(v, bc_val, boundary, seg, lower, nb, bc_index);
+    DD out = face_out_u(pc, y, coef);
+    if (boundary && !dirichlet) out = dd_two_prod(area, y.h);      // Neumann: |e| g_N outward
+    return out;
 }
 
 __global__ void __launch_bounds__(256) residual_cells_kernel(DevView v, const double* __restrict__ q,
@@ -95,7 +110,7 @@ __global__ void __launch_bounds__(256) residual_cells_kernel(DevView v, const do
         const long long fx = G.fx0 + i + (long long)(G.nx + 1) * j;
         const long long fy = G.fy0 + i + (long long)G.nx * j;
         const long long b0 = G.b0;
-        DD E = dd_two_sum(0.0, -q[c]);
+        DD E = {0.0 - q[c], 0.0};
         E = dd_acc_u(E, cell_face(v, bc_val, G.bc[0], i == 0, i > 0 ? v.xface_seg[fx] : -1, false, v.cxU[fx], G.hy,
                                   pc, c - 1, b0 + j));
         E = dd_acc_u(E, cell_face(v, bc_val, G.bc[1], i == G.nx - 1, i < G.nx - 1 ? v.xface_seg[fx + 1] : -1, true,
@@ -168,27 +183,20 @@ __global__ void __launch_bounds__(256) residual_cells_fp64_kernel(DevView v, con
         const long long fx = G.fx0 + i + (long long)(G.nx + 1) * j;
         const long long fy = G.fy0 + i + (long long)G.nx * j;
         const long long b0 = G.b0;
-        // outward flux of the cell through one face
-        auto face = [&](int dirichlet, bool boundary, int seg, bool lower, double coef, double area, long long nb,
-                        long long bc_index) -> double {
-            if (boundary) {
-                const double g = bc_val[bc_index];
-                return dirichlet ? coef * (pc - g) : area * g;
-            }
-            if (seg >= 0) {
-                const double2 l = v.seg_lam_dd[2 * seg + (lower ? 0 : 1)];
-                return coef * (pc - (l.x + l.y));
-            }
-            return coef * (pc - (v.p_hi[nb] + v.p_lo[nb]));
-        };
+        // outward flux of the cell through one face, added to E
         double E = -q[c];
-        E += face(G.bc[0], i == 0, i > 0 ? v.xface_seg[fx] : -1, false, v.cxU[fx], G.hy, c - 1, b0 + j);
-        E += face(G.bc[1], i == G.nx - 1, i < G.nx - 1 ? v.xface_seg[fx + 1] : -1, true, v.cxL[fx + 1], G.hy, c + 1,
-                  b0 + G.ny + j);
-        E += face(G.bc[2], j == 0, j > 0 ? v.yface_seg[fy] : -1, false, v.cyU[fy], G.hx, c - G.nx,
-                  b0 + 2 * G.ny + i);
-        E += face(G.bc[3], j == G.ny - 1, j < G.ny - 1 ? v.yface_seg[fy + G.nx] : -1, true, v.cyL[fy + G.nx], G.hx,
-                  c + G.nx, b0 + 2 * G.ny + G.nx + i);
+        auto face = [&](int dirichlet, bool boundary, int seg, bool lower, double coef, double area, long long nb,
+                        long long bc_index) {
+            const DD y = across(v, bc_val, boundary, seg, lower, nb, bc_index);
+            const bool neumann = boundary && !dirichlet;
+            E = fma(neumann ? area : coef, neumann ? y.h : pc - (y.h + y.l), E);
+        };
+        face(G.bc[0], i == 0, i > 0 ? v.xface_seg[fx] : -1, false, v.cxU[fx], G.hy, c - 1, b0 + j);
+        face(G.bc[1], i == G.nx - 1, i < G.nx - 1 ? v.xface_seg[fx + 1] : -1, true, v.cxL[fx + 1], G.hy, c + 1,
+             b0 + G.ny + j);
+        face(G.bc[2], j == 0, j > 0 ? v.yface_seg[fy] : -1, false, v.cyU[fy], G.hx, c - G.nx, b0 + 2 * G.ny + i);
+        face(G.bc[3], j == G.ny - 1, j < G.ny - 1 ? v.yface_seg[fy + G.nx] : -1, true, v.cyL[fy + G.nx], G.hx,
+             c + G.nx, b0 + 2 * G.ny + G.nx + i);
         e = E;
         v.rcell[c] = -e;
     }
@@ -301,16 +309,23 @@ __global__ void face_flux_kernel(DevView v, const double* __restrict__ bc_val, d
             F = G.bc[2 * axis + 1] ? cL[fl] * (pres(ca) - g) : area * g;
         } else {
             const int t = axis == 0 ? v.xface_seg[fl] : v.yface_seg[fl];
-            if (t >= 0) {
-                const double2 la = v.seg_lam_dd[2 * t], lb = v.seg_lam_dd[2 * t + 1];
-                const double da = cL[fl] * (pres(ca) - (la.x + la.y));
-                const double db = cU[fl] * (pres(cb) - (lb.x + lb.y));
-                fa = da;
-                fb = -db;
-                F = 0.5 * (da - db);
-                skel = true;
+            // lanes on and off the skeleton share the arithmetic of the side
+            // below where it counts (every warp of x faces has both)
+            if (kMode == 1 && t < 0) {
+                F = cL[fl] * (v.p_hi[ca] - v.p_hi[cb]);
             } else {
-                F = cL[fl] * (pres(ca) - pres(cb));
+                DD y;
+                if (t >= 0) y = seg_lam(v, t, 0);
+                else y = state_p(v, cb);
+                F = cL[fl] * (pres(ca) - (y.h + y.l));
+                if (t >= 0) {
+                    const double2 lb = v.seg_lam_dd[2 * t + 1];
+                    const double db = cU[fl] * (pres(cb) - (lb.x + lb.y));
+                    fa = F;
+                    fb = -db;
+                    F = 0.5 * (F - db);
+                    skel = true;
+                }
             }
         }
     } else if (line == 0) {
@@ -323,17 +338,17 @@ __global__ void face_flux_kernel(DevView v, const double* __restrict__ bc_val, d
         F = out.h + out.l;
     } else {
         const int t = axis == 0 ? v.xface_seg[fl] : v.yface_seg[fl];
+        DD y = state_p(v, cb);
+        if (t >= 0) y = seg_lam(v, t, 0);
+        const DD da = face_out_u(state_p(v, ca), y, cL[fl]);
+        F = da.h + da.l;
         if (t >= 0) {
-            const DD da = face_out_u(state_p(v, ca), seg_lam(v, t, 0), cL[fl]);
             const DD db = face_out_u(state_p(v, cb), seg_lam(v, t, 1), cU[fl]);
-            fa = da.h + da.l;
+            fa = F;
             fb = -(db.h + db.l);
             const DD dm = dd_sub_u(da, db);
             F = 0.5 * (dm.h + dm.l);
             skel = true;
-        } else {
-            const DD d = face_out_u(state_p(v, ca), state_p(v, cb), cL[fl]);
-            F = d.h + d.l;
         }
     }
     if (xface) {
