@@ -1907,7 +1907,7 @@ static cudaError_t launch_merge_build_t(const DevView& v, int first, int count, 
     {
         HookScope hs(hook, factor ? kPhRootFactor : kPhGjSweep);
         e = invert_launch<F>(v, first, count, max_g2, scratch, barrier, sms, tune.sweep_per_sm, factor, s);
-        ++*launches;
+        *launches += !factor && max_g2 > kNodeMax && phase_level(count, max_g2) ? phase_sweep_launches(max_g2) : 1;
         if (e != cudaSuccess) return e;
     }
     if (max_m > 0) {

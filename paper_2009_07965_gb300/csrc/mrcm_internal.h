@@ -399,6 +399,7 @@ cudaError_t launch_merge_r(const DevView& v, int first, int count, int max_g2, i
 // T^-1 -> W of one height in blocks of 64 on the tensor cores; scratch:
 // sweep_node_scratch(max_g2) values of the arithmetic type per node.
 __host__ __device__ constexpr long long sweep_node_scratch(int nmax) { return 2LL * nmax * 64 + 2 * 64 * 64; }
+inline int phase_sweep_launches(int max_g2) { return 2 + 3 * ((max_g2 + 63) / 64); }   // form, back; 3 per step
 cudaError_t launch_phase_sweep(const DevView& v, int first, int count, int max_g2, bool fp32, double* scratch,
                                cudaStream_t s);
 cudaError_t launch_block_sweep(const DevView& v, int first, int count, int max_g2, bool fp32, double* scratch,

@@ -138,3 +138,39 @@ def test_phase_sweep_gives_the_bits_of_the_cooperative_one(mrcm_lib, nx, ny, seg
     assert len(maps[0]) == len(maps[1]) > 4
     for x, y in zip(*maps):
         assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("nx,ny,seg", [(170, 147, 1), (163, 150, 1)])
+def test_strips_give_the_bits_of_the_tiles(mrcm_lib, nx, ny, seg, precision):
+    # 40 problems have heights wide enough for the strips of X and R
+    # (2g <= 128), 6 problems take the tiles; g, m and the children's
+    # shares of m on and off the edges of the 64 x 32 tiles and of
+    # the 16-entry steps of k.  One chunk of k: exact digit products in both
+    import torch
+    import paper_2009_07965_gb300 as mr
+    probs = [inputs.darcy_problem(nx, ny, sigma2=2.0, corr=0.1, seed=k % 5, bc="left_right", seg=(seg, seg))
+             for k in range(40)]
+    maps, n_small = [], 6
+    for n in (40, n_small):
+        b = mr.BatchSolver([torch.from_numpy(p.K).cuda() for p in probs[:n]], [(p.Lx, p.Ly) for p in probs[:n]],
+                           [p.bc_type for p in probs[:n]], sub=probs[0].sub, seg=(seg, seg), alpha=1.0,
+                           precision=mr.binding.MRCM_FP64 if precision == "fp64" else mr.binding.MRCM_MIXED)
+        b.build_basis()
+        nodes = mr.mrcm_query(b.ctx, "NODES")
+        info = [mr.mrcm_node_info(b.ctx, v) for v in range(nodes)]
+        heights = {}
+        for v, i in enumerate(info):
+            if i["height"] > 0:
+                heights.setdefault(i["height"], []).append(v)
+        out = []
+        for h in sorted(heights):
+            width = max(2 * info[v]["g"] for v in heights[h])
+            # the same inverses in both: up to 2g = 64, or enough work for the block sweep in the small batch
+            if 32 < width <= 64 or 64 < width <= 128 and len(heights[h]) * n_small / n * width ** 2 >= 540000:
+                out += [((h, v - heights[h][0]), mr.mrcm_node_operator(b.ctx, v)) for v in heights[h][:6]]
+        maps.append(out)
+        b.close()
+    assert len(maps[0]) == len(maps[1]) >= 12
+    for (k0, x), (k1, y) in zip(*maps):
+        assert k0 == k1 and np.array_equal(x, y), k0
