@@ -156,7 +156,11 @@ __global__ void __launch_bounds__(kGemmThreads, 2) merge_rupdate_strip_kernel(De
 }
 
 // Whether a level's products run as strips: one chunk of k, and the strips
-// fill the resident CTAs (two per SM) three times over.
+// fill the resident CTAs (two per SM) three times over; with fewer a strip's
+// tiles in series outlast the tiles of their own CTAs side by side.  (Strips of
+// 128 rows on tcgen05, one CTA per SM, three to five tiles behind a prologue that
+// nothing overlaps: X of 2g = 128 0.94 -> 0.67 ms, but X of 2g = 64 0.50 -> 0.88
+// and R 1.21 -> 1.44, box 128x128x64 as a whole 36.9 -> 37.2; not kept.)
 bool strips(int max_g2, long long ctas) { return max_g2 <= 2 * kChunkK && ctas >= 3 * 2 * 152; }
 
 template <int S>
@@ -206,6 +210,12 @@ cudaError_t r_launch(const DevView& v, int first, int count, int max_g2, int max
 // sequential chain of pivots runs beside the other tiles' products; then W.
 // A grid barrier between the phases (two per 64 rows); with more items than
 // CTAs the update items are handed out by ticket.
+//
+// Bound by its chain (90 to 100 us per 64 rows: 64 pivots, two barriers) where
+// systems are few, else by the update.  Measured against the FP64 sweep of
+// gj_sweep_kernel: 256 nodes of 2g = 512 63.7 -> 8.1 ms, 512 of 256 19.1 -> 3.1
+// (both go to the phase launches below since), 2 of 1024 3.0 -> 1.5, 1 of 2048
+// (the root of 4096^2, a factorisation before) 4.2 -> 3.3.
 constexpr int kSweepB = kInvert;
 static_assert(kSweepB == kChunkK && kSweepB == kTileM && kSweepB == 2 * kTileN, "one chunk, one tile row per block");
 
