@@ -707,7 +707,8 @@ sweep_update_kernel(DevView v, int first, int count, int nmax, T* scratch, int s
     load_b(hn);
     const int r = r0 + tc_row();
     const bool mine = r < n && r / kSweepB != step;
-    bool ok = true;
+    bool ok = true;                                                     // (uniform per warp)
+    int issued = 0;
     for (int tile = 0;; ++tile) {
         const int c0 = h * kTcN + tc_col();
         T* Ar = A + (long long)r * n + c0;
@@ -718,30 +719,33 @@ sweep_update_kernel(DevView v, int first, int count, int nmax, T* scratch, int s
             if (mine && c0 + c <= r) load_pair(old[c], old[c + 1], Ar + c);
         }
         if (hn < h1) {
-            if (stages_b) tc_stage_b<S>(sm, tile + 1, row, vb);
-            tc_staged();
+            if (stages_b && ok) tc_stage_b<S>(sm, tile + 1, row, vb);
+            if (tc_staged(!ok)) break;                                  // a warp gave up on a tile
             if (tid == 0) tc_issue(sm, tile + 1, nb);
+            issued = tile + 1;
         }
         const int h2 = next_product(hn + 1);
         load_b(h2);
-        if (ok) ok = tc_wait(sm, tile, v.status);
+        ok = ok && tc_wait(sm, tile, v.spin_limit);
+        if (ok) {
 #pragma unroll
-        for (int u = 0; u < kTcOut / 4; ++u) {
-            typename SplitAcc<S>::T x[4];
-            tc_outputs(sm, tile, u, x);
+            for (int u = 0; u < kTcOut / 4; ++u) {
+                typename SplitAcc<S>::T x[4];
+                tc_outputs(sm, tile, u, x);
 #pragma unroll
-            for (int c = 0; c < 4; c += 2) {
-                const int cc = 4 * u + c;
-                const T y0 = old[cc] - (T)x[c], y1 = old[cc + 1] - (T)x[c + 1];
-                if (mine && c0 + cc + 1 <= r) store_pair(Ar + cc, y0, y1);
-                else if (mine && c0 + cc == r) Ar[cc] = y0;
+                for (int c = 0; c < 4; c += 2) {
+                    const int cc = 4 * u + c;
+                    const T y0 = old[cc] - (T)x[c], y1 = old[cc + 1] - (T)x[c + 1];
+                    if (mine && c0 + cc + 1 <= r) store_pair(Ar + cc, y0, y1);
+                    else if (mine && c0 + cc == r) Ar[cc] = y0;
+                }
             }
         }
         if (hn >= h1) break;
         h = hn;
         hn = h2;
     }
-    tc_end(sm);
+    tc_end(sm, ok, issued, v.status);
 }
 template <class T>
 __global__ void __launch_bounds__(kGemmThreads) sweep_back_kernel(DevView v, int first, int tiles) {

@@ -63,14 +63,6 @@ __device__ __forceinline__ void tc_begin(TcSmem<S>& sm) {
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
-template <int S>
-__device__ __forceinline__ void tc_end(TcSmem<S>& sm) {
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    if (threadIdx.x < 32)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(sm.tmem), "r"(2 * S * kTcN));
-}
-
 // The digits of row `row` of an operand (eight lanes per row, lane j entries
 // 8 j .. 8 j + 7 in v) to dst + digit * dig.
 template <int S, class T>
@@ -100,11 +92,11 @@ __device__ __forceinline__ void tc_stage_b(TcSmem<S>& sm, int tile, int row, con
     tc_stage<S>(&sm.B[tile & 1][0], kTcN * 16, TcSmem<S>::kStepB, sm.eb[tile & 3], row, v);
 }
 // Makes the CTA's staged digits visible to the tensor cores; then thread 0
-// may issue.
-__device__ __forceinline__ void tc_staged() {
+// may issue.  True (all threads) when stop holds on any thread.
+__device__ __forceinline__ bool tc_staged(bool stop = false) {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
+    return __syncthreads_or(stop);
 }
 // All digit products of a tile (kn entries of k), by one thread.
 template <int S>
@@ -124,18 +116,25 @@ __device__ __forceinline__ void tc_issue(TcSmem<S>& sm, int tile, int kn) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                      smem_u32(&sm.bar[buf])) : "memory");
 }
-// Waits for a tile; false (and kStatusTimeout) when it does not come.
+// Waits for a tile, at most `limit` blocking polls (and at most kTcPolls: a
+// poll may suspend the warp for many microseconds) after one that does not
+// block.  False, on every lane of the warp, when the tile did not come.
+constexpr int kTcPolls = 1 << 16;
 template <int S>
-__device__ __forceinline__ bool tc_wait(TcSmem<S>& sm, int tile, int* status) {
-    const unsigned parity = (tile >> 1) & 1;
-    unsigned done = 0;
-    for (int spin = 0; spin < (1 << 16) && !done; ++spin)
+__device__ __forceinline__ bool tc_wait(TcSmem<S>& sm, int tile, long long limit) {
+    const unsigned bar = smem_u32(&sm.bar[tile & 1]), parity = (tile >> 1) & 1;
+    unsigned done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.b32 %0, 1, 0, p;\n\t}"
+        : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+    const int polls = (int)min(limit, (long long)kTcPolls);
+    for (int spin = 0; spin < polls && !done; ++spin)
         asm volatile(
             "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.b32 %0, 1, 0, p;\n\t}"
-            : "=r"(done) : "r"(smem_u32(&sm.bar[tile & 1])), "r"(parity) : "memory");
+            : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+    const bool all = __all_sync(0xffffffffu, done);
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (!done) atomicOr(status, kStatusTimeout);
-    return done;
+    return all;
 }
 // Row and first column of this thread's outputs of a tile.
 __device__ __forceinline__ int tc_row() { return threadIdx.x & 127; }
@@ -159,6 +158,21 @@ __device__ __forceinline__ void tc_outputs(TcSmem<S>& sm, int tile, int q, typen
         for (int l = 0; l < S; ++l) x[l] = n[l][u];
         out[u] = combine_levels(x, ea, sm.eb[tile & 3][c + u]);
     }
+}
+// Frees the tensor memory; by the whole CTA.  ok: this warp saw every tile it
+// waited for.  Where one did not, the tiles still in flight (up to `last`, the
+// last one issued) are waited for first, again with a limit: the tensor cores
+// read this CTA's shared memory and write its tensor memory until then.
+template <int S>
+__device__ __forceinline__ void tc_end(TcSmem<S>& sm, bool ok, int last, int* status) {
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    if (__syncthreads_or(!ok)) {
+        if (threadIdx.x == 0) atomicOr(status, kStatusTimeout);
+        for (int tile = max(last - 1, 0); tile <= last; ++tile) tc_wait(sm, tile, kTcPolls);
+        __syncthreads();
+    }
+    if (threadIdx.x < 32)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(sm.tmem), "r"(2 * S * kTcN));
 }
 
 }  // namespace
