@@ -46,10 +46,15 @@ __device__ __forceinline__ void tc_mma(unsigned d, unsigned long long a, unsigne
 // FP16 x FP16 -> FP32, both operands K-major, M = 128
 __device__ __forceinline__ unsigned tc_idesc(int n) { return 1u << 4 | (unsigned)(n >> 3) << 17 | (kTcM >> 4) << 24; }
 
+// The .sync.aligned forms of tcgen05 want every lane of the warp together; what
+// comes before them here (predicated loads and stores, loops with early ends)
+// may leave a warp split, so each is preceded by a __syncwarp().
+//
 // Tensor memory for the two accumulator sets, and the barriers; by the whole CTA.
 template <int S>
 __device__ __forceinline__ void tc_begin(TcSmem<S>& sm) {
     if (threadIdx.x < 32) {
+        __syncwarp();
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sm.tmem)),
                      "r"(2 * S * kTcN) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
@@ -145,6 +150,7 @@ __device__ __forceinline__ void tc_outputs(TcSmem<S>& sm, int tile, int q, typen
     const int c = tc_col() + 4 * q;
     const unsigned t = sm.tmem + (tile & 1) * S * kTcN + c + ((threadIdx.x & 96) << 16);
     float n[S][4];
+    __syncwarp();
 #pragma unroll
     for (int l = 0; l < S; ++l)
         asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
@@ -171,8 +177,10 @@ __device__ __forceinline__ void tc_end(TcSmem<S>& sm, bool ok, int last, int* st
         for (int tile = max(last - 1, 0); tile <= last; ++tile) tc_wait(sm, tile, kTcPolls);
         __syncthreads();
     }
-    if (threadIdx.x < 32)
+    if (threadIdx.x < 32) {
+        __syncwarp();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(sm.tmem), "r"(2 * S * kTcN));
+    }
 }
 
 }  // namespace
