@@ -129,10 +129,12 @@ __device__ __forceinline__ void digit_pair(T x, T y, int E, unsigned (&out)[S]) 
     }
 }
 // The biased FP64 exponent of a row from the largest exponent field of its
-// entries (FP32's 255, an infinity or NaN, as 2047).
+// entries (FP32's 255, an infinity or NaN, as 2047; a row without numbers,
+// whose digits mean nothing, far below all others).
+constexpr int kZeroExp = -(1 << 14);
 template <class T>
 __device__ __forceinline__ int common_exponent(int E) {
-    return sizeof(T) == 8 || E == 0 ? E : (E == 255 ? 2047 : E + 896);
+    return E == 0 ? kZeroExp : (sizeof(T) == 8 ? E : (E == 255 ? 2047 : E + 896));
 }
 
 // Writes the digit pairs of this lane's entries of one row (eight lanes).
@@ -227,12 +229,15 @@ __device__ __forceinline__ double combine_levels(const float (&n)[8], int ea, in
 }
 // The same for S = 4 in FP32 (the levels are exact integers; one rounding
 // per step of the Horner sum).
-__device__ __forceinline__ float pow2f(int e) {         // 2^e, flushed to 0 / infinity outside the FP32 range
-    return __int_as_float(e < -126 ? 0 : (e > 127 ? 0x7f800000 : (e + 127) << 23));
+__device__ __forceinline__ float pow2f(int e) {         // 2^e, kept within the normal FP32 range, 0 below it
+    return __int_as_float(e < -126 ? 0 : (min(e, 127) + 127) << 23);
 }
 __device__ __forceinline__ float combine_levels(const float (&n)[4], int ea, int eb) {
     const float v = fmaf(fmaf(fmaf(n[0], 256.f, n[1]), 256.f, n[2]), 256.f, n[3]);
-    const float f = v * pow2f(ea - 1041) * pow2f(eb - 1041);
+    // 2^(ea + eb - 2082) as two factors: either exponent may be far out of the
+    // FP32 range where their sum is not
+    const int e = max(ea + eb - 2082, 2 * kZeroExp), h = e >> 1;
+    const float f = v * pow2f(h) * pow2f(e - h);
     return (ea == 2047 || eb == 2047) ? __int_as_float(0x7fc00000) : f;
 }
 // x as a double by integer operations (a conversion instruction holds the
