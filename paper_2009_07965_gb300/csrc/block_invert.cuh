@@ -192,13 +192,17 @@ __device__ bool invert_block(InvertSmem<T>& S, int nb, Ok&& pivot_ok) {
         auto c_entry = [&](int bx, int r, int k) -> T {
             return bx > kb ? S.A[bx * kPlane + r][k0 + k] : S.A[k0 + k][bx * kPlane + r];
         };
+        // the powers of two that level the products over this block's columns
+        int sk[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) sk[i] = half_exponent(S.P[frag_k(i)][frag_k(i)]);
         // U = C P, A_KK = -P
         for (int item = warp; item < 2 * (nblk - 1); item += NW) {
             const int q = item >> 1, nt = item & 1, bx = q < kb ? q : q + 1;
             FragA<SL> a;
             FragB<SL> b;
-            load_frag_a<SL, T>(a, [&](int r, int k) { return c_entry(bx, r, k); });
-            load_frag_b<SL, T>(b, [&](int n, int k) { return S.P[8 * nt + n][k]; });
+            load_frag_a<SL, T>(a, sk, 1, [&](int r, int k) { return c_entry(bx, r, k); });
+            load_frag_b<SL, T>(b, sk, -1, [&](int n, int k) { return S.P[8 * nt + n][k]; });
             typename SplitAcc<SL>::T out[4];
             frag_product(a, b, out);
 #pragma unroll
@@ -221,10 +225,10 @@ __device__ bool invert_block(InvertSmem<T>& S, int nb, Ok&& pivot_ok) {
                 if (bx == kb || by == kb) continue;
                 for (int nt = 0; nt < 2; ++nt, ++item) {
                     if (item < lo || item >= hi) continue;
-                    if (have != bx) load_frag_a<SL, T>(a, [&](int r, int k) { return c_entry(bx, r, k); });
+                    if (have != bx) load_frag_a<SL, T>(a, sk, 1, [&](int r, int k) { return c_entry(bx, r, k); });
                     have = bx;
                     FragB<SL> b;
-                    load_frag_b<SL, T>(b, [&](int n, int k) { return S.U[by * kPlane + 8 * nt + n][k]; });
+                    load_frag_b<SL, T>(b, sk, -1, [&](int n, int k) { return S.U[by * kPlane + 8 * nt + n][k]; });
                     typename SplitAcc<SL>::T out[4];
                     frag_product(a, b, out);
 #pragma unroll

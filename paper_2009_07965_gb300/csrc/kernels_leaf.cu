@@ -266,7 +266,10 @@ leaf_build_kernel(DevView v, int mp, int cz, int bytes) {
             }
             // stage 0: V = P Z; stage 1: R += Z^T V, entries (row, n), row >= n, of
             // the column order; 16 x 8 tiles dealt to the warps
-            int item = 0;
+            // (P goes as P_kk^1/2 over k, Z as P_kk^-1/2, V as P_kk^1/2 again)
+            int item = 0, sk[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) sk[i] = half_exponent(s.P[h][tri_at(frag_k(i), frag_k(i))]);
 #pragma unroll 1
             for (int stage = 0; stage < 2; ++stage) {
                 const int mt = stage ? (cc + 15) / 16 : 1;
@@ -281,7 +284,7 @@ leaf_build_kernel(DevView v, int mp, int cz, int bytes) {
                         if (NW > 1 && (item + ni) % NW != warp) continue;
                         if (!loaded) {
                             const T *zp = &zs[16 * ri][0], *pp = s.P[h];
-                            load_frag_a<S, T>(a, [&](int r, int k) {
+                            load_frag_a<S, T>(a, sk, stage ? 1 : -1, [&](int r, int k) {
                                 return r < rows ? (stage ? zp[r * (kPlane + 1) + k] : pp[tri_at(r, k)]) : (T)0;
                             });
                             loaded = true;
@@ -289,7 +292,7 @@ leaf_build_kernel(DevView v, int mp, int cz, int bytes) {
                         const T* bp = &(stage ? vs : zs)[8 * ni][0];
                         FragB<S> b;
                         load_frag_b<S, T>(
-                            b, [&](int n, int k) { return 8 * ni + n < cc ? bp[n * (kPlane + 1) + k] : (T)0; });
+                            b, sk, stage ? -1 : 1, [&](int n, int k) { return 8 * ni + n < cc ? bp[n * (kPlane + 1) + k] : (T)0; });
                         typename SplitAcc<S>::T out[4];
                         frag_product(a, b, out, rows);
 #pragma unroll

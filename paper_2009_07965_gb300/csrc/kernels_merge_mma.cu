@@ -17,6 +17,14 @@ namespace {
 // of X's columns are cut on either side of o1.  W is symmetric: its row r is
 // read as column r, contiguous in k, and the map of a child is symmetric:
 // column j of C is read along the map's row of that segment.
+//
+// Powers of two of the two products: column k of W (and row k of X) goes as
+// D_k^-1/2, row k of C as D_k^1/2, D the Robin coefficient of the segment.
+struct GammaScale {
+    const double* sq;                      // D^1/2 of the node's gamma segments
+    int sign;
+    __device__ __forceinline__ int operator()(int k) const { return sign * whole_exponent(sq[k]); }
+};
 template <int S>
 __global__ void __launch_bounds__(kGemmThreads, 2) merge_x_kernel(DevView v, int first) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -38,7 +46,8 @@ __global__ void __launch_bounds__(kGemmThreads, 2) merge_x_kernel(DevView v, int
     typename SplitAcc<S>::T sum[2][4];
     split_product<S, double, false, true>(
         sm, g, gpos, [&](int r) { return r0 + r < g2 ? W + (long long)(r0 + r) * g2 : nullptr; },
-        [&](int j) { return j0 + j < jend ? Rc + (long long)opos[j0 + j] * mc : nullptr; }, sum);
+        [&](int j) { return j0 + j < jend ? Rc + (long long)opos[j0 + j] * mc : nullptr; },
+        GammaScale{v.gam_sq + D.gamma_off, 1}, sum);
     double* X = v.X + D.X_off;
 #pragma unroll
     for (int mt = 0; mt < 2; ++mt)
@@ -74,7 +83,8 @@ __global__ void __launch_bounds__(kGemmThreads, 2) merge_rupdate_kernel(DevView 
     typename SplitAcc<S>::T sum[2][4];
     split_product<S, double, true, false>(
         sm, g, gpos, [&](int i) { return i0 + i < iend ? Rc + (long long)opos[i0 + i] * mc : nullptr; },
-        [&](int j) { return j0 + j < m ? X + (long long)(j0 + j) * g2 : nullptr; }, sum);
+        [&](int j) { return j0 + j < m ? X + (long long)(j0 + j) * g2 : nullptr; },
+        GammaScale{v.gam_sq + D.gamma_off, -1}, sum);
     double* Rp = v.R + D.R_off;
 #pragma unroll
     for (int mt = 0; mt < 2; ++mt)
@@ -116,7 +126,7 @@ __global__ void __launch_bounds__(kGemmThreads, 2) merge_x_strip_kernel(DevView 
             const int j = jbeg + t * kTileN + c;
             return j < jend ? Rc + (long long)opos[j] * mc : nullptr;
         },
-        [](int, int, int) { return 0.0; },
+        GammaScale{v.gam_sq + D.gamma_off, 1}, [](int, int, int) { return 0.0; },
         [&](int t, int i, int c, double x, double) {
             const int r = r0 + i, j = jbeg + t * kTileN + c;
             if (r < g2 && j < jend) X[(long long)j * g2 + r] = neg_bits(x);
@@ -143,6 +153,7 @@ __global__ void __launch_bounds__(kGemmThreads, 2) merge_rupdate_strip_kernel(De
         sm, g, half ? N.gpos2 : N.gpos1, 0, (iend + kTileN - 1) / kTileN,
         [&](int i) { return i0 + i < iend ? Rc + (long long)opos[i0 + i] * mc : nullptr; },
         [&](int t, int c) { return t * kTileN + c < m ? X + (long long)(t * kTileN + c) * g2 : nullptr; },
+        GammaScale{v.gam_sq + D.gamma_off, -1},
         [&](int t, int r, int c) {
             const int i = i0 + r, j = t * kTileN + c;                   // R_oo: both on one child
             return i < iend && j <= i && half == (j >= o1) ? Rc[(long long)opos[i] * mc + opos[j]] : 0.0;
@@ -234,6 +245,13 @@ struct SweepScratch {
         P = U + (long long)nmax * kSweepB;
     }
     __device__ __forceinline__ T* p(int step) const { return P + (step & 1) * kSweepB * kSweepB; }
+};
+// Powers of two of the products over a swept block's columns: C_xk goes as
+// P_kk^-1/2 of its inverse, P_kc and U_xk as P_kk^1/2.
+template <class T>
+struct BlockScale {
+    const T* P;
+    __device__ __forceinline__ int operator()(int k) const { return half_exponent(P[k * (kSweepB + 1)]); }
 };
 
 // 1 / sum D of a pinned node's gamma segments (the regularised all-Neumann
@@ -336,7 +354,7 @@ __device__ void panel_item(const DevView& v, const MergeDesc& D, const SweepScra
     typename SplitAcc<S>::T sum[2][4];
     split_product<S, T, false, false>(
         sm, nb, nullptr, [&](int x) { return x < nx ? rows + x * ld : nullptr; },
-        [&](int c) { return h0 + c < nb ? P + (h0 + c) * kSweepB : nullptr; }, sum);
+        [&](int c) { return h0 + c < nb ? P + (h0 + c) * kSweepB : nullptr; }, BlockScale<T>{P}, sum);
     T* U = sc.U + (long long)x0 * kSweepB;
 #pragma unroll
     for (int mt = 0; mt < 2; ++mt)
@@ -409,6 +427,7 @@ __device__ void update_strip(const DevView& v, const MergeDesc& D, const SweepSc
     }
     int h = next_product(h0);
     if (h >= h1) return;
+    const int power = tid < nb ? BlockScale<T>{P}(tid) : 0;             // in flight with the rows
     T vb[kLaneK];
     load_scratch_row(vb, sc.U + (long long)(h * kTileN + row) * kSweepB, h * kTileN + row < n, nb);
     {
@@ -418,13 +437,20 @@ __device__ void update_strip(const DevView& v, const MergeDesc& D, const SweepSc
             const int r = r0 + row + p * kPassRows;
             load_scratch_row(va[p], sc.C + (long long)r * kSweepB, r < n, nb);
         }
-        __syncthreads();                                                // the CTA's previous item is done with sm
+        if (tid < kChunkK) sm.sk[tid] = power;                          // (the CTA's previous item has ended)
+        __syncthreads();
+        int s[kLaneK];
+        load_scale(s, sm.sk);
 #pragma unroll
-        for (int p = 0; p < 2; ++p) stage_row<S>(sm.A, sm.ea, row + p * kPassRows, nb, va[p]);
+        for (int p = 0; p < 2; ++p) stage_row<S, 1>(sm.A, sm.ea, row + p * kPassRows, nb, va[p], s);
     }
     for (;;) {
         const int c0 = h * kTileN;
-        stage_row<S>(sm.B, sm.eb, row, nb, vb);
+        {
+            int s[kLaneK];
+            load_scale(s, sm.sk);
+            stage_row<S, -1>(sm.B, sm.eb, row, nb, vb, s);
+        }
         __syncthreads();
         const int hn = next_product(h + 1);
         if (hn < h1) load_scratch_row(vb, sc.U + (long long)(hn * kTileN + row) * kSweepB, hn * kTileN + row < n, nb);
@@ -474,7 +500,7 @@ __device__ void next_inverse(const DevView& v, const MergeDesc& D, const SweepSc
         split_product<S, T, false, false>(
             sm, kSweepB, nullptr, [&](int x) { return x < nb1 ? sc.C + (long long)(k1 + x) * kSweepB : nullptr; },
             [&](int c) { return h * kTileN + c < nb1 ? sc.U + (long long)(k1 + h * kTileN + c) * kSweepB : nullptr; },
-            sum[h]);
+            BlockScale<T>{sc.p(step)}, sum[h]);
     }
     __syncthreads();
 #pragma unroll
@@ -662,6 +688,7 @@ sweep_update_kernel(DevView v, int first, int count, int nmax, T* scratch, int s
         return h;
     };
     const T* P = sc.p(step);
+    const int power = tid < nb ? BlockScale<T>{P}(tid) : 0;             // in flight with what follows
     for (int h = h0; h < h1; ++h) {
         const int tj = h >> 1, c0 = h * kTcN;
         for (int ti = 2 * p; ti < 2 * p + 2; ++ti) {
@@ -684,6 +711,7 @@ sweep_update_kernel(DevView v, int first, int count, int nmax, T* scratch, int s
     }
     int h = next_product(h0);
     if (h >= h1) return;
+    if (tid < kSweepB) sm.sk[tid] = power;
     tc_begin(sm);
     const int row = tid >> 3;                                           // (B: the first 32 of the CTA's 64 rows)
     const bool stages_b = row < kTcN;                                   // uniform per warp

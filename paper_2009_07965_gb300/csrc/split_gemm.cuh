@@ -16,10 +16,23 @@
 // of a chunk the eight integers of an output are combined in 64-bit integer
 // arithmetic, rounded once to FP64 and added to the running sum.
 //
-// Against an FP64 fused multiply-add loop: an operand is exact unless it is
-// more than 2^10 below the largest entry of its row in the chunk (then it is
-// rounded to 2^-63 of that entry), and one rounding per 64 terms takes the
-// place of one per term.
+// Accuracy.  An operand is exact unless it is more than 2^10 below the largest
+// entry of its row in the chunk; then it is cut off at 2^-62 of that entry.
+// With the dropped levels the error of a chunk's sum is below a few 2^-62
+// max_k |a_k| max_k |b_k|, plus the one rounding (an FP64 loop: 2^-53 of every
+// partial sum).  Where the terms themselves are as large as that product of
+// maxima, this is the smaller error; where a and b are large at different k
+// (a = (1, 2^-20), b = (2^-20, 1): 3e-13 of the sum) it would be the larger.
+// The operands of the merges and leaves are graded like that by the contrast
+// of the permeability, but by factors that are known: the column k of one
+// operand goes as 1 / d_k, the row k of the other as d_k, with d = D^1/2 of
+// the interface segments, or the square root of a diagonal of an inverse.  So
+// each product takes the power of two nearest below d_k (sc), which the cutting
+// adds to the exponents: no rounding, and both rows are level in k.  (K
+// contrast 1e11, one-face segments, node maps against quadruple precision,
+// entries over the roots of their diagonals: without the powers 7.5e-15 to
+// 1.2e-14, with them and in FMA loops 1e-16 to 1.6e-15.  They cost 0.3 to 1%
+// of a build in FP64, 1 to 2% of a mixed one, whose cutting is the larger part.)
 //
 // S = 4 (31 bits, 10 digit products) serves the FP32 merges of the mixed
 // form: more than an FP32 operand's 24 bits of the largest entry, sums
@@ -36,9 +49,9 @@
 // unit u at u ^ (row % 8): the eight rows an ldmatrix reads and the four rows
 // a staging warp writes then lie in distinct banks.
 //
-// Measured (one GB300, all heights): 4096^2 X 14.46 -> 2.33 ms, R 12.65 -> 2.41
+// Measured (one GB300, all heights): 4096^2 X 14.46 -> 2.41 ms, R 12.65 -> 2.43
 // against FP64 FMA loops at 97 and 92% of the FP64 peak; box 128x128x64 X
-// 27.5 -> 4.7, R 23.6 -> 5.5.  Seven digits in four warps per CTA were as fast
+// 27.5 -> 4.8, R 23.6 -> 5.5.  Seven digits in four warps per CTA were as fast
 // (2.25 and 2.67 ms) and less exact: node maps against quadruple precision 2.1e-15
 // at alpha = 100 (now 1.9e-16, the FMA loops 2.4e-16), boxes against a dense
 // FP64 solution 6.3e-13 (now 2.6e-13, the FMA loops 2.7e-13).
@@ -61,6 +74,7 @@ struct SplitSmem {
     __half A[S][kTileM][kChunkK];
     __half B[S][kTileN][kChunkK];
     int ea[kTileM], eb[kTileN];          // largest biased exponent of each row in the chunk
+    __align__(8) int sk[kChunkK];        // powers of two of the chunk's k (where a strip keeps them)
 };
 // Position of entry k of a staged row.
 __device__ __forceinline__ int swizzled(int row, int k) { return ((k >> 3) ^ (row & 7)) * 8 + (k & 7); }
@@ -86,33 +100,55 @@ __device__ __forceinline__ int out_row(int mt, int r) {
 }
 __device__ __forceinline__ int out_col(int r) { return warp_n0() + 2 * (threadIdx.x & 3) + (r & 1); }
 
-// The digits of |x| relative to the row exponent E, one byte each (the
-// leading digit as it is, in [0, 128]; the others + 128), the last digit in
-// the lowest byte.
+// Exponents of rows without numbers, and of rows with an infinity or a NaN.
+constexpr int kZeroExp = -(1 << 14), kNonFiniteExp = 1 << 14;
 __device__ __forceinline__ unsigned high_word(double x) { return (unsigned)__double2hiint(x); }
 __device__ __forceinline__ unsigned high_word(float x) { return __float_as_uint(x); }
-__device__ __forceinline__ int exponent_bits(double x) { return __double2hiint(x) & 0x7ff00000; }
-__device__ __forceinline__ int exponent_bits(float x) { return __float_as_int(x) & 0x7f800000; }
+__device__ __forceinline__ int exponent_field(double x) { return (int)((high_word(x) >> 20) & 0x7ffu); }
+__device__ __forceinline__ int exponent_field(float x) { return (int)((high_word(x) >> 23) & 0xffu); }
+// Biased exponent of x 2^s, |s| <= 512 (FP32: 64; the square root of a number's
+// range).  Zeros, and subnormals with them, must lie 63 (31) places below
+// every number of a row: an FP64 zero's exponent is s itself, below the 640
+// that common_exponent() asks of a row; FP32 has no such room and takes a
+// select.
+__device__ __forceinline__ int scaled_exponent(double x, int s) { return exponent_field(x) + s; }
+__device__ __forceinline__ int scaled_exponent(float x, int s) {
+    const int f = exponent_field(x);
+    return f + (f == 0 ? kZeroExp : s);
+}
+// floor(log2(x^(1/2))), 0 for what has none: the power of two that levels the
+// products with an inverse of diagonal x.
+template <class T>
+__device__ __forceinline__ int half_exponent(T x) {
+    const int f = exponent_field(x);
+    return (f == 0 || f == (sizeof(T) == 8 ? 2047 : 255)) ? 0 : (f - (sizeof(T) == 8 ? 1023 : 127)) >> 1;
+}
+// floor(log2(x)) of a positive normal x
+__device__ __forceinline__ int whole_exponent(double x) { return exponent_field(x) - 1023; }
+
+// The digits of |x|, d binary places below the row's exponent, one byte each
+// (the leading digit as it is, in [0, 128]; the others + 128), the last digit
+// in the lowest byte.
 template <int S>
-__device__ __forceinline__ unsigned long long digit_bytes(double x, int E) {
+__device__ __forceinline__ unsigned long long digit_bytes(double x, int d) {
     const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-    const int d = min(E - (int)((hi >> 20) & 0x7ffu), S == 8 ? 63 : 31);
+    d = min(d, S == 8 ? 63 : 31);
     const unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 42) | ((unsigned long long)lo << 10);
     if (S == 8) return (m >> d) + 0x0080808080808080ull;
     return (m >> (d + 32)) + 0x00808080ull;
 }
 template <int S>
-__device__ __forceinline__ unsigned digit_bytes(float x, int E) {       // S = 4
+__device__ __forceinline__ unsigned digit_bytes(float x, int d) {       // S = 4
     const unsigned b = __float_as_uint(x);
-    return ((((b & 0x7fffffu) | 0x800000u) << 7) >> min(E - (int)((b >> 23) & 0xffu), 31)) + 0x00808080u;
+    return ((((b & 0x7fffffu) | 0x800000u) << 7) >> min(d, 31)) + 0x00808080u;
 }
 
 // The digits of two entries of a row as FP16 pairs (the layout of an MMA
-// operand register).
+// operand register), dx and dy places below their row's exponent.
 template <int S, class T>
-__device__ __forceinline__ void digit_pair(T x, T y, int E, unsigned (&out)[S]) {
+__device__ __forceinline__ void digit_pair(T x, T y, int dx, int dy, unsigned (&out)[S]) {
     const unsigned ha = high_word(x), hb = high_word(y);
-    const unsigned long long ua = digit_bytes<S>(x, E), ub = digit_bytes<S>(y, E);
+    const unsigned long long ua = digit_bytes<S>(x, dx), ub = digit_bytes<S>(y, dy);
     // the signs as FP16 factors sigma = +-1, and -1152 sigma, -1024 sigma: a
     // digit is (1024 + byte) sigma - (1024 or 1152) sigma, exact
     const unsigned sg = __byte_perm(ha, hb, 0x7030);
@@ -128,33 +164,38 @@ __device__ __forceinline__ void digit_pair(T x, T y, int E, unsigned (&out)[S]) 
         out[s] = *reinterpret_cast<const unsigned*>(&h);
     }
 }
-// The biased FP64 exponent of a row from the largest exponent field of its
-// entries (FP32's 255, an infinity or NaN, as 2047; a row without numbers,
-// whose digits mean nothing, far below all others).
-constexpr int kZeroExp = -(1 << 14);
+// The biased FP64 exponent of a row from the largest exponent of its entries:
+// below 2^-383 (FP64) a row counts as zero, and from 2^512 (FP32: 2^64) on,
+// where an infinity or NaN lies whatever its power of two, as not finite.
+// Scaled entries go as the square root of the data's range and stay inside.
 template <class T>
 __device__ __forceinline__ int common_exponent(int E) {
-    return E == 0 ? kZeroExp : (sizeof(T) == 8 ? E : (E == 255 ? 2047 : E + 896));
+    if (sizeof(T) == 8) return E < 640 ? kZeroExp : (E >= 1535 ? kNonFiniteExp : E);
+    return E >= 191 ? kNonFiniteExp : E + 896;
 }
 
-// Writes the digit pairs of this lane's entries of one row (eight lanes).
-template <int S, int ROWS, class T>
-__device__ __forceinline__ void stage_row(__half (*dst)[ROWS][kChunkK], int* e, int row, int kn, const T (&v)[kLaneK]) {
-    int E = 0;
+// Writes the digit pairs of this lane's entries of one row (eight lanes),
+// entry i times 2^(SIGN s[i]).
+template <int S, int SIGN, int ROWS, class T>
+__device__ __forceinline__ void stage_row(__half (*dst)[ROWS][kChunkK], int* e, int row, int kn, const T (&v)[kLaneK],
+                                          const int (&s)[kLaneK]) {
+    int ex[kLaneK], E = kZeroExp;
 #pragma unroll
-    for (int i = 0; i < kLaneK; ++i) E = max(E, exponent_bits(v[i]));
+    for (int i = 0; i < kLaneK; ++i) {
+        ex[i] = scaled_exponent(v[i], SIGN * s[i]);
+        E = max(E, ex[i]);
+    }
 #pragma unroll
     for (int w = 1; w < 8; w <<= 1) E = max(E, __shfl_xor_sync(0xffffffffu, E, w));
-    E = sizeof(T) == 8 ? E >> 20 : E >> 23;
     if (stage_q() == 0) e[row] = common_exponent<T>(E);
     const int kend = (kn + 15) & ~15;
 #pragma unroll
     for (int i = 0; i < kLaneK; i += 2) {
         if (8 * i >= kend) break;
         unsigned d[S];
-        digit_pair<S>(v[i], v[i + 1], E, d);
+        digit_pair<S>(v[i], v[i + 1], E - ex[i], E - ex[i + 1], d);
 #pragma unroll
-        for (int s = 0; s < S; ++s) *reinterpret_cast<unsigned*>(&dst[s][row][swizzled(row, lane_k(i))]) = d[s];
+        for (int j = 0; j < S; ++j) *reinterpret_cast<unsigned*>(&dst[j][row][swizzled(row, lane_k(i))]) = d[j];
     }
 }
 
@@ -224,7 +265,7 @@ __device__ __forceinline__ double combine_levels(const float (&n)[8], int ea, in
     unsigned long long bits = ((unsigned long long)(be - 1) << 52) + mant;
     if (u == 0 || be <= 0) bits = 0;                                          // zero or underflow
     if (be >= 2047) bits = 0x7ff0000000000000ull;                             // overflow
-    if (ea == 2047 || eb == 2047) bits = 0x7ff8000000000000ull;               // an infinity or NaN among the entries
+    if (max(ea, eb) >= kNonFiniteExp) bits = 0x7ff8000000000000ull;           // an infinity or NaN among the entries
     return __longlong_as_double((long long)(bits | (s & 0x8000000000000000ull)));
 }
 // The same for S = 4 in FP32 (the levels are exact integers; one rounding
@@ -238,7 +279,7 @@ __device__ __forceinline__ float combine_levels(const float (&n)[4], int ea, int
     // FP32 range where their sum is not
     const int e = max(ea + eb - 2082, 2 * kZeroExp), h = e >> 1;
     const float f = v * pow2f(h) * pow2f(e - h);
-    return (ea == 2047 || eb == 2047) ? __int_as_float(0x7fc00000) : f;
+    return max(ea, eb) >= kNonFiniteExp ? __int_as_float(0x7fc00000) : f;
 }
 // x as a double by integer operations (a conversion instruction holds the
 // FP64 pipe like an FP64 instruction); FP32 subnormals count as zero.
@@ -264,21 +305,39 @@ __device__ __forceinline__ void load_index(int (&ix)[kLaneK], const int* idx, in
     for (int i = 0; i < kLaneK; ++i) ix[i] = (ON && lane_k(i) < kn) ? idx[lane_k(i)] : 0;
 }
 
+// The powers of this lane's entries of the chunk from k0 on.
+template <class Scale>
+__device__ __forceinline__ void load_scale(int (&s)[kLaneK], Scale&& sc, int k0, int kn) {
+#pragma unroll
+    for (int i = 0; i < kLaneK; ++i) s[i] = lane_k(i) < kn ? sc(k0 + lane_k(i)) : 0;
+}
+// ... from the CTA's shared copy
+__device__ __forceinline__ void load_scale(int (&s)[kLaneK], const int* sk) {
+#pragma unroll
+    for (int i = 0; i < kLaneK; i += 2) {
+        const int2 x = *reinterpret_cast<const int2*>(sk + lane_k(i));
+        s[i] = x.x;
+        s[i + 1] = x.y;
+    }
+}
+
 // The warp's part of sum_k A(row, k) B(col, k), k < K (K >= 1), at row
 // out_row(mt, r), column out_col(r).  arow(row) / brow(col): pointer to the
 // operand's row (nullptr: zeros), entry k at [k], or at [idx[k]] where AG /
-// BG say that the operand is gathered.
-template <int S, class T, bool AG, bool BG, class ASrc, class BSrc>
+// BG say that the operand is gathered.  sc(k): A's column k is cut as
+// A 2^sc(k), B's as B 2^-sc(k).
+template <int S, class T, bool AG, bool BG, class ASrc, class BSrc, class Scale>
 __device__ __forceinline__ void split_product(SplitSmem<S>& sm, int K, const int* idx, ASrc&& arow, BSrc&& brow,
-                                              typename SplitAcc<S>::T (&sum)[2][4]) {
+                                              Scale&& sc, typename SplitAcc<S>::T (&sum)[2][4]) {
     const int row = stage_slot();
     const T *pa[2] = {arow(row), arow(row + kPassRows)}, *pb = brow(row);
 #pragma unroll 1
     for (int k0 = 0; k0 < K; k0 += kChunkK) {
         const int kn = min(kChunkK, K - k0);
         {
-            int ix[kLaneK];
+            int ix[kLaneK], s[kLaneK];
             load_index<AG || BG>(ix, idx + k0, kn);
+            load_scale(s, sc, k0, kn);
             // every row's entries in flight together
             T va[2][kLaneK], vb[kLaneK];
 #pragma unroll
@@ -286,8 +345,8 @@ __device__ __forceinline__ void split_product(SplitSmem<S>& sm, int K, const int
             load_row<BG>(vb, pb ? pb + (BG ? 0 : k0) : nullptr, ix, kn);
             if (k0) __syncthreads();                  // the previous chunk's digits are read
 #pragma unroll
-            for (int p = 0; p < 2; ++p) stage_row<S>(sm.A, sm.ea, row + p * kPassRows, kn, va[p]);
-            stage_row<S>(sm.B, sm.eb, row, kn, vb);
+            for (int p = 0; p < 2; ++p) stage_row<S, 1>(sm.A, sm.ea, row + p * kPassRows, kn, va[p], s);
+            stage_row<S, -1>(sm.B, sm.eb, row, kn, vb, s);
         }
         __syncthreads();
         float acc[S][2][4];
@@ -310,10 +369,11 @@ __device__ __forceinline__ void split_product(SplitSmem<S>& sm, int K, const int
 // B and the values pre(t, row, column) that its epilogue needs are loaded
 // while the products of the tile before run; epi(t, row, column, product,
 // pre) receives every entry.
-template <int S, bool AG, bool BG, class ASrc, class BSrc, class Pre, class Epi>
+template <int S, bool AG, bool BG, class ASrc, class BSrc, class Scale, class Pre, class Epi>
 __device__ __forceinline__ void strip_product(SplitSmem<S>& sm, int K, const int* idx, int t0, int t1, ASrc&& arow,
-                                              BSrc&& brow, Pre&& pre, Epi&& epi) {
+                                              BSrc&& brow, Scale&& sc, Pre&& pre, Epi&& epi) {
     const int row = stage_slot();
+    const int power = threadIdx.x < K ? sc(threadIdx.x) : 0;          // in flight with the rows
     int ix[kLaneK];
     load_index<AG || BG>(ix, idx, K);
     double vb[kLaneK];
@@ -322,12 +382,20 @@ __device__ __forceinline__ void strip_product(SplitSmem<S>& sm, int K, const int
         double va[2][kLaneK];
 #pragma unroll
         for (int p = 0; p < 2; ++p) load_row<AG>(va[p], arow(row + p * kPassRows), ix, K);
+        if (threadIdx.x < kChunkK) sm.sk[threadIdx.x] = power;
+        __syncthreads();
+        int s[kLaneK];
+        load_scale(s, sm.sk);
 #pragma unroll
-        for (int p = 0; p < 2; ++p) stage_row<S>(sm.A, sm.ea, row + p * kPassRows, K, va[p]);
+        for (int p = 0; p < 2; ++p) stage_row<S, 1>(sm.A, sm.ea, row + p * kPassRows, K, va[p], s);
     }
     for (int t = t0; t < t1; ++t) {
         if (t > t0) __syncthreads();                  // the tile before is done with sm.B
-        stage_row<S>(sm.B, sm.eb, row, K, vb);
+        {
+            int s[kLaneK];
+            load_scale(s, sm.sk);
+            stage_row<S, -1>(sm.B, sm.eb, row, K, vb, s);
+        }
         __syncthreads();
         if (t + 1 < t1) load_row<BG>(vb, brow(t + 1, row), ix, K);
         double old[2][4];
@@ -367,49 +435,57 @@ struct FragB {
     int e;                      // exponent of column g
 };
 template <class T>
-__device__ __forceinline__ int quad_exponent(T a, T b, T c, T d) {
-    int E = max(max(exponent_bits(a), exponent_bits(b)), max(exponent_bits(c), exponent_bits(d)));
+__device__ __forceinline__ int quad_exponent(const T (&v)[4], const int (&s)[4], int sign, int (&ex)[4]) {
+    int E = kZeroExp;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        ex[i] = scaled_exponent(v[i], sign * s[i]);
+        E = max(E, ex[i]);
+    }
     E = max(E, __shfl_xor_sync(0xffffffffu, E, 1));
-    E = max(E, __shfl_xor_sync(0xffffffffu, E, 2));
-    return sizeof(T) == 8 ? E >> 20 : E >> 23;
+    return max(E, __shfl_xor_sync(0xffffffffu, E, 2));
 }
-// at(row, k): the operand's entry
+// k of a lane's four entries of a fragment row
+__device__ __forceinline__ int frag_k(int i) { return 2 * (threadIdx.x & 3) + (i & 1) + 8 * (i >> 1); }
+// at(row, k): the operand's entry; entries i times 2^(sign s[i])
 template <int S, class T, class At>
-__device__ __forceinline__ void load_frag_a(FragA<S>& f, At&& at) {
-    const int g = (threadIdx.x & 31) >> 2, t = threadIdx.x & 3;
+__device__ __forceinline__ void load_frag_a(FragA<S>& f, const int (&s)[4], int sign, At&& at) {
+    const int g = (threadIdx.x & 31) >> 2;
     T v[2][4];
 #pragma unroll
     for (int h = 0; h < 2; ++h)
 #pragma unroll
-        for (int i = 0; i < 4; ++i) v[h][i] = at(g + 8 * h, 2 * t + (i & 1) + 8 * (i >> 1));
+        for (int i = 0; i < 4; ++i) v[h][i] = at(g + 8 * h, frag_k(i));
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-        const int E = quad_exponent(v[h][0], v[h][1], v[h][2], v[h][3]);
+        int ex[4];
+        const int E = quad_exponent(v[h], s, sign, ex);
         (h ? f.e1 : f.e0) = common_exponent<T>(E);
 #pragma unroll
         for (int p = 0; p < 2; ++p) {
             unsigned d[S];
-            digit_pair<S>(v[h][2 * p], v[h][2 * p + 1], E, d);
+            digit_pair<S>(v[h][2 * p], v[h][2 * p + 1], E - ex[2 * p], E - ex[2 * p + 1], d);
 #pragma unroll
-            for (int s = 0; s < S; ++s) f.d[s][h + 2 * p] = d[s];
+            for (int j = 0; j < S; ++j) f.d[j][h + 2 * p] = d[j];
         }
     }
 }
 // at(col, k)
 template <int S, class T, class At>
-__device__ __forceinline__ void load_frag_b(FragB<S>& f, At&& at) {
-    const int g = (threadIdx.x & 31) >> 2, t = threadIdx.x & 3;
+__device__ __forceinline__ void load_frag_b(FragB<S>& f, const int (&s)[4], int sign, At&& at) {
+    const int g = (threadIdx.x & 31) >> 2;
     T v[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) v[i] = at(g, 2 * t + (i & 1) + 8 * (i >> 1));
-    const int E = quad_exponent(v[0], v[1], v[2], v[3]);
+    for (int i = 0; i < 4; ++i) v[i] = at(g, frag_k(i));
+    int ex[4];
+    const int E = quad_exponent(v, s, sign, ex);
     f.e = common_exponent<T>(E);
 #pragma unroll
     for (int p = 0; p < 2; ++p) {
         unsigned d[S];
-        digit_pair<S>(v[2 * p], v[2 * p + 1], E, d);
+        digit_pair<S>(v[2 * p], v[2 * p + 1], E - ex[2 * p], E - ex[2 * p + 1], d);
 #pragma unroll
-        for (int s = 0; s < S; ++s) f.d[s][p] = d[s];
+        for (int j = 0; j < S; ++j) f.d[j][p] = d[j];
     }
 }
 // out[r]: row g + 8 (r / 2), column 2 t + r % 2 of the 16 x 8 product, of whose

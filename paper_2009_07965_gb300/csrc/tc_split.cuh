@@ -27,6 +27,7 @@ struct TcSmem {
     __align__(16) unsigned char A[S][8 * kStepA];
     __align__(16) unsigned char B[2][8 * kStepB];
     int ea[kTcM], eb[4][kTcN];           // (eb: by tile, a tile ahead of the one being combined)
+    __align__(16) int sk[64];            // powers of two of the k (A's entries; B's the inverse ones)
     __align__(8) unsigned long long bar[2];
     unsigned int tmem;
 };
@@ -69,20 +70,28 @@ __device__ __forceinline__ void tc_begin(TcSmem<S>& sm) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 // The digits of row `row` of an operand (eight lanes per row, lane j entries
-// 8 j .. 8 j + 7 in v) to dst + digit * dig.
-template <int S, class T>
-__device__ __forceinline__ void tc_stage(unsigned char* dst, int dig, int kstep, int* e, int row, const T (&v)[8]) {
+// 8 j .. 8 j + 7 in v, times 2^(SIGN sk)) to dst + digit * dig.
+template <int S, int SIGN, class T>
+__device__ __forceinline__ void tc_stage(unsigned char* dst, int dig, int kstep, int* e, int row, const T (&v)[8],
+                                         const int* sk) {
     const int j = threadIdx.x & 7;
-    int E = 0;
+    int ex[8], E = kZeroExp;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) E = max(E, exponent_bits(v[i]));
+    for (int i = 0; i < 8; i += 4) {
+        const int4 s = *reinterpret_cast<const int4*>(sk + 8 * j + i);
+        ex[i] = scaled_exponent(v[i], SIGN * s.x);
+        ex[i + 1] = scaled_exponent(v[i + 1], SIGN * s.y);
+        ex[i + 2] = scaled_exponent(v[i + 2], SIGN * s.z);
+        ex[i + 3] = scaled_exponent(v[i + 3], SIGN * s.w);
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) E = max(E, ex[i]);
 #pragma unroll
     for (int w = 1; w < 8; w <<= 1) E = max(E, __shfl_xor_sync(0xffffffffu, E, w));
-    E = sizeof(T) == 8 ? E >> 20 : E >> 23;
     if (j == 0) e[row] = common_exponent<T>(E);
     unsigned d[4][S];
 #pragma unroll
-    for (int p = 0; p < 4; ++p) digit_pair<S>(v[2 * p], v[2 * p + 1], E, d[p]);
+    for (int p = 0; p < 4; ++p) digit_pair<S>(v[2 * p], v[2 * p + 1], E - ex[2 * p], E - ex[2 * p + 1], d[p]);
     unsigned char* at = dst + j * kstep + row * 16;
 #pragma unroll
     for (int s = 0; s < S; ++s)
@@ -90,11 +99,11 @@ __device__ __forceinline__ void tc_stage(unsigned char* dst, int dig, int kstep,
 }
 template <int S, class T>
 __device__ __forceinline__ void tc_stage_a(TcSmem<S>& sm, int row, const T (&v)[8]) {
-    tc_stage<S>(&sm.A[0][0], 8 * TcSmem<S>::kStepA, TcSmem<S>::kStepA, sm.ea, row, v);
+    tc_stage<S, 1>(&sm.A[0][0], 8 * TcSmem<S>::kStepA, TcSmem<S>::kStepA, sm.ea, row, v, sm.sk);
 }
 template <int S, class T>
 __device__ __forceinline__ void tc_stage_b(TcSmem<S>& sm, int tile, int row, const T (&v)[8]) {
-    tc_stage<S>(&sm.B[tile & 1][0], kTcN * 16, TcSmem<S>::kStepB, sm.eb[tile & 3], row, v);
+    tc_stage<S, -1>(&sm.B[tile & 1][0], kTcN * 16, TcSmem<S>::kStepB, sm.eb[tile & 3], row, v, sm.sk);
 }
 // Makes the CTA's staged digits visible to the tensor cores; then thread 0
 // may issue.  True (all threads) when stop holds on any thread.
