@@ -804,6 +804,7 @@ cudaError_t pressure_launch(const DevView& v, bool accumulate, int mp, int cz, c
 cudaError_t launch_leaf_build(const DevView& v, int max_m, int max_c, cudaStream_t s) {
     const int mp = std::max(max_m, 1), cz = std::max(max_c, 1);
     if (v.dim == 3) return build_dispatch<3, double>(v, mp, cz, s);
+    if (v.banded) return launch_banded_build(v, max_m, s);
     return v.leaf32 ? build_dispatch<2, float>(v, mp, cz, s) : build_dispatch<2, double>(v, mp, cz, s);
 }
 
@@ -811,6 +812,7 @@ cudaError_t launch_leaf_particular(const DevView& v, const double* q, const doub
                                    int max_c, cudaStream_t s) {
     const int mp = std::max(max_m, 1), cz = std::max(max_c, 1);
     if (v.dim == 3) return particular_launch<3, double>(v, q, bc_val, with_sadj, mp, cz, s);
+    if (v.banded) return launch_banded_particular(v, q, bc_val, with_sadj, s);
     return v.leaf32 ? particular_launch<2, float>(v, q, bc_val, with_sadj, mp, cz, s)
                     : particular_launch<2, double>(v, q, bc_val, with_sadj, mp, cz, s);
 }
@@ -818,12 +820,14 @@ cudaError_t launch_leaf_particular(const DevView& v, const double* q, const doub
 cudaError_t launch_leaf_pressure(const DevView& v, bool accumulate, int max_m, int max_c, cudaStream_t s) {
     const int mp = std::max(max_m, 1), cz = std::max(max_c, 1);
     if (v.dim == 3) return pressure_launch<3, double>(v, accumulate, mp, cz, s);
+    if (v.banded) return launch_banded_pressure(v, accumulate, s);
     return v.leaf32 ? pressure_launch<2, float>(v, accumulate, mp, cz, s)
                     : pressure_launch<2, double>(v, accumulate, mp, cz, s);
 }
 
 cudaError_t launch_leaf_fields(const DevView& v, const int* ids, int count, float* psi, cudaStream_t s) {
-    if (count == 0) return cudaSuccess;
+    if (count <= 0) return cudaSuccess;
+    if (v.banded) return launch_banded_fields(v, ids, count, psi, s);
     const int grid = (count + kSolveWarps - 1) / kSolveWarps;
     if (v.leaf32) leaf_fields_kernel<float><<<grid, 32 * kSolveWarps, 0, s>>>(v, ids, count, psi);
     else leaf_fields_kernel<double><<<grid, 32 * kSolveWarps, 0, s>>>(v, ids, count, psi);

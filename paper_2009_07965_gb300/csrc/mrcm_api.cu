@@ -57,6 +57,7 @@ struct Plan {
     std::vector<int> level_first, level_count, level_max_g2, level_max_m;  // index by height-1
     std::vector<int> node_map, gamma_segs;
     int max_m_leaf = 0, max_c_leaf = 0, max_g2 = 0;
+    bool banded = false;                 // leaves eliminated cell by cell
     // storage sizes (doubles / ints)
     long long nR = 0, nr = 0, nW = 0, nX = 0, nL = 0, nZ = 0, nzb = 0;
     std::vector<long long> node_R_off, node_r_off;
@@ -143,6 +144,31 @@ void finish_tree(Plan& P) {
 }
 
 void finish_merges(Plan& P);
+
+// Whether a 2D context's leaves are eliminated cell by cell instead of plane by
+// plane, by the shape (w x h cells, m segments) and number of its leaves.  The
+// lines follow a sweep over w, h <= 16 and segments of 1 to 16 faces, build
+// plus two solve passes, cells over planes (below 1: cells faster), 20000 to
+// 600000 cells: w <= 4 and few segments 0.2 to 0.85 whatever the count; w = 6 to
+// 8 0.6 to 0.95 where 4 w + m < 44, and a few planes of few cells (10 x 4: 0.79,
+// 12 x 6: 0.91), but 1.25 to 1.5 below some 2400 leaves, where the chain of
+// cells is the longer one; 12 x 12 and 16 x 16 with one segment a side 0.90 and
+// 0.97 at 4096 leaves, 1.1 at 2304 (the planes' waves are 1824 leaves); as many
+// segments as cells, or one plane, 1.05 to 1.7; more than 16 segments 0.5 to
+// 0.86 for w <= 2, else 0.95 to 5.8.
+bool banded_leaves(const Plan& P) {
+    int w = 0, h = 0;
+    for (const LeafDesc& L : P.leaves) {
+        w = std::max(w, L.w);
+        h = std::max(h, L.h);
+    }
+    const int n = w * h, m = P.max_m_leaf;
+    if (m > 16) return w <= 2;
+    if (w == 1) return true;
+    if (w > 4 && P.nleaf <= 2400) return false;
+    if (h == 1 || (m >= n && w >= 4)) return m <= 4;
+    return 4 * w + m < 44 || (n < 64 && m <= 8) || (m <= 4 && P.nleaf > 2 * 1824);
+}
 
 int make_plan(Plan& P) {
     const int ngrid = (int)P.grids.size();
@@ -297,6 +323,7 @@ int make_plan(Plan& P) {
         P.height = std::max(P.height, P.nodes[root].height);
     }
     finish_tree(P);
+    P.banded = banded_leaves(P);
     for (int id = 0; id < P.nleaf; ++id) {
         LeafDesc& L = P.leaves[id];
         const long long n = (long long)L.w * L.h;
@@ -306,8 +333,8 @@ int make_plan(Plan& P) {
         L.R_off = P.node_R_off[id];
         L.r_off = P.node_r_off[id];
         const LeafGeo geo = leaf_geo2(L, P.gx, P.gy);
-        P.nL += n * L.w;
-        P.nZ += geo.zsize();
+        P.nL += P.banded ? n * (kMaxLeafSide + 1) : n * L.w;
+        P.nZ += P.banded ? n * L.m : geo.zsize();
         P.nzb += n;
         P.max_c_leaf = std::max(P.max_c_leaf, std::max(geo.ncols(0), geo.ncols(1)));
         // flop model of the leaf kernel: LDL^T band steps, forward solve of
@@ -1088,6 +1115,7 @@ static int setup3_impl(mrcm_ctx* c, const mrcm_grid* g, const double* K_dev, con
     v.g3 = P.g3;
     v.mixed = precision == MRCM_MIXED ? 1 : 0;
     v.leaf32 = 0;                  // 3D blocks are factored in FP64
+    v.banded = 0;
     v.res_dd = 0;                  // 3D refinement residuals in FP64
     c->precision = precision;
     c->refine_steps = v.mixed ? kMixedRefineDefault3D : 0;
@@ -1171,6 +1199,7 @@ static int setup_impl(mrcm_ctx* c, int count, const mrcm_grid* g, const double* 
     DevView& v = c->v;
     v.mixed = precision == MRCM_MIXED ? 1 : 0;
     v.leaf32 = 0;                  // the mixed form's leaves in FP64 unless mrcm_set_mixed_leaves(1)
+    v.banded = P.banded;
     v.res_dd = v.mixed ? 0 : 1;    // FP64 residuals suffice for the mixed form's tolerance
     c->precision = precision;
     if (v.mixed) c->refine_steps = kMixedRefineDefault;

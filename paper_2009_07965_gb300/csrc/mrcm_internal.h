@@ -47,9 +47,9 @@ struct LeafDesc {
     int side_off[4];   // local index of the first segment of side x-, x+, y-,
                        // y+ (-1 when the side lies on the domain boundary)
     int seg_off;       // offset of the leaf's segment ids in leaf_segs
-    long long L_off;   // P_k of every plane (h of w x w)
-    long long Z_off;   // Z_k of every plane (leaf_geometry.cuh)
-    long long zb_off;  // particular right-hand sides y_k: n values
+    long long L_off;   // P_k of every plane (h of w x w); banded: L (n x 16) and 1 / d (n)
+    long long Z_off;   // Z_k of every plane (leaf_geometry.cuh); banded: Z (n x m)
+    long long zb_off;  // particular right-hand sides y_k (banded: L^-1 b): n values
     long long R_off;   // node R (m x m) of the leaf
     long long r_off;   // node rbar / lambda (m values each, separate arrays)
 };
@@ -146,6 +146,7 @@ struct DevView {
     float* leafL32;     // the same in FP32 (mixed precision: leaf work in FP32)
     float* leafZ32;
     int mixed;          // 1: the mixed form (the merges of FP32 levels in FP32)
+    int banded;         // 1: leaves eliminated cell by cell (kernels_leaf_banded.cu; 2D)
     int leaf32;         // 1: leaf factors in FP32 (mixed form, mrcm_set_mixed_leaves)
     int res_dd;         // 1: refinement residuals in double-double, 0: in FP64 (mrcm_set_residual)
     double* leafzb;     // particular right-hand sides y_k
@@ -338,6 +339,13 @@ cudaError_t launch_leaf_particular(const DevView& v, const double* q, const doub
 // p = A^-1 (bbar + B lambda) per leaf into the double-double state
 // (p_hi, p_lo): set, or accumulate (double-double add of the correction).
 cudaError_t launch_leaf_pressure(const DevView& v, bool accumulate, int max_m, int max_c, cudaStream_t s);
+// The same for contexts of small or narrow leaves (DevView::banded), which the
+// launchers above pass on (kernels_leaf_banded.cu).
+cudaError_t launch_banded_build(const DevView& v, int max_m, cudaStream_t s);
+cudaError_t launch_banded_particular(const DevView& v, const double* q, const double* bc_val, bool with_sadj,
+                                     cudaStream_t s);
+cudaError_t launch_banded_pressure(const DevView& v, bool accumulate, cudaStream_t s);
+cudaError_t launch_banded_fields(const DevView& v, const int* ids, int count, float* psi, cudaStream_t s);
 // interface unknowns from the two Robin data of each segment (set or add)
 cudaError_t launch_lam_to_PU(const DevView& v, bool accumulate, cudaStream_t s);
 // residual of the discrete equations in double-double; fills rcell, sadj
