@@ -334,7 +334,9 @@ leaf_build_kernel(DevView v, int mp, int cz, int bytes) {
 // ---------------------------------------------------------------------------
 // Solve phase, one warp per leaf: lanes 0-15 the planes below the middle one
 // (lane = cell), lanes 16-31 those above, in step; the middle plane by both
-// (each half of the warp takes half of the products).
+// (each half of the warp takes half of the products).  FP32 factors are widened
+// by integer operations: a conversion holds the FP64 pipe like the FP64
+// multiply-add it feeds.
 constexpr int kSolveWarps = 4;
 
 // Right-hand side of the particular problem at one cell (Eqs. addu/addp):
@@ -386,7 +388,7 @@ __device__ __forceinline__ double row_product_next(TS (&p)[kPlane], const double
     double a = 0.0;
 #pragma unroll
     for (int j = 0; j < kPlane; ++j) {
-        a = fma((double)p[j], y[j], a);
+        a = fma(widen(p[j]), y[j], a);
         p[j] = j < n ? c[j * nb] : (TS)0;
     }
     return a;
@@ -397,7 +399,7 @@ __device__ __forceinline__ double half_product(const TS (&p)[kPlane], const doub
     double a = 0.0;
 #pragma unroll
     for (int j = 0; j < kPlane / 2; ++j)
-        a = fma((double)(part ? p[j + kPlane / 2] : p[j]), y[j + part * (kPlane / 2)], a);
+        a = fma(widen(part ? p[j + kPlane / 2] : p[j]), y[j + part * (kPlane / 2)], a);
     return a;
 }
 
@@ -472,10 +474,10 @@ leaf_particular_kernel(DevView v, const double* __restrict__ q, const double* __
         if (SMALL) {
 #pragma unroll
             for (int c = 0; c < 8; ++c)
-                if (c < ccw) part[c] = fma((double)z[c], wn, part[c]);
+                if (c < ccw) part[c] = fma(widen(z[c]), wn, part[c]);
         } else {
             for (int c = 0; c < cc; ++c)
-                acc[h * cz + c][l] = fma(act ? (double)Zk[c * nb + l] : 0.0, wn, acc[h * cz + c][l]);
+                acc[h * cz + c][l] = fma(act ? widen(Zk[c * nb + l]) : 0.0, wn, acc[h * cz + c][l]);
         }
         __syncwarp();
     }
@@ -510,7 +512,7 @@ leaf_particular_kernel(DevView v, const double* __restrict__ q, const double* __
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
             const int t = 8 * h + c;
-            zm[c] = l < nb && t < g.m ? (double)Zm[t * nb + l] * w : 0.0;
+            zm[c] = l < nb && t < g.m ? widen(Zm[t * nb + l]) * w : 0.0;
         }
         double* rs = &ysh[warp][0][0];                             // rbar by segment (m <= 16)
         const double r = reduce_columns8(zm, l);
@@ -525,7 +527,7 @@ leaf_particular_kernel(DevView v, const double* __restrict__ q, const double* __
         if (lane < g.m) store(lane, rs[lane]);
         return;
     }
-    for (int t = h; t < g.m; t += 2) acc[2 * cz + t][l] = l < nb ? (double)Zm[t * nb + l] * w : 0.0;
+    for (int t = h; t < g.m; t += 2) acc[2 * cz + t][l] = l < nb ? widen(Zm[t * nb + l]) * w : 0.0;
     __syncwarp();
     // each row summed by one lane (over the 16 cells), then the halves' rows
     // added to their segments
@@ -622,14 +624,14 @@ __global__ void __launch_bounds__(32 * kSolveWarps) leaf_pressure_kernel(DevView
 #pragma unroll
             for (int u = 0; u < 8; ++u) z[u] = Zk[(c + u * step) * nb];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) a = fma((double)z[u], lm[c + u * step], a);
+            for (int u = 0; u < 8; ++u) a = fma(widen(z[u]), lm[c + u * step], a);
         }
         TS z[8];
 #pragma unroll
         for (int u = 0; u < 7; ++u) z[u] = c + u * step < cc ? Zk[(c + u * step) * nb] : (TS)0;
 #pragma unroll
         for (int u = 0; u < 7; ++u)
-            if (c + u * step < cc) a = fma((double)z[u], lm[c + u * step], a);
+            if (c + u * step < cc) a = fma(widen(z[u]), lm[c + u * step], a);
         return a;
     };
     solve_outward<DIM, TS>(v, leaf, g, leaf_L<TS>(v) + g.L_off, ysh[warp], lane, rhs, [&](int k, int l, double x) {
@@ -678,8 +680,8 @@ __global__ void __launch_bounds__(32 * kSolveWarps) leaf_fields_kernel(DevView v
                 if (g.segment(h, p) == s) pos[h] = p;
         auto rhs = [&](int h, int k, int l) -> double {
             if (l >= nb) return 0.0;
-            if (h < 0) return lane < 16 ? (double)Zg[g.zoff(0, k) + s * nb + l] : 0.0;
-            return pos[h] >= 0 && pos[h] < g.cols(h, k) ? (double)Zg[g.zoff(h, k) + pos[h] * nb + l] : 0.0;
+            if (h < 0) return lane < 16 ? widen(Zg[g.zoff(0, k) + s * nb + l]) : 0.0;
+            return pos[h] >= 0 && pos[h] < g.cols(h, k) ? widen(Zg[g.zoff(h, k) + pos[h] * nb + l]) : 0.0;
         };
         solve_outward<2, TS>(v, id, g, leaf_L<TS>(v) + g.L_off, ysh[warp], lane, rhs, [&](int k, int l, double x) {
             psi[((long long)item * 256 + k * nb + l) * 16 + s] = (float)x;
