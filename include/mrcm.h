@@ -365,9 +365,10 @@ int mrcm_set_mixed_leaves(mrcm_ctx* ctx, int fp32);
  * on it (64-row blocks, each waiting only for the blocks it depends on).
  * MRCM_ROOT_INVERSE: the explicit inverse, as at every other blocked height;
  * each solve pass then applies it as a matrix-vector product.
- * MRCM_ROOT_AUTO (the default): the inverse (its products run on the tensor
- * cores, so that it takes less time than the factor at every size measured,
- * and its solve passes are the shorter).
+ * MRCM_ROOT_AUTO (the default): the factor for a single FP64 root system of
+ * 1024 <= 2g < 1408, the inverse elsewhere (below, its passes are the shorter
+ * and the elimination no longer; above, its products run on the tensor cores:
+ * measured up to 2g = 6144, 45 against 101 ms).
  * Applies to tree heights with 2g > 32 whose nodes all lack outer segments.
  * Both forms solve the same equations (to rounding).  Invalidates the basis
  * (call mrcm_build_basis again).  Errors: MRCM_ERR_INVALID_ARG,

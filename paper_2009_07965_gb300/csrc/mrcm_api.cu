@@ -71,9 +71,10 @@ struct Plan {
     double phase_build[MRCM_PHASE_COUNT] = {};   // per build call
     double phase_pass[MRCM_PHASE_COUNT] = {};    // per solve pass
     // the above count root levels in the inverse form; these differences are
-    // added where they take the factor form (MRCM_ROOT_FACTOR)
-    double root_build[MRCM_PHASE_COUNT] = {}, root_pass[MRCM_PHASE_COUNT] = {};
-    double root_merge = 0, root_solve = 0, root_model_sweep = 0;
+    // added where they take the factor form: [0] every root level
+    // (MRCM_ROOT_FACTOR), [1] those MRCM_ROOT_AUTO factors in FP64
+    double root_build[2][MRCM_PHASE_COUNT] = {}, root_pass[2][MRCM_PHASE_COUNT] = {};
+    double root_merge[2] = {}, root_solve[2] = {}, root_model_sweep[2] = {};
     double residual_flops = 0, finish_flops = 0;
     // 3D contexts: the grid, the blocks (leaves), the second tangential
     // extent of each segment and the z-face map
@@ -475,13 +476,16 @@ void finish_merges(Plan& P) {
                 // forward sweep (N^2), the inverse diagonal blocks (2 kGJ N)
                 // and the backward sweep (N^2) instead of the product (2 N^2)
                 const double fac = N * (N * N - 1.0) / 3.0;
-                P.root_build[MRCM_PHASE_GJ_SWEEP] -= sym;
-                P.root_build[MRCM_PHASE_ROOT_FACTOR] += fac;
-                P.root_merge += fac - sym;
-                P.root_model_sweep -= 2.0 / 3.0 * N * N * N;
-                P.root_pass[MRCM_PHASE_TREE_UP] += N * N;
-                P.root_pass[MRCM_PHASE_TREE_DOWN] += N * N + 2.0 * kMergeBlock * N - 2.0 * N * N;
-                P.root_solve += 2.0 * kMergeBlock * N;
+                for (int a = 0; a < 2; ++a) {
+                    if (a == 1 && !root_factor_pays(P.level_count[h - 1], P.level_max_g2[h - 1])) continue;
+                    P.root_build[a][MRCM_PHASE_GJ_SWEEP] -= sym;
+                    P.root_build[a][MRCM_PHASE_ROOT_FACTOR] += fac;
+                    P.root_merge[a] += fac - sym;
+                    P.root_model_sweep[a] -= 2.0 / 3.0 * N * N * N;
+                    P.root_pass[a][MRCM_PHASE_TREE_UP] += N * N;
+                    P.root_pass[a][MRCM_PHASE_TREE_DOWN] += N * N + 2.0 * kMergeBlock * N - 2.0 * N * N;
+                    P.root_solve[a] += 2.0 * kMergeBlock * N;
+                }
             }
             P.phase_build[MRCM_PHASE_MERGE_X] += 2.0 * N * gd * md;
             P.phase_build[MRCM_PHASE_MERGE_R] += md * (md + 1.0) * gd;
@@ -1001,22 +1005,26 @@ static void fill_plan_inputs(Plan& P, int count, const mrcm_grid* g, const int s
     P.gx = seg[0]; P.gy = seg[1];
 }
 
-// whether a root form keeps factors (then the plan's root_* differences apply)
-static double root_factored(int form) { return form == MRCM_ROOT_FACTOR ? 1.0 : 0.0; }
+// which of the plan's root_* differences applies to a root form, times f
+static int root_set(int form, bool mixed, double& f) {
+    f = form == MRCM_ROOT_FACTOR || (form == MRCM_ROOT_AUTO && !mixed) ? 1.0 : 0.0;
+    return form == MRCM_ROOT_AUTO ? 1 : 0;
+}
 
-static int plan_value(const Plan& P, int what, long long* value, int form = MRCM_ROOT_AUTO) {
-    const double f = root_factored(form);
+static int plan_value(const Plan& P, int what, long long* value, int form = MRCM_ROOT_AUTO, bool mixed = false) {
+    double f;
+    const int a = root_set(form, mixed, f);
     switch (what) {
         case MRCM_Q_LEAVES: *value = P.nleaf; break;
         case MRCM_Q_SEGMENTS: *value = P.nseg; break;
         case MRCM_Q_LEVELS: *value = P.height; break;
         case MRCM_Q_NODES: *value = (long long)P.nodes.size(); break;
         case MRCM_Q_MAX_GAMMA: *value = P.max_g2; break;
-        case MRCM_Q_BUILD_FLOPS: *value = P.leaf_flops + P.merge_flops + (long long)(f * P.root_merge); break;
-        case MRCM_Q_SOLVE_FLOPS: *value = P.solve_flops + (long long)(f * P.root_solve); break;  // one pass
+        case MRCM_Q_BUILD_FLOPS: *value = P.leaf_flops + P.merge_flops + (long long)(f * P.root_merge[a]); break;
+        case MRCM_Q_SOLVE_FLOPS: *value = P.solve_flops + (long long)(f * P.root_solve[a]); break;  // one pass
         case MRCM_Q_LEAF_FLOPS: *value = P.leaf_flops; break;
         case MRCM_Q_MODEL_BUILD_FLOPS: *value = (long long)P.model_build; break;
-        case MRCM_Q_MODEL_SWEEP_FLOPS: *value = (long long)(P.model_sweep + f * P.root_model_sweep); break;
+        case MRCM_Q_MODEL_SWEEP_FLOPS: *value = (long long)(P.model_sweep + f * P.root_model_sweep[a]); break;
         case MRCM_Q_GRIDS: *value = (long long)P.grids.size(); break;
         case MRCM_Q_CELLS: *value = P.ncell; break;
         default: return MRCM_ERR_INVALID_ARG;
@@ -1045,8 +1053,11 @@ int mrcm_plan_query(const mrcm_grid* g, const int sub_cells[3], const int seg_ce
 // form of the context.
 static bool level_factor(const mrcm_ctx* c, int h) {
     const Plan& P = c->P;
-    return c->root_form == MRCM_ROOT_FACTOR && P.level_max_m[h - 1] == 0 &&
-           merge_level_blocked(P.level_count[h - 1], P.level_max_g2[h - 1], P.level_max_m[h - 1]);
+    if (c->root_form == MRCM_ROOT_INVERSE || P.level_max_m[h - 1] != 0 ||
+        !merge_level_blocked(P.level_count[h - 1], P.level_max_g2[h - 1], P.level_max_m[h - 1]))
+        return false;
+    return c->root_form == MRCM_ROOT_FACTOR ||
+           (!c->v.mixed && root_factor_pays(P.level_count[h - 1], P.level_max_g2[h - 1]));
 }
 static void set_tree_forms(mrcm_ctx* c) {
     for (int h = 1; h <= c->P.height; ++h) c->tree.form[h - 1] = level_factor(c, h) ? 1 : 0;
@@ -1732,7 +1743,7 @@ int mrcm_query(const mrcm_ctx* c, int what, long long* value) {
         case MRCM_Q_KERNEL_LAUNCHES_BUILD: *value = c->launches_build; return MRCM_OK;
         case MRCM_Q_KERNEL_LAUNCHES_SOLVE: *value = c->launches_solve; return MRCM_OK;
         case MRCM_Q_GRAPH_REPLAYS: *value = c->graph_replays; return MRCM_OK;
-        default: return plan_value(c->P, what, value, c->root_form);
+        default: return plan_value(c->P, what, value, c->root_form, c->v.mixed);
     }
 }
 
@@ -1844,10 +1855,12 @@ int mrcm_group_times(mrcm_ctx* c, int* phase, double* ms, int cap) {
 int mrcm_phase_flops(const mrcm_ctx* c, double* flops) {
     if (!c || !flops) return MRCM_ERR_INVALID_ARG;
     const Plan& P = c->P;
-    const double passes = 1.0 + c->refine_steps, f = root_factored(c->root_form);
+    const double passes = 1.0 + c->refine_steps;
+    double f;
+    const int a = root_set(c->root_form, c->v.mixed, f);
     for (int p = 0; p < MRCM_PHASE_COUNT; ++p)
-        flops[p] = P.phase_build[p] + f * P.root_build[p] +
-                   passes * (P.phase_pass[p] + f * P.root_pass[p]);
+        flops[p] = P.phase_build[p] + f * P.root_build[a][p] +
+                   passes * (P.phase_pass[p] + f * P.root_pass[a][p]);
     flops[MRCM_PHASE_RESIDUAL] = (c->refine_steps + (c->refine_check ? 1 : 0)) * P.residual_flops;
     flops[MRCM_PHASE_FINISH] = P.finish_flops;
     return MRCM_OK;

@@ -434,6 +434,18 @@ size_t merge_scratch_doubles(int count, int max_g2, int max_m);
 constexpr int kMergeBlock = 16;      // block size of the blocked Gauss-Jordan sweep (flop model)
 constexpr int kTriBlock = 64;        // solve blocks of the factor form's triangular sweeps
 
+// Whether MRCM_ROOT_AUTO keeps the factor of a root level: a single FP64 system
+// of 1024 <= 2g < 1408.  The factor's FP64 sweep is the shorter elimination
+// there (factor / inverse, ms: 2g = 1024 1.04 / 1.46, 1280 1.58 / 2.01, 1408 1.97 /
+// 2.21, 1664 2.86 / 2.66), by more than its triangular sweeps add to two solve
+// passes (0.16 ms a pass at 1024, 0.20 at 1280, 0.21 at 1408); more systems gain
+// by the block sweep's products, and the mixed form has passes enough to lose.
+// Below 1024 the FP64 inverse's chain is no longer than the factor's.
+constexpr int kRootFactorMin = 1024, kRootFactorEnd = 1408;
+inline bool root_factor_pays(int count, int max_g2) {
+    return count == 1 && max_g2 >= kRootFactorMin && max_g2 < kRootFactorEnd;
+}
+
 // The merge levels of the tree for the fused up / down sweeps of the solve
 // (passed by value as a kernel argument; index h - 1 for height h).
 constexpr int kMaxTreeLevels = 48;
