@@ -113,7 +113,8 @@ def _nodes(mr, s):
 
 
 @pytest.mark.parametrize("kind,decades,alpha", [("channels", 5, 1.0), ("channels", 8, 1.0), ("channels", 11, 1.0),
-                                                ("channels", 11, 10.0), ("random", 8, 1.0), ("random", 11, 1.0)])
+                                                ("channels", 11, 10.0), ("random", 2, 1.0), ("random", 2, 100.0),
+                                                ("random", 8, 1.0), ("random", 11, 1.0)])
 def test_maps_of_high_contrast_fields_keep_fp64_accuracy(mrcm_lib, kind, decades, alpha):
     import torch
     import paper_2009_07965_gb300 as mr
