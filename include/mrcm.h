@@ -263,7 +263,9 @@ enum {
     MRCM_PHASE_MERGE_SMALL = 2,    /* whole merges of small interface systems       */
     MRCM_PHASE_GJ_SWEEP = 3,       /* blocked merges: Gauss-Jordan inversion of the
                                       quasi-definite form (one system per CTA up to
-                                      2g = 64, a cooperative sweep above)          */
+                                      2g = 64; above, a cooperative sweep, or one
+                                      launch per phase and 64 rows for 64 systems
+                                      or more)                                     */
     MRCM_PHASE_MERGE_FORM = 4,     /* blocked merges: the quasi-definite form of the
                                       interface matrix and its back transform; now
                                       done inside the sweep's launch (timed as
@@ -316,9 +318,10 @@ int mrcm_set_refinement(mrcm_ctx* ctx, int steps, int check);
 int mrcm_set_residual(mrcm_ctx* ctx, int dd);
 
 /*
- * mrcm_set_wait_limit -- polls after which a bounded wait between the CTAs
- * of one cooperative launch (the blocked interface sweeps and the solve's
- * tree sweeps) gives up; the paper has no counterpart.  polls < 0 restores
+ * mrcm_set_wait_limit -- polls after which a bounded wait gives up: between the
+ * CTAs of one cooperative launch (the blocked interface sweeps and the solve's
+ * tree sweeps), or for the tensor cores in the sweep of many systems (at most
+ * 65536 polls there, each of which may block); the paper has no counterpart.  polls < 0 restores
  * the default (about a second of polling); 0 gives up at the first check
  * that finds the awaited condition unmet.  A wait that gives up makes the
  * call return MRCM_ERR_TIMEOUT; every CTA then leaves the launch at its
@@ -380,18 +383,19 @@ int mrcm_set_root_form(mrcm_ctx* ctx, int form);
 /*
  * mrcm_autotune -- picks the launch shapes of every blocked merge level by
  * timing them on this device: CTAs per SM of the cooperative sweeps (1 or 2
- * of the block sweep, 1 to 4 of the FP64 sweep); each candidate is run `reps` times (1..100) on the
- * context's stream and the fastest kept per tree height.  Every shape computes the
- * same numbers, so the basis stays valid; later builds use the choices (the
- * captured build graph is dropped).  The paper has no counterpart.  Needs a
+ * of the block sweep, 1 to 4 of the FP64 sweep); each candidate is run `reps`
+ * times (1..100) on the context's stream and the fastest kept per tree height.
+ * Every shape computes the same numbers, so the basis stays valid; later builds
+ * use the choices (the captured build graph is dropped).  The paper has no counterpart.  Needs a
  * built basis (MRCM_ERR_NOT_BUILT otherwise).  Errors: MRCM_ERR_INVALID_ARG,
  * MRCM_ERR_NOT_BUILT, MRCM_ERR_TIMEOUT, MRCM_ERR_CUDA.
  *
  * mrcm_tune_info -- the choices for tree height `height` (1 = the leaves'
  * parents): out[0] CTAs per SM of the sweep; 0 where the built-in heuristic
  * applies (before mrcm_autotune, and on heights merged by the small-system
- * kernel) and on heights inverted one system per CTA (2g <= 64: no launch
- * shape to choose).
+ * kernel) and on heights without a launch shape to choose: inverted one system
+ * per CTA (2g <= 64), or by plain launches, one per phase (64 systems or more
+ * with count (2g)^2 >= 2^20).
  * out[1] and out[2] (the products X and R) are 0: they have one shape.
  */
 int mrcm_autotune(mrcm_ctx* ctx, int reps);

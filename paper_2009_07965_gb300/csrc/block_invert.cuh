@@ -17,12 +17,12 @@ namespace {
 
 constexpr int kPlane = 16;        // largest block swept by one warp
 
-// Distribution of the lower triangle of a 16 x 16 block over GL lanes (8, 16
-// or 32): lane l of 8 owns rows l and 15 - l, 17 entries, split over GL / 8
-// lanes where there are more.
+// Distribution of the lower triangle of a 16 x 16 block over GL lanes (8 or
+// 16): lane l of 8 owns rows l and 15 - l, 17 entries, split over two lanes
+// where there are 16.
 template <int GL>
 struct BlockSlots {
-    static constexpr int kN = GL == 8 ? 17 : (GL == 16 ? 9 : 5);
+    static constexpr int kN = GL == 8 ? 17 : 9;
     int l, s0;
     __device__ __forceinline__ BlockSlots() {
         const int lane = threadIdx.x & (GL - 1);

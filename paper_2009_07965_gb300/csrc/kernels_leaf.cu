@@ -131,8 +131,8 @@ leaf_build_kernel(DevView v, int mp, int cz, int bytes) {
     const int tid = threadIdx.x - 32 * team, lane = tid & 31, warp = tid >> 5;
     const int leaf0 = (blockIdx.x * TM + team) * LPC;
     // the warp that inverts: warps of one index share a scheduler, so CTAs
-    // take turns (152 of them are dealt to the SMs at a time)
-    const int wsweep = NW == 1 ? 0 : (blockIdx.x / 152) % NW;
+    // take turns (as many as SMs are dealt at a time)
+    const int wsweep = NW == 1 ? 0 : (blockIdx.x / kRuleSMs) % NW;
     // this lane's block in the inversions: half hf of leaf lf
     const int q = lane / GL, lf = q >> 1, hf = q & 1, gl = lane & (GL - 1);
     const bool present = leaf0 + lf < v.nleaf;
@@ -765,15 +765,19 @@ template <int DIM, class T>
 cudaError_t build_dispatch(const DevView& v, int mp, int cz, cudaStream_t s) {
     // 2D leaves of up to 16 segments: one warp per two leaves (the FP64
     // instructions of the inversions serve four blocks: a quarter fewer per
-    // leaf).  One leaf per warp while two would leave a last wave nearly empty
-    // (a wave of the former is 3648 leaves; 4096 leaves: 0.76 ms, two per warp
-    // 0.85; 24576: two per warp 5.2), and four warps to a leaf where not even
-    // that fills the schedulers (16 leaves: 0.20 ms; one warp per leaf in the
-    // elimination by cells before 0.62).  More segments: four warps per leaf
-    // share the products.
+    // leaf), one leaf per warp for fewer, and four warps to a leaf where not even
+    // that fills the schedulers.  Waves are 1824 leaves one per warp, 3648 two
+    // per warp; 16 x 16 leaves, ms four warps / one / two leaves per warp: 160
+    // 0.201 / 0.199 / 0.351, 304 0.204 / 0.199 / 0.354, 800 0.417 / 0.245 / 0.355,
+    // 1824 0.71 / 0.307 / 0.439, 2432 0.96 / 0.477 / 0.443, 3648 1.46 / 0.603 /
+    // 0.542, 4096 1.63 / 0.750 / 0.844, 4864 1.93 / 0.820 / 0.851, 6000 2.38 / 1.033 /
+    // 0.951, 12000 4.74 / 1.96 / 1.85.  The line lies past the one-per-warp
+    // form's third wave; between its first and its second the other form would
+    // be up to 10% shorter.  More segments: four warps per leaf share the
+    // products.
     if (DIM == 2 && mp <= 16) {
-        if (v.nleaf <= 152 * 2) return build_launch<2, T, 4, 1>(v, mp, cz, s);
-        if (v.nleaf <= 152 * 32) return build_launch<2, T, 1, 1, kTeams>(v, mp, cz, s);
+        if (v.nleaf <= kRuleSMs * 2) return build_launch<2, T, 4, 1>(v, mp, cz, s);
+        if (v.nleaf <= kRuleSMs * 32) return build_launch<2, T, 1, 1, kTeams>(v, mp, cz, s);
         return build_launch<2, T, 1, 2, kTeams>(v, mp, cz, s);
     }
     return build_launch<DIM, T, 4, 1>(v, mp, cz, s);

@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(kGemmThreads, 2) merge_rupdate_strip_kernel(De
 // 128 rows on tcgen05, one CTA per SM, three to five tiles behind a prologue that
 // nothing overlaps: X of 2g = 128 0.94 -> 0.67 ms, but X of 2g = 64 0.50 -> 0.88
 // and R 1.21 -> 1.44, box 128x128x64 as a whole 36.9 -> 37.2; not kept.)
-bool strips(int max_g2, long long ctas) { return max_g2 <= 2 * kChunkK && ctas >= 3 * 2 * 152; }
+bool strips(int max_g2, long long ctas) { return max_g2 <= 2 * kChunkK && ctas >= 3 * 2 * kRuleSMs; }
 
 template <int S>
 cudaError_t x_launch(const DevView& v, int first, int count, int max_g2, int max_m, cudaStream_t s) {

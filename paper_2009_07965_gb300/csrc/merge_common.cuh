@@ -79,10 +79,14 @@ __device__ __forceinline__ unsigned int ld_acquire_gpu(const unsigned int* p) {
 }
 // Grid-wide barrier of a cooperative launch: a monotonic arrival counter
 // (reset before the launch); round n ends when it reaches (n + 1) * grid.
-// Data written by other CTAs before a barrier is read after it with L2-only
-// loads (__ldcg).  Every wait is bounded (`limit` polls, about a second by
-// default); a CTA that gives up sets kStatusTimeout and the caller returns.
-
+// What a CTA wrote before the barrier is visible to the others after it, plain
+// loads included: its threads' writes are ordered before thread 0's fence and
+// arrival by the CTA barrier, thread 0 of the reader acquires the counter, and
+// its CTA barrier orders the reader's loads behind that.  (Kernels that read a
+// location both before and after a barrier through __ldcg do so to keep it out
+// of L1, not for correctness.)  Every wait is bounded (`limit` polls, about a
+// second by default); a CTA that gives up sets kStatusTimeout and the caller
+// returns.
 __device__ bool grid_barrier(unsigned int* counter, unsigned int& round, int* status, long long limit) {
     __shared__ int s_ok;
     __syncthreads();

@@ -154,7 +154,7 @@ void finish_merges(Plan& P);
 // 8 0.6 to 0.95 where 4 w + m < 44, and a few planes of few cells (10 x 4: 0.79,
 // 12 x 6: 0.91), but 1.25 to 1.5 below some 2400 leaves, where the chain of
 // cells is the longer one; 12 x 12 and 16 x 16 with one segment a side 0.90 and
-// 0.97 at 4096 leaves, 1.1 at 2304 (the planes' waves are 1824 leaves); as many
+// 0.97 at 4096 leaves, 1.1 at 2304 (the planes' waves are 12 leaves per SM); as many
 // segments as cells, or one plane, 1.05 to 1.7; more than 16 segments 0.5 to
 // 0.86 for w <= 2, else 0.95 to 5.8.
 bool banded_leaves(const Plan& P) {
@@ -168,7 +168,7 @@ bool banded_leaves(const Plan& P) {
     if (w == 1) return true;
     if (w > 4 && P.nleaf <= 2400) return false;
     if (h == 1 || (m >= n && w >= 4)) return m <= 4;
-    return 4 * w + m < 44 || (n < 64 && m <= 8) || (m <= 4 && P.nleaf > 2 * 1824);
+    return 4 * w + m < 44 || (n < 64 && m <= 8) || (m <= 4 && P.nleaf > 24 * kRuleSMs);
 }
 
 int make_plan(Plan& P) {

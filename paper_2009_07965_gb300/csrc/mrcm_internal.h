@@ -9,6 +9,9 @@ namespace mrcm {
 
 // Largest leaf side handled by the leaf kernels (cells).
 constexpr int kMaxLeafSide = 16;
+// SMs of the part that the rules on sizes were measured on (a threshold, not the
+// device's count, so that a rule takes the same form on every device).
+constexpr int kRuleSMs = 152;
 // Device status word bits (host maps them to MRCM_ERR_* codes).
 enum : int {
     kStatusBadK = 1,
