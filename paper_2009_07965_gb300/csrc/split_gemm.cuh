@@ -31,8 +31,8 @@
 // adds to the exponents: no rounding, and both rows are level in k.  (K
 // contrast 1e11, one-face segments, node maps against quadruple precision,
 // entries over the roots of their diagonals: without the powers 7.5e-15 to
-// 1.2e-14, with them and in FMA loops 1e-16 to 1.6e-15.  They cost 0.3 to 1%
-// of a build in FP64, 1 to 2% of a mixed one, whose cutting is the larger part.)
+// 1.2e-14, with them and in FMA loops 1e-16 to 1.6e-15.  They cost up to 0.6%
+// of an FP64 step and 1% of a mixed one, whose cutting is the larger part.)
 //
 // S = 4 (31 bits, 10 digit products) serves the FP32 merges of the mixed
 // form: more than an FP32 operand's 24 bits of the largest entry, sums
@@ -132,10 +132,10 @@ __device__ __forceinline__ int whole_exponent(double x) { return exponent_field(
 template <int S>
 __device__ __forceinline__ unsigned long long digit_bytes(double x, int d) {
     const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-    d = min(d, S == 8 ? 63 : 31);
-    const unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 42) | ((unsigned long long)lo << 10);
-    if (S == 8) return (m >> d) + 0x0080808080808080ull;
-    return (m >> (d + 32)) + 0x00808080ull;
+    const unsigned top = (hi & 0xfffffu) | 0x100000u;
+    if (S == 4) return (__funnelshift_l(lo, top, 10) >> min(d, 31)) + 0x00808080u;    // the upper 31 bits alone
+    const unsigned long long m = ((unsigned long long)top << 42) | ((unsigned long long)lo << 10);
+    return (m >> min(d, 63)) + 0x0080808080808080ull;
 }
 template <int S>
 __device__ __forceinline__ unsigned digit_bytes(float x, int d) {       // S = 4
@@ -275,11 +275,13 @@ __device__ __forceinline__ float pow2f(int e) {         // 2^e, kept within the 
 }
 __device__ __forceinline__ float combine_levels(const float (&n)[4], int ea, int eb) {
     const float v = fmaf(fmaf(fmaf(n[0], 256.f, n[1]), 256.f, n[2]), 256.f, n[3]);
-    // 2^(ea + eb - 2082) as two factors: either exponent may be far out of the
-    // FP32 range where their sum is not
-    const int e = max(ea + eb - 2082, 2 * kZeroExp), h = e >> 1;
-    const float f = v * pow2f(h) * pow2f(e - h);
-    return max(ea, eb) >= kNonFiniteExp ? __int_as_float(0x7fc00000) : f;
+    const int e = ea + eb - 2082;
+    if ((unsigned)(e + 126) <= 253u) return v * __int_as_float((e + 127) << 23);
+    // 2^e as two factors, so that v 2^e itself decides whether it leaves the range
+    // (a row of zeros: e far below); beyond that an infinity or NaN in a row
+    if (max(ea, eb) >= kNonFiniteExp) return __int_as_float(0x7fc00000);
+    const int h = max(e, 2 * kZeroExp) >> 1;
+    return v * pow2f(h) * pow2f(max(e, 2 * kZeroExp) - h);
 }
 // x as a double by integer operations (a conversion instruction holds the
 // FP64 pipe like an FP64 instruction); FP32 subnormals count as zero.
@@ -305,13 +307,7 @@ __device__ __forceinline__ void load_index(int (&ix)[kLaneK], const int* idx, in
     for (int i = 0; i < kLaneK; ++i) ix[i] = (ON && lane_k(i) < kn) ? idx[lane_k(i)] : 0;
 }
 
-// The powers of this lane's entries of the chunk from k0 on.
-template <class Scale>
-__device__ __forceinline__ void load_scale(int (&s)[kLaneK], Scale&& sc, int k0, int kn) {
-#pragma unroll
-    for (int i = 0; i < kLaneK; ++i) s[i] = lane_k(i) < kn ? sc(k0 + lane_k(i)) : 0;
-}
-// ... from the CTA's shared copy
+// The powers of this lane's entries of the chunk.
 __device__ __forceinline__ void load_scale(int (&s)[kLaneK], const int* sk) {
 #pragma unroll
     for (int i = 0; i < kLaneK; i += 2) {
@@ -337,13 +333,15 @@ __device__ __forceinline__ void split_product(SplitSmem<S>& sm, int K, const int
         {
             int ix[kLaneK], s[kLaneK];
             load_index<AG || BG>(ix, idx + k0, kn);
-            load_scale(s, sc, k0, kn);
+            const int power = threadIdx.x < kn ? sc(k0 + (int)threadIdx.x) : 0;
             // every row's entries in flight together
             T va[2][kLaneK], vb[kLaneK];
 #pragma unroll
             for (int p = 0; p < 2; ++p) load_row<AG>(va[p], pa[p] ? pa[p] + (AG ? 0 : k0) : nullptr, ix, kn);
             load_row<BG>(vb, pb ? pb + (BG ? 0 : k0) : nullptr, ix, kn);
-            if (k0) __syncthreads();                  // the previous chunk's digits are read
+            if (threadIdx.x < kChunkK) sm.sk[threadIdx.x] = power;
+            __syncthreads();                          // the previous chunk's digits are read
+            load_scale(s, sm.sk);
 #pragma unroll
             for (int p = 0; p < 2; ++p) stage_row<S, 1>(sm.A, sm.ea, row + p * kPassRows, kn, va[p], s);
             stage_row<S, -1>(sm.B, sm.eb, row, kn, vb, s);
