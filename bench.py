@@ -19,7 +19,9 @@ and the boundary values and the device->host copies of p, Fx, Fy inside
 the timed region.
 
 The roofline denominators are measured in the same run by the library's
-pipe probes (mrcm_probe_peak: FP64 FMA, FP64 MMA, FP32 FMA).
+pipe probes (mrcm_probe_peak): FP64 FMA, or, for the phases whose products run
+on the tensor cores, BF16 mma.sync over the 36 digit products of an FP64
+multiply-add.
 
 N > 1 (torchrun): every rank solves its own realisation (independent
 replicas, no collective on the data path); value = all ranks' cells / max
@@ -85,10 +87,29 @@ CPU_WINDOW = 256
 # dram__bytes_write.sum).  A family missing here reports traffic null.
 TRAFFIC_PER_LAUNCH = {
     ("square4096", "gj_sweep"): dict(bytes=20.9e6, source="ncu capture of one profiled step "
-                                     "(profiles/dram_traffic_square4096.md), mean over block_sweep_kernel's 6 launches"),
+                                     "(profiles/dram_traffic_square4096.md), mean over block_sweep_kernel's 6 launches "
+                                     "(the phase's other kernels not counted)"),
     ("square4096", "leaf_build"): dict(bytes=4168.1e6, source="ncu capture of one profiled step "
                                        "(profiles/dram_traffic_square4096.md)"),
 }
+
+
+# Phases whose products run as split products: one FP64 multiply-add is 36 digit
+# products on the FP16 tensor cores (mma.sync, same rate as BF16)
+SPLIT_PHASES = ("leaf_build", "gj_sweep", "merge_x", "merge_r")
+
+
+def phase_peak(peaks, phase):
+    """Roofline denominator of a phase: the measured rate, in FP64 flops, of the
+    pipe that its products run on, and where it comes from."""
+    if phase in SPLIT_PHASES:
+        return dict(peak=peaks["BF16"] / 36,
+                    peak_source="measured in this run: BF16 mma.sync probe (mrcm_probe_peak BF16) over 36 digit products "
+                                "per multiply-add, of measured; diagonal-block inverses and heights with few systems "
+                                "run on the FP64 pipe (DFMA probe in peaks_measured_tflops)",
+                    peak_nominal=None)
+    return dict(peak=peaks["DFMA"], peak_source="measured in this run: FP64 FMA probe (mrcm_probe_peak DFMA), of measured",
+                peak_nominal=FP64_NOMINAL_TFLOPS)
 
 
 def time_copies(stream, *pairs, reps=3):
@@ -649,13 +670,13 @@ def run_ours(args):
     # the dominant kernel family: the phase with the largest share of the step
     dom = max(mr.PHASES, key=lambda k: ph[k])
     achieved = pf[dom] / (ph[dom] / 1e3) / 1e12
-    peak = peaks["DFMA"]
+    peak = phase_peak(peaks, dom)
     model = {}
     if dom == "gj_sweep":
         mflops = mr.mrcm_query(solver.ctx, "MODEL_SWEEP_FLOPS")
         model = dict(achieved_model=mflops / (ph[dom] / 1e3) / 1e12,
                      model="(2/3) N^3 per blocked interface system (LU count)")
-        model["frac_model"] = model["achieved_model"] / peak
+        model["frac_model"] = model["achieved_model"] / peak["peak"]
     build_ms = sum(ph[k] for k in ("coef", "leaf_build", "merge_small", "gj_sweep", "merge_form", "merge_x",
                                    "merge_r", "root_factor"))
     model_build = mr.mrcm_query(solver.ctx, "MODEL_BUILD_FLOPS")
@@ -664,12 +685,12 @@ def run_ours(args):
     impl_build = sum(pf[k] for k in build_phases)
     basis = dict(ms=build_ms, model_gflop=model_build / 1e9,
                  model_tflops=model_build / (build_ms / 1e3) / 1e12,
-                 frac_model=model_build / (build_ms / 1e3) / 1e12 / peak,
+                 times_fp64_rate_model=model_build / (build_ms / 1e3) / 1e12 / peaks["DFMA"],
                  model="banded-Cholesky leaves + LU merges (MRCM_Q_MODEL_BUILD_FLOPS)",
                  # the implementation's own flops over the whole build against the
-                 # measured FP64 rate: how busy the FP64 pipe is across all phases
+                 # measured FP64 FMA rate (above 1: the products leave that pipe)
                  impl_gflop=impl_build / 1e9, impl_tflops=impl_build / (build_ms / 1e3) / 1e12,
-                 frac_impl=impl_build / (build_ms / 1e3) / 1e12 / peak)
+                 times_fp64_rate_impl=impl_build / (build_ms / 1e3) / 1e12 / peaks["DFMA"])
     # per tree height of the build: the launch groups in order
     heights, by_kernel = [], []
     for name, ms in groups:
@@ -702,16 +723,13 @@ def run_ours(args):
                     levels=mr.mrcm_query(solver.ctx, "LEVELS"),
                     l2="inputs larger than L2; L2 also flushed between timed steps (256 MiB write outside the events)",
                     parallelism=f"replicas x{world}"),
-        roofline=dict(bound="alu", achieved=achieved, peak=peak, unit="TFLOP/s",
-                      frac=achieved / peak,
+        roofline=dict(bound="alu", achieved=achieved, unit="TFLOP/s", frac=achieved / peak["peak"], **peak,
                       traffic=traffic["bytes"] if traffic else None,
                       traffic_unit="bytes per launch",
                       traffic_source=traffic["source"] if traffic else None,
                       kernel=mr.PHASE_KERNELS[dom], phase=dom, share=ph[dom] / (total_ms / args.steps),
                       flop_count="algorithmic flops of the implemented algorithm (mrcm_phase_flops)",
-                      peak_source=("measured in this run: FP64 FMA probe (mrcm_probe_peak DFMA), "
-                                   "of measured"),
-                      peak_nominal=FP64_NOMINAL_TFLOPS, **model),
+                      **model),
         peaks_measured_tflops=peaks,
         basis_build=basis,
         merge_ms_per_height=heights,
@@ -906,7 +924,7 @@ def run_ensemble(args):
     ph = {k: v / args.steps for k, v in phases.items()}
     dom = max(mr.PHASES, key=lambda k: ph[k])
     achieved = pf[dom] / (ph[dom] / 1e3) / 1e12
-    peak = peaks["DFMA"]
+    peak = phase_peak(peaks, dom)
     cpu = None
     if not args.no_cpu_baseline:
         cpu = time_ensemble_oracle(wl, probs)
@@ -917,11 +935,9 @@ def run_ensemble(args):
         config=dict(workload=wl["desc"], realisations=len(probs), cells=cells,
                     leaves=mr.mrcm_query(b.ctx, "LEAVES"), levels=mr.mrcm_query(b.ctx, "LEVELS"),
                     l2="inputs larger than L2; L2 also flushed between timed steps", parallelism="one context"),
-        roofline=dict(bound="alu", achieved=achieved, peak=peak, unit="TFLOP/s", frac=achieved / peak,
+        roofline=dict(bound="alu", achieved=achieved, unit="TFLOP/s", frac=achieved / peak["peak"], **peak,
                       traffic=None, kernel=mr.PHASE_KERNELS[dom], phase=dom,
-                      share=ph[dom] / (total_ms / args.steps),
-                      peak_source="measured in this run: FP64 FMA probe (mrcm_probe_peak DFMA), of measured",
-                      peak_nominal=FP64_NOMINAL_TFLOPS),
+                      share=ph[dom] / (total_ms / args.steps)),
         peaks_measured_tflops=peaks,
         autotuned_shapes=tuned,
         phases={k: dict(ms=ph[k], gflop=pf[k] / 1e9, tflops=(pf[k] / (ph[k] / 1e3) / 1e12) if ph[k] > 0 else None)
@@ -1041,7 +1057,7 @@ def run_box3d(args):
     ph = {k: v / args.steps for k, v in phases.items()}
     dom = max(mr.PHASES, key=lambda k: ph[k])
     achieved = pf[dom] / (ph[dom] / 1e3) / 1e12
-    peak = peaks["DFMA"]
+    peak = phase_peak(peaks, dom)
     plan = {w: mr.mrcm_query(sol.ctx, w.upper()) for w in ("leaves", "segments", "levels")}
     sol.close()
     del K_d, q_d, bc_d, outs_h
@@ -1097,11 +1113,9 @@ def run_box3d(args):
                     else wl["desc"].replace("256x256x64", "x".join(map(str, args.box_n))) + " (reduced box)",
                     cells=cells, **plan,
                     l2="inputs larger than L2; L2 also flushed between timed steps", parallelism="one context"),
-        roofline=dict(bound="alu", achieved=achieved, peak=peak, unit="TFLOP/s", frac=achieved / peak,
+        roofline=dict(bound="alu", achieved=achieved, unit="TFLOP/s", frac=achieved / peak["peak"], **peak,
                       traffic=None, kernel=mr.PHASE_KERNELS[dom], phase=dom,
-                      share=ph[dom] / (total_ms / args.steps),
-                      peak_source="measured in this run: FP64 FMA probe (mrcm_probe_peak DFMA), of measured",
-                      peak_nominal=FP64_NOMINAL_TFLOPS),
+                      share=ph[dom] / (total_ms / args.steps)),
         peaks_measured_tflops=peaks,
         autotuned_shapes=tuned,
         gflop_per_step=sum(pf.values()) / 1e9,
