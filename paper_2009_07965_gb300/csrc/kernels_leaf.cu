@@ -40,7 +40,7 @@
 // 0.47, box 256x256x64 34.9 -> 16.8; particular problems and pressures of
 // 1500x700 per pass 0.20 and 0.22 -> 0.11 and 0.12, of 256x256x64 3.3 and 3.0 ->
 // 2.1 and 1.1 (4096^2 1.21 and 1.08 -> 1.22 and 1.11: FP64 pipe either way).
-// Of the build's 9.4 ms, 6.0 are FP64 instructions (1690 per leaf, 64 cycles
+// Of the build's 9.3 ms, 6.0 are FP64 instructions (1690 per leaf, 64 cycles
 // each).
 //
 // Stored for the solve phase: P_k (nb x nb per plane, planes in order) and Z_k
@@ -332,12 +332,34 @@ leaf_build_kernel(DevView v, int mp, int cz, int bytes) {
 }
 
 // ---------------------------------------------------------------------------
-// Solve phase, one warp per leaf: lanes 0-15 the planes below the middle one
-// (lane = cell), lanes 16-31 those above, in step; the middle plane by both
-// (each half of the warp takes half of the products).  FP32 factors are widened
-// by integer operations: a conversion holds the FP64 pipe like the FP64
-// multiply-add it feeds.
+// Solve phase, 2 PL lanes per leaf (one warp: PL = 16; four blocks per warp:
+// PL = 4): lanes 0 .. PL - 1 the planes below the middle one (lane = cell), the
+// others those above, in step; the middle plane by both (each half takes half
+// of the products).  FP32 factors are widened by integer operations: a
+// conversion holds the FP64 pipe like the FP64 multiply-add it feeds.
+//
+// PL = 4 serves 3D blocks whose planes have at most four cells, where most lanes
+// of a warp per block idle (particular problems / pressures, ms a pass: 16384
+// blocks of 1^3 0.075 / 0.042 -> 0.020 / 0.018, 4096 of 2^3 0.049 / 0.035 -> 0.024 /
+// 0.025, 32768 of 2^3 0.293 / 0.180 -> 0.079 / 0.076; the kernels before the planes
+// 0.053 / 0.030, 0.054 / 0.038, 0.352 / 0.208).
 constexpr int kSolveWarps = 4;
+template <int PL>
+struct SolveLanes {
+    int sg, gl, h, l;             // leaf of the warp, lane of the leaf, half, cell of the plane
+    int leaf;
+    bool on;                      // (past the last leaf the lanes follow it and store nothing)
+    __device__ __forceinline__ SolveLanes(int warp_leaves0, int n) {
+        const int lane = threadIdx.x & 31;
+        sg = lane / (2 * PL);
+        gl = lane % (2 * PL);
+        h = gl / PL;
+        l = gl % PL;
+        leaf = warp_leaves0 + sg;
+        on = leaf < n;
+        leaf = min(leaf, n - 1);
+    }
+};
 
 // Right-hand side of the particular problem at one cell (Eqs. addu/addp):
 // the source plus Dirichlet and Neumann data of its domain-boundary faces.
@@ -370,36 +392,35 @@ __device__ __forceinline__ double particular_rhs(const DevView& v, int leaf, con
 }
 
 // Column l of the stored P of plane k (P is symmetric: entry j is P(l, j)).
-template <class TS>
-__device__ __forceinline__ void load_p(TS (&p)[kPlane], const TS* Lg, int nb, int k, int l, bool on) {
+template <int PL, class TS>
+__device__ __forceinline__ void load_p(TS (&p)[PL], const TS* Lg, int nb, int k, int l, bool on) {
     const TS* c = Lg + (long long)k * nb * nb + l;
 #pragma unroll
-    for (int j = 0; j < kPlane; ++j) p[j] = (on && l < nb && j < nb) ? c[j * nb] : (TS)0;
+    for (int j = 0; j < PL; ++j) p[j] = (on && l < nb && j < nb) ? c[j * nb] : (TS)0;
 }
 // sum_j p[j] y[j], and column l of plane k in p's place: each entry is loaded
 // as soon as the one before it is used, a plane ahead of its own use.  One
 // chain: its latency (75 cycles) is little above what an FP64 instruction
 // holds the pipe for, and partial sums would only add to it.
-template <class TS>
-__device__ __forceinline__ double row_product_next(TS (&p)[kPlane], const double* y, const TS* Lg, int nb, int k, int l,
+template <int PL, class TS>
+__device__ __forceinline__ double row_product_next(TS (&p)[PL], const double* y, const TS* Lg, int nb, int k, int l,
                                                    bool on) {
     const TS* c = Lg + (long long)k * nb * nb + l;
     const int n = on && l < nb ? nb : 0;
     double a = 0.0;
 #pragma unroll
-    for (int j = 0; j < kPlane; ++j) {
+    for (int j = 0; j < PL; ++j) {
         a = fma(widen(p[j]), y[j], a);
         p[j] = j < n ? c[j * nb] : (TS)0;
     }
     return a;
 }
-// the half of the product over j in [8 part, 8 part + 8)
-template <class TS>
-__device__ __forceinline__ double half_product(const TS (&p)[kPlane], const double* y, int part) {
+// the half of the product over j in [PL / 2 part, PL / 2 (part + 1))
+template <int PL, class TS>
+__device__ __forceinline__ double half_product(const TS (&p)[PL], const double* y, int part) {
     double a = 0.0;
 #pragma unroll
-    for (int j = 0; j < kPlane / 2; ++j)
-        a = fma(widen(part ? p[j + kPlane / 2] : p[j]), y[j + part * (kPlane / 2)], a);
+    for (int j = 0; j < PL / 2; ++j) a = fma(widen(part ? p[j + PL / 2] : p[j]), y[j + part * (PL / 2)], a);
     return a;
 }
 
@@ -420,30 +441,38 @@ __device__ __forceinline__ double reduce_columns8(double (&x)[8], int l) {
 
 // y_k (into leafzb), w_k = P_k y_k and rbar = sum_k Z_k^T w_k.  SMALL: at most
 // 8 columns meet a plane off the middle one and m <= 16 (partial sums in
-// registers); otherwise they go through shared memory (acc: (2 cz + mp) rows
-// of 17 doubles per warp).  TS: storage type of the factors (float in the
+// registers; PL = 16 only); otherwise they go through shared memory (acc: (2 cz +
+// mp) rows of PL + 1 doubles per leaf).  TS: storage type of the factors (float in the
 // mixed form's FP32 leaves); the arithmetic is FP64.
-template <int DIM, class TS, bool SMALL>
+template <int DIM, class TS, bool SMALL, int PL>
 __global__ void __launch_bounds__(32 * kSolveWarps)
 leaf_particular_kernel(DevView v, const double* __restrict__ q, const double* __restrict__ bc_val, bool with_sadj,
                        int mp, int cz) {
-    __shared__ double ysh[kSolveWarps][2][kPlane];
+    static_assert(!SMALL || PL == 16, "partial sums in registers over 16 lanes");
+    __shared__ double ysh_all[kSolveWarps][32];
     extern __shared__ __align__(16) double acc_raw[];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, h = lane >> 4, l = lane & 15;
-    const int leaf = blockIdx.x * kSolveWarps + warp;
-    if (leaf >= v.nleaf) return;                      // uniform over the warp
+    constexpr int kLeaves = 16 / PL;                  // leaves per warp
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int first = (blockIdx.x * kSolveWarps + warp) * kLeaves;
+    if (first >= v.nleaf) return;                     // uniform over the warp
+    const SolveLanes<PL> q4(first, v.nleaf);
+    const int h = q4.h, l = q4.l, leaf = q4.leaf;
+    double* ysh = ysh_all[warp] + (2 * q4.sg + h) * PL;   // y of the lane's plane
     const LeafGeo g = leaf_geo<DIM>(v, leaf);
-    const int nb = g.nb, hp = g.halfplanes(h), steps = max(g.halfplanes(0), g.halfplanes(1));
+    const int nb = g.nb, hp = g.halfplanes(h);
+    int steps = max(g.halfplanes(0), g.halfplanes(1));
+    if (kLeaves > 1) steps = __reduce_max_sync(0xffffffffu, steps);
     const TS* Lg = leaf_L<TS>(v) + g.L_off;
     const TS* Zg = leaf_Z<TS>(v) + g.Z_off;
     double* zb = v.leafzb + g.zb_off;
-    double (*acc)[kPlane + 1] = reinterpret_cast<double (*)[kPlane + 1]>(acc_raw) + (size_t)warp * (2 * cz + mp);
+    double (*acc)[PL + 1] =
+        reinterpret_cast<double (*)[PL + 1]>(acc_raw) + (size_t)(warp * kLeaves + q4.sg) * (2 * cz + mp);
     double part[8];
 #pragma unroll
     for (int p = 0; p < 8; ++p) part[p] = 0.0;
     if constexpr (!SMALL)
         for (int p = 0; p < cz; ++p) acc[h * cz + p][l] = 0.0;
-    TS p[kPlane];
+    TS p[PL];
     double w = 0.0, yn = 0.0, tn = 0.0;
     // right-hand side and coupling to the plane before, a plane ahead
     auto ahead = [&](int j) {
@@ -459,17 +488,17 @@ leaf_particular_kernel(DevView v, const double* __restrict__ q, const double* __
         const bool act = j < hp && l < nb;
         const int k = h ? g.H - 1 - j : j;
         const double y = act ? (j > 0 ? fma(tn, w, yn) : yn) : 0.0;
-        if (act) zb[k * nb + l] = y;
+        if (act && q4.on) zb[k * nb + l] = y;
         const int cc = j < hp ? g.cols(h, k) : 0;
         const TS* Zk = Zg + g.zoff(h, k);
         TS z[8];
         if (SMALL)
 #pragma unroll
             for (int c = 0; c < 8; ++c) z[c] = act && c < cc ? Zk[c * nb + l] : (TS)0;
-        ysh[warp][h][l] = y;
+        ysh[l] = y;
         __syncwarp();
         ahead(j + 1);
-        const double wn = row_product_next(p, ysh[warp][h], Lg, nb, h ? k - 1 : k + 1, l, j + 1 < hp);
+        const double wn = row_product_next(p, ysh, Lg, nb, h ? k - 1 : k + 1, l, j + 1 < hp);
         if (act) w = wn;
         if (SMALL) {
 #pragma unroll
@@ -484,7 +513,7 @@ leaf_particular_kernel(DevView v, const double* __restrict__ q, const double* __
     // the middle plane
     {
         load_p(p, Lg, nb, g.M, l, true);
-        const double other = __shfl_xor_sync(0xffffffffu, w, 16);
+        const double other = __shfl_xor_sync(0xffffffffu, w, PL);
         const double wt = h ? other : w, wb = h ? w : other;       // (0 for a half without planes)
         double y = 0.0;
         if (l < nb) {
@@ -492,21 +521,21 @@ leaf_particular_kernel(DevView v, const double* __restrict__ q, const double* __
             y = particular_rhs<DIM>(v, leaf, f, q, bc_val);
             if (g.halfplanes(0) > 0) y = fma(f.down(), wt, y);
             if (g.halfplanes(1) > 0) y = fma(f.up(), wb, y);
-            if (h == 0) zb[g.M * nb + l] = y;
+            if (h == 0 && q4.on) zb[g.M * nb + l] = y;
         }
-        ysh[warp][h][l] = y;
+        ysh[l] = y;
         __syncwarp();
-        w = half_product(p, ysh[warp][h], h);
-        w += __shfl_xor_sync(0xffffffffu, w, 16);
+        w = half_product(p, ysh, h);
+        w += __shfl_xor_sync(0xffffffffu, w, PL);
     }
     const TS* Zm = Zg + g.zoff(0, g.M);
     double* rb = v.rbar + g.r_off;
     auto store = [&](int t, double x) {
         // a right-hand side sigma on this segment's interface row,
         // F - D (lambda_other - lambda_own) = sigma, acts as rbar - sigma
-        rb[t] = with_sadj ? x - v.sadj[g.r_off + t] : x;
+        if (q4.on) rb[t] = with_sadj ? x - v.sadj[g.r_off + t] : x;
     };
-    if (SMALL) {
+    if constexpr (SMALL) {
         // columns 8 h + c of the middle plane
         double zm[8];
 #pragma unroll
@@ -514,7 +543,7 @@ leaf_particular_kernel(DevView v, const double* __restrict__ q, const double* __
             const int t = 8 * h + c;
             zm[c] = l < nb && t < g.m ? widen(Zm[t * nb + l]) * w : 0.0;
         }
-        double* rs = &ysh[warp][0][0];                             // rbar by segment (m <= 16)
+        double* rs = ysh_all[warp];                                // rbar by segment (m <= 16)
         const double r = reduce_columns8(zm, l);
         __syncwarp();
         if (!(l & 1) && 8 * h + (l >> 1) < g.m) rs[8 * h + (l >> 1)] = r;
@@ -529,12 +558,12 @@ leaf_particular_kernel(DevView v, const double* __restrict__ q, const double* __
     }
     for (int t = h; t < g.m; t += 2) acc[2 * cz + t][l] = l < nb ? widen(Zm[t * nb + l]) * w : 0.0;
     __syncwarp();
-    // each row summed by one lane (over the 16 cells), then the halves' rows
+    // each row summed by one lane (over the cells), then the halves' rows
     // added to their segments
-    for (int p = lane; p < 2 * cz + g.m; p += 32) {
+    for (int p = q4.gl; p < 2 * cz + g.m; p += 2 * PL) {
         double s0 = 0.0, s1 = 0.0;
 #pragma unroll
-        for (int c = 0; c < kPlane; c += 2) {
+        for (int c = 0; c < PL; c += 2) {
             s0 += acc[p][c];
             s1 += acc[p][c + 1];
         }
@@ -542,21 +571,23 @@ leaf_particular_kernel(DevView v, const double* __restrict__ q, const double* __
     }
     __syncwarp();
     for (int s = 0; s < 2; ++s) {
-        for (int p = lane; p < g.ncols(s); p += 32) acc[2 * cz + g.segment(s, p)][0] += acc[s * cz + p][0];
+        for (int p = q4.gl; p < g.ncols(s); p += 2 * PL) acc[2 * cz + g.segment(s, p)][0] += acc[s * cz + p][0];
         __syncwarp();
     }
-    for (int t = lane; t < g.m; t += 32) store(t, acc[2 * cz + t][0]);
+    for (int t = q4.gl; t < g.m; t += 2 * PL) store(t, acc[2 * cz + t][0]);
 }
 
 // x = A^-1 (A-elimination's right-hand sides), from the middle plane outwards;
 // rhs(h, k, l, Zk, cc): y_k + Z_k lambda at cell l (h < 0: the middle plane,
-// where each half warp returns its share), out(k, l, x).
-template <int DIM, class TS, class Rhs, class Out>
-__device__ __forceinline__ void solve_outward(const DevView& v, int leaf, const LeafGeo& g, const TS* Lg,
-                                              double (*ysh)[kPlane], int lane, Rhs&& rhs, Out&& out) {
-    const int h = lane >> 4, l = lane & 15, nb = g.nb, hp = g.halfplanes(h);
-    const int steps = max(g.halfplanes(0), g.halfplanes(1));
-    TS p[kPlane];
+// where each half of the lanes returns its share), out(k, l, x); ysh: PL doubles
+// of the lane's leaf and half.
+template <int DIM, int PL, class TS, class Rhs, class Out>
+__device__ __forceinline__ void solve_outward(const DevView& v, const SolveLanes<PL>& q4, const LeafGeo& g,
+                                              const TS* Lg, double* ysh, Rhs&& rhs, Out&& out) {
+    const int h = q4.h, l = q4.l, nb = g.nb, hp = g.halfplanes(h), leaf = q4.leaf;
+    int steps = max(g.halfplanes(0), g.halfplanes(1));
+    if (PL < 16) steps = __reduce_max_sync(0xffffffffu, steps);
+    TS p[PL];
     double x, tn = 0.0;
     auto ahead = [&](int d) {                                      // coupling to the plane before, a plane ahead
         if (d > hp || l >= nb) return;
@@ -565,55 +596,57 @@ __device__ __forceinline__ void solve_outward(const DevView& v, int leaf, const 
     };
     ahead(1);
     {
-        TS pm[kPlane];
+        TS pm[PL];
         load_p(pm, Lg, nb, g.M, l, true);
         load_p(p, Lg, nb, h ? g.M + 1 : g.M - 1, l, hp > 0);
         double y = rhs(-1, g.M, l);
-        y += __shfl_xor_sync(0xffffffffu, y, 16);
-        ysh[h][l] = y;
+        y += __shfl_xor_sync(0xffffffffu, y, PL);
+        ysh[l] = y;
         __syncwarp();
-        x = half_product(pm, ysh[h], h);
-        x += __shfl_xor_sync(0xffffffffu, x, 16);
+        x = half_product(pm, ysh, h);
+        x += __shfl_xor_sync(0xffffffffu, x, PL);
         __syncwarp();
-        if (h == 0 && l < nb) out(g.M, l, x);
+        if (h == 0 && l < nb && q4.on) out(g.M, l, x);
     }
     double r = steps > 0 && hp > 0 ? rhs(h, h ? g.M + 1 : g.M - 1, l) : 0.0;
     for (int d = 1; d <= steps; ++d) {
         const bool act = d <= hp;
         const int k = h ? g.M + d : g.M - d;
-        ysh[h][l] = act && l < nb ? fma(tn, x, r) : 0.0;
+        ysh[l] = act && l < nb ? fma(tn, x, r) : 0.0;
         __syncwarp();
         ahead(d + 1);
-        const double xn = row_product_next(p, ysh[h], Lg, nb, h ? k + 1 : k - 1, l, d + 1 <= hp);
+        const double xn = row_product_next(p, ysh, Lg, nb, h ? k + 1 : k - 1, l, d + 1 <= hp);
         if (d + 1 <= hp) r = rhs(h, h ? k + 1 : k - 1, l);         // the next plane's
         if (act) x = xn;
-        if (act && l < nb) out(k, l, x);
+        if (act && l < nb && q4.on) out(k, l, x);
         __syncwarp();
     }
 }
 
 // Final pressures p = A^-1 (bbar + B lambda), written into the state (p_hi,
 // p_lo) or added to it in double-double (refinement corrections).
-template <int DIM, class TS>
+template <int DIM, class TS, int PL>
 __global__ void __launch_bounds__(32 * kSolveWarps) leaf_pressure_kernel(DevView v, bool accumulate, int mp, int cz) {
-    __shared__ double ysh[kSolveWarps][2][kPlane];
-    extern __shared__ __align__(16) double lam_raw[];              // per warp: lambda in the halves' orders
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int leaf = blockIdx.x * kSolveWarps + warp;
-    if (leaf >= v.nleaf) return;                                   // uniform over the warp
+    __shared__ double ysh[kSolveWarps][32];
+    extern __shared__ __align__(16) double lam_raw[];              // per leaf: lambda in the halves' orders
+    constexpr int kLeaves = 16 / PL;                               // leaves per warp
+    const int warp = threadIdx.x >> 5, first = (blockIdx.x * kSolveWarps + warp) * kLeaves;
+    if (first >= v.nleaf) return;                                  // uniform over the warp
+    const SolveLanes<PL> q4(first, v.nleaf);
+    const int leaf = q4.leaf;
     const LeafGeo g = leaf_geo<DIM>(v, leaf);
-    double* lam = lam_raw + (size_t)warp * (2 * cz + mp);
-    for (int t = lane; t < g.m; t += 32) lam[2 * cz + t] = v.lam[g.r_off + t];
+    double* lam = lam_raw + (size_t)(warp * kLeaves + q4.sg) * (2 * cz + mp);
+    for (int t = q4.gl; t < g.m; t += 2 * PL) lam[2 * cz + t] = v.lam[g.r_off + t];
     __syncwarp();
     for (int s = 0; s < 2; ++s)
-        for (int p = lane; p < g.ncols(s); p += 32) lam[s * cz + p] = lam[2 * cz + g.segment(s, p)];
+        for (int p = q4.gl; p < g.ncols(s); p += 2 * PL) lam[s * cz + p] = lam[2 * cz + g.segment(s, p)];
     __syncwarp();
     const TS* Zg = leaf_Z<TS>(v) + g.Z_off;
     const double* zb = v.leafzb + g.zb_off;
     const int nb = g.nb;
     auto rhs = [&](int h, int k, int l) -> double {
         const bool mid = h < 0;
-        const int half = lane >> 4, cc = mid ? g.m : g.cols(h, k), step = mid ? 2 : 1;
+        const int half = q4.h, cc = mid ? g.m : g.cols(h, k), step = mid ? 2 : 1;
         const TS* Zk = Zg + g.zoff(mid ? 0 : h, k) + l;
         const double* lm = lam + (mid ? 2 * cz : h * cz);
         if (l >= nb) return 0.0;
@@ -634,7 +667,8 @@ __global__ void __launch_bounds__(32 * kSolveWarps) leaf_pressure_kernel(DevView
             if (c + u * step < cc) a = fma(widen(z[u]), lm[c + u * step], a);
         return a;
     };
-    solve_outward<DIM, TS>(v, leaf, g, leaf_L<TS>(v) + g.L_off, ysh[warp], lane, rhs, [&](int k, int l, double x) {
+    double* ys = ysh[warp] + (2 * q4.sg + q4.h) * PL;
+    solve_outward<DIM, PL, TS>(v, q4, g, leaf_L<TS>(v) + g.L_off, ys, rhs, [&](int k, int l, double x) {
         long long c;
         if constexpr (DIM == 2) {
             const LeafDesc& L = v.leaves[leaf];
@@ -661,7 +695,7 @@ __global__ void __launch_bounds__(32 * kSolveWarps) leaf_pressure_kernel(DevView
 template <class TS>
 __global__ void __launch_bounds__(32 * kSolveWarps) leaf_fields_kernel(DevView v, const int* __restrict__ ids,
                                                                       int count, float* __restrict__ psi) {
-    __shared__ double ysh[kSolveWarps][2][kPlane];
+    __shared__ double ysh[kSolveWarps][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int item = blockIdx.x * kSolveWarps + warp;
     if (item >= count) return;                                     // uniform over the warp
@@ -671,6 +705,7 @@ __global__ void __launch_bounds__(32 * kSolveWarps) leaf_fields_kernel(DevView v
         return;
     }
     const LeafGeo g = leaf_geo<2>(v, id);
+    const SolveLanes<16> q4(id, v.nleaf);
     const TS* Zg = leaf_Z<TS>(v) + g.Z_off;
     const int nb = g.nb;
     for (int s = 0; s < g.m; ++s) {
@@ -683,7 +718,8 @@ __global__ void __launch_bounds__(32 * kSolveWarps) leaf_fields_kernel(DevView v
             if (h < 0) return lane < 16 ? widen(Zg[g.zoff(0, k) + s * nb + l]) : 0.0;
             return pos[h] >= 0 && pos[h] < g.cols(h, k) ? widen(Zg[g.zoff(h, k) + pos[h] * nb + l]) : 0.0;
         };
-        solve_outward<2, TS>(v, id, g, leaf_L<TS>(v) + g.L_off, ysh[warp], lane, rhs, [&](int k, int l, double x) {
+        double* ys = ysh[warp] + q4.h * 16;
+        solve_outward<2, 16, TS>(v, q4, g, leaf_L<TS>(v) + g.L_off, ys, rhs, [&](int k, int l, double x) {
             psi[((long long)item * 256 + k * nb + l) * 16 + s] = (float)x;
         });
     }
@@ -782,27 +818,44 @@ cudaError_t build_dispatch(const DevView& v, int mp, int cz, cudaStream_t s) {
     }
     return build_launch<DIM, T, 4, 1>(v, mp, cz, s);
 }
+template <int DIM, class TS, bool SMALL, int PL>
+cudaError_t particular_go(const DevView& v, const double* q, const double* bc_val, bool with_sadj, int mp, int cz,
+                          cudaStream_t s) {
+    constexpr int per = kSolveWarps * (16 / PL);
+    const int bytes = SMALL ? 0 : (int)sizeof(double) * per * (2 * cz + mp) * (PL + 1);
+    auto* kern = leaf_particular_kernel<DIM, TS, SMALL, PL>;
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e != cudaSuccess) return e;
+    kern<<<(v.nleaf + per - 1) / per, 32 * kSolveWarps, bytes, s>>>(v, q, bc_val, with_sadj, mp, cz);
+    return cudaGetLastError();
+}
+// Planes of at most four cells (3D): four blocks per warp, as long as their
+// partial sums fit in shared memory.
+bool narrow_planes(const DevView& v, int mp, int cz) {
+    return v.nb3 <= 4 && (size_t)kSolveWarps * 4 * (2 * cz + mp) * 5 * sizeof(double) <= 200 * 1024;
+}
 template <int DIM, class TS>
 cudaError_t particular_launch(const DevView& v, const double* q, const double* bc_val, bool with_sadj, int mp, int cz,
                               cudaStream_t s) {
-    const int grid = (v.nleaf + kSolveWarps - 1) / kSolveWarps;
-    if (cz <= 8 && mp <= 16) {
-        leaf_particular_kernel<DIM, TS, true><<<grid, 32 * kSolveWarps, 0, s>>>(v, q, bc_val, with_sadj, mp, cz);
-        return cudaGetLastError();
-    }
-    const int bytes = (int)sizeof(double) * kSolveWarps * (2 * cz + mp) * (kPlane + 1);
-    auto* kern = leaf_particular_kernel<DIM, TS, false>;
+    if (DIM == 3 && narrow_planes(v, mp, cz))
+        return particular_go<DIM, TS, false, DIM == 3 ? 4 : 16>(v, q, bc_val, with_sadj, mp, cz, s);
+    if (cz <= 8 && mp <= 16) return particular_go<DIM, TS, true, 16>(v, q, bc_val, with_sadj, mp, cz, s);
+    return particular_go<DIM, TS, false, 16>(v, q, bc_val, with_sadj, mp, cz, s);
+}
+template <int DIM, class TS, int PL>
+cudaError_t pressure_go(const DevView& v, bool accumulate, int mp, int cz, cudaStream_t s) {
+    constexpr int per = kSolveWarps * (16 / PL);
+    const int bytes = (int)sizeof(double) * per * (2 * cz + mp);
+    auto* kern = leaf_pressure_kernel<DIM, TS, PL>;
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     if (e != cudaSuccess) return e;
-    kern<<<grid, 32 * kSolveWarps, bytes, s>>>(v, q, bc_val, with_sadj, mp, cz);
+    kern<<<(v.nleaf + per - 1) / per, 32 * kSolveWarps, bytes, s>>>(v, accumulate, mp, cz);
     return cudaGetLastError();
 }
 template <int DIM, class TS>
 cudaError_t pressure_launch(const DevView& v, bool accumulate, int mp, int cz, cudaStream_t s) {
-    const int grid = (v.nleaf + kSolveWarps - 1) / kSolveWarps;
-    const int bytes = (int)sizeof(double) * kSolveWarps * (2 * cz + mp);
-    leaf_pressure_kernel<DIM, TS><<<grid, 32 * kSolveWarps, bytes, s>>>(v, accumulate, mp, cz);
-    return cudaGetLastError();
+    if (DIM == 3 && narrow_planes(v, mp, cz)) return pressure_go<DIM, TS, DIM == 3 ? 4 : 16>(v, accumulate, mp, cz, s);
+    return pressure_go<DIM, TS, 16>(v, accumulate, mp, cz, s);
 }
 
 }  // namespace

@@ -1127,6 +1127,8 @@ static int setup3_impl(mrcm_ctx* c, const mrcm_grid* g, const double* K_dev, con
     v.mixed = precision == MRCM_MIXED ? 1 : 0;
     v.leaf32 = 0;                  // 3D blocks are factored in FP64
     v.banded = 0;
+    v.nb3 = 0;
+    for (const LeafDesc3& B : P.leaves3) v.nb3 = std::max(v.nb3, B.w[0] * B.w[1]);
     v.res_dd = 0;                  // 3D refinement residuals in FP64
     c->precision = precision;
     c->refine_steps = v.mixed ? kMixedRefineDefault3D : 0;

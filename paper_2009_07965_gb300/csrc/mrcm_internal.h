@@ -149,6 +149,7 @@ struct DevView {
     float* leafL32;     // the same in FP32 (mixed precision: leaf work in FP32)
     float* leafZ32;
     int mixed;          // 1: the mixed form (the merges of FP32 levels in FP32)
+    int nb3;            // most cells of a block's x-y plane (3D)
     int banded;         // 1: leaves eliminated cell by cell (kernels_leaf_banded.cu; 2D)
     int leaf32;         // 1: leaf factors in FP32 (mixed form, mrcm_set_mixed_leaves)
     int res_dd;         // 1: refinement residuals in double-double, 0: in FP64 (mrcm_set_residual)
