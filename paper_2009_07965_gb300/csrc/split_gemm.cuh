@@ -49,9 +49,9 @@
 // unit u at u ^ (row % 8): the eight rows an ldmatrix reads and the four rows
 // a staging warp writes then lie in distinct banks.
 //
-// Measured (one GB300, all heights): 4096^2 X 14.46 -> 2.41 ms, R 12.65 -> 2.43
+// Measured (one GB300, all heights): 4096^2 X 14.46 -> 2.37 ms, R 12.65 -> 2.49
 // against FP64 FMA loops at 97 and 92% of the FP64 peak; box 128x128x64 X
-// 27.5 -> 4.8, R 23.6 -> 5.5.  Seven digits in four warps per CTA were as fast
+// 27.5 -> 4.7, R 23.6 -> 5.6.  Seven digits in four warps per CTA were as fast
 // (2.25 and 2.67 ms) and less exact: node maps against quadruple precision 2.1e-15
 // at alpha = 100 (now 1.9e-16, the FMA loops 2.4e-16), boxes against a dense
 // FP64 solution 6.3e-13 (now 2.6e-13, the FMA loops 2.7e-13).
